@@ -182,8 +182,9 @@ int64_t vptq_linear_workspace_bytes(const vptq_layer_desc *desc, int32_t B);
  * over the FP16-rounded weights by at most ~1e-3 of max|out|).
  *   x    [B][N] row-major, desc->x_dtype;  out [B][M] row-major, desc->out_dtype.
  * B <= 16 runs the split-K decode kernels; larger B runs the tensor-core path
- * (tcgen05) when the layer qualifies (v = 8, k1 > 8192, x bf16/fp16), otherwise the
- * decode kernels over groups of 16 tokens.  Calls on one stream are ordered; calls
+ * (tcgen05) when the layer qualifies (v = 6, 8 or 12, any codebook sizes, groups and outlier columns, scale and
+ * bias per input column), otherwise the decode kernels over groups of 16 tokens.  From 5 tokens on the paths
+ * "decode_l2_fma" and "decode_gl_fma" run the tensor-core kernel as well.  Calls on one stream are ordered; calls
  * on different streams must not share a workspace.
  * The tensor-core path splits the input dimension of some output tiles over CTAs.  With long shares the CTA
  * that holds a tile's last piece stores it and raises a flag, and the CTAs that hold the other pieces wait for
@@ -208,7 +209,7 @@ int vptq_linear(const vptq_layer_desc *desc, const void *x, int32_t B,
  *   descs, ptrs  host arrays of n_layers descriptors / pointer sets; all layers have the same N and
  *                x_dtype (else VPTQ_E_SHAPE); M, codebooks, scale/bias and out_dtype are per layer
  *   outs         host array of n_layers DEVICE pointers, outs[l] = [B][M_l] row-major
- * When every layer takes the same one of the decode paths "decode_l2_fma" (B <= 16), "decode_smem_fma"
+ * When every layer takes the same one of the decode paths "decode_l2_fma" (B <= 8), "decode_smem_fma"
  * or "decode_gl_fma" (B <= 4; for these two the layers must also share their format apart from M: v,
  * codebook sizes, outlier columns, groups, scale flag) and whole vector rows of the layers spread evenly
  * over the SMs, one kernel per token group serves all layers (no launch, prologue and ragged tail per

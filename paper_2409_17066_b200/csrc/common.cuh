@@ -126,6 +126,10 @@ __device__ __forceinline__ void store_out(void *out, long long i, float val, int
 // streaming multiprocessors of the current device, cached per device ordinal (device_info.cu)
 int device_sm_count();
 
+// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per kernel, device and size instead of at every launch
+// (device_info.cu)
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes);
+
 // limit, in clock cycles, of the bounded device-side waits: 0 = each kernel's default (about two seconds);
 // set by vptq_debug_set_wait_limit, for tests that let a wait run out (device_info.cu)
 unsigned long long debug_wait_limit();

@@ -2,6 +2,7 @@
 #include "common.cuh"
 
 #include <atomic>
+#include <mutex>
 #include <stdlib.h>
 #include <string.h>
 
@@ -31,6 +32,53 @@ int device_sm_count()
     if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) return 148;
     if (dev < kMaxDevices) g_sm_count[dev].store(v, std::memory_order_relaxed);
     return v;
+}
+
+// What has been allowed so far, per (kernel, device): a small open-addressed table that only ever grows and is read without
+// a lock (a slot's key is written last).  More kernels than slots fall back to setting the attribute at every launch.
+namespace {
+struct SmemSlot {
+    std::atomic<const void *> kernel{nullptr};
+    int dev;
+    std::atomic<size_t> bytes{0};
+};
+constexpr int kSmemSlots = 1024;
+SmemSlot g_smem[kSmemSlots];
+std::mutex g_smem_mutex;
+}
+
+cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes)
+{
+    if (bytes <= 48 * 1024) return cudaSuccess;           // what every kernel may use without asking
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const size_t h = ((size_t)kernel >> 4) * 31 + (size_t)dev;
+    for (int i = 0; i < kSmemSlots; i++) {
+        SmemSlot &s = g_smem[(h + i) % kSmemSlots];
+        const void *k = s.kernel.load(std::memory_order_acquire);
+        if (k == nullptr) break;
+        if (k == kernel && s.dev == dev) {
+            if (s.bytes.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
+            break;
+        }
+    }
+    std::lock_guard<std::mutex> lock(g_smem_mutex);
+    SmemSlot *slot = nullptr;
+    for (int i = 0; i < kSmemSlots && slot == nullptr; i++) {
+        SmemSlot &s = g_smem[(h + i) % kSmemSlots];
+        const void *k = s.kernel.load(std::memory_order_relaxed);
+        if (k == nullptr || (k == kernel && s.dev == dev)) slot = &s;
+    }
+    if (slot != nullptr && slot->kernel.load(std::memory_order_relaxed) == kernel && slot->bytes.load(std::memory_order_relaxed) >= bytes)
+        return cudaSuccess;                                // another thread was faster
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && slot != nullptr) {
+        slot->dev = dev;
+        slot->bytes.store(bytes, std::memory_order_release);
+        slot->kernel.store(kernel, std::memory_order_release);
+    }
+    return e;
 }
 
 bool pdl_enabled(const char *family)

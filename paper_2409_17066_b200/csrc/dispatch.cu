@@ -34,6 +34,14 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
     return PATH_GENERIC;
 }
 
+// 5 to 16 tokens of the families that read their tables out of L2 take at most four tokens per launch and gather every
+// centroid again for the next four; the batched kernel gathers it once whatever the batch (4096 x 4096 over the 1 MiB table:
+// 25 us at any batch up to 64, against 14 us per four tokens).
+static bool batched_decode(LinearPath path, const LayerView &L, int B)
+{
+    return (path == PATH_DECODE_L2_FMA || path == PATH_DECODE_GL_FMA) && B >= 5 && !L.deterministic && gemm_tcgen05_supported(L, B);
+}
+
 const char *linear_path_name(const LayerView &L, int B, int flags)
 {
     switch (choose_path(L, B, flags)) {
@@ -49,7 +57,9 @@ const char *linear_path_name(const LayerView &L, int B, int flags)
 
 long long linear_workspace_bytes(const LayerView &L, int B, int flags)
 {
-    switch (choose_path(L, B, flags)) {
+    const LinearPath path = choose_path(L, B, flags);
+    if (batched_decode(path, L, B)) return gemm_tcgen05_workspace_bytes(L, B);
+    switch (path) {
     case PATH_DECODE_SMEM_FMA: return 0;
     case PATH_DECODE_SMEM_MMA: return smem_mma_workspace_bytes(L, decode_group(B));
     case PATH_DECODE_L2_FMA: return l2_fma_workspace_bytes(L, decode_group(B));
@@ -64,7 +74,9 @@ int linear_launches(const LayerView &L, int B, int flags)
 {
     const int groups = (B + DECODE_MAX_B - 1) / DECODE_MAX_B;
     const int last = B - (groups - 1) * DECODE_MAX_B;
-    switch (choose_path(L, B, flags)) {
+    const LinearPath path = choose_path(L, B, flags);
+    if (batched_decode(path, L, B)) return gemm_tcgen05_launches(L, B);
+    switch (path) {
     case PATH_DECODE_SMEM_FMA:
         return (groups - 1) * smem_fma_launches(L, DECODE_MAX_B) + smem_fma_launches(L, last);
     case PATH_DECODE_SMEM_MMA: return groups * (smem_tc_supported(L, decode_group(B)) ? 2 : 1);      // pre-pass + main kernel
@@ -85,7 +97,7 @@ int linear_dispatch(const LayerView &L, int flags, const void *x, int B, void *o
     const LinearPath path = choose_path(L, B, flags);
     if (path == PATH_GENERIC) {
         e = launch_linear_generic(L, x, B, out, ws, st);
-    } else if (path == PATH_GEMM_TCGEN05) {
+    } else if (path == PATH_GEMM_TCGEN05 || batched_decode(path, L, B)) {
         e = launch_gemm_tcgen05(L, x, B, out, ws, st);
     } else if (path == PATH_DECODE_BUCKET_FMA) {
         const void *img = L.prepared;
@@ -128,6 +140,10 @@ LinearPath fused_path(const LayerView *Ls, const int *flags, int n, int B)
         }
         return (n <= MAX_FUSED && ctas <= device_sm_count()) ? path : PATH_GENERIC;
     }
+    // The layers one by one through the batched kernel are faster than several fused launches: past 8 tokens with the 1 MiB
+    // table (q+k+v+o of 4096 x 4096 at 9 tokens 133 -> 87 us; 8 tokens 82 fused), always with group-wise tables (v = 12
+    // gate+up+down of a 7B layer at 8 tokens 580 -> 164 us)
+    if (batched_decode(path, Ls[0], B) && (B > 8 || path == PATH_DECODE_GL_FMA)) return PATH_GENERIC;
     if (path == PATH_DECODE_L2_FMA && l2_fma_fused_supported(Ls, n, B)) return path;
     if (path == PATH_DECODE_SMEM_FMA && smem_fma_fused_supported(Ls, n, B)) return path;
     if (path == PATH_DECODE_GL_FMA && gl_fma_fused_supported(Ls, n, B)) return path;

@@ -2,40 +2,43 @@
 // operand is dequantised on the fly into shared memory (the FP16 weight matrix never exists in
 // global memory; App. D.2 describes the paper's two-phase scheme that this replaces).
 //
-//   D[m][t] (TMEM, FP32, 128 lanes x 512 columns) += A[m][k] * B[t][k]
-//   A = W tile, 128 output rows x 32 input columns, written by producer warps: one 16-byte
-//       centroid (8 consecutive output rows of one input column) = C1[i1] + C2[i2] per store,
-//       in the MN-major 128-byte-swizzled layout tcgen05.mma reads;
-//   B = x*s tile (FP16, scale folded into the activations by a pre-pass), 512 tokens x 32
-//       columns, K-major with the 64-byte swizzle.  The pre-pass writes the activations as the
-//       shared-memory image of these tiles ([256-token half][k block] -> 16 KB, swizzle applied),
-//       so a tile half arrives by one linear bulk copy of whole 128-byte lines (a tiled TMA load of
-//       64-byte rows asks L2 for twice as many pieces);
-//   tcgen05.mma.cta_group::1.kind::f16, M = 128, N = 256 (two per token tile), K = 16.
+//   D[m][t] (TMEM, FP32, 128 lanes x up to 512 columns) += A[m][k] * B[t][k]
+//   A = W tile, NV whole vector rows (16 x 8, 20 x 6 or 10 x 12 output rows) x KS input columns, written by producer
+//       warps from C1[i1] + C2[i2]:
+//         v = 8:      KS = 32, one 16-byte store per centroid in the MN-major 128-byte-swizzled layout;
+//         v = 6, 12:  KS = 64, a lane takes 8 columns of a vector row, turns them into rows in registers (one byte
+//                     permute per pair) and stores 16 bytes per output row in the K-major 128-byte-swizzled layout: the
+//                     MN-major form would need 4- or 8-byte stores at a time (12- and 24-byte vectors);
+//   B = x*s (FP16, scale folded into the activations by a pre-pass), the tile's tokens x 32 columns per ring element,
+//       K-major with the 64-byte swizzle.  The pre-pass writes the activations as the shared-memory image of these
+//       elements, so one arrives by one linear bulk copy of whole 128-byte lines;
+//   tcgen05.mma.cta_group::1.kind::f16, M = 128, N = the tile's tokens (16 .. 256, one or two per token tile), K = 16.
+// Columns: the main columns first, then the outlier columns (a few k blocks of their own, A written from C0).
+// Tables: a main codebook of at most 64 KB (16-byte rows) and a residual one of at most 16 KB sit in shared memory
+// (small ones as several skewed copies); larger or group-wise ones are read out of L2, rows of 12 and 24 bytes from a copy
+// with rows padded to 16 and 32 bytes that the pre-pass writes (one load instruction and one 32-byte sector per row).
 //
-// Warp roles (640 threads): warp 0 bulk loads of B; warp 1 TMEM allocation + MMA issue (one
-// thread); warps 2-11 dequant producers (a pair per k block: a1 unpack with the next visit's
-// indices already in flight, a3 main lookup from the L2-resident codebook, a4 residual lookup
-// from shared memory, add, store); warps 12-19 epilogue (tcgen05.ld -> + bias term -> shared
-// memory -> TMA store or reduce-add), two per TMEM lane quarter.  Twenty warps are five per
-// scheduler: the register budget per thread is the same from 17 to 20 warps.
-// A and B have rings of their own: A has a stage per producer pair and one to spare (the
-// producers' gathers need a few microseconds), B holds 32 KB per stage and is shallow.
-// What bounds the k loop is the SM's request path to L2 (about one request per clock): per k block
-// 512 centroid reads and 256 lines of activations.  Two ways of sharing the activation tiles in a
-// CTA pair were measured and dropped: tcgen05 cta_group::2 (each CTA loads half of the tokens; the
-// pair advances at the pace of its slower half: 103 us against 88 us on the 14336 x 4096 layer at
-// 512 tokens) and forwarding the own half into the partner's shared memory (the forwarded bytes
-// load the same outgoing path: 117 us).
-// Persistent grid, one CTA per SM.  The work is the list of (tile, k block) units, tile =
-// (token tile, 128-row tile); with an FP32 output every CTA takes an equal, contiguous share of
-// the units, whatever tile they fall in, so all SMs stay busy; other output types are dealt out in
-// whole tiles.  When a share is long (FLAG_ORDER_MIN_SHARE k blocks or more) the pieces of a split
-// tile meet in the output without a zero-fill: the piece that holds the tile's last k blocks is the
-// first thing its CTA works on, so it finishes early; it stores and then raises the tile's flag in
-// the workspace; the other pieces (the last thing their CTAs work on) wait for the flag (a bounded
-// wait that is normally over before it starts) and reduce-add.  With short shares all pieces end
-// together, so there the pre-pass clears the output and every piece reduce-adds.
+// Warp roles: warp 0 bulk loads of B; warp 1 TMEM allocation + MMA issue (one thread); warps 4-19 the dequant producers in
+// GROUPS groups, a k block each in turn (the next visit's packed indices in flight); warps 20-27 the epilogue
+// (tcgen05.ld -> + bias term -> output), two per TMEM lane quarter.
+// What bounds the k loop is the SM's shared-memory/L1 data pipe (128 bytes per clock), which everything passes: per 32
+// columns at 512 tokens the MMAs read 48 KB (384 clocks) and the bulk copies write 32 KB (256), the producers' stores take 64
+// and 512 gathers out of L2 a wavefront each (512) plus the residual reads: about 1280 of the 1070-1330 clocks measured
+// against 512 of the MMAs alone.  More producer warps (10, 12, 16), a converged or a single-lane issue loop, a scheduler
+// kept free for the MMA issuer: all the same.  CTA pairs that forward half of every activation tile into the partner's
+// shared memory were slower (117 us against 88 us on 14336 x 4096 at 512 tokens).
+//
+// Persistent grid, one CTA per SM.  The work is the list of (tile, k block) units, tile = (token tile, row tile); every
+// CTA takes an equal, contiguous share of the units, whatever tile they fall in (a deterministic call: whole tiles).
+// The pieces of a split tile meet
+//   - FP32 output with 16-byte rows, long shares (FLAG_ORDER_MIN_COLS columns): in the output, without a zero-fill: the
+//     piece that holds the tile's last k blocks is the first thing its CTA works on, so it finishes early; it stores and
+//     then raises the tile's flag in the workspace; the other pieces (the last thing their CTAs work on) wait for the flag
+//     (a bounded wait that is normally over before it starts) and reduce-add;
+//   - FP32 output, short shares or a call that shares the GPU: in the output, cleared by the pre-pass, every piece adds;
+//   - any other output: in an FP32 scratch tile cleared by the pre-pass; every piece adds and counts itself in, and
+//     whichever warp finds its part complete converts and stores it (nobody waits).  Whole tiles per CTA, the form before,
+//     left 84 of 148 SMs idle on an 8192 x 8192 layer at 333 tokens and 140 on a 1024 x 8192 one.
 //
 // Every mbarrier wait is bounded: after about two seconds a waiter records VPTQ_E_TIMEOUT in
 // the status word of the workspace, raises a CTA-wide abort flag and every role leaves its
@@ -44,6 +47,7 @@
 
 #include "common.cuh"
 #include "gemm.cuh"
+#include "index_words.cuh"
 #include "tcgen05_ptx.cuh"
 
 namespace vptq {
@@ -52,45 +56,89 @@ namespace {
 
 using namespace tc;
 
-constexpr int TILE_M = 128;
-constexpr int TILE_K = 32;
-constexpr int TILE_N = 512;
-constexpr int MMA_N = 256;
-constexpr int A_STAGES = 6;                              // ring of dequantised weight tiles
-constexpr int A_STAGE_BYTES = TILE_M * TILE_K * 2;       // 8 KB
-constexpr int B_STAGES = 3;                              // ring of activation tiles
-constexpr int B_HALF_BYTES = MMA_N * TILE_K * 2;         // 256 tokens x 32 columns: 16 KB, one bulk copy
-constexpr int B_STAGE_BYTES = 2 * B_HALF_BYTES;          // 32 KB
-constexpr int PAIRS = 5;                                 // producer warp pairs; pair p fills k blocks p, p+PAIRS, ...
-constexpr int PRODUCER_WARPS = 2 * PAIRS;
+constexpr int MAX_TILE_N = 512;                          // tokens of a tile: all TMEM columns
+constexpr int IMG_COLS = 32;                             // columns of a B ring element
+constexpr int MAX_B_STAGES = 8;
 constexpr int EPI_WARPS = 8;
-constexpr int EPI_BUF_BYTES = 16 * 32 * 4;                // one staged piece of the output: 16 tokens x 32 rows, FP32
+constexpr int EPI_TOKENS = 32;                            // tokens an epilogue warp reads out of TMEM at a time
+constexpr int PIECE_TOKENS = 16;                          // ... and hands to the copy engine at a time
+constexpr int EPI_BUF_BYTES = PIECE_TOKENS * 32 * 4;      // one staged piece of the output: 16 tokens x 32 rows, FP32
 constexpr int EPI_STAGE_BYTES = EPI_WARPS * 2 * EPI_BUF_BYTES;   // two buffers per epilogue warp: 32 KB
-constexpr int CB2_REPLICAS = 4;                          // copies of a small residual table (16-byte skew)
-static_assert(A_STAGES >= PAIRS, "a producer pair needs a stage of its own");
-constexpr int GEMM_THREADS = 32 * (2 + PRODUCER_WARPS + EPI_WARPS);   // 640
-constexpr int A_SBO = 2048;   // bytes between consecutive 8-column groups of the A stage
-constexpr int A_LBO = 1024;   // bytes between the two 64-row blocks of the A stage
-constexpr int B_SBO = 512;    // bytes between consecutive 8-token groups of the B stage (8 x 64 B)
-
+constexpr int B_SBO = 512;    // bytes between consecutive 8-token groups of a B element (8 x 64 B)
 constexpr int WS_STATUS_BYTES = 256;
-constexpr int FLAG_ORDER_MIN_SHARE = 24;
+constexpr int DRAIN_COLS = 160;                          // columns of a k loop that take as long as draining 512 tokens of a tile
+constexpr int FLAG_ORDER_MIN_COLS = 768;                 // columns of a share from which split tiles meet by flag order
+constexpr int SMEM_LIMIT = 227 * 1024, SMEM_LIMIT_L1 = 195 * 1024;
+
+// per vector length: geometry of the A tile and the producers
+template <int V> struct Tile;
+template <> struct Tile<8> {
+    static constexpr int NV = 16, KS = 32, A_STAGES = 6, GROUP_WARPS = 2, GROUPS = 6;
+};
+template <> struct Tile<6> {
+    static constexpr int NV = 20, KS = 64, A_STAGES = 3, GROUP_WARPS = 5, GROUPS = 2;
+};
+template <> struct Tile<12> {
+    static constexpr int NV = 10, KS = 64, A_STAGES = 5, GROUP_WARPS = 3, GROUPS = 4;
+};
+template <int V> constexpr int a_stage_bytes() { return 128 * Tile<V>::KS * 2; }
+// Warps by role, in whole warpgroups (register shares move between warpgroups): 4 with the loader and the MMA issuer, 12
+// producers, 8 for the epilogue.  24 warps start with 80 registers a thread; the producers take 104, the others keep 56:
+// 12 x 104 + 12 x 56 = 24 x 80.  (16 producer warps with 96 registers fill the A ring no faster: the shared-memory pipe bounds.)
+constexpr int PRODUCER_WARP0 = 4, PRODUCER_WARPS = 12, EPI_WARP0 = PRODUCER_WARP0 + PRODUCER_WARPS;
+constexpr int GEMM_THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
+constexpr int REGS_PRODUCER = 104, REGS_OTHER = 56;
+
+// where a table's rows come from
+enum TableSource { TABLE_NONE = 0, TABLE_SHARED = 1, TABLE_GLOBAL = 2 };
+
+// token rows of a scratch tile: whole pieces
+__host__ __device__ __forceinline__ int scratch_rows(int tile_n) { return (tile_n + EPI_TOKENS - 1) / EPI_TOKENS * EPI_TOKENS; }
+
+// How the units (k blocks of all tiles, tile by tile) are cut into one contiguous share per CTA.  Draining a tile costs a CTA
+// about as much as `drain` k blocks, so the cuts are even on a line on which every tile is that much longer (a cut that
+// falls into a tile's extra length is moved to the tile's end).  A v = 12 decoder layer of a 7B model at 512 tokens: 676 -> 617
+// us.  whole_tiles: cuts only between tiles.
+struct Shares {
+    unsigned kb, len, workers, whole_tiles;      // k blocks of a tile; its length on the line, kb + drain
+    unsigned each, rest;                         // line (or tiles) per worker, and how many workers get one more
+    __host__ __device__ unsigned begin(unsigned w) const        // first unit of worker w (w = workers: the end)
+    {
+        const unsigned at = w * each + (w < rest ? w : rest);
+        if (whole_tiles) return at * kb;
+        const unsigned tile = at / len, off = at - tile * len;
+        return tile * kb + (off < kb ? off : kb);
+    }
+    __host__ __device__ unsigned worker_of(unsigned u) const    // the worker whose share holds unit u
+    {
+        const unsigned tile = u / kb, at = whole_tiles ? tile : tile * len + (u - tile * kb);
+        unsigned w = at / (each + 1);
+        while (w + 1 < workers && begin(w + 1) <= u) w++;
+        return w;
+    }
+};
 
 struct GemmParams {
     LayerView L;
     void *out;
     int B;
-    int tiles_m, tiles_t, kb_total;
-    int unit_gran;       // a CTA's share of the units is a multiple of this (1, or kb_total = whole tiles)
-    long long units;     // tiles_m * tiles_t * kb_total
-    int cb2_replicated;
-    int cb2_bytes;
+    int tiles_m, tiles_t, tile_n;   // row tiles, token tiles, tokens of a token tile (a multiple of 16)
+    int n0;                         // tokens of the first MMA of a k step; the second takes tile_n - n0
+    int kb_main, kb_total;          // k blocks of KS columns: main region, all
+    Shares shares;       // how the (tile, k block) units are dealt out to the CTAs
+    int b_stages;
+    int cb1_shift, cb2_shift;       // log2 of the copies of a table in shared memory
+    int cb1_bytes, cb2_bytes;
     int flag_order;      // split tiles: 1 = last piece stores and raises a flag, the others wait and add; 0 = all add
     int tma_out;         // FP32 output written by TMA store / reduce from shared memory (needs M % 4 == 0)
     int *status;         // workspace status word
-    const float *bterm;  // [B]
-    int *tile_flags;     // [tiles]: epilogue warps that have stored the piece with the tile's last k blocks
-    const uint8_t *xs;   // activation tile images, [ceil(B / 256)][kb_total][16 KB]
+    const float *bpart;  // [bias_parts][tiles_t * tile_n]: partial sums of x*b
+    int bias_parts;
+    int *tile_flags;     // [tiles][EPI_WARPS]: flag order: [tile][0] counts the epilogue warps that have stored the last
+                         // piece; scratch: arrivals per epilogue warp
+    float *scratch;      // [tiles][4][scratch_rows(tile_n)][32] FP32 sums of split tiles, or null
+    const uint8_t *xs;   // activation images, [tiles_t][kb_total * KS / 32][tile_n * 64 bytes]
+    const uint8_t *tab1, *tab2;     // tables read from global memory: rows of 16 (v <= 8) or 32 bytes
 };
 
 // ---- PTX wrappers ----------------------------------------------------------------------------
@@ -116,28 +164,18 @@ __device__ __forceinline__ bool flag_wait(const int *flag, int target, volatile 
     }
 }
 
-// kind::f16, FP16 x FP16 -> FP32, A MN-major, B K-major, M = 128, N = 256
-constexpr uint32_t IDESC = (1u << 4) | (0u << 7) | (0u << 10) | (1u << 15) | (0u << 16) |
-                           ((uint32_t)(MMA_N >> 3) << 17) | ((uint32_t)(TILE_M >> 4) << 24);
-
-__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t accumulate)
+// kind::f16, FP16 x FP16 -> FP32, B K-major, M = 128, N = n; A MN-major or K-major
+__device__ __forceinline__ uint32_t instr_desc(bool a_mn_major, int n)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(IDESC), "r"(accumulate) : "memory");
+    return (1u << 4) | ((a_mn_major ? 1u : 0u) << 15) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
-// The MMAs of one 32-column k block: two k16 steps x one or two 256-token halves, issued back to back.
-// `ad`/`bd` describe the k16 = 0 slice of the stage; the second slice lies 2 * A_SBO (A) and 32 bytes (B)
-// further, the second token half B_HALF_BYTES further (descriptor address units are 16 bytes).
-__device__ __forceinline__ void umma_kblock(uint32_t d_tmem, uint64_t ad, uint64_t bd, uint32_t accumulate, bool two_halves)
+// (descriptors as two words: only the low one, which holds the address, changes from MMA to MMA)
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t accumulate)
 {
-    const uint64_t ad1 = ad + (uint64_t)((2 * A_SBO) >> 4);
-    const uint64_t bd1 = bd + 2u;
-    const uint64_t bh = (uint64_t)(B_HALF_BYTES >> 4);
-    umma_f16(d_tmem, ad, bd, accumulate);
-    if (two_halves) umma_f16(d_tmem + MMA_N, ad, bd + bh, accumulate);
-    umma_f16(d_tmem, ad1, bd1, 1u);
-    if (two_halves) umma_f16(d_tmem + MMA_N, ad1, bd1 + bh, 1u);
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %6, 0;\n\t"
+                 "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
 {
@@ -148,16 +186,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32])
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
                    "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
                    "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -172,149 +200,243 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, uint32_t sr
                      ::"l"(map), "r"(src), "r"(x), "r"(y) : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
+// linear reduce-add of a staged piece into the scratch tile
+__device__ __forceinline__ void bulk_add(float *dst, uint32_t src)
+{
+    asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;"
+                 ::"l"(dst), "r"(src), "r"(EPI_BUF_BYTES) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void st_shared16(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+__device__ __forceinline__ uint32_t hadd2_bits(uint32_t a, uint32_t b)
+{
+    const __half2 r = __hadd2(*reinterpret_cast<const __half2 *>(&a), *reinterpret_cast<const __half2 *>(&b));
+    return *reinterpret_cast<const uint32_t *>(&r);
+}
 
-// ---- pre-pass: xs = fp16(x * s) written as tile images, bterm[t] = sum_n x[t][n] * b[n], status = 0, tile
-//      flags = 0; clears row t of an FP32 output in which all pieces of split tiles reduce-add (zero_out != nullptr).
-// Image of the tile half (256 tokens) x (k block of 32 columns): token r, 16-byte chunk q (8 columns) at
+// One row of a table of V-component vectors as V / 2 words; the rows of a table in shared memory take 16 bytes, of one in
+// global memory 16 (V <= 8) or 32.  No L1 allocation: the tensor core's operand reads share the L1 data path.
+template <int V>
+__device__ __forceinline__ void row_global(const uint8_t *tab, uint32_t e, uint32_t (&w)[V / 2])
+{
+    uint32_t r[8];
+    if (V <= 8) {
+        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "l"(tab + 16ull * e));
+    } else {
+        asm volatile("ld.global.nc.L1::no_allocate.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "l"(tab + 32ull * e));
+    }
+#pragma unroll
+    for (int i = 0; i < V / 2; i++) w[i] = r[i];
+}
+template <int V>
+__device__ __forceinline__ void row_shared(const uint4 *tab, uint32_t e, uint32_t (&w)[V / 2])
+{
+    const uint4 q = tab[e];
+    const uint32_t r[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+    for (int i = 0; i < V / 2; i++) w[i] = r[i < 4 ? i : 0];
+}
+
+// ---- pre-pass: xs = fp16(x * s) written as B images, partial sums of x * b per token, padded tables, and everything of the
+//      workspace (and output) that has to start at zero.
+// Image of (token tile, 32 columns): token row r of the tile, 16-byte chunk q (8 columns) at
 //      (r / 8) * 512 + (r % 8) * 64 + ((q ^ ((r % 8) / 2)) * 16: the K-major 64-byte-swizzled operand layout.
-// One block per token of the padded range; tokens >= B and columns >= N are written as zeros. ---------------
-constexpr int PRE_THREADS = 128;
+// Block (g, y): tokens 8g .. 8g+7 of the padded range, every gridDim.y-th run of 8 images; a warp takes four tokens x two
+// images (128 bytes of a row of x), a lane 8 columns of a token; tokens >= B and columns beyond a region are zeros. -------
+constexpr int PRE_THREADS = 256;
 
-__global__ void __launch_bounds__(PRE_THREADS)
-gemm_prepass_kernel(LayerView L, const void *__restrict__ x, int B, uint8_t *__restrict__ xs,
-                    float *__restrict__ bterm, int *status, int *__restrict__ tile_flags, int n_tiles,
-                    float *__restrict__ zero_out)
+struct PrepassParams {
+    LayerView L;
+    const void *x;
+    int B, tile_n;
+    int img_main, img_total;        // 32-column images: main region, all
+    uint8_t *xs;
+    float *bpart;
+    int *status;
+    int *tile_flags; int n_flags;
+    float *zero; long long n_zero;  // FP32 words to clear (a multiple of 4 unless the address is not 16-byte aligned)
+    uint8_t *pad1, *pad2;           // null, or where the tables go with their rows padded to pad_bytes
+    int pad_bytes;
+};
+
+// table [rows][v] -> rows of `pad` bytes (16 or 32), zero-filled
+__device__ __forceinline__ void pad_table(uint8_t *dst, const __half *src, long long rows, int v, int pad, long long first, long long step)
+{
+    for (long long i = first; i < rows; i += step) {
+        const uint32_t *p = reinterpret_cast<const uint32_t *>(src + i * v);     // even v: rows are 4-byte aligned
+        uint32_t w[8];
+#pragma unroll
+        for (int k = 0; k < 8; k++) w[k] = 2 * k < v ? __ldg(p + k) : 0u;
+        *reinterpret_cast<uint4 *>(dst + i * pad) = make_uint4(w[0], w[1], w[2], w[3]);
+        if (pad == 32) *reinterpret_cast<uint4 *>(dst + i * pad + 16) = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+}
+
+__global__ void __launch_bounds__(PRE_THREADS, 4)
+gemm_prepass_kernel(const __grid_constant__ PrepassParams P)
 {
     // the GEMM is launched as a programmatic dependent: its CTAs may become resident and run their set-up and
     // first centroid reads as soon as every block of this grid has started; whatever reads this kernel's
     // output waits for the whole grid (griddepcontrol.wait) first
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int t = blockIdx.x;
-    for (int i = t * PRE_THREADS + threadIdx.x; i < n_tiles; i += gridDim.x * PRE_THREADS) tile_flags[i] = 0;
-    const int kb_total = (L.N + TILE_K - 1) / TILE_K;
-    // where token t's 64 bytes of k block 0 start; the other k blocks follow at B_HALF_BYTES each
-    uint8_t *img_row = xs + (long long)(t / MMA_N) * kb_total * B_HALF_BYTES + ((t % MMA_N) >> 3) * B_SBO + (t & 7) * 64;
-    const int sw = (t & 7) >> 1;
-    if (t >= B) {
-        for (int q = threadIdx.x; q < 4 * kb_total; q += PRE_THREADS)
-            *reinterpret_cast<uint4 *>(img_row + (long long)(q >> 2) * B_HALF_BYTES + (((q & 3) ^ sw) << 4)) = make_uint4(0, 0, 0, 0);
-        return;
+    pdl_launch_dependents();
+    const LayerView &L = P.L;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long tid = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * PRE_THREADS + threadIdx.x;
+    const long long n_tid = (long long)gridDim.x * gridDim.y * PRE_THREADS;
+    pdl_wait();          // the activations may be the previous kernel's output, and that kernel may use this workspace
+    if (tid == 0) *P.status = 0;
+    for (long long i = tid; i < P.n_flags; i += n_tid) P.tile_flags[i] = 0;
+    if ((P.n_zero & 3) == 0) {
+        for (long long i = tid; i < (P.n_zero >> 2); i += n_tid) reinterpret_cast<float4 *>(P.zero)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+        for (long long i = tid; i < P.n_zero; i += n_tid) P.zero[i] = 0.f;
     }
-    if (t == 0 && threadIdx.x == 0) *status = 0;
-    if (zero_out != nullptr) {
-        float *row = zero_out + (long long)t * L.M;
-        if ((L.M & 3) == 0) {
-            float4 *r4 = reinterpret_cast<float4 *>(row);          // rows of M floats start 16-byte aligned
-            for (int i = threadIdx.x; i < (L.M >> 2); i += PRE_THREADS) r4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        } else {
-            for (int i = threadIdx.x; i < L.M; i += PRE_THREADS) row[i] = 0.f;
-        }
-    }
+    if (P.pad1) pad_table(P.pad1, L.c1, (long long)L.G * L.k1, L.v, P.pad_bytes, tid, n_tid);
+    if (P.pad2) pad_table(P.pad2, L.c2, (long long)L.G * L.k2, L.v, P.pad_bytes, tid, n_tid);
+
+    const int tok = 4 * (warp & 1) + (lane >> 3), q = lane & 3;
+    const int tg = blockIdx.x * 8 + tok;                 // token of the padded range
+    const int tile = tg / P.tile_n, row = tg - tile * P.tile_n;
+    const int t = tg;                                    // token tiles are consecutive runs of tile_n tokens
+    const bool live = t < P.B;
+    uint8_t *dst = P.xs + (long long)tile * P.img_total * (P.tile_n * 64) + (row >> 3) * B_SBO + (row & 7) * 64 + ((q ^ ((row & 7) >> 1)) << 4);
+    const uint16_t *xr = reinterpret_cast<const uint16_t *>(P.x) + (long long)(live ? t : 0) * L.N;
+    const bool wide = L.perm == nullptr && (L.N & 7) == 0 && (L.n_out & 7) == 0;
     float acc = 0.f;
-    if ((L.N & 7) == 0 && L.perm == nullptr) {
-        // 8 columns = one chunk per thread and step, 128-bit loads and stores; the loads of four steps are
-        // issued together (a thread with one load in flight at a time leaves the memory system idle)
-        constexpr int UNROLL = 4;
-        const uint4 one = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u), zero = make_uint4(0, 0, 0, 0);
-        for (int n0 = 8 * threadIdx.x; n0 < kb_total * TILE_K; n0 += UNROLL * 8 * PRE_THREADS) {
-            uint4 xq[UNROLL], sq[UNROLL], bq[UNROLL];
+    constexpr int UNROLL = 2;
+    const int stride = gridDim.y * 8;
+    for (int img0 = blockIdx.y * 8 + (warp >> 1) * 2 + ((lane >> 2) & 1); img0 < P.img_total; img0 += UNROLL * stride) {
+        uint4 xq[UNROLL], sq[UNROLL], bq[UNROLL];            // 8 activations as they are, 8 scales, 8 biases
 #pragma unroll
-            for (int u = 0; u < UNROLL; u++) {
-                const int n = n0 + u * 8 * PRE_THREADS;
-                xq[u] = zero; sq[u] = one; bq[u] = zero;
-                if (n < L.N) {
-                    xq[u] = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(x) + (long long)t * L.N + n));
+        for (int u = 0; u < UNROLL; u++) {
+            const int img = img0 + u * stride;
+            const bool main_cols = img < P.img_main;
+            const int c = (main_cols ? img : img - P.img_main) * IMG_COLS + q * 8;     // first column, counted in its region
+            const int n_cols = img >= P.img_total ? 0 : main_cols ? L.Nc : L.n_out, base = main_cols ? L.n_out : 0;
+            xq[u] = make_uint4(0, 0, 0, 0); sq[u] = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u); bq[u] = xq[u];
+            if (wide) {
+                if (c < n_cols) {                                // (regions are multiples of 8 columns here)
+                    if (live) xq[u] = __ldg(reinterpret_cast<const uint4 *>(xr + base + c));
                     if (L.has_scale) {
-                        sq[u] = __ldg(reinterpret_cast<const uint4 *>(L.scale + n));
-                        bq[u] = __ldg(reinterpret_cast<const uint4 *>(L.bias + n));
+                        sq[u] = __ldg(reinterpret_cast<const uint4 *>(L.scale + base + c));
+                        bq[u] = __ldg(reinterpret_cast<const uint4 *>(L.bias + base + c));
                     }
                 }
-            }
+            } else {
+                uint16_t xe[8], se[8], be[8];
 #pragma unroll
-            for (int u = 0; u < UNROLL; u++) {
-                const int n = n0 + u * 8 * PRE_THREADS;
-                if (n >= kb_total * TILE_K) break;
-                const uint32_t xw[4] = {xq[u].x, xq[u].y, xq[u].z, xq[u].w}, sc[4] = {sq[u].x, sq[u].y, sq[u].z, sq[u].w},
-                               bw[4] = {bq[u].x, bq[u].y, bq[u].z, bq[u].w};
-                uint32_t ow[4];
-#pragma unroll
-                for (int i = 0; i < 4; i++) {       // columns >= N were loaded as zeros: they store zeros and add nothing
-                    float2 xv;
-                    if (L.x_bf16) xv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xw[i]));
-                    else xv = __half22float2(*reinterpret_cast<const __half2 *>(&xw[i]));
-                    const float2 sv = __half22float2(*reinterpret_cast<const __half2 *>(&sc[i]));
-                    const float2 bv = __half22float2(*reinterpret_cast<const __half2 *>(&bw[i]));
-                    const __half2 o = __floats2half2_rn(xv.x * sv.x, xv.y * sv.y);
-                    ow[i] = *reinterpret_cast<const uint32_t *>(&o);
-                    acc += xv.x * bv.x + xv.y * bv.y;
+                for (int i = 0; i < 8; i++) {
+                    const int n = base + c + i;
+                    const bool in = c + i < n_cols;
+                    xe[i] = (in && live) ? __ldg(xr + in_col(L, n)) : (uint16_t)0;
+                    se[i] = (in && L.has_scale) ? __ldg(reinterpret_cast<const uint16_t *>(L.scale) + n) : (uint16_t)0x3C00;
+                    be[i] = (in && L.has_scale) ? __ldg(reinterpret_cast<const uint16_t *>(L.bias) + n) : (uint16_t)0;
                 }
-                const int q = n >> 3;
-                *reinterpret_cast<uint4 *>(img_row + (long long)(q >> 2) * B_HALF_BYTES + (((q & 3) ^ sw) << 4)) =
-                    make_uint4(ow[0], ow[1], ow[2], ow[3]);
+                auto pack = [](const uint16_t (&e)[8]) {
+                    return make_uint4(e[0] | ((uint32_t)e[1] << 16), e[2] | ((uint32_t)e[3] << 16), e[4] | ((uint32_t)e[5] << 16), e[6] | ((uint32_t)e[7] << 16));
+                };
+                xq[u] = pack(xe); sq[u] = pack(se); bq[u] = pack(be);
             }
         }
-    } else {
-        for (int n = threadIdx.x; n < kb_total * TILE_K; n += PRE_THREADS) {
-            float xv = 0.f, sc = 1.f, bi = 0.f;
-            if (n < L.N) {
-                xv = load_act(x, (long long)t * L.N + in_col(L, n), L.x_bf16);
-                if (L.has_scale) {
-                    sc = __half2float(__ldg(L.scale + n));
-                    bi = __half2float(__ldg(L.bias + n));
-                }
+#pragma unroll
+        for (int u = 0; u < UNROLL; u++) {
+            const int img = img0 + u * stride;
+            if (img >= P.img_total) break;
+            const uint32_t xw[4] = {xq[u].x, xq[u].y, xq[u].z, xq[u].w}, sw[4] = {sq[u].x, sq[u].y, sq[u].z, sq[u].w}, bw[4] = {bq[u].x, bq[u].y, bq[u].z, bq[u].w};
+            uint32_t o[4];
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                const float2 a = L.x_bf16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xw[i]))
+                                          : __half22float2(*reinterpret_cast<const __half2 *>(&xw[i]));
+                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&sw[i]));
+                const float2 h = __half22float2(*reinterpret_cast<const __half2 *>(&bw[i]));
+                const __half2 y = __floats2half2_rn(a.x * f.x, a.y * f.y);
+                o[i] = *reinterpret_cast<const uint32_t *>(&y);
+                acc += a.x * h.x + a.y * h.y;
             }
-            const int q = n >> 3;
-            *reinterpret_cast<__half *>(img_row + (long long)(q >> 2) * B_HALF_BYTES + (((q & 3) ^ sw) << 4) + (n & 7) * 2) =
-                __float2half_rn(xv * sc);
-            acc += xv * bi;
+            *reinterpret_cast<uint4 *>(dst + (long long)img * (P.tile_n * 64)) = make_uint4(o[0], o[1], o[2], o[3]);
         }
     }
-    __shared__ float red[PRE_THREADS / 32];
+    __shared__ float red[PRE_THREADS / 64][8];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((lane & 7) == 0) red[warp >> 1][tok] = acc;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 8) {
         float a = 0.f;
-        for (int w = 0; w < PRE_THREADS / 32; w++) a += red[w];
-        bterm[t] = a;
+        for (int w = 0; w < PRE_THREADS / 64; w++) a += red[w][threadIdx.x];
+        P.bpart[(long long)blockIdx.y * gridDim.x * 8 + blockIdx.x * 8 + threadIdx.x] = a;
     }
 }
 
-// ---- the GEMM ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, GemmParams P)
+// ---- outlier columns (Sec. 3.2.3): value of stored column n < n_out at output row m -------------------------------------
+__device__ __forceinline__ uint32_t outlier_bits(const LayerView &L, int m, int n)
 {
-    extern __shared__ uint8_t smem_raw[];
+    if (m >= L.M || n >= L.n_out) return 0u;
+    const int r = m / L.v0;
+    const int i = clamp_index(load_index(L.s0.ptr + (long long)r * L.s0.stride, n, L.s0.bits), L.k0);
+    return __ldg(reinterpret_cast<const unsigned short *>(L.c0) + (long long)i * L.v0 + (m - r * L.v0));
+}
+// four output rows m0 .. m0+3 (m0 a multiple of 4) of column n as two words, for v0 = 4
+__device__ __forceinline__ uint2 outlier_vector4(const LayerView &L, int m0, int n)
+{
+    if (m0 >= L.M || n >= L.n_out) return make_uint2(0u, 0u);
+    const int i = clamp_index(load_index(L.s0.ptr + (long long)(m0 >> 2) * L.s0.stride, n, L.s0.bits), L.k0);
+    return __ldg(reinterpret_cast<const uint2 *>(L.c0) + i);
+}
+
+// ---- the GEMM ------------------------------------------------------------------------------------
+template <int V, int T1, int T2>
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
+gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, const __grid_constant__ GemmParams P)
+{
+    constexpr bool MN = V == 8;                              // A layout
+    constexpr int KS = Tile<V>::KS, NV = Tile<V>::NV, A_STAGES = Tile<V>::A_STAGES, A_BYTES = a_stage_bytes<V>();
+    constexpr int GROUPS = Tile<V>::GROUPS, GROUP_WARPS = Tile<V>::GROUP_WARPS;
+    constexpr int SUBS = KS / IMG_COLS, TILE_M = NV * V, W2 = V / 2;
+    constexpr int A_SBO = MN ? 2048 : 1024, A_LBO = MN ? 1024 : 16;
+    static_assert(A_STAGES >= GROUPS, "a producer group needs a stage of its own");
+    static_assert(GROUPS * GROUP_WARPS <= PRODUCER_WARPS, "producer warps");
+    extern __shared__ __align__(1024) uint8_t sm[];          // swizzled operand stages need 1024-byte alignment
     const LayerView &L = P.L;
-    // carve shared memory; swizzled operand stages need 1024-byte alignment
-    const uint32_t raw = smem_addr(smem_raw);
-    const uint32_t base = (raw + 1023u) & ~1023u;
-    uint8_t *sm = smem_raw + (base - raw);
-    const uint32_t sA = base;                                   // A_STAGES x 8 KB
-    const uint32_t sB = sA + A_STAGES * A_STAGE_BYTES;          // B_STAGES x 32 KB
-    uint8_t *cb2_ptr = sm + A_STAGES * A_STAGE_BYTES + B_STAGES * B_STAGE_BYTES;
+    const uint32_t base = smem_addr(sm);
+    if (base & 1023u) {                                      // (every thread of the grid answers alike)
+        grid_dependency_wait();
+        if (threadIdx.x == 0) atomicExch(P.status, VPTQ_E_UNSUPPORTED);
+        return;
+    }
+    const int b_bytes = P.tile_n * 64, b_stages = P.b_stages;
+    const uint32_t sA = base;
+    const uint32_t sB = sA + A_STAGES * A_BYTES;
+    uint8_t *cb1_ptr = sm + A_STAGES * A_BYTES + b_stages * b_bytes;
+    uint8_t *cb2_ptr = cb1_ptr + P.cb1_bytes;
     const uint32_t sEpi = smem_addr(cb2_ptr + P.cb2_bytes);     // EPI_WARPS x 2 x 2 KB output staging
-    uint8_t *misc = cb2_ptr + P.cb2_bytes + EPI_STAGE_BYTES;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(misc);   // fullA[] emptyA[] fullB[] emptyB[] accum_full accum_empty
+    float *bias = reinterpret_cast<float *>(cb2_ptr + P.cb2_bytes + EPI_STAGE_BYTES);       // [tile_n] bias terms of the token tile
+    uint64_t *bars = reinterpret_cast<uint64_t *>(bias + MAX_TILE_N);   // fullA[] emptyA[] fullB[] emptyB[] accum_full accum_empty
     const uint32_t bar0 = smem_addr(bars);
     auto bar_fullA = [&](int s) { return bar0 + 8u * s; };
     auto bar_emptyA = [&](int s) { return bar0 + 8u * (A_STAGES + s); };
     auto bar_fullB = [&](int s) { return bar0 + 8u * (2 * A_STAGES + s); };
-    auto bar_emptyB = [&](int s) { return bar0 + 8u * (2 * A_STAGES + B_STAGES + s); };
-    constexpr int N_RING_BARS = 2 * A_STAGES + 2 * B_STAGES;
+    auto bar_emptyB = [&](int s) { return bar0 + 8u * (2 * A_STAGES + MAX_B_STAGES + s); };
+    constexpr int N_RING_BARS = 2 * A_STAGES + 2 * MAX_B_STAGES;
     const uint32_t bar_accum_full = bar0 + 8u * N_RING_BARS;
     const uint32_t bar_accum_empty = bar0 + 8u * (N_RING_BARS + 1);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(misc + 8 * (N_RING_BARS + 2));
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + N_RING_BARS + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int s = 0; s < A_STAGES; s++) {
-            mbar_init(bar_fullA(s), 2);       // one arrival per producer warp of a pair
-            mbar_init(bar_emptyA(s), 1);      // tcgen05.commit
+            mbar_init(bar_fullA(s), GROUP_WARPS);       // one arrival per producer warp of a group
+            mbar_init(bar_emptyA(s), 1);                // tcgen05.commit
         }
-        for (int s = 0; s < B_STAGES; s++) {
+        for (int s = 0; s < b_stages; s++) {
             mbar_init(bar_fullB(s), 1);       // the expect_tx arrival
             mbar_init(bar_emptyB(s), 1);      // tcgen05.commit
         }
@@ -327,178 +449,283 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, GemmParams P)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // residual codebook -> shared memory (all threads)
-    if (L.k2) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(L.c2);
-        uint4 *dst = reinterpret_cast<uint4 *>(cb2_ptr);
-        // (loads of 4 entries are issued before the first store: one L2 round trip per 4 entries)
-        const int n2 = P.cb2_replicated ? L.k2 * CB2_REPLICAS : L.k2, sh = P.cb2_replicated ? 2 : 0;
-        for (int i0 = threadIdx.x; i0 < n2; i0 += 4 * GEMM_THREADS) {
+    // tables -> shared memory as 16-byte rows (all threads; the loads of 4 rows are issued before the first store)
+    auto stage_table = [&](uint8_t *dst, const __half *src, int k, int shift) {
+        uint4 *d = reinterpret_cast<uint4 *>(dst);
+        const int n = k << shift;
+        for (int i0 = threadIdx.x; i0 < n; i0 += 4 * GEMM_THREADS) {
             uint4 row[4];
 #pragma unroll
             for (int u = 0; u < 4; u++)
-                if (i0 + u * GEMM_THREADS < n2) row[u] = __ldg(src + ((i0 + u * GEMM_THREADS) >> sh));
+                if (i0 + u * GEMM_THREADS < n) row[u] = load_centroid_row(src, (i0 + u * GEMM_THREADS) >> shift, V);
 #pragma unroll
             for (int u = 0; u < 4; u++)
-                if (i0 + u * GEMM_THREADS < n2) dst[i0 + u * GEMM_THREADS] = row[u];
+                if (i0 + u * GEMM_THREADS < n) d[i0 + u * GEMM_THREADS] = row[u];
         }
-    }
+    };
+    if (T1 == TABLE_SHARED) stage_table(cb1_ptr, L.c1, L.k1, P.cb1_shift);
+    if (T2 == TABLE_SHARED) stage_table(cb2_ptr, L.c2, L.k2, P.cb2_shift);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
-    // this CTA's share of the (tile, k block) units: [u_begin, u_end), boundaries multiples of unit_gran
-    const long long n_workers = gridDim.x, worker = blockIdx.x;
-    const long long groups = P.units / P.unit_gran;
-    const long long u_begin = groups * worker / n_workers * P.unit_gran;
-    const long long u_end = groups * (worker + 1) / n_workers * P.unit_gran;
+    // this CTA's share of the (tile, k block) units
+    const unsigned u_begin = P.shares.begin(blockIdx.x), u_end = P.shares.begin(blockIdx.x + 1);
     // A segment is the part of one tile inside the share: k blocks [kb0, kb1) of tile `tile`.
 #define FOR_EACH_SEGMENT                                                                          \
-    for (long long u = u_begin; u < u_end && ok; u += kb1 - kb0)                                    \
-        if (tile = (int)(u / P.kb_total), kb0 = (int)(u % P.kb_total),                              \
-            kb1 = (int)min((long long)P.kb_total, kb0 + (u_end - u)), true)
+    for (unsigned u = u_begin; u < u_end && ok; u += (unsigned)(kb1 - kb0))                         \
+        if (tile = (int)(u / (unsigned)P.kb_total), kb0 = (int)(u % (unsigned)P.kb_total),          \
+            kb1 = (int)min((unsigned)P.kb_total, kb0 + (u_end - u)), true)
     int tile = 0, kb0 = 0, kb1 = 0;
     bool ok = true;
 
-    if (warp == 0) {
-        // ================= bulk copies: B tiles =================
-        if (lane == 0) {
-            grid_dependency_wait();                              // the tile images are the pre-pass's output
+    if (warp < PRODUCER_WARP0) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
+        // ================= bulk copies: B ring =================
+        if (warp == 0 && lane == 0) {
+            grid_dependency_wait();                              // the images are the pre-pass's output
             int it = 0;
-            uint32_t s = 0, ps = 1;                              // ring position, parity to wait for
+            int s = 0;
+            uint32_t ps = 1;                                     // ring position, parity to wait for
             FOR_EACH_SEGMENT {
-                const int tt = tile / P.tiles_m;
-                const int t0 = tt * TILE_N;
-                const int halves = (P.B - t0 > MMA_N) ? 2 : 1;
-                for (int kb = kb0; kb < kb1; kb++, it++, s = (s + 1 == B_STAGES ? 0 : s + 1), ps ^= (s == 0 ? 1u : 0u)) {
+                const uint8_t *src = P.xs + ((long long)(tile / P.tiles_m) * P.kb_total * SUBS + (long long)kb0 * SUBS) * b_bytes;
+                for (int i = 0; i < (kb1 - kb0) * SUBS; i++, it++, src += b_bytes) {
                     if (!(ok = mbar_wait(bar_emptyB(s), ps, abort_flag, P.status))) break;
-                    mbar_expect_tx(bar_fullB(s), halves * B_HALF_BYTES);
-                    for (int h = 0; h < halves; h++)
-                        bulk_load(sB + s * B_STAGE_BYTES + h * B_HALF_BYTES,
-                                  P.xs + ((long long)(2 * tt + h) * P.kb_total + kb) * B_HALF_BYTES, B_HALF_BYTES, bar_fullB(s));
+                    mbar_expect_tx(bar_fullB(s), b_bytes);
+                    bulk_load(sB + s * b_bytes, src, b_bytes, bar_fullB(s));
+                    if (++s == b_stages) { s = 0; ps ^= 1u; }
                 }
             }
             if (!ok) {
                 // abandoned: give copies still in flight a bounded time to land before the CTA exits
-                const int first = it > B_STAGES ? it - B_STAGES : 0;
+                const int first = it > b_stages ? it - b_stages : 0;
                 for (int j = first; j < it; j++) {
                     const long long t0c = clock64();
-                    while (!mbar_try(bar_fullB(j % B_STAGES), (j / B_STAGES) & 1) && clock64() - t0c < 20000000ll) {}
+                    while (!mbar_try(bar_fullB(j % b_stages), (j / b_stages) & 1) && clock64() - t0c < 20000000ll) {}
                 }
             }
         }
-    } else if (warp == 1) {
         // ================= MMA issue =================
-        if (lane == 0) {
-            // One thread runs this loop as a serial instruction chain, so it is kept short: descriptors
-            // are a constant plus a stage offset, stage numbers and parities are running counters, and the
-            // MMAs of a k block go out in one asm block.
+        if (warp == 1) {
+            // The whole warp runs this loop, converged, and an elected lane issues (see elect_one); the loop is a serial
+            // chain, so it is kept short: descriptors are a constant plus a stage offset, stage numbers and parities are
+            // running counters.
             const uint64_t adesc0 = make_smem_desc(sA, A_LBO, A_SBO, LAYOUT_SW128);
             const uint64_t bdesc0 = make_smem_desc(sB, 16, B_SBO, LAYOUT_SW64);
-            uint32_t sa = 0, pa = 0, sb = 0, pb = 0;          // ring positions and their phase parities
+            const uint32_t a_lo0 = (uint32_t)adesc0, a_hi = (uint32_t)(adesc0 >> 32), b_lo0 = (uint32_t)bdesc0, b_hi = (uint32_t)(bdesc0 >> 32);
+            const int n1 = P.tile_n - P.n0;
+            const uint32_t id0 = instr_desc(MN, P.n0), id1 = instr_desc(MN, n1);
+            const uint32_t bh = (uint32_t)((P.n0 * 64) >> 4);        // second MMA's token rows
+            const uint32_t tmem0 = __shfl_sync(0xffffffffu, tmem_base, 0), tmem1 = tmem0 + (uint32_t)P.n0;
+            int sa = 0, sb = 0;                                      // ring positions and their phase parities
+            uint32_t pa = 0, pb = 0, gave_up = 0;
             int seg_no = 0;
             FOR_EACH_SEGMENT {
-                const int tt = tile / P.tiles_m;
-                const bool two_halves = P.B - tt * TILE_N > MMA_N;
                 // the accumulators must have been drained by the epilogues of the previous segment
-                if (!(ok = mbar_wait(bar_accum_empty, (seg_no & 1) ^ 1, abort_flag, P.status))) break;
+                mbar_wait_uniform(bar_accum_empty, (seg_no & 1) ^ 1, gave_up);
                 tc_fence_after();
+                uint32_t acc = 0;
                 for (int kb = kb0; kb < kb1; kb++) {
-                    if (!(ok = mbar_wait(bar_fullA(sa), pa, abort_flag, P.status))) break;
-                    if (!(ok = mbar_wait(bar_fullB(sb), pb, abort_flag, P.status))) break;
+                    mbar_wait_uniform(bar_fullA(sa), pa, gave_up);
                     // (stage offsets only touch the 14-bit address field of the descriptors: no carry)
-                    const uint64_t ad = adesc0 + (uint64_t)((sa * A_STAGE_BYTES) >> 4);
-                    const uint64_t bd = bdesc0 + (uint64_t)((sb * B_STAGE_BYTES) >> 4);
-                    umma_kblock(tmem_base, ad, bd, kb > kb0 ? 1u : 0u, two_halves);
-                    umma_commit(bar_emptyA(sa));      // the stages may be refilled once these MMAs have read them
-                    umma_commit(bar_emptyB(sb));
+                    const uint32_t a_lo = a_lo0 + (uint32_t)((sa * A_BYTES) >> 4);
+#pragma unroll
+                    for (int sub = 0; sub < SUBS; sub++) {
+                        mbar_wait_uniform(bar_fullB(sb), pb, gave_up);
+                        const uint32_t b_lo = b_lo0 + (uint32_t)((sb * b_bytes) >> 4);
+                        if (elect_one()) {
+#pragma unroll
+                            for (int h = 0; h < 2; h++) {                // k = 16 at a time
+                                // MN-major: two 8-column groups further; K-major: 32 bytes further inside the swizzled row
+                                const uint32_t ak = a_lo + (uint32_t)(MN ? (h * 2 * A_SBO) >> 4 : (sub * 2 + h) * 2);
+                                const uint32_t bk = b_lo + (uint32_t)(h * 2);
+                                umma_f16(tmem0, ak, a_hi, bk, b_hi, id0, acc);
+                                if (n1) umma_f16(tmem1, ak, a_hi, bk + bh, b_hi, id1, acc);
+                                acc = 1;
+                            }
+                            umma_commit(bar_emptyB(sb));      // the stages may be refilled once these MMAs have read them
+                            if (sub == SUBS - 1) umma_commit(bar_emptyA(sa));
+                        }
+                        acc = 1;
+                        if (++sb == b_stages) { sb = 0; pb ^= 1u; }
+                    }
                     if (++sa == A_STAGES) { sa = 0; pa ^= 1u; }
-                    if (++sb == B_STAGES) { sb = 0; pb ^= 1u; }
                 }
-                if (ok) umma_commit(bar_accum_full);  // accumulators complete
+                if (__any_sync(0xffffffffu, gave_up != 0)) {         // some wait ran out: what was issued is in bounds and worthless
+                    *abort_flag = 1;
+                    if (lane == 0) { grid_dependency_wait(); atomicExch(P.status, VPTQ_E_TIMEOUT); }
+                    ok = false;
+                } else if (elect_one()) {
+                    umma_commit(bar_accum_full);                     // accumulators complete
+                }
+                __syncwarp();
                 seg_no++;
             }
         }
-    } else if (warp < 2 + PRODUCER_WARPS) {
+    } else if (warp < EPI_WARP0) {
         // ================= dequant producers: A tiles =================
-        const int pw = warp - 2, pair = pw >> 1, half = pw & 1;
-        const int c = lane & 7, grp = lane >> 3;             // row chunk within the 64-row block, 8-column group
-        const uint4 *cb1 = reinterpret_cast<const uint4 *>(L.c1);
-        const uint4 *cb2 = reinterpret_cast<const uint4 *>(cb2_ptr);
-        const int rep = P.cb2_replicated ? (lane & (CB2_REPLICAS - 1)) : 0, rshift = P.cb2_replicated ? 2 : 0;
-        const uint32_t kmax1 = (uint32_t)(L.k1 - 1), kmax2 = L.k2 ? (uint32_t)(L.k2 - 1) : 0u;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_PRODUCER));
+        const int pw = warp - PRODUCER_WARP0, group = pw / GROUP_WARPS, wi = pw % GROUP_WARPS;
+        // v = 8: lane = (row chunk within the 64-row half `wi`, 8-column group of 4); else lane = (vector row of 4, group of 8)
+        const int vr = MN ? 8 * wi + (lane & 7) : 4 * wi + (lane >> 3);         // vector row within the tile
+        const int cg = MN ? lane >> 3 : lane & 7;
+        const uint4 *cb1 = reinterpret_cast<const uint4 *>(cb1_ptr) + (lane & ((1 << P.cb1_shift) - 1));
+        const uint4 *cb2 = reinterpret_cast<const uint4 *>(cb2_ptr) + (lane & ((1 << P.cb2_shift) - 1));
+        if (group >= GROUPS) ok = false;                     // a warp beyond the last whole group has no work
+        bool waited = false;                                 // padded tables are the pre-pass's output
         int it0 = 0;                                         // k blocks of earlier segments
         FOR_EACH_SEGMENT {
             const int mt = tile % P.tiles_m;
-            const int vrow = mt * (TILE_M / 8) + 8 * half + c;
-            const bool row_ok = vrow < L.R;
-            const uint8_t *row1 = L.s1.ptr + (long long)vrow * L.s1.stride;
-            const uint8_t *row2 = L.k2 ? L.s2.ptr + (long long)vrow * L.s2.stride : nullptr;
-            // this pair's k blocks of the segment: those whose running number is = pair (mod PAIRS)
-            int kb = kb0 + ((pair - it0 % PAIRS) + PAIRS) % PAIRS;
-            // a1: packed indices of 8 columns; the next visit's are loaded one visit ahead
-            uint4 raw1 = make_uint4(0, 0, 0, 0);
-            uint2 raw2 = make_uint2(0, 0);
-            if (kb < kb1 && row_ok && kb * TILE_K + 8 * grp < L.N) {
-                raw1 = __ldg(reinterpret_cast<const uint4 *>(row1 + 2LL * (kb * TILE_K + 8 * grp)));
-                if (L.k2) raw2 = __ldg(reinterpret_cast<const uint2 *>(row2 + (kb * TILE_K + 8 * grp)));
+            const int vrow = mt * NV + vr;
+            const bool row_ok = vr < NV && vrow < L.R;
+            const uint8_t *row1 = L.s1.ptr + (long long)(row_ok ? vrow : 0) * L.s1.stride;
+            const uint8_t *row2 = T2 ? L.s2.ptr + (long long)(row_ok ? vrow : 0) * L.s2.stride : nullptr;
+            // this group's k blocks of the segment: those whose running number is = group (mod GROUPS)
+            int kb = kb0 + ((group - it0 % GROUPS) + GROUPS) % GROUPS;
+            // a1: packed indices of 8 columns; the next visit's are loaded one visit ahead (a column group beyond the main
+            // columns reads as zeros)
+            const int limit = row_ok ? L.Nc : 0;
+            uint4 raw1 = make_uint4(0, 0, 0, 0), raw2 = make_uint4(0, 0, 0, 0);
+            if (kb < kb1) {
+                raw1 = load_raw8(row1, L.s1.stride, kb * (KS / 8) + cg, limit, L.s1.bits);
+                if (T2) raw2 = load_raw8(row2, L.s2.stride, kb * (KS / 8) + cg, limit, L.s2.bits);
             }
-            for (; kb < kb1; kb += PAIRS) {
+            if ((T1 == TABLE_GLOBAL || T2 == TABLE_GLOBAL) && V != 8 && !waited) { grid_dependency_wait(); waited = true; }
+            for (; kb < kb1; kb += GROUPS) {
                 const int it = it0 + (kb - kb0);
                 const int s = it % A_STAGES;
-                const int col0 = kb * TILE_K + 8 * grp;
-                const bool live = row_ok && col0 < L.N;
-                const uint32_t w1[4] = {raw1.x, raw1.y, raw1.z, raw1.w};
-                const uint2 cur2 = raw2;
-                {
-                    const int ncol = col0 + PAIRS * TILE_K;
-                    if (kb + PAIRS < kb1 && row_ok && ncol < L.N) {
-                        raw1 = __ldg(reinterpret_cast<const uint4 *>(row1 + 2LL * ncol));
-                        if (L.k2) raw2 = __ldg(reinterpret_cast<const uint2 *>(row2 + ncol));
-                    }
-                }
-                // a3: main centroids, 8 reads in flight (issued before the wait: they do not touch the stage)
-                uint4 cw[8];
+                const uint32_t stage = sA + s * A_BYTES;
+                if (kb >= P.kb_main) {
+                    // a5: outlier columns; few k blocks, written element by element
+                    ok = __all_sync(0xffffffffu, mbar_wait(bar_emptyA(s), ((it / A_STAGES) & 1) ^ 1, abort_flag, P.status));
+                    if (!ok) break;
+                    const int n0c = (kb - P.kb_main) * KS, m_tile = mt * TILE_M;
+                    const bool quads = L.v0 == 4 && TILE_M % 4 == 0;
+                    if (MN) {
+                        // (chunk of 8 rows, column): 16 x 32 of them
+                        for (int i = wi * 32 + lane; i < 16 * KS; i += GROUP_WARPS * 32) {
+                            const int ch = i & 15, k = i >> 4, m0 = m_tile + 8 * ch;
+                            uint32_t w[4];
+                            if (quads) {
+                                const uint2 a = outlier_vector4(L, m0, n0c + k), b = outlier_vector4(L, m0 + 4, n0c + k);
+                                w[0] = a.x; w[1] = a.y; w[2] = b.x; w[3] = b.y;
+                            } else {
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    uint32_t id = (w1[j >> 1] >> (16 * (j & 1))) & 0xFFFFu;
-                    id = min(id, kmax1);
-                    // (no L1 allocation: the tensor core's operand reads share the L1 data path)
-                    if (live) asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
-                                           : "=r"(cw[j].x), "=r"(cw[j].y), "=r"(cw[j].z), "=r"(cw[j].w) : "l"(cb1 + id));
-                    else cw[j] = make_uint4(0, 0, 0, 0);
-                }
-                // a4: residual centroids from shared memory, all 8 before the wait as well: one shared-memory
-                // round trip per visit instead of one per store
-                uint4 rv[8];
+                                for (int j = 0; j < 4; j++) w[j] = outlier_bits(L, m0 + 2 * j, n0c + k) | (outlier_bits(L, m0 + 2 * j + 1, n0c + k) << 16);
+                            }
+                            st_shared16(stage + (k >> 3) * 2048 + (ch >> 3) * 1024 + (k & 7) * 128 + (((ch & 7) ^ (k & 7)) << 4), w[0], w[1], w[2], w[3]);
+                        }
+                    } else if (quads) {
+                        // (4 rows, 8 columns): 30 x 8 of them, turned into rows
+                        for (int i = wi * 32 + lane; i < (TILE_M / 4) * 8; i += GROUP_WARPS * 32) {
+                            const int q = i & 7, m = (i >> 3) * 4;
+                            uint2 a[8];
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    rv[j] = make_uint4(0, 0, 0, 0);
-                    if (L.k2 && live) {
-                        uint32_t id2 = ((j < 4 ? cur2.x : cur2.y) >> (8 * (j & 3))) & 0xFFu;
-                        id2 = min(id2, kmax2);
-                        rv[j] = cb2[(id2 << rshift) + rep];
-                    }
-                }
-                // the whole warp takes the same decision: the stores below end in a warp-wide barrier
-                ok = __all_sync(0xffffffffu, mbar_wait(bar_emptyA(s), ((it / A_STAGES) & 1) ^ 1, abort_flag, P.status));
-                if (!ok) break;
-                const uint32_t dst0 = sA + s * A_STAGE_BYTES + grp * A_SBO + half * A_LBO;
+                            for (int j = 0; j < 8; j++) a[j] = outlier_vector4(L, m_tile + m, n0c + q * 8 + j);
 #pragma unroll
-                for (int j = 0; j < 8; j++) {
-                    uint4 w = cw[j];
-                    {   // sum in FP16 (adding zero when there is no residual stage changes nothing)
-                        __half2 a0 = __hadd2(*reinterpret_cast<__half2 *>(&w.x), *reinterpret_cast<const __half2 *>(&rv[j].x));
-                        __half2 a1 = __hadd2(*reinterpret_cast<__half2 *>(&w.y), *reinterpret_cast<const __half2 *>(&rv[j].y));
-                        __half2 a2 = __hadd2(*reinterpret_cast<__half2 *>(&w.z), *reinterpret_cast<const __half2 *>(&rv[j].z));
-                        __half2 a3 = __hadd2(*reinterpret_cast<__half2 *>(&w.w), *reinterpret_cast<const __half2 *>(&rv[j].w));
-                        w.x = *reinterpret_cast<uint32_t *>(&a0); w.y = *reinterpret_cast<uint32_t *>(&a1);
-                        w.z = *reinterpret_cast<uint32_t *>(&a2); w.w = *reinterpret_cast<uint32_t *>(&a3);
+                            for (int r = 0; r < 4; r++) {
+                                uint32_t w[4];
+#pragma unroll
+                                for (int j = 0; j < 4; j++) {
+                                    const uint32_t lo = r < 2 ? a[2 * j].x : a[2 * j].y, hi = r < 2 ? a[2 * j + 1].x : a[2 * j + 1].y;
+                                    w[j] = __byte_perm(lo, hi, (r & 1) ? 0x7632 : 0x5410);
+                                }
+                                st_shared16(stage + ((m + r) >> 3) * 1024 + ((m + r) & 7) * 128 + ((q ^ ((m + r) & 7)) << 4), w[0], w[1], w[2], w[3]);
+                            }
+                        }
+                    } else {
+                        for (int i = wi * 32 + lane; i < TILE_M * 8; i += GROUP_WARPS * 32) {
+                            const int q = i & 7, m = i >> 3;
+                            uint32_t w[4];
+#pragma unroll
+                            for (int j = 0; j < 4; j++)
+                                w[j] = outlier_bits(L, m_tile + m, n0c + q * 8 + 2 * j) | (outlier_bits(L, m_tile + m, n0c + q * 8 + 2 * j + 1) << 16);
+                            st_shared16(stage + (m >> 3) * 1024 + (m & 7) * 128 + ((q ^ (m & 7)) << 4), w[0], w[1], w[2], w[3]);
+                        }
                     }
-                    if (col0 + j >= L.N) w = make_uint4(0, 0, 0, 0);
-                    const uint32_t dst = dst0 + j * 128 + ((c ^ j) << 4);
-                    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(w.x), "r"(w.y), "r"(w.z), "r"(w.w) : "memory");
+                } else {
+                    const int col0 = kb * KS + 8 * cg;
+                    // (a lane without a row or columns holds zeros and so reads entry 0 along with the others)
+                    uint32_t w1[4], w2[4] = {0, 0, 0, 0};
+                    decode8(raw1, L.s1.bits, L.k1, w1);
+                    if (T2) decode8(raw2, L.s2.bits, L.k2, w2);
+                    if (kb + GROUPS < kb1) {
+                        raw1 = load_raw8(row1, L.s1.stride, (kb + GROUPS) * (KS / 8) + cg, limit, L.s1.bits);
+                        if (T2) raw2 = load_raw8(row2, L.s2.stride, (kb + GROUPS) * (KS / 8) + cg, limit, L.s2.bits);
+                    }
+                    // Sec. 3.1: a column's tables are those of its group
+                    uint32_t g = 0;
+                    int g_next = 0x7fffffff;
+                    if ((T1 == TABLE_GLOBAL || T2 == TABLE_GLOBAL) && L.G > 1) { g = (uint32_t)(col0 / L.cpg); g_next = (int)(g + 1) * L.cpg; }
+                    auto next_group = [&](int j) { if (col0 + j >= g_next && (int)g + 1 < L.G) { g++; g_next += L.cpg; } };
+                    auto id = [&](const uint32_t (&w)[4], int j) { return (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu; };
+                    uint32_t cw[8][W2];
+                    if (V <= 8) {
+                        // a3: main centroids, a4: residual centroids; all reads in flight before the wait (they do not touch the stage)
+                        uint32_t rv[8][W2];
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            next_group(j);
+                            if (T1 == TABLE_SHARED) row_shared<V>(cb1, id(w1, j) << P.cb1_shift, cw[j]);
+                            else row_global<V>(P.tab1, g * (uint32_t)L.k1 + id(w1, j), cw[j]);
+                            if (T2 == TABLE_SHARED) row_shared<V>(cb2, id(w2, j) << P.cb2_shift, rv[j]);
+                            else if (T2 == TABLE_GLOBAL) row_global<V>(P.tab2, g * (uint32_t)L.k2 + id(w2, j), rv[j]);
+                        }
+                        // the whole warp takes the same decision: the stores below end in a warp-wide barrier
+                        ok = __all_sync(0xffffffffu, mbar_wait(bar_emptyA(s), ((it / A_STAGES) & 1) ^ 1, abort_flag, P.status));
+                        if (!ok) break;
+                        if (T2) {            // sum in FP16 (one rounding of 2^-11)
+#pragma unroll
+                            for (int j = 0; j < 8; j++)
+#pragma unroll
+                                for (int i = 0; i < W2; i++) cw[j][i] = hadd2_bits(cw[j][i], rv[j][i]);
+                        }
+                    } else {
+                        // two 32-byte rows per column: four columns in flight at a time
+#pragma unroll
+                        for (int j0 = 0; j0 < 8; j0 += 4) {
+                            uint32_t rv[4][W2];
+#pragma unroll
+                            for (int u = 0; u < 4; u++) {
+                                const int j = j0 + u;
+                                next_group(j);
+                                row_global<V>(P.tab1, g * (uint32_t)L.k1 + id(w1, j), cw[j]);
+                                if (T2) row_global<V>(P.tab2, g * (uint32_t)L.k2 + id(w2, j), rv[u]);
+                            }
+                            if (T2) {
+#pragma unroll
+                                for (int u = 0; u < 4; u++)
+#pragma unroll
+                                    for (int i = 0; i < W2; i++) cw[j0 + u][i] = hadd2_bits(cw[j0 + u][i], rv[u][i]);
+                            }
+                        }
+                        ok = __all_sync(0xffffffffu, mbar_wait(bar_emptyA(s), ((it / A_STAGES) & 1) ^ 1, abort_flag, P.status));
+                        if (!ok) break;
+                    }
+                    if (col0 + 8 > L.Nc) {
+#pragma unroll
+                        for (int j = 0; j < 8; j++)
+                            if (col0 + j >= L.Nc)
+#pragma unroll
+                                for (int i = 0; i < W2; i++) cw[j][i] = 0u;
+                    }
+                    if (MN) {
+                        const uint32_t dst0 = stage + cg * 2048 + wi * 1024;
+#pragma unroll
+                        for (int j = 0; j < 8; j++)
+                            st_shared16(dst0 + j * 128 + (((lane & 7) ^ j) << 4), cw[j][0], cw[j][1], cw[j][2], cw[j][W2 - 1]);
+                    } else if (vr < NV) {
+                        // 8 columns x V rows -> V rows of 8 columns
+#pragma unroll
+                        for (int r = 0; r < V; r++) {
+                            const int m = vr * V + r;
+                            uint32_t w[4];
+#pragma unroll
+                            for (int j = 0; j < 4; j++) w[j] = __byte_perm(cw[2 * j][r >> 1], cw[2 * j + 1][r >> 1], (r & 1) ? 0x7632 : 0x5410);
+                            st_shared16(stage + (m >> 3) * 1024 + (m & 7) * 128 + ((cg ^ (m & 7)) << 4), w[0], w[1], w[2], w[3]);
+                        }
+                    }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic-proxy stores -> visible to the MMA
                 __syncwarp();
@@ -507,111 +734,106 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, GemmParams P)
             it0 += kb1 - kb0;
         }
     } else {
-        // ================= epilogue: two warps per TMEM lane quarter, one per 256-token half =================
+        // ================= epilogue: two warps per TMEM lane quarter, taking turns at chunks of 32 tokens =================
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
+        const int ew = warp - EPI_WARP0, h = ew >> 2;
         const int q = warp & 3;                                  // TMEM lane quarter this warp may read
-        const int h = (warp - (2 + PRODUCER_WARPS)) >> 2;        // token half of the tile
-        const bool fp32_out = L.out_dtype == VPTQ_DTYPE_FP32;
-        const unsigned Mu = (unsigned)L.M;
-        int seg_no = 0;
-        unsigned epi_piece = 0;                                  // staged pieces so far (buffer parity)
-        grid_dependency_wait();                                  // bias terms, tile flags and a cleared output come from the pre-pass
+        const int padded_b = P.tiles_t * P.tile_n;
+        int seg_no = 0, bias_tile = -1;
+        grid_dependency_wait();                                  // bias terms, flags and cleared sums come from the pre-pass
         FOR_EACH_SEGMENT {
             const int mt = tile % P.tiles_m, tt = tile / P.tiles_m;
-            const int t0 = tt * TILE_N;
+            const int t0 = tt * P.tile_n;
             const int m = mt * TILE_M + 32 * q + lane;
-            const int t_cnt = min(TILE_N, P.B - t0);
+            const bool m_ok = 32 * q + lane < TILE_M && m < L.M;
+            const int t_cnt = min(P.tile_n, P.B - t0);
+            if (tt != bias_tile) {
+                // the token tile's bias terms: the parts in order (a fixed order, whoever adds)
+                asm volatile("bar.sync 1, %0;" ::"r"(EPI_WARPS * 32) : "memory");
+                for (int t = ew * 32 + lane; t < P.tile_n; t += EPI_WARPS * 32) {
+                    float a = 0.f;
+#pragma unroll 8
+                    for (int c = 0; c < P.bias_parts; c++) a += __ldg(P.bpart + (long long)c * padded_b + t0 + t);
+                    bias[t] = a;
+                }
+                asm volatile("bar.sync 1, %0;" ::"r"(EPI_WARPS * 32) : "memory");
+                bias_tile = tt;
+            }
             // a split tile: the piece with the last k blocks stores and announces it, the others add afterwards
             const bool split = kb0 != 0 || kb1 != P.kb_total;
+            const bool to_scratch = split && P.scratch != nullptr;
             const bool add = P.flag_order ? kb1 != P.kb_total : split;
             const bool announce = P.flag_order && kb0 != 0 && kb1 == P.kb_total;
-            // bias terms of this warp's 256 tokens, loaded before the wait (a load inside the drain would
-            // cost an L2 round trip under load): lane l holds token 32*i + l of chunk i
-            float bt_chunk[MMA_N / 32];
-#pragma unroll
-            for (int i = 0; i < MMA_N / 32; i++) {
-                const int t = t0 + h * MMA_N + 32 * i + lane;
-                bt_chunk[i] = (kb0 == 0 && t < P.B) ? __ldg(P.bterm + t) : 0.f;
+            int pieces = 0;                                  // shares that hold some of the tile (worked out while the MMAs run)
+            if (to_scratch) {
+                const unsigned first_u = (unsigned)tile * P.kb_total, end_u = first_u + P.kb_total;
+                unsigned at = 0;
+                for (unsigned w = P.shares.worker_of(first_u); at < end_u; w++) {
+                    const unsigned next = P.shares.begin(w + 1);
+                    pieces += next > at;                                     // (an empty share holds nothing)
+                    at = next;
+                }
             }
             ok = __all_sync(0xffffffffu, mbar_wait(bar_accum_full, seg_no & 1, abort_flag, P.status));
             if (!ok) break;
             tc_fence_after();
             if (add && P.flag_order) {
-                ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(P.tile_flags + tile, EPI_WARPS, abort_flag, P.status));
+                ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(P.tile_flags + tile * EPI_WARPS, EPI_WARPS, abort_flag, P.status));
                 if (!ok) break;
                 asm volatile("fence.proxy.async;" ::: "memory");     // the reduce-adds below go through the async proxy
             }
-            if (P.tma_out) {
-                // FP32 output through shared memory: per 16 tokens a warp stages its [16][32] piece (lane =
-                // output row: conflict free) and one lane hands it to TMA (store, or reduce-add for a partial
-                // tile); two staging buffers per warp, so the copy of one piece overlaps the next.
-                const uint32_t ebuf = sEpi + (uint32_t)(warp - (2 + PRODUCER_WARPS)) * (2 * EPI_BUF_BYTES);
-                const int m0 = mt * TILE_M + 32 * q;
+            const uint32_t ebuf = sEpi + (uint32_t)(ew * 2 * EPI_BUF_BYTES);
+            const int m0 = mt * TILE_M + 32 * q;
+            // rows of this quarter that belong to the tile: a 120-row tile leaves 8 lanes of the last quarter unused, and a
+            // 32-row box of the output must not touch the next tile's rows, so that quarter stores element by element
+            const bool box = P.tma_out && 32 * q + 32 <= TILE_M;
+            float *sc = to_scratch ? P.scratch + ((long long)tile * 4 + q) * scratch_rows(P.tile_n) * 32 : nullptr;
+            for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += 2 * EPI_TOKENS) {
+                uint32_t r[EPI_TOKENS];
+                tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c1, r);
+                if (kb0 == 0) {
+                    const float4 *b4 = reinterpret_cast<const float4 *>(bias + c1);
 #pragma unroll
-                for (int ci = 0; ci < MMA_N / 32; ci++) {    // unrolled: bt_chunk[] stays in registers
-                    const int c0 = h * MMA_N + 32 * ci;
-                    if (c0 >= t_cnt) break;
-                    const float bt_lane = bt_chunk[ci];
-#pragma unroll
-                    for (int hh = 0; hh < 2; hh++) {
-                        const int c1 = c0 + 16 * hh;
-                        if (c1 >= t_cnt) break;
-                        uint32_t r[16];
-                        tmem_ld16(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c1, r);
-                        if (kb0 == 0) {
-#pragma unroll
-                            for (int j = 0; j < 16; j++)
-                                r[j] = __float_as_uint(__uint_as_float(r[j]) + __shfl_sync(0xffffffffu, bt_lane, 16 * hh + j));
-                        }
-                        // the buffer written two pieces ago must have been read by its copy
-                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
-                        __syncwarp();
-                        const uint32_t buf = ebuf + (uint32_t)(epi_piece & 1) * EPI_BUF_BYTES;
-#pragma unroll
-                        for (int j = 0; j < 16; j++)
-                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + j * 128u + lane * 4u), "r"(r[j]) : "memory");
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0 && m0 < L.M) tma_store_2d(&tmap_out, buf, m0, t0 + c1, add);
-                        epi_piece++;
+                    for (int j = 0; j < EPI_TOKENS / 4; j++) {
+                        const float4 bv = b4[j];
+                        r[4 * j] = __float_as_uint(__uint_as_float(r[4 * j]) + bv.x);
+                        r[4 * j + 1] = __float_as_uint(__uint_as_float(r[4 * j + 1]) + bv.y);
+                        r[4 * j + 2] = __float_as_uint(__uint_as_float(r[4 * j + 2]) + bv.z);
+                        r[4 * j + 3] = __float_as_uint(__uint_as_float(r[4 * j + 3]) + bv.w);
                     }
                 }
-            } else
+                if (box || to_scratch) {
+                    // through shared memory: a warp stages a [16][32] piece (lane = output row: conflict free) and one
+                    // lane hands it to the copy engine (store or reduce-add); two staging buffers per warp, so the copy of
+                    // one piece overlaps the next.  The buffer written two pieces ago must have been read by its copy.
 #pragma unroll
-            for (int ci = 0; ci < MMA_N / 32; ci++) {        // unrolled: bt_chunk[] stays in registers
-                const int c0 = h * MMA_N + 32 * ci;
-                if (c0 >= t_cnt) break;
-                const float bt_lane = bt_chunk[ci];
-                uint32_t r[32];
-                tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, r);
-                if (kb0 == 0) {
+                    for (int p = 0; p < EPI_TOKENS / PIECE_TOKENS; p++) {
+                        const int c2 = c1 + p * PIECE_TOKENS;
+                        if (c2 >= t_cnt) break;
+                        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                        __syncwarp();
+                        const uint32_t buf = ebuf + (uint32_t)(p & 1) * EPI_BUF_BYTES;
 #pragma unroll
-                    for (int j = 0; j < 32; j++)
-                        r[j] = __float_as_uint(__uint_as_float(r[j]) + __shfl_sync(0xffffffffu, bt_lane, j));
-                }
-                if (m < L.M) {
-                    const int nt = min(32, P.B - (t0 + c0));           // tokens of this chunk that exist
-                    if (fp32_out) {
-                        // one element per token row; independent addresses, no serial pointer chain
-                        float *p = reinterpret_cast<float *>(P.out) + (long long)(t0 + c0) * L.M + m;
-                        if (nt == 32 && !add) {
-#pragma unroll
-                            for (int j = 0; j < 32; j++) p[(unsigned)j * Mu] = __uint_as_float(r[j]);
-                        } else if (nt == 32) {
-#pragma unroll
-                            for (int j = 0; j < 32; j++) atomicAdd(p + (unsigned)j * Mu, __uint_as_float(r[j]));
-                        } else {
-#pragma unroll
-                            for (int j = 0; j < 32; j++) {
-                                if (j < nt) {
-                                    if (!add) p[(unsigned)j * Mu] = __uint_as_float(r[j]);
-                                    else atomicAdd(p + (unsigned)j * Mu, __uint_as_float(r[j]));
-                                }
-                            }
+                        for (int j = 0; j < PIECE_TOKENS; j++)
+                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + j * 128u + lane * 4u), "r"(r[p * PIECE_TOKENS + j]) : "memory");
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) {
+                            if (to_scratch) bulk_add(sc + c2 * 32, buf);
+                            else if (m0 < L.M) tma_store_2d(&tmap_out, buf, m0, t0 + c2, add);
                         }
+                    }
+                } else if (m_ok) {
+                    const int nt = min(EPI_TOKENS, t_cnt - c1);                // tokens of this chunk that exist
+                    const long long o0 = (long long)(t0 + c1) * L.M + m;
+                    if (add) {
+#pragma unroll
+                        for (int j = 0; j < EPI_TOKENS; j++)
+                            if (j < nt) atomicAdd(reinterpret_cast<float *>(P.out) + o0 + (long long)j * L.M, __uint_as_float(r[j]));
                     } else {
 #pragma unroll
-                        for (int j = 0; j < 32; j++)
-                            if (j < nt) store_out(P.out, (long long)(t0 + c0 + j) * L.M + m, __uint_as_float(r[j]), L.out_dtype);
+                        for (int j = 0; j < EPI_TOKENS; j++)
+                            if (j < nt) store_out(P.out, o0 + (long long)j * L.M, __uint_as_float(r[j]), L.out_dtype);
                     }
                 }
             }
@@ -620,19 +842,59 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, GemmParams P)
             if (lane == 0) mbar_arrive(bar_accum_empty);
             if (announce) {
                 // this warp's part of the tile is in memory before the flag counts it
+                if (lane == 0 && P.tma_out) {
+                    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+                    asm volatile("fence.proxy.async;" ::: "memory");
+                }
+                __threadfence();
+                __syncwarp();
+                if (lane == 0) atomicAdd(P.tile_flags + tile * EPI_WARPS, 1);
+            }
+            if (to_scratch) {
+                // count this warp's part in; the CTA that finds all pieces counted converts and stores the part
+                int before = 0;
                 if (lane == 0) {
-                    if (P.tma_out) {
-                        asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-                        asm volatile("fence.proxy.async;" ::: "memory");
-                    }
+                    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+                    asm volatile("fence.proxy.async;" ::: "memory");
                     __threadfence();
-                    atomicAdd(P.tile_flags + tile, 1);
+                    before = atomicAdd(P.tile_flags + tile * EPI_WARPS + ew, 1);
+                    __threadfence();
+                }
+                before = __shfl_sync(0xffffffffu, before, 0);
+                if (before == pieces - 1) {
+                    const int rq = 4 * (lane & 7), mq = m0 + rq;              // this lane's four rows
+                    const bool rows4 = 32 * q + rq + 4 <= TILE_M && mq + 4 <= L.M && (L.M & 3) == 0;
+                    for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += 2 * EPI_TOKENS)
+#pragma unroll
+                    for (int c2 = c1; c2 < c1 + EPI_TOKENS; c2 += 16) {
+                        float4 v[4];
+#pragma unroll
+                        for (int i = 0; i < 4; i++) v[i] = __ldcg(reinterpret_cast<const float4 *>(sc + (c2 + 4 * i + (lane >> 3)) * 32 + rq));
+#pragma unroll
+                        for (int i = 0; i < 4; i++) {
+                            const int t = c2 + 4 * i + (lane >> 3);
+                            if (t >= t_cnt) continue;
+                            const long long o = (long long)(t0 + t) * L.M + mq;
+                            if (rows4 && L.out_dtype == VPTQ_DTYPE_FP16) {
+                                __half2 p[2] = {__floats2half2_rn(v[i].x, v[i].y), __floats2half2_rn(v[i].z, v[i].w)};
+                                *reinterpret_cast<uint2 *>(reinterpret_cast<__half *>(P.out) + o) = *reinterpret_cast<const uint2 *>(p);
+                            } else if (rows4 && L.out_dtype == VPTQ_DTYPE_BF16) {
+                                __nv_bfloat162 p[2] = {__floats2bfloat162_rn(v[i].x, v[i].y), __floats2bfloat162_rn(v[i].z, v[i].w)};
+                                *reinterpret_cast<uint2 *>(reinterpret_cast<__nv_bfloat16 *>(P.out) + o) = *reinterpret_cast<const uint2 *>(p);
+                            } else {
+                                const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+                                for (int k = 0; k < 4; k++)
+                                    if (32 * q + rq + k < TILE_M && mq + k < L.M) store_out(P.out, o + k, e[k], L.out_dtype);
+                            }
+                        }
+                    }
                 }
             }
             seg_no++;
         }
         // the staging buffers must outlive the copies that read them, the copies must land before the end
-        if (P.tma_out && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     }
 #undef FOR_EACH_SEGMENT
 
@@ -667,106 +929,101 @@ EncodeTiledFn get_encode_fn()
 }
 
 struct GemmPlan {
-    int tiles_m, tiles_t, kb_total, unit_gran, grid, any_split, flag_order, cb2_rep, cb2_bytes;
-    long long units;
+    int t1, t2;                      // TableSource of the main and the residual table
+    Shares shares;
+    int tiles_m, tiles_t, tile_n, n0, ks, kb_main, kb_total, grid, any_split, flag_order, tma_out, scratch;
+    int b_stages, cb1_shift, cb2_shift, cb1_bytes, cb2_bytes;
+    int pre_x, pre_y;                // pre-pass grid; pre_y = parts of a bias term
+    long long n_scratch;
     size_t smem;
-    long long ws_bytes, off_flags, off_bterm, off_xs;
+    int pad_bytes;                   // rows of padded table copies, 0 = none
+    long long ws_bytes, off_flags, off_bpart, off_pad1, off_pad2, off_scratch, off_xs;
 };
 
-size_t gemm_smem_bytes(int cb2_bytes)
+template <int V>
+GemmPlan plan_gemm_v(const LayerView &L, int B)
 {
-    return 1024 + (size_t)A_STAGES * A_STAGE_BYTES + (size_t)B_STAGES * B_STAGE_BYTES + cb2_bytes +
-           EPI_STAGE_BYTES + 8 * (2 * A_STAGES + 2 * B_STAGES + 2) + 16;
+    GemmPlan p;
+    memset(&p, 0, sizeof(p));
+    int workers = device_sm_count();
+    // tables: small ones of a single group in shared memory, with copies where that costs little
+    p.t1 = (V <= 8 && L.G == 1 && (long long)L.k1 * 16 <= 64 * 1024) ? TABLE_SHARED : TABLE_GLOBAL;
+    p.t2 = L.k2 == 0 ? TABLE_NONE : (V <= 8 && L.G == 1 && L.k2 * 16 <= 16 * 1024) ? TABLE_SHARED : TABLE_GLOBAL;
+    if (p.t1 == TABLE_SHARED) {
+        while (p.cb1_shift < 3 && (L.k1 * 16 << (p.cb1_shift + 1)) <= 32 * 1024) p.cb1_shift++;
+        p.cb1_bytes = L.k1 * 16 << p.cb1_shift;
+    }
+    // token tiles of equal size, at most MAX_TILE_N tokens each
+    p.tiles_t = ceil_div(B, MAX_TILE_N);
+    p.tile_n = (ceil_div(B, p.tiles_t) + 15) / 16 * 16;
+    p.n0 = p.tile_n <= 256 ? p.tile_n : (p.tile_n / 2 + 15) / 16 * 16;
+    p.tiles_m = ceil_div(L.R, Tile<V>::NV);
+    p.ks = Tile<V>::KS;
+    p.kb_main = ceil_div(L.Nc, p.ks);
+    p.kb_total = p.kb_main + ceil_div(L.n_out, p.ks);
+    // a deterministic call gets whole tiles: sums of several pieces arrive in no fixed order
+    Shares &sh = p.shares;
+    const unsigned tiles = (unsigned)p.tiles_m * p.tiles_t;
+    sh.kb = p.kb_total; sh.whole_tiles = L.deterministic ? 1 : 0;
+    sh.len = p.kb_total + DRAIN_COLS * p.tile_n / MAX_TILE_N / p.ks;
+    // (a share of a few k blocks is not worth a CTA of its own: it costs a piece of the output and its meeting)
+    const unsigned most = L.deterministic ? tiles : (tiles * sh.kb * p.ks + 127) / 128;
+    if (most < (unsigned)workers) workers = (int)most;
+    sh.workers = p.grid = workers;
+    const unsigned line = sh.whole_tiles ? tiles : tiles * sh.len;
+    sh.each = line / workers; sh.rest = line % workers;
+    for (int c = 1; c < workers; c++)
+        if (sh.begin(c) % p.kb_total != 0) p.any_split = 1;
+    p.tma_out = (L.out_dtype == VPTQ_DTYPE_FP32 && (L.M & 3) == 0) ? 1 : 0;
+    p.scratch = p.any_split && !p.tma_out;
+    // flag order makes CTAs wait for one another: only for a call that has the GPU to itself
+    p.flag_order = (p.any_split && p.tma_out && tiles * sh.kb / workers * p.ks >= FLAG_ORDER_MIN_COLS && !L.concurrent) ? 1 : 0;
+    // Shared memory: tables, A ring, then a B ring of up to 96 KB.  Three stages of it come before
+    // copies of the residual table (eight copies are free of bank conflicts).  A table in L2
+    // needs the L1 that is left, whose lines hold the reads in flight: past 196 KB a CTA (with the 1 KB the system keeps)
+    // leaves 28 KB of L1 instead of 60 KB, and 14336 x 4096 at 512 tokens takes 101 us instead of 90.
+    const int b_bytes = p.tile_n * 64;
+    const int limit = p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL ? SMEM_LIMIT_L1 : SMEM_LIMIT;
+    const bool copies = p.t2 == TABLE_SHARED && L.k2 <= 256;
+    p.cb2_shift = copies ? 3 : 0;
+    while (true) {
+        p.cb2_bytes = p.t2 == TABLE_SHARED ? L.k2 * 16 << p.cb2_shift : 0;
+        const int fixed = Tile<V>::A_STAGES * a_stage_bytes<V>() + p.cb1_bytes + p.cb2_bytes + EPI_STAGE_BYTES +
+                          MAX_TILE_N * 4 + 8 * (2 * Tile<V>::A_STAGES + 2 * MAX_B_STAGES + 2) + 16;
+        int room = limit - fixed;
+        if (room > 96 * 1024) room = 96 * 1024;
+        p.b_stages = room / b_bytes < MAX_B_STAGES ? room / b_bytes : MAX_B_STAGES;
+        p.smem = (size_t)fixed + (size_t)(p.b_stages > 0 ? p.b_stages : 0) * b_bytes;
+        if (p.b_stages >= 3 || p.cb2_shift == 0) break;
+        p.cb2_shift--;
+    }
+    // pre-pass: enough blocks to fill the GPU (each of them is one part of eight tokens' bias terms)
+    const int images = p.kb_total * (p.ks / IMG_COLS);
+    p.pre_x = p.tiles_t * p.tile_n / 8;
+    p.pre_y = ceil_div(4 * device_sm_count(), p.pre_x);
+    if (p.pre_y > ceil_div(images, 8)) p.pre_y = ceil_div(images, 8);
+    p.pad_bytes = (V != 8 && (p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL)) ? (V <= 8 ? 16 : 32) : 0;
+    auto take = [&](long long bytes) { const long long at = p.ws_bytes; p.ws_bytes += (bytes + 255) / 256 * 256; return at; };
+    take(WS_STATUS_BYTES);
+    p.off_flags = take((long long)tiles * EPI_WARPS * 4);
+    p.off_bpart = take((long long)p.pre_y * p.tiles_t * p.tile_n * 4);
+    p.off_pad1 = take(p.pad_bytes && p.t1 == TABLE_GLOBAL ? (long long)L.G * L.k1 * p.pad_bytes : 0);
+    p.off_pad2 = take(p.pad_bytes && p.t2 == TABLE_GLOBAL ? (long long)L.G * L.k2 * p.pad_bytes : 0);
+    p.n_scratch = p.scratch ? (long long)tiles * 4 * scratch_rows(p.tile_n) * 32 : 0;
+    p.off_scratch = take(p.n_scratch * 4);
+    p.off_xs = take((long long)p.tiles_t * images * b_bytes);
+    return p;
 }
 
 GemmPlan plan_gemm(const LayerView &L, int B)
 {
-    GemmPlan p;
-    int workers = device_sm_count();
-    p.cb2_rep = (L.k2 > 0 && L.k2 <= 256) ? 1 : 0;
-    p.cb2_bytes = L.k2 ? L.k2 * 16 * (p.cb2_rep ? CB2_REPLICAS : 1) : 0;
-    p.tiles_m = ceil_div(L.M, TILE_M);
-    p.tiles_t = ceil_div(B, TILE_N);
-    p.kb_total = ceil_div(L.N, TILE_K);
-    p.units = (long long)p.tiles_m * p.tiles_t * p.kb_total;
-    // the pieces of a split tile meet in an FP32 output by red.add; other output types get whole tiles
-    // (and so does a deterministic call: reduce-adds of several pieces arrive in no fixed order)
-    p.unit_gran = (L.out_dtype == VPTQ_DTYPE_FP32 && !L.deterministic) ? 1 : p.kb_total;
-    const long long groups = p.units / p.unit_gran;
-    if (groups < workers) workers = (int)groups;
-    p.grid = workers;
-    p.any_split = 0;
-    for (int c = 1; c < workers; c++)
-        if ((groups * c / workers * p.unit_gran) % p.kb_total != 0) p.any_split = 1;
-    // flag order makes CTAs wait for one another: only for a call that has the GPU to itself
-    p.flag_order = (p.any_split && p.units / workers >= FLAG_ORDER_MIN_SHARE && !L.concurrent) ? 1 : 0;
-    p.smem = gemm_smem_bytes(p.cb2_bytes);
-    p.off_flags = WS_STATUS_BYTES;
-    p.off_bterm = p.off_flags + ((long long)p.tiles_m * p.tiles_t * 4 + 255) / 256 * 256;
-    p.off_xs = p.off_bterm + ((long long)B * 4 + 255) / 256 * 256;
-    // activation tile images: whole 256-token halves and whole k blocks
-    p.ws_bytes = p.off_xs + (long long)ceil_div(B, MMA_N) * p.kb_total * B_HALF_BYTES;
-    return p;
+    return L.v == 8 ? plan_gemm_v<8>(L, B) : L.v == 6 ? plan_gemm_v<6>(L, B) : plan_gemm_v<12>(L, B);
 }
 
-}  // namespace
-
-bool gemm_tcgen05_supported(const LayerView &L, int B)
+template <int V, int T1, int T2>
+cudaError_t launch_gemm(const GemmPlan &pl, const CUtensorMap &map, const GemmParams &P, cudaStream_t st)
 {
-    if (L.G > 1) return false;          // one codebook pair per layer here
-    if (B <= 16) return false;
-    if (L.v != 8 || L.n_out != 0 || L.scale_rows) return false;
-    if (L.s1.bits != 16) return false;
-    if (L.k2 && (L.s2.bits != 8 || L.k2 > 2048)) return false;
-    return true;
-}
-
-// (the scratch layout does not depend on the device, so this query makes no CUDA call)
-long long gemm_tcgen05_workspace_bytes(const LayerView &L, int B) { return plan_gemm(L, B).ws_bytes; }
-
-int gemm_tcgen05_launches(const LayerView &, int) { return 2; }   // pre-pass + GEMM
-
-bool gemm_tcgen05_waits_between_ctas(const LayerView &L, int B) { return plan_gemm(L, B).flag_order != 0; }
-
-cudaError_t launch_gemm_tcgen05(const LayerView &L, const void *x, int B, void *out, void *ws, cudaStream_t st)
-{
-    const GemmPlan pl = plan_gemm(L, B);
-    uint8_t *w8 = reinterpret_cast<uint8_t *>(ws);
-    int *status = reinterpret_cast<int *>(w8);
-    int *tile_flags = reinterpret_cast<int *>(w8 + pl.off_flags);
-    float *bterm = reinterpret_cast<float *>(w8 + pl.off_bterm);
-    uint8_t *xs = w8 + pl.off_xs;
-
-    // FP32 output with 16-byte aligned rows: the epilogue goes through shared memory and TMA
-    const int tma_out = (L.out_dtype == VPTQ_DTYPE_FP32 && (L.M & 3) == 0) ? 1 : 0;
-    CUtensorMap tmap_out;
-    memset(&tmap_out, 0, sizeof(tmap_out));      // not read by the kernel when tma_out == 0
-    if (tma_out) {
-        EncodeTiledFn encode = get_encode_fn();
-        if (encode == nullptr) return cudaErrorNotSupported;
-        const cuuint64_t odim[2] = {(cuuint64_t)L.M, (cuuint64_t)B};
-        const cuuint64_t ostride[1] = {(cuuint64_t)L.M * 4};
-        const cuuint32_t obox[2] = {32, 16};
-        const cuuint32_t estr[2] = {1, 1};
-        const CUresult r = encode(&tmap_out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, out, odim, ostride, obox, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    }
-
-    cudaError_t e;
-    gemm_prepass_kernel<<<ceil_div(B, MMA_N) * MMA_N, PRE_THREADS, 0, st>>>(
-        L, x, B, xs, bterm, status, tile_flags, pl.tiles_m * pl.tiles_t,
-        (pl.any_split && !pl.flag_order) ? reinterpret_cast<float *>(out) : nullptr);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    GemmParams P;
-    P.L = L; P.out = out; P.B = B;
-    P.tiles_m = pl.tiles_m; P.tiles_t = pl.tiles_t; P.kb_total = pl.kb_total;
-    P.unit_gran = pl.unit_gran; P.units = pl.units;
-    P.cb2_replicated = pl.cb2_rep; P.cb2_bytes = pl.cb2_bytes;
-    P.status = status; P.bterm = bterm; P.xs = xs; P.tile_flags = tile_flags; P.flag_order = pl.flag_order; P.tma_out = tma_out;
-    e = cudaFuncSetAttribute(gemm_tcgen05_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2>), pl.smem);
     if (e != cudaSuccess) return e;
     // programmatic dependent launch: set-up and the producers' first reads overlap the pre-pass
     cudaLaunchConfig_t cfg = {};
@@ -778,7 +1035,99 @@ cudaError_t launch_gemm_tcgen05(const LayerView &L, const void *x, int B, void *
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel, tmap_out, P);
+    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2>, map, P);
+}
+
+template <int V>
+cudaError_t launch_gemm_v(const GemmPlan &pl, const CUtensorMap &map, const GemmParams &P, cudaStream_t st)
+{
+    if (pl.t1 == TABLE_SHARED) {
+        if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_SHARED, TABLE_NONE>(pl, map, P, st);
+        if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_SHARED, TABLE_SHARED>(pl, map, P, st);
+        return launch_gemm<V, TABLE_SHARED, TABLE_GLOBAL>(pl, map, P, st);
+    }
+    if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_GLOBAL, TABLE_NONE>(pl, map, P, st);
+    if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_GLOBAL, TABLE_SHARED>(pl, map, P, st);
+    return launch_gemm<V, TABLE_GLOBAL, TABLE_GLOBAL>(pl, map, P, st);
+}
+
+}  // namespace
+
+bool gemm_tcgen05_supported(const LayerView &L, int B)
+{
+    if (B < 1 || L.scale_rows || L.Nc <= 0) return false;
+    // (unit numbers are 32-bit: more than any batch that fits the device's memory needs)
+    return (L.v == 6 || L.v == 8 || L.v == 12) && ((long long)L.M / 96 + 1) * (B / 256 + 1) * (L.N / 16 + 16) < 0x7fffffffLL;
+}
+
+long long gemm_tcgen05_workspace_bytes(const LayerView &L, int B) { return plan_gemm(L, B).ws_bytes; }
+
+int gemm_tcgen05_launches(const LayerView &, int) { return 2; }   // pre-pass + GEMM
+
+bool gemm_tcgen05_waits_between_ctas(const LayerView &L, int B) { return plan_gemm(L, B).flag_order != 0; }
+
+cudaError_t launch_gemm_tcgen05(const LayerView &L, const void *x, int B, void *out, void *ws, cudaStream_t st)
+{
+    const GemmPlan pl = plan_gemm(L, B);
+    uint8_t *w8 = reinterpret_cast<uint8_t *>(ws);
+
+    // FP32 output with 16-byte aligned rows: the epilogue goes through shared memory and TMA
+    CUtensorMap tmap_out;
+    memset(&tmap_out, 0, sizeof(tmap_out));      // not read by the kernel when tma_out == 0
+    if (pl.tma_out) {
+        EncodeTiledFn encode = get_encode_fn();
+        if (encode == nullptr) return cudaErrorNotSupported;
+        const cuuint64_t odim[2] = {(cuuint64_t)L.M, (cuuint64_t)B};
+        const cuuint64_t ostride[1] = {(cuuint64_t)L.M * 4};
+        const cuuint32_t obox[2] = {32, PIECE_TOKENS};
+        const cuuint32_t estr[2] = {1, 1};
+        const CUresult r = encode(&tmap_out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, out, odim, ostride, obox, estr,
+                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+    }
+
+    PrepassParams Q;
+    memset(&Q, 0, sizeof(Q));
+    Q.L = L; Q.x = x; Q.B = B; Q.tile_n = pl.tile_n;
+    Q.img_main = pl.kb_main * (pl.ks / IMG_COLS); Q.img_total = pl.kb_total * (pl.ks / IMG_COLS);
+    Q.xs = w8 + pl.off_xs;
+    Q.bpart = reinterpret_cast<float *>(w8 + pl.off_bpart);
+    Q.status = reinterpret_cast<int *>(w8);
+    Q.tile_flags = reinterpret_cast<int *>(w8 + pl.off_flags); Q.n_flags = pl.tiles_m * pl.tiles_t * EPI_WARPS;
+    if (pl.scratch) { Q.zero = reinterpret_cast<float *>(w8 + pl.off_scratch); Q.n_zero = pl.n_scratch; }
+    else if (pl.any_split && !pl.flag_order) { Q.zero = reinterpret_cast<float *>(out); Q.n_zero = (long long)B * L.M; }
+    if (pl.pad_bytes && pl.t1 == TABLE_GLOBAL) Q.pad1 = w8 + pl.off_pad1;
+    if (pl.pad_bytes && pl.t2 == TABLE_GLOBAL) Q.pad2 = w8 + pl.off_pad2;
+    Q.pad_bytes = pl.pad_bytes;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(pl.pre_x, pl.pre_y, 1);
+    cfg.blockDim = dim3(PRE_THREADS, 1, 1);
+    cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_prepass_kernel, Q);
+    if (e != cudaSuccess) return e;
+
+    GemmParams P;
+    memset(&P, 0, sizeof(P));
+    P.L = L; P.out = out; P.B = B;
+    P.tiles_m = pl.tiles_m; P.tiles_t = pl.tiles_t; P.tile_n = pl.tile_n; P.n0 = pl.n0;
+    P.kb_main = pl.kb_main; P.kb_total = pl.kb_total; P.shares = pl.shares;
+    P.b_stages = pl.b_stages; P.cb1_shift = pl.cb1_shift; P.cb2_shift = pl.cb2_shift;
+    P.cb1_bytes = pl.cb1_bytes; P.cb2_bytes = pl.cb2_bytes;
+    P.flag_order = pl.flag_order; P.tma_out = pl.tma_out;
+    P.status = Q.status; P.bpart = Q.bpart; P.bias_parts = pl.pre_y; P.tile_flags = Q.tile_flags;
+    P.scratch = pl.scratch ? reinterpret_cast<float *>(w8 + pl.off_scratch) : nullptr;
+    P.xs = Q.xs;
+    P.tab1 = Q.pad1 ? Q.pad1 : reinterpret_cast<const uint8_t *>(L.c1);
+    P.tab2 = Q.pad2 ? Q.pad2 : reinterpret_cast<const uint8_t *>(L.c2);
+    if (L.v == 8) return launch_gemm_v<8>(pl, tmap_out, P, st);
+    if (L.v == 6) return launch_gemm_v<6>(pl, tmap_out, P, st);
+    return pl.t2 == TABLE_NONE ? launch_gemm<12, TABLE_GLOBAL, TABLE_NONE>(pl, tmap_out, P, st)
+                               : launch_gemm<12, TABLE_GLOBAL, TABLE_GLOBAL>(pl, tmap_out, P, st);
 }
 
 }  // namespace vptq

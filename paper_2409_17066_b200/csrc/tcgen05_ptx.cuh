@@ -56,6 +56,36 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// One lane of a converged warp.  A warp that runs its issue loop together and lets an elected lane execute the tcgen05
+// instructions keeps descriptors and barrier addresses in uniform registers; a loop that only one lane runs moves every
+// operand there first, one serial move after another.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t is;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(is));
+    return is != 0;
+}
+// Bounded wait for such a loop: the spin is one opaque block, so that the loop around it stays uniform for the compiler, and
+// giving up only sets `gave_up` (checked by the caller where it is cheap; a wait entered with it set polls once).
+__device__ __forceinline__ void mbar_wait_uniform(uint32_t bar, uint32_t parity, uint32_t &gave_up)
+{
+    asm volatile("{\n\t.reg .pred p, q;\n\t.reg .u64 t0, t1;\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "@p bra DONE;\n\t"
+                 "mov.u64 t0, %%clock64;\n\t"
+                 "AGAIN:\n\t"
+                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+                 "@p bra DONE;\n\t"
+                 "mov.u64 t1, %%clock64;\n\t"
+                 "sub.u64 t1, t1, t0;\n\t"
+                 "setp.lt.u64 q, t1, %3;\n\t"
+                 "setp.eq.and.u32 q, %0, 0, q;\n\t"
+                 "@q bra AGAIN;\n\t"
+                 "mov.u32 %0, 1;\n\t"
+                 "DONE:\n\t}"
+                 : "+r"(gave_up) : "r"(bar), "r"(parity), "n"(WAIT_LIMIT_CYCLES) : "memory");
+}
+
 // linear bulk copy global -> shared memory (16-byte aligned addresses, size a multiple of 16)
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
 {

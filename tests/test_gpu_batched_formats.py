@@ -1,0 +1,61 @@
+"""The batched tensor-core kernel where its tiles and pieces have edges: every vector length it takes, tables staged and in
+L2, outlier columns of both kinds, groups that end inside a column group, odd index widths, split tiles in every output type,
+several token tiles, few tokens (the decode families it serves from 5 tokens on)."""
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from oracle import oracle
+from paper_2409_17066_b200 import synth
+
+from helpers import TOL, rel_err
+
+pytestmark = pytest.mark.gpu
+
+V6 = dict(v=6, k1=4096, k2=256, n_out=7, v0=4, k0=4096)
+V12 = dict(v=12, k1=4096, k2=4096, n_out=13, v0=4, k0=8192, n_groups=4)
+
+
+@pytest.mark.parametrize("M,N,B,kw", [
+    (130, 700, 17, V6),                                                           # one tile and a short last row
+    (721, 1003, 300, dict(V6, out_dtype="fp32")),                                 # rows of an FP32 output that are no multiple of 4
+    (720, 1301, 256, dict(V6, n_out=33, v0=3, k0=100, permuted=True)),            # outlier vectors that straddle the tiles
+    (1210, 2100, 49, dict(v=6, k1=5000, k2=5000, out_dtype="bf16")),              # 13-bit indices, both tables padded in the workspace
+    (900, 515, 33, dict(v=6, k1=256, out_dtype="fp32")),                          # staged with copies, no residual
+    (1201, 1034, 40, dict(V12, out_dtype="bf16")),                                # groups that end inside a lane's 8 columns
+    (2400, 2222, 530, V12),                                                       # two token tiles, split tiles
+    (600, 640, 512, dict(v=12, k1=4096, out_dtype="fp32", has_scale=False)),      # no residual, no scale
+    (1100, 1000, 64, dict(v=8, k1=256, k2=256, n_out=9, v0=5, k0=37)),            # outlier vectors of 5
+    (1024, 2051, 97, dict(v=8, k1=4096, k2=4096, n_groups=3, x_dtype="bf16")),    # group-wise with v = 8
+    (1000, 4100, 5, dict(v=8, k1=65536, k2=256)),                                 # the decode families' batches
+    (1000, 1411, 16, dict(v=8, k1=65536, x_dtype="bf16", out_dtype="fp32")),
+    (1300, 1500, 6, V12),
+])
+def test_batched_kernel_formats_and_edges(M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    spec = synth.LayerSpec("bf", M, N, **kw)
+    d = synth.make_layer(spec, 89, B % 5, B)
+    dl = b.DeviceLayer(d)
+    y_ref = oracle.Layer.from_synth(d).linear(d["x"])
+    x = dl.upload_x(d["x"])
+    tol = TOL if spec.out_dtype != "bf16" else 2.0 ** -8
+    for _ in range(2):                                  # the workspace is reused
+        y = dl.linear(x)
+        assert b.vptq_workspace_status(dl.workspace(B)) == b.OK
+        assert rel_err(y.float().cpu().numpy(), y_ref) <= tol
+    shared = dl.with_flags(dl.desc.flags | b.FLAG_CONCURRENT)
+    assert b.lib.vptq_linear_waits_between_ctas(C.byref(shared.desc), B) == 0
+    assert rel_err(shared.linear(x).float().cpu().numpy(), y_ref) <= tol
+
+
+def test_batched_kernel_repeats_bit_for_bit_when_asked():
+    from paper_2409_17066_b200 import binding as b
+    spec = synth.LayerSpec("bd", 1210, 2100, **V6)
+    d = synth.make_layer(spec, 90, 0, 100)
+    dl = b.DeviceLayer(d)
+    det = dl.with_flags(dl.desc.flags | b.FLAG_DETERMINISTIC)
+    x = dl.upload_x(d["x"])
+    ys = [det.linear(x).clone() for _ in range(3)]
+    assert all(np.array_equal(y.cpu().numpy().view(np.uint16), ys[0].cpu().numpy().view(np.uint16)) for y in ys)
+    assert rel_err(ys[0].float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
