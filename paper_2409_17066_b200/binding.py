@@ -3,7 +3,9 @@
 Argument marshalling only: every function here passes device pointers of torch tensors
 (and torch's current CUDA stream) straight to the entry point of the same name.  torch is
 used for device memory and streams, nothing else; there is no CPU fallback — if the
-shared library is missing, importing this module fails.
+shared library is missing, importing this module fails.  The calls a decode loop makes per
+projection (vptq_linear, DeviceLayer.linear, FusedLayers.linear) marshal their arguments in
+the extension module _native (csrc/native_binding.cpp), the others through ctypes.
 """
 from __future__ import annotations
 
@@ -17,12 +19,14 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libvptq.so")
 
-if not os.path.exists(LIB_PATH):
-    raise ImportError(
-        f"{LIB_PATH} is missing: build it with `python -m paper_2409_17066_b200.build` "
-        "(there is no CPU fallback)")
+for _path in (LIB_PATH, os.path.join(_HERE, "_native.so")):
+    if not os.path.exists(_path):
+        raise ImportError(
+            f"{_path} is missing: build it with `python -m paper_2409_17066_b200.build` "
+            "(there is no CPU fallback)")
 
 lib = C.CDLL(LIB_PATH)
+from . import _native  # noqa: E402  (needs torch's and the library's symbols)
 
 OK = 0
 E_NULL, E_SHAPE, E_ALIGN, E_UNSUPPORTED, E_WORKSPACE, E_INDEX_RANGE, E_CUDA, E_TIMEOUT = range(-1, -9, -1)
@@ -112,6 +116,9 @@ class VptqError(RuntimeError):
         if code == E_CUDA:
             msg += ": " + lib.vptq_last_cuda_error().decode()
         super().__init__(f"libvptq error {code}: {msg}")
+
+
+_native.set_error_class(VptqError)
 
 
 def _check(code: int) -> None:
@@ -295,14 +302,8 @@ def vptq_linear_workspace_bytes(desc: LayerDesc, B: int) -> int:
 
 def vptq_linear(desc: LayerDesc, x: torch.Tensor, ptrs: LayerPtrs, out: torch.Tensor,
                 workspace: Optional[torch.Tensor]) -> torch.Tensor:
-    assert x.is_cuda and x.is_contiguous() and out.is_cuda and out.is_contiguous()
-    assert x.dtype == _TORCH_DT[desc.x_dtype] and out.dtype == _TORCH_DT[desc.out_dtype]
-    B = x.shape[0]
-    assert tuple(x.shape) == (B, desc.N) and tuple(out.shape) == (B, desc.M)
-    ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
-    _check(lib.vptq_linear(C.byref(desc), _ptr(x), B, C.byref(ptrs), _ptr(out),
-                           _ptr(workspace), ws_bytes, _stream()))
-    return out
+    """out [B][M] = x [B][N] * W^T; contiguous CUDA tensors of the descriptor's types (AssertionError otherwise)."""
+    return _native.linear(desc, x, ptrs, out, workspace)
 
 
 def _desc_array(descs: Sequence[LayerDesc]):
@@ -474,10 +475,11 @@ class DeviceLayer:
         return vptq_dequant(self.desc, self.ptrs, W)
 
     def linear(self, x: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
-        B = x.shape[0]
-        if out is None:
-            out = torch.empty((B, self.spec.M), dtype=_TORCH_DT[self.desc.out_dtype], device=self.device)
-        return vptq_linear(self.desc, x, self.ptrs, out, self.workspace(B))
+        y = _native.layer_linear(self.desc, self.ptrs, self._ws, x, out)
+        if y is None:                                    # first call at this batch size
+            self.workspace(x.shape[0])
+            y = _native.layer_linear(self.desc, self.ptrs, self._ws, x, out)
+        return y
 
 
 class FusedLayers:
@@ -506,12 +508,11 @@ class FusedLayers:
         return self._ws[B]
 
     def linear(self, x: torch.Tensor, outs: Sequence[torch.Tensor]) -> Sequence[torch.Tensor]:
-        B = x.shape[0]
-        ws = self.workspace(B)
-        out_ptrs = (C.c_void_p * self.n)(*[o.data_ptr() for o in outs])
-        _check(lib.vptq_linear_fused(self.descs, self.ptrs, self.n, _ptr(x), B, out_ptrs, _ptr(ws),
-                                     0 if ws is None else ws.numel(), _stream()))
-        return outs
+        r = _native.fused_linear(self.descs, self.ptrs, self.n, self._ws, x, outs)
+        if r is None:                                    # first call at this batch size
+            self.workspace(x.shape[0])
+            r = _native.fused_linear(self.descs, self.ptrs, self.n, self._ws, x, outs)
+        return r
 
     def linear_host_io(self, x_host: torch.Tensor, outs_host: Sequence[torch.Tensor], x_dev: torch.Tensor,
                        outs_dev: Sequence[torch.Tensor]) -> Sequence[torch.Tensor]:

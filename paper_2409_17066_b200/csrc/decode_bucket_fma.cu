@@ -517,7 +517,7 @@ cudaError_t launch_decode_bucket_fma(const LayerView *Ls, const void *const *ima
     const bool res = Ls[0].k2 > 0;
     const size_t smem = bucket_smem_bytes();
     auto kern = res ? decode_bucket_fma_kernel<true> : decode_bucket_fma_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
     // programmatic dependent launch: the prologue (barriers, tables, first blocks) runs under the previous kernel's tail
     return launch_dependent("bucket", kern, grid, BK_THREADS, smem, st, P);

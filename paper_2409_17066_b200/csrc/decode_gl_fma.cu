@@ -342,8 +342,7 @@ GlFmaPlan plan_gl_fma(const LayerView &L, int TB)
 template <int TB, int VV, bool RES, bool FUSED>
 cudaError_t launch_kernel(const GlFmaParams &P, const GlFmaPlan &pl, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(decode_gl_fma_kernel<TB, VV, RES, FUSED>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_gl_fma_kernel<TB, VV, RES, FUSED>), pl.smem);
     if (e != cudaSuccess) return e;
     decode_gl_fma_kernel<TB, VV, RES, FUSED><<<pl.grid, GL_WARPS * 32, pl.smem, st>>>(P);
     return cudaGetLastError();

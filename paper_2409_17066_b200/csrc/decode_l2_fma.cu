@@ -456,8 +456,7 @@ bool plan_l2_fused(const LayerView *Ls, int n, int TB, L2Plan *out)
 template <int TB, bool RES, bool OWNER, int WARPS, bool FUSED>
 cudaError_t launch_one(const L2FmaParams &P, const L2Plan &pl, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(decode_l2_fma_kernel<TB, RES, OWNER, WARPS, FUSED>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_l2_fma_kernel<TB, RES, OWNER, WARPS, FUSED>), pl.smem);
     if (e != cudaSuccess) return e;
     // Launched the ordinary way: as a programmatic dependent this kernel measured slower back to back (the
     // 70B-shaped layer 377 us per pass instead of 295 us), although its prologue is short.  It still lets the

@@ -348,8 +348,7 @@ SmemFmaPlan plan_smem_fma(const LayerView &L, int TB)
 template <int TB, int VV, bool RES, int WARPS, bool FUSED>
 cudaError_t launch_kernel(const SmemFmaParams &P, const SmemFmaPlan &pl, cudaStream_t st)
 {
-    cudaError_t e = cudaFuncSetAttribute(decode_smem_fma_kernel<TB, VV, RES, WARPS, FUSED>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_fma_kernel<TB, VV, RES, WARPS, FUSED>), pl.smem);
     if (e != cudaSuccess) return e;
     return launch_dependent("smem_fma", decode_smem_fma_kernel<TB, VV, RES, WARPS, FUSED>, pl.grid, WARPS * 32, pl.smem, st, P);
 }

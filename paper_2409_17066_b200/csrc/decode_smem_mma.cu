@@ -415,11 +415,11 @@ cudaError_t launch_variant(const SmemMmaParams &P, bool perm, int grid, size_t s
 {
     cudaError_t e;
     if (perm) {
-        e = cudaFuncSetAttribute(decode_smem_mma_kernel<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_mma_kernel<NT, true>), smem);
         if (e != cudaSuccess) return e;
         decode_smem_mma_kernel<NT, true><<<grid, THREADS, smem, st>>>(P);
     } else {
-        e = cudaFuncSetAttribute(decode_smem_mma_kernel<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_mma_kernel<NT, false>), smem);
         if (e != cudaSuccess) return e;
         decode_smem_mma_kernel<NT, false><<<grid, THREADS, smem, st>>>(P);
     }

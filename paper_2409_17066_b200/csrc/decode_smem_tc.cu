@@ -398,12 +398,12 @@ cudaError_t launch_decode_smem_tc(const LayerView &L, const void *x, int B, void
     if (e != cudaSuccess) return e;
     if (NT == 2) {
         auto kern = res ? decode_smem_tc_kernel<2, true> : decode_smem_tc_kernel<2, false>;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+        e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), pl.smem);
         if (e != cudaSuccess) return e;
         return launch_dependent("smem_tc", kern, pl.grid, TC_THREADS, pl.smem, st, P);
     }
     auto kern = res ? decode_smem_tc_kernel<1, true> : decode_smem_tc_kernel<1, false>;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+    e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), pl.smem);
     if (e != cudaSuccess) return e;
     return launch_dependent("smem_tc", kern, pl.grid, TC_THREADS, pl.smem, st, P);
 }

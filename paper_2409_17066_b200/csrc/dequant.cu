@@ -348,7 +348,7 @@ cudaError_t launch_restore(const RestoreParams &P, size_t smem, int cps, int gri
 {
     constexpr int CPL = restore_cpl<V>();
     auto kern = cps == CPL ? restore_kernel<V, RES, SMEM, CPL> : cps == 2 ? restore_kernel<V, RES, SMEM, 2> : restore_kernel<V, RES, SMEM, 1>;
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), smem);
     if (e != cudaSuccess) return e;
     kern<<<grid, RS_THREADS, smem, st>>>(P);
     return cudaGetLastError();

@@ -49,7 +49,7 @@ std::mutex g_smem_mutex;
 
 cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes)
 {
-    if (bytes <= 48 * 1024) return cudaSuccess;           // what every kernel may use without asking
+    if (bytes <= 40 * 1024) return cudaSuccess;           // with its static part inside the 48 KB every kernel may use
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
