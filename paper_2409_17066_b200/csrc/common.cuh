@@ -130,6 +130,10 @@ int device_sm_count();
 // (device_info.cu)
 cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes);
 
+// Clusters of `size` CTAs of `kernel` (threads and dynamic shared memory given) that are resident at once on the current
+// device, looked up once per kernel and device; 0 when the question has no answer (device_info.cu)
+int max_resident_clusters(const void *kernel, int size, int threads, size_t smem);
+
 // limit, in clock cycles, of the bounded device-side waits: 0 = each kernel's default (about two seconds);
 // set by vptq_debug_set_wait_limit, for tests that let a wait run out (device_info.cu)
 unsigned long long debug_wait_limit();

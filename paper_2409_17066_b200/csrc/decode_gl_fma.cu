@@ -2,7 +2,15 @@
 // (Sec. 3.1), vector lengths up to 16 (the published 2-bit models use v = 12 with two 4096-entry
 // codebooks per group, App. B table), any index width; batch 1..4 per launch, FP32 FMAs.
 //
-// Codebooks stay in global memory (a group's pair is 2 x k x 2v bytes; all groups together are a
+// Two kernels.  decode_gs_fma_kernel, for tables that fit shared memory group by group and layers large enough to fill
+// them, one or two tokens per launch: a cluster of G CTAs owns whole vector rows, each CTA the columns of one group with that
+// group's pair of tables staged (a plane of 16-byte pieces and one of 8- or 16-byte pieces per table: v = 12 takes one 16- and
+// one 8-byte read per row), and the partial sums meet through distributed shared memory.  What bounds it: the shared-memory
+// pipe, about 35 wavefronts per 32 index pairs with random rows (v = 12), and about 8 us of launch, staging and meeting.
+// 11008 x 4096, v = 12, two 4096-entry tables in each of four groups, one token: 65.7 -> 28.2 us (4096 x 4096 32.8 -> 17.3); a
+// decoder layer of a 7B model in that setting: 311 -> 129 us.
+//
+// decode_gl_fma_kernel, for everything else: codebooks stay in global memory (a group's pair is 2 x k x 2v bytes; all groups together are a
 // few hundred KB, L2-resident and partly L1-resident) and every index costs one random read of a
 // 2v-byte row (a3, a4).  Organisation as in the other decode kernels: persistent grid, one CTA per
 // SM owning whole vector rows; (vector row, 256-column chunk) tasks dealt out evenly over the warps;
@@ -62,6 +70,438 @@ __device__ __forceinline__ void load_row_words(const __half *__restrict__ tab, l
         for (int i = 0; i < VW; i++) w[i] = i < vw ? __ldg(p + i) : 0u;
     }
 }
+
+// ---- group tables in shared memory ---------------------------------------------------------------------------------
+
+constexpr size_t GS_SMEM_LIMIT = 226 * 1024;
+constexpr int GS_TABLE_BUDGET = 200 * 1024;
+constexpr int GS_MAX_CLUSTER = 8;
+constexpr int GS_WARPS = 32;
+
+struct GsFmaParams {
+    LayerView L[MAX_FUSED];        // layer l is the work of clusters [cluster_begin[l], cluster_begin[l + 1])
+    void *out[MAX_FUSED];
+    int cluster_begin[MAX_FUSED + 1];
+    int n_layers;
+    const void *x;
+    int B;                 // tokens in this launch (<= TB)
+    int slab_cols;         // columns of x*s staged at a time (a multiple of 256)
+    int n_out_pad;
+    int part_floats;
+};
+
+__device__ __forceinline__ float ld_cluster_f32(const float *p, int rank)
+{
+    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+    uint32_t r;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// dense table [k][v] -> plane A (components 0..7, 16 bytes) and plane B (components 8.., PB bytes), zero beyond v
+template <int PB>
+__device__ __forceinline__ void stage_planes(const __half *__restrict__ src, int k, int v, uint4 *pa, uint8_t *pb, int threads)
+{
+    const int vw = v >> 1;
+    if (PB == 8 && v == 12 && (k & 1) == 0) {
+        // 24-byte rows from a 16-byte aligned table (an even k keeps every group's table aligned): a thread takes two rows with
+        // three 16-byte loads, two such pairs in flight
+        const uint4 *s = reinterpret_cast<const uint4 *>(src);
+        for (int i0 = threadIdx.x; i0 < (k >> 1); i0 += 2 * threads) {
+            uint4 w[2][3];
+#pragma unroll
+            for (int u = 0; u < 2; u++)
+#pragma unroll
+                for (int c = 0; c < 3; c++)
+                    if (i0 + u * threads < (k >> 1)) w[u][c] = __ldg(s + 3 * (i0 + u * threads) + c);
+#pragma unroll
+            for (int u = 0; u < 2; u++) {
+                const int e = 2 * (i0 + u * threads);
+                if (e >= k) break;
+                pa[e] = w[u][0];
+                pa[e + 1] = make_uint4(w[u][1].z, w[u][1].w, w[u][2].x, w[u][2].y);
+                *reinterpret_cast<uint4 *>(pb + (size_t)e * 8) = make_uint4(w[u][1].x, w[u][1].y, w[u][2].z, w[u][2].w);
+            }
+        }
+        return;
+    }
+    for (int e = threadIdx.x; e < k; e += threads) {
+        const uint32_t *p = reinterpret_cast<const uint32_t *>(src) + (long long)e * vw;
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) w[i] = i < vw ? __ldg(p + i) : 0u;
+        pa[e] = make_uint4(w[0], w[1], w[2], w[3]);
+        if (PB == 8) reinterpret_cast<uint2 *>(pb)[e] = make_uint2(w[4], w[5]);
+        if (PB == 16) reinterpret_cast<uint4 *>(pb)[e] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+}
+
+template <int TB, int PB, bool RES>
+__global__ void __launch_bounds__(GS_WARPS * 32, 1)
+decode_gs_fma_kernel(const __grid_constant__ GsFmaParams P)
+{
+    constexpr int WARPS = GS_WARPS, THREADS = WARPS * 32;
+    constexpr int VW = 4 + PB / 4, VV = 2 * VW;                     // words and components of a staged row
+    extern __shared__ __align__(16) uint8_t smem[];
+    pdl_launch_dependents();
+    int li = 0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // rank within the cluster = column group; all layers of a launch have the same number of groups
+    const int G = P.L[0].G, g = (int)blockIdx.x % G, cid = (int)blockIdx.x / G;
+    while (li + 1 < P.n_layers && cid >= P.cluster_begin[li + 1]) li++;
+    const LayerView &L = P.L[li];
+    const int bid = cid - P.cluster_begin[li], gdim = P.cluster_begin[li + 1] - P.cluster_begin[li];
+
+    uint4 *t1a = reinterpret_cast<uint4 *>(smem);                                            // [k1]
+    uint4 *t2a = t1a + L.k1;                                                                 // [k2]
+    uint8_t *t1b = reinterpret_cast<uint8_t *>(t2a + (RES ? L.k2 : 0));                      // [k1][PB]
+    uint8_t *t2b = t1b + (size_t)L.k1 * PB;                                                  // [k2][PB]
+    uint8_t *end = t2b + (RES ? (size_t)L.k2 * PB : 0);
+    __half *xs = reinterpret_cast<__half *>(smem + ((size_t)(end - smem) + 15) / 16 * 16);   // [TB][slab_cols]
+    __half *xs_out = xs + (size_t)TB * P.slab_cols;                                          // [TB][n_out_pad]
+    float *part = reinterpret_cast<float *>(xs_out + (size_t)TB * P.n_out_pad);              // [rows][TB][16]
+    float *bterm = part + P.part_floats;                                                     // [4]
+    float *red = bterm + 4;                                                                  // [WARPS][4]
+
+    const int r0 = (int)((long long)L.R * bid / gdim), r1 = (int)((long long)L.R * (bid + 1) / gdim);
+    const int m_lo = r0 * L.v, m_hi = min(L.M, r1 * L.v);
+    // this group's main columns, and the 8-column boundary at or before the first of them
+    const int c_first = min(L.Nc, g * L.cpg), c_last = min(L.Nc, c_first + L.cpg);
+    const int c_base = c_first & ~7;
+
+    stage_planes<PB>(L.c1 + (long long)g * L.k1 * L.v, L.k1, L.v, t1a, t1b, THREADS);
+    if (RES) stage_planes<PB>(L.c2 + (long long)g * L.k2 * L.v, L.k2, L.v, t2a, t2b, THREADS);
+    for (int i = threadIdx.x; i < P.part_floats; i += THREADS) part[i] = 0.f;
+    if (threadIdx.x < 4) bterm[threadIdx.x] = 0.f;
+
+    const int cols = c_last - c_base;                            // columns to walk (at most 7 for a group without columns)
+    const int n_slabs = (cols + P.slab_cols - 1) / P.slab_cols;
+    for (int slab = 0; slab < max(1, n_slabs); slab++) {
+        const int s_begin = c_base + slab * P.slab_cols;
+        const int s_end = min(c_last, s_begin + P.slab_cols);
+        const int chunks = max(0, s_end - s_begin + 255) >> 8;
+
+        // ---- this warp's task range: (row, chunk of the slab), chunk fastest; first task's packed words ----
+        const int n_tasks = (r1 - r0) * chunks;
+        int q = (int)((long long)n_tasks * warp / WARPS);
+        const int q_end = (int)((long long)n_tasks * (warp + 1) / WARPS);
+        int r = r0 + (chunks ? q / chunks : 0), ch = chunks ? q % chunks : 0;
+        uint4 raw1 = make_uint4(0, 0, 0, 0), raw2 = make_uint4(0, 0, 0, 0);
+        if (q < q_end) {
+            const int grp = (s_begin >> 3) + ch * 32 + lane;
+            raw1 = load_raw8(L.s1.ptr + (long long)r * L.s1.stride, L.s1.stride, grp, s_end, L.s1.bits);
+            if (RES) raw2 = load_raw8(L.s2.ptr + (long long)r * L.s2.stride, L.s2.stride, grp, s_end, L.s2.bits);
+        }
+
+        // ---- x*s (FP16) of the slab, zero outside the group; the bias term of the group's own columns; slab 0 of the
+        // first CTA of the cluster adds the outlier columns' share (the activations may be the previous kernel's output)
+        pdl_wait();
+        {
+            float bacc[TB];
+#pragma unroll
+            for (int t = 0; t < TB; t++) bacc[t] = 0.f;
+#pragma unroll 2
+            for (int i = threadIdx.x; i < chunks * 256; i += THREADS) {
+                const int c = s_begin + i, n = L.n_out + c;
+                const bool mine = c >= c_first && c < s_end;
+                float sc = 1.f, bi = 0.f;
+                if (mine && L.has_scale) { sc = __half2float(__ldg(L.scale + n)); bi = __half2float(__ldg(L.bias + n)); }
+                const long long f = mine ? in_col(L, n) : 0;
+#pragma unroll
+                for (int t = 0; t < TB; t++) {
+                    const float xv = mine && t < P.B ? load_act(P.x, (long long)t * L.N + f, L.x_bf16) : 0.f;
+                    xs[t * P.slab_cols + i] = __float2half_rn(xv * sc);
+                    bacc[t] += xv * bi;
+                }
+            }
+            if (slab == 0) {
+                for (int n = threadIdx.x; n < L.n_out; n += THREADS) {
+                    float sc = 1.f, bi = 0.f;
+                    if (L.has_scale) { sc = __half2float(__ldg(L.scale + n)); bi = __half2float(__ldg(L.bias + n)); }
+                    const long long f = in_col(L, n);
+#pragma unroll
+                    for (int t = 0; t < TB; t++) {
+                        const float xv = t < P.B ? load_act(P.x, (long long)t * L.N + f, L.x_bf16) : 0.f;
+                        xs_out[t * P.n_out_pad + n] = __float2half_rn(xv * sc);
+                        if (g == 0) bacc[t] += xv * bi;
+                    }
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < TB; t++) {
+                float a = bacc[t];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                if (lane == 0) red[warp * 4 + t] = a;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < TB) {
+            float a = bterm[threadIdx.x];
+            for (int w = 0; w < WARPS; w++) a += red[w * 4 + threadIdx.x];
+            bterm[threadIdx.x] = a;
+        }
+
+        // ---- a5: outlier columns, the outlier rows shared out over the cluster's warps ----
+        if (slab == 0 && L.n_out > 0) {
+            const int q_lo = m_lo / L.v0, q_hi = (m_hi + L.v0 - 1) / L.v0;
+            for (int qq = q_lo + warp * G + g; qq < q_hi; qq += WARPS * G) {
+                const uint8_t *row0 = L.s0.ptr + (long long)qq * L.s0.stride;
+                float oacc[8][TB];
+#pragma unroll
+                for (int j = 0; j < 8; j++)
+#pragma unroll
+                    for (int t = 0; t < TB; t++) oacc[j][t] = 0.f;
+                for (int n = lane; n < L.n_out; n += 32) {
+                    const int i0 = clamp_index(load_index(row0, n, L.s0.bits), L.k0);
+                    const uint4 cw = load_centroid_row(L.c0, i0, L.v0);
+                    const float2 c01 = h2f(cw.x), c23 = h2f(cw.y), c45 = h2f(cw.z), c67 = h2f(cw.w);
+                    const float cj[8] = {c01.x, c01.y, c23.x, c23.y, c45.x, c45.y, c67.x, c67.y};
+#pragma unroll
+                    for (int t = 0; t < TB; t++) {
+                        const float xv = __half2float(xs_out[t * P.n_out_pad + n]);
+#pragma unroll
+                        for (int j = 0; j < 8; j++) oacc[j][t] += xv * cj[j];
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < 8; j++) {
+                    if (j >= L.v0) break;
+#pragma unroll
+                    for (int t = 0; t < TB; t++) {
+                        float a = oacc[j][t];
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+                        const int m = qq * L.v0 + j;
+                        if (lane == 0 && m >= m_lo && m < m_hi) {
+                            const int rr = m / L.v, jj = m - rr * L.v;
+                            atomicAdd(part + ((rr - r0) * TB + t) * 16 + jj, a);
+                        }
+                    }
+                }
+            }
+        }
+
+        // ---- main tasks ----
+        float acc[TB][VV];
+#pragma unroll
+        for (int t = 0; t < TB; t++)
+#pragma unroll
+            for (int j = 0; j < VV; j++) acc[t][j] = 0.f;
+        while (q < q_end) {
+            uint32_t w1[4], w2[4] = {0, 0, 0, 0};
+            decode8(raw1, L.s1.bits, L.k1, w1);
+            if (RES) decode8(raw2, L.s2.bits, L.k2, w2);
+            const int cur_r = r, cur_ch = ch;
+            q++;
+            if (++ch == chunks) { ch = 0; r++; }
+            if (q < q_end) {
+                const int grp = (s_begin >> 3) + ch * 32 + lane;
+                raw1 = load_raw8(L.s1.ptr + (long long)r * L.s1.stride, L.s1.stride, grp, s_end, L.s1.bits);
+                if (RES) raw2 = load_raw8(L.s2.ptr + (long long)r * L.s2.stride, L.s2.stride, grp, s_end, L.s2.bits);
+            }
+            if (s_begin + cur_ch * 256 + lane * 8 < s_end) {
+                uint4 xv4[TB];
+#pragma unroll
+                for (int t = 0; t < TB; t++)
+                    xv4[t] = *reinterpret_cast<const uint4 *>(xs + t * P.slab_cols + cur_ch * 256 + lane * 8);
+#pragma unroll
+                for (int s0 = 0; s0 < 8; s0 += 2) {
+                    // two columns' rows in flight
+                    uint32_t cw[2][VW], rw[2][VW];
+#pragma unroll
+                    for (int u = 0; u < 2; u++) {
+                        const int s = s0 + u;
+                        auto fetch = [&](const uint4 *ta, const uint8_t *tb, uint32_t id, uint32_t (&w)[VW]) {
+                            const uint4 a = ta[id];
+                            w[0] = a.x; w[1] = a.y; w[2] = a.z; w[3] = a.w;
+                            if (PB == 8) { const uint2 b = reinterpret_cast<const uint2 *>(tb)[id]; w[4 % VW] = b.x; w[5 % VW] = b.y; }
+                            if (PB == 16) {
+                                const uint4 b = reinterpret_cast<const uint4 *>(tb)[id];
+                                w[4 % VW] = b.x; w[5 % VW] = b.y; w[6 % VW] = b.z; w[7 % VW] = b.w;
+                            }
+                        };
+                        fetch(t1a, t1b, (w1[s >> 1] >> (16 * (s & 1))) & 0xFFFFu, cw[u]);
+                        if (RES) fetch(t2a, t2b, (w2[s >> 1] >> (16 * (s & 1))) & 0xFFFFu, rw[u]);
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; u++) {
+                        const int s = s0 + u;
+#pragma unroll
+                        for (int i = 0; i < VW; i++) {
+                            uint32_t w = cw[u][i];
+                            if (RES) {      // summed in FP16 (one rounding of 2^-11)
+                                const __half2 a = __hadd2(*reinterpret_cast<__half2 *>(&w), *reinterpret_cast<const __half2 *>(&rw[u][i]));
+                                w = *reinterpret_cast<const uint32_t *>(&a);
+                            }
+#pragma unroll
+                            for (int t = 0; t < TB; t++) {
+                                const uint32_t xw = (s >> 1) == 0 ? xv4[t].x : (s >> 1) == 1 ? xv4[t].y : (s >> 1) == 2 ? xv4[t].z : xv4[t].w;
+                                fma_f16x2(acc[t][2 * i], acc[t][2 * i + 1], xw, (s & 1) != 0, w);
+                            }
+                        }
+                    }
+                }
+            }
+            if (q < q_end && r == cur_r) continue;
+
+            // ---- row change (or end of range): halving butterfly over 16*TB values per lane ----
+            constexpr int NV = 16 * TB;
+            float v[NV];
+#pragma unroll
+            for (int t = 0; t < TB; t++)
+#pragma unroll
+                for (int j = 0; j < 16; j++) {
+                    v[t * 16 + j] = j < VV ? acc[t][j < VV ? j : 0] : 0.f;
+                    if (j < VV) acc[t][j < VV ? j : 0] = 0.f;
+                }
+            const int vi = halving_butterfly<NV>(v, lane);
+            constexpr int KEEP = NV >= 32 ? NV / 32 : 1;
+            constexpr int dup = NV >= 32 ? 1 : 32 / NV;
+            if ((lane & (dup - 1)) == 0) {
+#pragma unroll
+                for (int k = 0; k < KEEP; k++) {
+                    const int idx = vi + k, t = idx >> 4, j = idx & 15;
+                    if (j < VV) atomicAdd(part + ((cur_r - r0) * TB + t) * 16 + j, v[k]);
+                }
+            }
+        }
+        __syncthreads();      // the slab's xs is dead; part[] complete after the last slab
+    }
+
+    // ---- the groups' sums meet: every CTA of the cluster finishes a share of the outputs ----
+    if (G > 1) cluster_sync();
+    const int n_m = m_hi - m_lo;
+    for (int i = g * THREADS + threadIdx.x; i < n_m * P.B; i += G * THREADS) {
+        const int t = i / n_m, ml = i % n_m;       // consecutive threads -> consecutive m
+        const int m = m_lo + ml, rr = m / L.v, jj = m - rr * L.v;
+        const float *p = part + ((rr - r0) * TB + t) * 16 + jj;
+        float y = 0.f;
+        if (G == 1) y = *p + bterm[t];
+        else for (int k = 0; k < G; k++) y += ld_cluster_f32(p, k) + ld_cluster_f32(bterm + t, k);
+        store_out(P.out[li], (long long)t * L.M + m, y, L.out_dtype);
+    }
+    if (G > 1) cluster_sync();                     // nobody leaves while its sums may still be read
+}
+
+struct GsFmaPlan {
+    int slab_cols, n_out_pad, part_floats, clusters, pb;
+    size_t smem;
+    bool ok;
+    int cluster_begin[MAX_FUSED + 1];
+};
+
+template <int TB, int PB, bool RES>
+const void *gs_kernel_ptr() { return reinterpret_cast<const void *>(decode_gs_fma_kernel<TB, PB, RES>); }
+template <int TB>
+const void *gs_kernel(int pb, bool res)
+{
+    if (pb == 0) return res ? gs_kernel_ptr<TB, 0, true>() : gs_kernel_ptr<TB, 0, false>();
+    if (pb == 8) return res ? gs_kernel_ptr<TB, 8, true>() : gs_kernel_ptr<TB, 8, false>();
+    return res ? gs_kernel_ptr<TB, 16, true>() : gs_kernel_ptr<TB, 16, false>();
+}
+
+// n layers of one format (apart from M), TB = 1 or 2
+GsFmaPlan plan_gs_fma(const LayerView *Ls, int n, int TB)
+{
+    GsFmaPlan p;
+    memset(&p, 0, sizeof(p));
+    const LayerView &L = Ls[0];
+    p.pb = L.v <= 8 ? 0 : L.v <= 12 ? 8 : 16;
+    const long long tables = ((long long)(L.k1 + L.k2) * (16 + p.pb) + 15) / 16 * 16;
+    if (TB > 2 || n < 1 || n > MAX_FUSED || L.G > GS_MAX_CLUSTER || (L.G & (L.G - 1)) != 0 || tables > GS_TABLE_BUDGET) return p;
+    long long rows = 0;
+    for (int l = 0; l < n; l++) rows += Ls[l].R;
+    // clusters that are resident at once: a GPC's SMs need not be a multiple of the cluster size
+    const void *kernel = TB == 2 ? gs_kernel<2>(p.pb, L.k2 > 0) : gs_kernel<1>(p.pb, L.k2 > 0);
+    p.clusters = L.G == 1 ? device_sm_count() : max_resident_clusters(kernel, L.G, GS_WARPS * 32, GS_SMEM_LIMIT);
+    if (p.clusters < 1) return p;
+    if (p.clusters > rows) p.clusters = (int)rows;
+    // Staging a group's tables (8192 rows of 24 bytes in about 3 us) pays from a few thousand index pairs per CTA on: a pair
+    // costs about 4 times as much out of L2.
+    if (rows * L.cpg * 4 < (long long)p.clusters * (L.k1 + L.k2)) return p;
+    int rows_cluster = ceil_div(Ls[0].R, p.clusters);
+    p.cluster_begin[1] = p.clusters;
+    if (n > 1) {
+        int R[MAX_FUSED];
+        for (int l = 0; l < n; l++) R[l] = Ls[l].R;
+        if (!split_ctas(R, n, p.clusters, p.cluster_begin, &rows_cluster)) return p;
+    }
+    p.part_floats = rows_cluster * TB * 16;
+    p.n_out_pad = (L.n_out + 7) / 8 * 8;
+    const long long fixed = tables + (long long)TB * p.n_out_pad * 2 + (long long)p.part_floats * 4 + 16 + GS_WARPS * 16;
+    long long slab = ((long long)GS_SMEM_LIMIT - fixed) / (2 * TB) / 256 * 256;
+    const int most = (L.cpg + 7 + 255) / 256 * 256;
+    if (slab > most) slab = most;
+    if (slab < 256) return p;
+    p.slab_cols = (int)slab;
+    p.smem = (size_t)(fixed + slab * 2 * TB);
+    p.ok = true;
+    return p;
+}
+
+template <int TB, int PB, bool RES>
+cudaError_t launch_gs(const GsFmaParams &P, const GsFmaPlan &pl, cudaStream_t st)
+{
+    const cudaError_t e = allow_dynamic_smem(gs_kernel_ptr<TB, PB, RES>(), GS_SMEM_LIMIT);
+    if (e != cudaSuccess) return e;
+    const int G = P.L[0].G;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(pl.clusters * G));
+    cfg.blockDim = dim3(GS_WARPS * 32);
+    cfg.dynamicSmemBytes = pl.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (pdl_enabled("gl_fma")) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (G > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = (unsigned)G; attr[na].val.clusterDim.y = 1; attr[na].val.clusterDim.z = 1;
+        na++;
+    }
+    cfg.attrs = attr; cfg.numAttrs = (unsigned)na;
+    return cudaLaunchKernelEx(&cfg, decode_gs_fma_kernel<TB, PB, RES>, P);
+}
+
+template <int TB>
+cudaError_t launch_gs_group(const GsFmaParams &P, const GsFmaPlan &pl, cudaStream_t st)
+{
+    const bool res = P.L[0].k2 > 0;
+    if (pl.pb == 0) return res ? launch_gs<TB, 0, true>(P, pl, st) : launch_gs<TB, 0, false>(P, pl, st);
+    if (pl.pb == 8) return res ? launch_gs<TB, 8, true>(P, pl, st) : launch_gs<TB, 8, false>(P, pl, st);
+    return res ? launch_gs<TB, 16, true>(P, pl, st) : launch_gs<TB, 16, false>(P, pl, st);
+}
+
+cudaError_t launch_decode_gs_fma(const LayerView *Ls, int n, const GsFmaPlan &pl, int TB, const void *x, int B, void *const *outs,
+                                 cudaStream_t st)
+{
+    for (int t0 = 0; t0 < B; t0 += TB) {
+        GsFmaParams P;
+        memset(&P, 0, sizeof(P));
+        for (int l = 0; l < n; l++) {
+            P.L[l] = Ls[l];
+            P.out[l] = reinterpret_cast<uint8_t *>(outs[l]) + (size_t)t0 * Ls[l].M * (Ls[l].out_dtype == VPTQ_DTYPE_FP32 ? 4 : 2);
+        }
+        for (int l = 0; l <= n; l++) P.cluster_begin[l] = pl.cluster_begin[l];
+        P.n_layers = n; P.B = (B - t0 < TB) ? (B - t0) : TB;
+        P.x = reinterpret_cast<const uint8_t *>(x) + (size_t)t0 * Ls[0].N * 2;
+        P.slab_cols = pl.slab_cols; P.n_out_pad = pl.n_out_pad; P.part_floats = pl.part_floats;
+        const cudaError_t e = TB == 2 ? launch_gs_group<2>(P, pl, st) : launch_gs_group<1>(P, pl, st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+// ---- tables in global memory ---------------------------------------------------------------------------------------
 
 template <int TB, int VV, bool RES, bool FUSED>
 __global__ void __launch_bounds__(GL_WARPS * 32, 1)
@@ -405,6 +845,8 @@ int gl_fma_launches(const LayerView &L, int B)
 cudaError_t launch_decode_gl_fma(const LayerView &L, const void *x, int B, void *out, cudaStream_t st)
 {
     const int TB = gl_token_group(B);
+    const GsFmaPlan gs = plan_gs_fma(&L, 1, TB);
+    if (gs.ok) return launch_decode_gs_fma(&L, 1, gs, TB, x, B, &out, st);
     const GlFmaPlan pl = plan_gl_fma(L, TB);
     const size_t xe = 2, oe = (L.out_dtype == VPTQ_DTYPE_FP32) ? 4 : 2;
     const bool res = L.k2 > 0;
@@ -439,6 +881,8 @@ cudaError_t launch_decode_gl_fma_fused(const LayerView *Ls, int n, const void *x
     const int TB = gl_token_group(B);
     GlFmaPlan pl;
     if (!plan_gl_fma_fused(Ls, n, TB, &pl)) return cudaErrorInvalidValue;
+    const GsFmaPlan gs = plan_gs_fma(Ls, n, TB);
+    if (gs.ok) return launch_decode_gs_fma(Ls, n, gs, TB, x, B, outs, st);
     const bool res = Ls[0].k2 > 0;
     for (int t0 = 0; t0 < B; t0 += TB) {
         GlFmaParams P;

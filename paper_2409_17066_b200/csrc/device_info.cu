@@ -81,6 +81,46 @@ cudaError_t allow_dynamic_smem(const void *kernel, size_t bytes)
     return e;
 }
 
+namespace {
+struct ClusterSlot { const void *kernel; int dev, size, answer; };
+ClusterSlot g_clusters[256];
+std::atomic<int> g_n_clusters{0};
+std::mutex g_clusters_mutex;
+}
+
+int max_resident_clusters(const void *kernel, int size, int threads, size_t smem)
+{
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 148 / size;      // size queries without a device: those of a B200
+    auto find = [&](int n) {
+        for (int i = 0; i < n; i++)
+            if (g_clusters[i].kernel == kernel && g_clusters[i].dev == dev && g_clusters[i].size == size) return g_clusters[i].answer;
+        return -1;
+    };
+    int a = find(g_n_clusters.load(std::memory_order_acquire));
+    if (a >= 0) return a;
+    std::lock_guard<std::mutex> lock(g_clusters_mutex);
+    const int n = g_n_clusters.load(std::memory_order_relaxed);
+    if ((a = find(n)) >= 0) return a;
+    a = 0;
+    if (allow_dynamic_smem(kernel, smem) == cudaSuccess) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)size * 1024u);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&a, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); a = 0; }
+    }
+    if (n < 256) {
+        g_clusters[n] = {kernel, dev, size, a};
+        g_n_clusters.store(n + 1, std::memory_order_release);
+    }
+    return a;
+}
+
 bool pdl_enabled(const char *family)
 {
     static const char *off = getenv("VPTQ_NO_PDL");          // read once

@@ -34,12 +34,12 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
     return PATH_GENERIC;
 }
 
-// 5 to 16 tokens of the families that read their tables out of L2 take at most four tokens per launch and gather every
-// centroid again for the next four; the batched kernel gathers it once whatever the batch (4096 x 4096 over the 1 MiB table:
-// 25 us at any batch up to 64, against 14 us per four tokens).
+// The families whose main tables are in L2 or group-wise take at most four or two tokens per launch and gather every centroid
+// again for the next ones; the batched kernel gathers it once whatever the batch.  4096 x 4096 over the 1 MiB table: 25 us
+// at any batch up to 64, against 14-17 us per four tokens; 11008 x 4096, v = 12 in four groups: 52 us against 31 us per two.
 static bool batched_decode(LinearPath path, const LayerView &L, int B)
 {
-    return (path == PATH_DECODE_L2_FMA || path == PATH_DECODE_GL_FMA) && B >= 5 && !L.deterministic && gemm_tcgen05_supported(L, B);
+    return ((path == PATH_DECODE_L2_FMA && B >= 5) || (path == PATH_DECODE_GL_FMA && B >= 3)) && !L.deterministic && gemm_tcgen05_supported(L, B);
 }
 
 const char *linear_path_name(const LayerView &L, int B, int flags)
