@@ -213,9 +213,13 @@ int vptq_linear(const vptq_layer_desc *desc, const void *x, int32_t B,
  * or "decode_gl_fma" (B <= 4; for these two the layers must also share their format apart from M: v,
  * codebook sizes, outlier columns, groups, scale flag) and whole vector rows of the layers spread evenly
  * over the SMs, one kernel per token group serves all layers (no launch, prologue and ragged tail per
- * layer; no scratch); otherwise the layers run one after the other on `stream`, sharing the workspace.
+ * layer; no scratch).  Layers of one format apart from M that the batched tensor-core kernel takes share
+ * one launch of it and of its pre-pass from 65 tokens on, and from 3 tokens on where that is faster than
+ * their own launches; its scratch starts with a status word like that of "gemm_tcgen05".  Otherwise the
+ * layers run one after the other on `stream`, sharing the workspace.
  * vptq_linear_fused_path() names which: "fused_decode_l2_fma", "fused_decode_smem_fma",
- * "fused_decode_gl_fma" or "one_by_one" ("invalid" for arguments the call would reject).  Each layer's
+ * "fused_decode_gl_fma", "fused_gemm_tcgen05" (up to 8 tokens over a table in L2 still
+ * "fused_decode_l2_fma") or "one_by_one" ("invalid" for arguments the call would reject).  Each layer's
  * result is the one vptq_linear gives for it (same arithmetic, same summation order within a vector
  * row).  Errors as for vptq_linear; nothing is launched when an argument is rejected. */
 #define VPTQ_MAX_FUSED_LAYERS 4

@@ -55,6 +55,7 @@ struct LayerView {
     const __half *c1, *c2, *c0;
     const __half *scale, *bias;
     const int *perm;       // nullptr, or [N]: stored column n is input feature perm[n] (Sec. 3.2.3)
+    int permuted;          // perm is (or, without pointers, will be) set
     const void *prepared;  // nullptr, or the prepared image of the layer
     int prep_parts;        // partitions of the prepared image
     int concurrent;        // the call may share the GPU: no waits between CTAs of a grid

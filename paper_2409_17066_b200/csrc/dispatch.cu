@@ -58,13 +58,13 @@ const char *linear_path_name(const LayerView &L, int B, int flags)
 long long linear_workspace_bytes(const LayerView &L, int B, int flags)
 {
     const LinearPath path = choose_path(L, B, flags);
-    if (batched_decode(path, L, B)) return gemm_tcgen05_workspace_bytes(L, B);
+    if (batched_decode(path, L, B)) return gemm_tcgen05_workspace_bytes(&L, 1, B);
     switch (path) {
     case PATH_DECODE_SMEM_FMA: return 0;
     case PATH_DECODE_SMEM_MMA: return smem_mma_workspace_bytes(L, decode_group(B));
     case PATH_DECODE_L2_FMA: return l2_fma_workspace_bytes(L, decode_group(B));
     case PATH_DECODE_GL_FMA: return 0;
-    case PATH_GEMM_TCGEN05: return gemm_tcgen05_workspace_bytes(L, B);
+    case PATH_GEMM_TCGEN05: return gemm_tcgen05_workspace_bytes(&L, 1, B);
     case PATH_DECODE_BUCKET_FMA: return (long long)bucket_fma_workspace_bytes(&L, &L.prep_parts, 1);
     default: return generic_workspace_bytes(L, B);
     }
@@ -98,7 +98,7 @@ int linear_dispatch(const LayerView &L, int flags, const void *x, int B, void *o
     if (path == PATH_GENERIC) {
         e = launch_linear_generic(L, x, B, out, ws, st);
     } else if (path == PATH_GEMM_TCGEN05 || batched_decode(path, L, B)) {
-        e = launch_gemm_tcgen05(L, x, B, out, ws, st);
+        e = launch_gemm_tcgen05(&L, 1, x, B, &out, ws, st);
     } else if (path == PATH_DECODE_BUCKET_FMA) {
         const void *img = L.prepared;
         void *o = out;
@@ -122,15 +122,34 @@ int linear_dispatch(const LayerView &L, int flags, const void *x, int B, void *o
 
 // ---- several layers that read the same activations ---------------------------------------------------
 
+// Whether layers whose own calls would take `path` are better off in one launch of the batched kernel, which costs one
+// set-up for all of them: a 7B layer's q+k+v+o (1024 rows of k and v) at 16 tokens takes 50 us instead of 76 over the 1 MiB
+// table, 70 instead of 100 with v = 12 in four groups.  Tables in shared memory have a decode kernel that takes a weight
+// for a little over half of the time, after 9 us (18 us with a residual table and 16 tokens) a layer: q+k+v+o with v = 6
+// 102 -> 65 us at 16 tokens, 82 -> 58 at 8, but gate+up of 11008 x 4096 79 -> 87 us at 8, and with 256 centroids and no
+// residual 42 -> 56.  From 17 to 64 tokens large layers, which fill the SMs on their own, keep sharing one layer's scratch.
+static bool fused_batched(LinearPath path, const LayerView *Ls, int n, int B)
+{
+    long long weights = 0;
+    for (int l = 0; l < n; l++) weights += (long long)Ls[l].M * Ls[l].N;
+    if (path == PATH_DECODE_SMEM_MMA) return weights <= ((n - 1LL) << (25 + (B > 8) + (Ls[0].k2 > 0)));
+    return path != PATH_GEMM_TCGEN05 || B > 64 || weights <= ((n - 1LL) << 26);
+}
+
 // The kernel family that serves all n layers with one launch per token group, or PATH_GENERIC when there is none.
 LinearPath fused_path(const LayerView *Ls, const int *flags, int n, int B)
 {
-    if (n < 2 || B > DECODE_MAX_B) return PATH_GENERIC;
+    if (n < 2) return PATH_GENERIC;
     for (int l = 0; l < n; l++)
         if (Ls[l].deterministic) return PATH_GENERIC;          // one layer after the other
     const LinearPath path = choose_path(Ls[0], B, flags[0]);
     for (int l = 1; l < n; l++)
         if (choose_path(Ls[l], B, flags[l]) != path) return PATH_GENERIC;
+    if (path == PATH_GEMM_TCGEN05 || batched_decode(path, Ls[0], B) || path == PATH_DECODE_SMEM_MMA) {
+        if (fused_batched(path, Ls, n, B) && gemm_tcgen05_fused_supported(Ls, n, B)) return PATH_GEMM_TCGEN05;
+        if (path != PATH_DECODE_L2_FMA || B > 8) return PATH_GENERIC;
+    }
+    if (B > DECODE_MAX_B) return PATH_GENERIC;
     if (path == PATH_DECODE_BUCKET_FMA) {
         // prepared layers share a launch when their partitions fit the SMs side by side
         int ctas = 0;
@@ -140,10 +159,6 @@ LinearPath fused_path(const LayerView *Ls, const int *flags, int n, int B)
         }
         return (n <= MAX_FUSED && ctas <= device_sm_count()) ? path : PATH_GENERIC;
     }
-    // The layers one by one through the batched kernel are faster than several fused launches: past 8 tokens with the 1 MiB
-    // table (q+k+v+o of 4096 x 4096 at 9 tokens 133 -> 87 us; 8 tokens 82 fused), always with group-wise tables (v = 12
-    // gate+up+down of a 7B layer at 8 tokens 580 -> 164 us)
-    if (batched_decode(path, Ls[0], B) && (B > 8 || path == PATH_DECODE_GL_FMA)) return PATH_GENERIC;
     if (path == PATH_DECODE_L2_FMA && l2_fma_fused_supported(Ls, n, B)) return path;
     if (path == PATH_DECODE_SMEM_FMA && smem_fma_fused_supported(Ls, n, B)) return path;
     if (path == PATH_DECODE_GL_FMA && gl_fma_fused_supported(Ls, n, B)) return path;
@@ -152,11 +167,15 @@ LinearPath fused_path(const LayerView *Ls, const int *flags, int n, int B)
 
 const char *linear_fused_path_name(const LayerView *Ls, const int *flags, int n, int B)
 {
-    switch (fused_path(Ls, flags, n, B)) {
+    const LinearPath path = fused_path(Ls, flags, n, B);
+    // (up to 8 tokens callers know these layers by the decode family's name, whichever kernel takes them)
+    if (path == PATH_GEMM_TCGEN05 && B <= 8 && choose_path(Ls[0], B, flags[0]) == PATH_DECODE_L2_FMA) return "fused_decode_l2_fma";
+    switch (path) {
     case PATH_DECODE_L2_FMA: return "fused_decode_l2_fma";
     case PATH_DECODE_SMEM_FMA: return "fused_decode_smem_fma";
     case PATH_DECODE_GL_FMA: return "fused_decode_gl_fma";
     case PATH_DECODE_BUCKET_FMA: return "fused_decode_bucket_fma";
+    case PATH_GEMM_TCGEN05: return "fused_gemm_tcgen05";
     default: return "one_by_one";
     }
 }
@@ -169,6 +188,7 @@ long long linear_fused_workspace_bytes(const LayerView *Ls, const int *flags, in
         for (int l = 0; l < n; l++) parts[l] = Ls[l].prep_parts;
         return (long long)bucket_fma_workspace_bytes(Ls, parts, n);
     }
+    if (fp == PATH_GEMM_TCGEN05) return gemm_tcgen05_workspace_bytes(Ls, n, B);
     if (fp != PATH_GENERIC) return 0;
     long long need = 0;       // one layer after the other on the stream: they share the scratch
     for (int l = 0; l < n; l++) {
@@ -185,6 +205,7 @@ int linear_fused_launches(const LayerView *Ls, const int *flags, int n, int B)
     if (path == PATH_DECODE_SMEM_FMA) return smem_fma_launches(Ls[0], B);      // one launch per token group
     if (path == PATH_DECODE_GL_FMA) return gl_fma_launches(Ls[0], B);
     if (path == PATH_DECODE_BUCKET_FMA) return 1;
+    if (path == PATH_GEMM_TCGEN05) return gemm_tcgen05_launches(Ls[0], B);
     int total = 0;
     for (int l = 0; l < n; l++) total += linear_launches(Ls[l], B, flags[l]);
     return total;
@@ -195,7 +216,8 @@ int linear_fused_dispatch(const LayerView *Ls, const int *flags, int n, const vo
 {
     const LinearPath path = fused_path(Ls, flags, n, B);
     if (path != PATH_GENERIC) {
-        if (path == PATH_DECODE_L2_FMA) *cuda_err = launch_decode_l2_fma_fused(Ls, n, x, B, outs, st);
+        if (path == PATH_GEMM_TCGEN05) *cuda_err = launch_gemm_tcgen05(Ls, n, x, B, outs, ws, st);
+        else if (path == PATH_DECODE_L2_FMA) *cuda_err = launch_decode_l2_fma_fused(Ls, n, x, B, outs, st);
         else if (path == PATH_DECODE_BUCKET_FMA) {
             const void *imgs[MAX_FUSED];
             int parts[MAX_FUSED];

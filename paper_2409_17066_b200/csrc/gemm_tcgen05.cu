@@ -46,6 +46,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "fused_split.cuh"
 #include "gemm.cuh"
 #include "index_words.cuh"
 #include "tcgen05_ptx.cuh"
@@ -139,6 +140,20 @@ struct GemmParams {
     float *scratch;      // [tiles][4][scratch_rows(tile_n)][32] FP32 sums of split tiles, or null
     const uint8_t *xs;   // activation images, [tiles_t][kb_total * KS / 32][tile_n * 64 bytes]
     const uint8_t *tab1, *tab2;     // tables read from global memory: rows of 16 (v <= 8) or 32 bytes
+};
+
+// One launch: layer l is the work of CTAs [cta_begin[l], cta_begin[l + 1]).  (A launch of one layer has kernels of its own:
+// parameters found by an index are loads instead of operands.  The maps are a parameter of their own for the same reason:
+// their address is taken, and with them in one struct 17 tokens x 8192 columns took 26.5 us instead of 24.)
+template <int NL>
+struct OutMaps {
+    CUtensorMap layer[NL];
+};
+template <int NL>
+struct GemmLaunch {
+    GemmParams layer[NL];
+    int cta_begin[NL + 1];
+    int n_layers;
 };
 
 // ---- PTX wrappers ----------------------------------------------------------------------------
@@ -250,6 +265,7 @@ __device__ __forceinline__ void row_shared(const uint4 *tab, uint32_t e, uint32_
 // Block (g, y): tokens 8g .. 8g+7 of the padded range, every gridDim.y-th run of 8 images; a warp takes four tokens x two
 // images (128 bytes of a row of x), a lane 8 columns of a token; tokens >= B and columns beyond a region are zeros. -------
 constexpr int PRE_THREADS = 256;
+constexpr long long PRE_ROWS_MIN = 1 << 20;      // activations of a launch
 
 struct PrepassParams {
     LayerView L;
@@ -278,18 +294,14 @@ __device__ __forceinline__ void pad_table(uint8_t *dst, const __half *src, long 
     }
 }
 
-__global__ void __launch_bounds__(PRE_THREADS, 4)
-gemm_prepass_kernel(const __grid_constant__ PrepassParams P)
+template <int NL>
+struct PrepassLaunch {
+    PrepassParams layer[NL];
+};
+
+// what has to start at zero, and the padded tables: thread tid of n_tid
+__device__ __forceinline__ void prepass_clear(const PrepassParams &P, long long tid, long long n_tid)
 {
-    // the GEMM is launched as a programmatic dependent: its CTAs may become resident and run their set-up and
-    // first centroid reads as soon as every block of this grid has started; whatever reads this kernel's
-    // output waits for the whole grid (griddepcontrol.wait) first
-    pdl_launch_dependents();
-    const LayerView &L = P.L;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long tid = ((long long)blockIdx.y * gridDim.x + blockIdx.x) * PRE_THREADS + threadIdx.x;
-    const long long n_tid = (long long)gridDim.x * gridDim.y * PRE_THREADS;
-    pdl_wait();          // the activations may be the previous kernel's output, and that kernel may use this workspace
     if (tid == 0) *P.status = 0;
     for (long long i = tid; i < P.n_flags; i += n_tid) P.tile_flags[i] = 0;
     if ((P.n_zero & 3) == 0) {
@@ -297,8 +309,171 @@ gemm_prepass_kernel(const __grid_constant__ PrepassParams P)
     } else {
         for (long long i = tid; i < P.n_zero; i += n_tid) P.zero[i] = 0.f;
     }
-    if (P.pad1) pad_table(P.pad1, L.c1, (long long)L.G * L.k1, L.v, P.pad_bytes, tid, n_tid);
-    if (P.pad2) pad_table(P.pad2, L.c2, (long long)L.G * L.k2, L.v, P.pad_bytes, tid, n_tid);
+    if (P.pad1) pad_table(P.pad1, P.L.c1, (long long)P.L.G * P.L.k1, P.L.v, P.pad_bytes, tid, n_tid);
+    if (P.pad2) pad_table(P.pad2, P.L.c2, (long long)P.L.G * P.L.k2, P.L.v, P.pad_bytes, tid, n_tid);
+}
+
+// eight activations x their scales -> FP16 pairs; returns the sum of activation x bias
+__device__ __forceinline__ float scale8(uint4 xq, uint4 sq, uint4 bq, int x_bf16, uint4 &out)
+{
+    const uint32_t xw[4] = {xq.x, xq.y, xq.z, xq.w}, sw[4] = {sq.x, sq.y, sq.z, sq.w}, bw[4] = {bq.x, bq.y, bq.z, bq.w};
+    uint32_t o[4];
+    float acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const float2 a = x_bf16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xw[i]))
+                                : __half22float2(*reinterpret_cast<const __half2 *>(&xw[i]));
+        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&sw[i]));
+        const float2 h = __half22float2(*reinterpret_cast<const __half2 *>(&bw[i]));
+        const __half2 y = __floats2half2_rn(a.x * f.x, a.y * f.y);
+        o[i] = *reinterpret_cast<const uint32_t *>(&y);
+        acc += a.x * h.x + a.y * h.y;
+    }
+    out = make_uint4(o[0], o[1], o[2], o[3]);
+    return acc;
+}
+__device__ __forceinline__ uint4 pack8(const uint16_t (&e)[8])
+{
+    return make_uint4(e[0] | ((uint32_t)e[1] << 16), e[2] | ((uint32_t)e[3] << 16), e[4] | ((uint32_t)e[5] << 16), e[6] | ((uint32_t)e[7] << 16));
+}
+
+// words shifted down by `by` < 2^S places
+template <int S, int NW>
+__device__ __forceinline__ void shift_words(uint32_t (&w)[NW], int by)
+{
+#pragma unroll
+    for (int b = S - 1; b >= 0; b--)
+        if (by & (1 << b)) {
+#pragma unroll
+            for (int i = 0; i + (1 << b) < NW; i++) w[i] = w[i + (1 << b)];
+        }
+}
+// Elements at .. at + 7 of p (16-byte aligned, len elements, zeros past them), which outlier columns push off 16-byte boundaries
+__device__ __forceinline__ uint4 load8(const uint16_t *p, long long at, long long len)
+{
+    const int sh = (int)(at & 7);
+    if (at - sh + (sh ? 16 : 8) <= len) {
+        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p + at - sh));
+        if (sh == 0) return a;
+        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p + at - sh + 8));
+        uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        shift_words<2>(w, sh >> 1);
+        const int h = 16 * (sh & 1);
+        return make_uint4(__funnelshift_r(w[0], w[1], h), __funnelshift_r(w[1], w[2], h), __funnelshift_r(w[2], w[3], h), __funnelshift_r(w[3], w[4], h));
+    }
+    uint16_t e[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) e[i] = at + i < len ? __ldg(p + at + i) : (uint16_t)0;
+    return pack8(e);
+}
+// input features of stored columns n .. n + 7
+__device__ __forceinline__ void load_features(const LayerView &L, int n, int (&f)[8])
+{
+    const int sh = n & 3;
+    if (n - sh + 12 <= L.N) {
+        uint32_t w[12];
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(L.perm + n - sh) + i);
+            w[4 * i] = a.x; w[4 * i + 1] = a.y; w[4 * i + 2] = a.z; w[4 * i + 3] = a.w;
+        }
+        shift_words<2>(w, sh);
+#pragma unroll
+        for (int i = 0; i < 8; i++) f[i] = (int)(w[i] < (unsigned)L.N ? w[i] : (unsigned)(L.N - 1));
+    } else {
+#pragma unroll
+        for (int i = 0; i < 8; i++) f[i] = in_col(L, n + i < L.N ? n + i : L.N - 1);
+    }
+}
+
+// Layers with a stored column order: a block keeps T whole rows of x in shared memory and gathers from there, a lane 8
+// columns for all T tokens.  2-byte gathers out of global memory take 32 L1 cycles per warp: 512 tokens x 11008 columns
+// 36.6 us.  Below a million
+// activations a block's rows are too many for its few columns (128 tokens x 4096: 28.6 us instead of 27.8 with the GEMM;
+// 128 x 11008: 35.4 instead of 37.3, 512 x 11008: 64.6 instead of 79.8).
+template <int T, int NL>
+__global__ void __launch_bounds__(PRE_THREADS)
+gemm_prepass_rows_kernel(const __grid_constant__ PrepassLaunch<NL> F)
+{
+    extern __shared__ __align__(16) uint16_t rows[];         // [T][N rounded up to 8]
+    pdl_launch_dependents();
+    const PrepassParams &P = F.layer[NL > 1 ? blockIdx.z : 0];
+    const LayerView &L = P.L;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_wait();          // the activations may be the previous kernel's output, and that kernel may use this workspace
+    prepass_clear(P, ((long long)blockIdx.y * gridDim.x + blockIdx.x) * PRE_THREADS + threadIdx.x, (long long)gridDim.x * gridDim.y * PRE_THREADS);
+
+    const int t0 = blockIdx.x * T, n_pad = (L.N + 7) / 8 * 8;
+    for (int i = 0; i < T; i++) {
+        const uint16_t *xr = reinterpret_cast<const uint16_t *>(P.x) + (long long)(t0 + i) * L.N;
+        if (t0 + i >= P.B) {
+            for (int n = 8 * threadIdx.x; n < n_pad; n += 8 * PRE_THREADS) *reinterpret_cast<uint4 *>(rows + i * n_pad + n) = make_uint4(0, 0, 0, 0);
+        } else if ((L.N & 7) == 0) {
+            for (int n = 8 * threadIdx.x; n < L.N; n += 8 * PRE_THREADS)
+                *reinterpret_cast<uint4 *>(rows + i * n_pad + n) = __ldg(reinterpret_cast<const uint4 *>(xr + n));
+        } else {
+#pragma unroll 4
+            for (int n = threadIdx.x; n < L.N; n += PRE_THREADS) rows[i * n_pad + n] = __ldg(xr + n);
+        }
+    }
+    __syncthreads();
+
+    const int tile = t0 / P.tile_n, row0 = t0 - tile * P.tile_n;          // (T divides tile_n)
+    uint8_t *base_dst = P.xs + (long long)tile * P.img_total * (P.tile_n * 64);
+    float acc[T];
+#pragma unroll
+    for (int i = 0; i < T; i++) acc[i] = 0.f;
+    for (int ch = (blockIdx.y * (PRE_THREADS / 32) + warp) * 32 + lane; ch < P.img_total * 4; ch += gridDim.y * PRE_THREADS) {
+        const int img = ch >> 2, q = ch & 3;
+        const bool main_cols = img < P.img_main;
+        const int c = (main_cols ? img : img - P.img_main) * IMG_COLS + q * 8;     // first column, counted in its region
+        const int n_cols = main_cols ? L.Nc : L.n_out, base = main_cols ? L.n_out : 0;
+        int f[8];
+        load_features(L, base + c, f);
+        uint4 sq = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u), bq = make_uint4(0, 0, 0, 0);
+        if (L.has_scale) {
+            sq = load8(reinterpret_cast<const uint16_t *>(L.scale), base + c, L.N);
+            bq = load8(reinterpret_cast<const uint16_t *>(L.bias), base + c, L.N);
+        }
+#pragma unroll
+        for (int i = 0; i < T; i++) {
+            uint16_t xe[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) xe[j] = c + j < n_cols ? rows[i * n_pad + f[j]] : (uint16_t)0;
+            uint4 o;
+            acc[i] += scale8(pack8(xe), sq, bq, L.x_bf16, o);
+            const int row = row0 + i;
+            *reinterpret_cast<uint4 *>(base_dst + (long long)img * (P.tile_n * 64) + (row >> 3) * B_SBO + (row & 7) * 64 + ((q ^ ((row & 7) >> 1)) << 4)) = o;
+        }
+    }
+    __shared__ float red[PRE_THREADS / 32][T];
+#pragma unroll
+    for (int i = 0; i < T; i++) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], o);
+        if (lane == 0) red[warp][i] = acc[i];
+    }
+    __syncthreads();
+    if (threadIdx.x < T) {
+        float a = 0.f;
+        for (int w = 0; w < PRE_THREADS / 32; w++) a += red[w][threadIdx.x];
+        P.bpart[(long long)blockIdx.y * gridDim.x * T + t0 + threadIdx.x] = a;
+    }
+}
+
+template <int NL>
+__global__ void __launch_bounds__(PRE_THREADS, 4)
+gemm_prepass_kernel(const __grid_constant__ PrepassLaunch<NL> F)
+{
+    // the GEMM is launched as a programmatic dependent: its CTAs may become resident and run their set-up and
+    // first centroid reads as soon as every block of this grid has started; whatever reads this kernel's
+    // output waits for the whole grid (griddepcontrol.wait) first
+    pdl_launch_dependents();
+    const PrepassParams &P = F.layer[NL > 1 ? blockIdx.z : 0];
+    const LayerView &L = P.L;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_wait();          // the activations may be the previous kernel's output, and that kernel may use this workspace
+    prepass_clear(P, ((long long)blockIdx.y * gridDim.x + blockIdx.x) * PRE_THREADS + threadIdx.x, (long long)gridDim.x * gridDim.y * PRE_THREADS);
 
     const int tok = 4 * (warp & 1) + (lane >> 3), q = lane & 3;
     const int tg = blockIdx.x * 8 + tok;                 // token of the padded range
@@ -338,29 +513,16 @@ gemm_prepass_kernel(const __grid_constant__ PrepassParams P)
                     se[i] = (in && L.has_scale) ? __ldg(reinterpret_cast<const uint16_t *>(L.scale) + n) : (uint16_t)0x3C00;
                     be[i] = (in && L.has_scale) ? __ldg(reinterpret_cast<const uint16_t *>(L.bias) + n) : (uint16_t)0;
                 }
-                auto pack = [](const uint16_t (&e)[8]) {
-                    return make_uint4(e[0] | ((uint32_t)e[1] << 16), e[2] | ((uint32_t)e[3] << 16), e[4] | ((uint32_t)e[5] << 16), e[6] | ((uint32_t)e[7] << 16));
-                };
-                xq[u] = pack(xe); sq[u] = pack(se); bq[u] = pack(be);
+                xq[u] = pack8(xe); sq[u] = pack8(se); bq[u] = pack8(be);
             }
         }
 #pragma unroll
         for (int u = 0; u < UNROLL; u++) {
             const int img = img0 + u * stride;
             if (img >= P.img_total) break;
-            const uint32_t xw[4] = {xq[u].x, xq[u].y, xq[u].z, xq[u].w}, sw[4] = {sq[u].x, sq[u].y, sq[u].z, sq[u].w}, bw[4] = {bq[u].x, bq[u].y, bq[u].z, bq[u].w};
-            uint32_t o[4];
-#pragma unroll
-            for (int i = 0; i < 4; i++) {
-                const float2 a = L.x_bf16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xw[i]))
-                                          : __half22float2(*reinterpret_cast<const __half2 *>(&xw[i]));
-                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&sw[i]));
-                const float2 h = __half22float2(*reinterpret_cast<const __half2 *>(&bw[i]));
-                const __half2 y = __floats2half2_rn(a.x * f.x, a.y * f.y);
-                o[i] = *reinterpret_cast<const uint32_t *>(&y);
-                acc += a.x * h.x + a.y * h.y;
-            }
-            *reinterpret_cast<uint4 *>(dst + (long long)img * (P.tile_n * 64)) = make_uint4(o[0], o[1], o[2], o[3]);
+            uint4 o;
+            acc += scale8(xq[u], sq[u], bq[u], L.x_bf16, o);
+            *reinterpret_cast<uint4 *>(dst + (long long)img * (P.tile_n * 64)) = o;
         }
     }
     __shared__ float red[PRE_THREADS / 64][8];
@@ -392,10 +554,17 @@ __device__ __forceinline__ uint2 outlier_vector4(const LayerView &L, int m0, int
 }
 
 // ---- the GEMM ------------------------------------------------------------------------------------
-template <int V, int T1, int T2>
+template <int V, int T1, int T2, int NL>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
-gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, const __grid_constant__ GemmParams P)
+gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_constant__ GemmLaunch<NL> F)
 {
+    // the layer this CTA works on, and its place among that layer's CTAs
+    int li = 0;
+    if (NL > 1)
+        while (li + 1 < F.n_layers && (int)blockIdx.x >= F.cta_begin[li + 1]) li++;
+    const GemmParams P = F.layer[NL > 1 ? li : 0];           // (a copy: through a reference gate+up of 11008 x 4096 at 300 tokens took 7 us more)
+    const CUtensorMap &tmap_out = maps.layer[NL > 1 ? li : 0];
+    const unsigned worker = blockIdx.x - (NL > 1 ? F.cta_begin[li] : 0);
     constexpr bool MN = V == 8;                              // A layout
     constexpr int KS = Tile<V>::KS, NV = Tile<V>::NV, A_STAGES = Tile<V>::A_STAGES, A_BYTES = a_stage_bytes<V>();
     constexpr int GROUPS = Tile<V>::GROUPS, GROUP_WARPS = Tile<V>::GROUP_WARPS;
@@ -471,7 +640,7 @@ gemm_tcgen05_kernel(const __grid_constant__ CUtensorMap tmap_out, const __grid_c
     const uint32_t tmem_base = *tmem_slot;
 
     // this CTA's share of the (tile, k block) units
-    const unsigned u_begin = P.shares.begin(blockIdx.x), u_end = P.shares.begin(blockIdx.x + 1);
+    const unsigned u_begin = P.shares.begin(worker), u_end = P.shares.begin(worker + 1);
     // A segment is the part of one tile inside the share: k blocks [kb0, kb1) of tile `tile`.
 #define FOR_EACH_SEGMENT                                                                          \
     for (unsigned u = u_begin; u < u_end && ok; u += (unsigned)(kb1 - kb0))                         \
@@ -934,18 +1103,19 @@ struct GemmPlan {
     int tiles_m, tiles_t, tile_n, n0, ks, kb_main, kb_total, grid, any_split, flag_order, tma_out, scratch;
     int b_stages, cb1_shift, cb2_shift, cb1_bytes, cb2_bytes;
     int pre_x, pre_y;                // pre-pass grid; pre_y = parts of a bias term
+    int pre_rows;                    // tokens per block of the pre-pass that keeps rows in shared memory, 0 = the other one
     long long n_scratch;
     size_t smem;
     int pad_bytes;                   // rows of padded table copies, 0 = none
     long long ws_bytes, off_flags, off_bpart, off_pad1, off_pad2, off_scratch, off_xs;
 };
 
+// `workers` CTAs at most, in a launch of n_layers layers
 template <int V>
-GemmPlan plan_gemm_v(const LayerView &L, int B)
+GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
 {
     GemmPlan p;
     memset(&p, 0, sizeof(p));
-    int workers = device_sm_count();
     // tables: small ones of a single group in shared memory, with copies where that costs little
     p.t1 = (V <= 8 && L.G == 1 && (long long)L.k1 * 16 <= 64 * 1024) ? TABLE_SHARED : TABLE_GLOBAL;
     p.t2 = L.k2 == 0 ? TABLE_NONE : (V <= 8 && L.G == 1 && L.k2 * 16 <= 16 * 1024) ? TABLE_SHARED : TABLE_GLOBAL;
@@ -999,8 +1169,11 @@ GemmPlan plan_gemm_v(const LayerView &L, int B)
     }
     // pre-pass: enough blocks to fill the GPU (each of them is one part of eight tokens' bias terms)
     const int images = p.kb_total * (p.ks / IMG_COLS);
-    p.pre_x = p.tiles_t * p.tile_n / 8;
-    p.pre_y = ceil_div(4 * device_sm_count(), p.pre_x);
+    const int row_bytes = (L.N + 7) / 8 * 16;
+    p.pre_rows = !L.permuted || (long long)B * L.N * n_layers < PRE_ROWS_MIN ? 0 : 4 * row_bytes <= 100 * 1024 ? 4 : 2 * row_bytes <= 200 * 1024 ? 2 : 0;
+    p.pre_x = p.tiles_t * p.tile_n / (p.pre_rows ? p.pre_rows : 8);
+    p.pre_y = p.pre_rows ? 2 * device_sm_count() / (p.pre_x * n_layers) : ceil_div(4 * device_sm_count(), p.pre_x * n_layers);
+    if (p.pre_y < 1) p.pre_y = 1;
     if (p.pre_y > ceil_div(images, 8)) p.pre_y = ceil_div(images, 8);
     p.pad_bytes = (V != 8 && (p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL)) ? (V <= 8 ? 16 : 32) : 0;
     auto take = [&](long long bytes) { const long long at = p.ws_bytes; p.ws_bytes += (bytes + 255) / 256 * 256; return at; };
@@ -1015,40 +1188,147 @@ GemmPlan plan_gemm_v(const LayerView &L, int B)
     return p;
 }
 
-GemmPlan plan_gemm(const LayerView &L, int B)
+GemmPlan plan_gemm(const LayerView &L, int B, int workers, int n_layers)
 {
-    return L.v == 8 ? plan_gemm_v<8>(L, B) : L.v == 6 ? plan_gemm_v<6>(L, B) : plan_gemm_v<12>(L, B);
+    return L.v == 8 ? plan_gemm_v<8>(L, B, workers, n_layers) : L.v == 6 ? plan_gemm_v<6>(L, B, workers, n_layers)
+                                                                         : plan_gemm_v<12>(L, B, workers, n_layers);
 }
 
-template <int V, int T1, int T2>
-cudaError_t launch_gemm(const GemmPlan &pl, const CUtensorMap &map, const GemmParams &P, cudaStream_t st)
+// The plans of the layers of one launch (n = 1: a launch of its own): the SMs are dealt out to the layers in proportion to
+// their vector rows, at least one each, leftover SMs where the most rows per CTA remain.  Returns the workspace bytes.
+long long plan_launch(const LayerView *Ls, int n, int B, GemmPlan *pl)
 {
-    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2>), pl.smem);
+    const int G = device_sm_count();
+    int ctas[MAX_FUSED], used = 0;
+    long long total = 0, ws = 0;
+    for (int l = 0; l < n; l++) total += Ls[l].R;
+    for (int l = 0; l < n; l++) {
+        ctas[l] = (int)(G * (long long)Ls[l].R / total);
+        if (ctas[l] < 1) ctas[l] = 1;
+        used += ctas[l];
+    }
+    for (; used < G; used++) {
+        int most = 0;
+        for (int l = 1; l < n; l++)
+            if ((long long)Ls[l].R * ctas[most] > (long long)Ls[most].R * ctas[l]) most = l;
+        ctas[most]++;
+    }
+    for (int l = 0; l < n; l++) {
+        pl[l] = plan_gemm(Ls[l], B, ctas[l], n);
+        ws += pl[l].ws_bytes;
+    }
+    return ws;
+}
+
+template <int V, int T1, int T2, int NL>
+cudaError_t launch_gemm(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmLaunch<NL> &F, cudaStream_t st)
+{
+    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2, NL>), pl.smem);
     if (e != cudaSuccess) return e;
     // programmatic dependent launch: set-up and the producers' first reads overlap the pre-pass
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(pl.grid, 1, 1);
+    cfg.gridDim = dim3(F.cta_begin[F.n_layers], 1, 1);
     cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2>, map, P);
+    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2, NL>, maps, F);
 }
 
-template <int V>
-cudaError_t launch_gemm_v(const GemmPlan &pl, const CUtensorMap &map, const GemmParams &P, cudaStream_t st)
+template <int V, int NL>
+cudaError_t launch_gemm_v(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmLaunch<NL> &F, cudaStream_t st)
 {
     if (pl.t1 == TABLE_SHARED) {
-        if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_SHARED, TABLE_NONE>(pl, map, P, st);
-        if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_SHARED, TABLE_SHARED>(pl, map, P, st);
-        return launch_gemm<V, TABLE_SHARED, TABLE_GLOBAL>(pl, map, P, st);
+        if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_SHARED, TABLE_NONE, NL>(pl, maps, F, st);
+        if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_SHARED, TABLE_SHARED, NL>(pl, maps, F, st);
+        return launch_gemm<V, TABLE_SHARED, TABLE_GLOBAL, NL>(pl, maps, F, st);
     }
-    if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_GLOBAL, TABLE_NONE>(pl, map, P, st);
-    if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_GLOBAL, TABLE_SHARED>(pl, map, P, st);
-    return launch_gemm<V, TABLE_GLOBAL, TABLE_GLOBAL>(pl, map, P, st);
+    if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_GLOBAL, TABLE_NONE, NL>(pl, maps, F, st);
+    if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_GLOBAL, TABLE_SHARED, NL>(pl, maps, F, st);
+    return launch_gemm<V, TABLE_GLOBAL, TABLE_GLOBAL, NL>(pl, maps, F, st);
+}
+
+template <int NL>
+cudaError_t launch_layers(const LayerView *Ls, int n, const void *x, int B, void *const *outs, void *ws, cudaStream_t st)
+{
+    GemmPlan pls[NL];
+    plan_launch(Ls, n, B, pls);
+    OutMaps<NL> maps;
+    GemmLaunch<NL> F;
+    PrepassLaunch<NL> Q;
+    memset(&maps, 0, sizeof(maps));      // not read by the kernel when tma_out == 0
+    memset(&F, 0, sizeof(F));
+    memset(&Q, 0, sizeof(Q));
+    F.n_layers = n;
+    uint8_t *w8 = reinterpret_cast<uint8_t *>(ws);
+    int *status = reinterpret_cast<int *>(ws);                 // the launch's: the first layer's
+    for (int l = 0; l < n; l++) {
+        const GemmPlan &pl = pls[l];
+        const LayerView &L = Ls[l];
+        // FP32 output with 16-byte aligned rows: the epilogue goes through shared memory and TMA
+        if (pl.tma_out) {
+            EncodeTiledFn encode = get_encode_fn();
+            if (encode == nullptr) return cudaErrorNotSupported;
+            const cuuint64_t odim[2] = {(cuuint64_t)L.M, (cuuint64_t)B};
+            const cuuint64_t ostride[1] = {(cuuint64_t)L.M * 4};
+            const cuuint32_t obox[2] = {32, PIECE_TOKENS};
+            const cuuint32_t estr[2] = {1, 1};
+            const CUresult r = encode(&maps.layer[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, outs[l], odim, ostride, obox, estr,
+                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+            if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+        }
+        PrepassParams &q = Q.layer[l];
+        q.L = L; q.x = x; q.B = B; q.tile_n = pl.tile_n;
+        q.img_main = pl.kb_main * (pl.ks / IMG_COLS); q.img_total = pl.kb_total * (pl.ks / IMG_COLS);
+        q.xs = w8 + pl.off_xs;
+        q.bpart = reinterpret_cast<float *>(w8 + pl.off_bpart);
+        q.status = status;
+        q.tile_flags = reinterpret_cast<int *>(w8 + pl.off_flags); q.n_flags = pl.tiles_m * pl.tiles_t * EPI_WARPS;
+        if (pl.scratch) { q.zero = reinterpret_cast<float *>(w8 + pl.off_scratch); q.n_zero = pl.n_scratch; }
+        else if (pl.any_split && !pl.flag_order) { q.zero = reinterpret_cast<float *>(outs[l]); q.n_zero = (long long)B * L.M; }
+        if (pl.pad_bytes && pl.t1 == TABLE_GLOBAL) q.pad1 = w8 + pl.off_pad1;
+        if (pl.pad_bytes && pl.t2 == TABLE_GLOBAL) q.pad2 = w8 + pl.off_pad2;
+        q.pad_bytes = pl.pad_bytes;
+
+        GemmParams &P = F.layer[l];
+        P.L = L; P.out = outs[l]; P.B = B;
+        P.tiles_m = pl.tiles_m; P.tiles_t = pl.tiles_t; P.tile_n = pl.tile_n; P.n0 = pl.n0;
+        P.kb_main = pl.kb_main; P.kb_total = pl.kb_total; P.shares = pl.shares;
+        P.b_stages = pl.b_stages; P.cb1_shift = pl.cb1_shift; P.cb2_shift = pl.cb2_shift;
+        P.cb1_bytes = pl.cb1_bytes; P.cb2_bytes = pl.cb2_bytes;
+        P.flag_order = pl.flag_order; P.tma_out = pl.tma_out;
+        P.status = status; P.bpart = q.bpart; P.bias_parts = pl.pre_y; P.tile_flags = q.tile_flags;
+        P.scratch = pl.scratch ? reinterpret_cast<float *>(w8 + pl.off_scratch) : nullptr;
+        P.xs = q.xs;
+        P.tab1 = q.pad1 ? q.pad1 : reinterpret_cast<const uint8_t *>(L.c1);
+        P.tab2 = q.pad2 ? q.pad2 : reinterpret_cast<const uint8_t *>(L.c2);
+        F.cta_begin[l + 1] = F.cta_begin[l] + pl.grid;
+        w8 += pl.ws_bytes;
+    }
+
+    // (the layers of a launch have one format, so their plans differ in the tiles only)
+    const GemmPlan &pl = pls[0];
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3(pl.pre_x, pl.pre_y, n);
+    cfg.blockDim = dim3(PRE_THREADS, 1, 1);
+    cfg.dynamicSmemBytes = (size_t)pl.pre_rows * ((Ls[0].N + 7) / 8 * 16);
+    cfg.stream = st;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    auto pre = pl.pre_rows == 4 ? gemm_prepass_rows_kernel<4, NL> : pl.pre_rows == 2 ? gemm_prepass_rows_kernel<2, NL> : gemm_prepass_kernel<NL>;
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(pre), cfg.dynamicSmemBytes);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, pre, Q);
+    if (e != cudaSuccess) return e;
+    if (Ls[0].v == 8) return launch_gemm_v<8, NL>(pl, maps, F, st);
+    if (Ls[0].v == 6) return launch_gemm_v<6, NL>(pl, maps, F, st);
+    return pl.t2 == TABLE_NONE ? launch_gemm<12, TABLE_GLOBAL, TABLE_NONE, NL>(pl, maps, F, st)
+                               : launch_gemm<12, TABLE_GLOBAL, TABLE_GLOBAL, NL>(pl, maps, F, st);
 }
 
 }  // namespace
@@ -1060,74 +1340,30 @@ bool gemm_tcgen05_supported(const LayerView &L, int B)
     return (L.v == 6 || L.v == 8 || L.v == 12) && ((long long)L.M / 96 + 1) * (B / 256 + 1) * (L.N / 16 + 16) < 0x7fffffffLL;
 }
 
-long long gemm_tcgen05_workspace_bytes(const LayerView &L, int B) { return plan_gemm(L, B).ws_bytes; }
+long long gemm_tcgen05_workspace_bytes(const LayerView *Ls, int n, int B)
+{
+    GemmPlan pl[MAX_FUSED];
+    return plan_launch(Ls, n, B, pl);
+}
+
+// Layers of one format (apart from M) can share a launch: q+k+v+o of a 70B layer at 333 tokens 265 -> 225 us (a 1024 x 8192
+// projection alone has 8 tiles for 148 SMs, 18 pieces of each meeting in one place).
+bool gemm_tcgen05_fused_supported(const LayerView *Ls, int n, int B)
+{
+    if (n < 2 || n > MAX_FUSED || n > device_sm_count()) return false;
+    for (int l = 0; l < n; l++)
+        if (!gemm_tcgen05_supported(Ls[l], B) || !same_geometry(Ls[0], Ls[l]) || Ls[l].permuted != Ls[0].permuted || Ls[l].deterministic) return false;
+    return true;
+}
 
 int gemm_tcgen05_launches(const LayerView &, int) { return 2; }   // pre-pass + GEMM
 
-bool gemm_tcgen05_waits_between_ctas(const LayerView &L, int B) { return plan_gemm(L, B).flag_order != 0; }
+bool gemm_tcgen05_waits_between_ctas(const LayerView &L, int B) { return plan_gemm(L, B, device_sm_count(), 1).flag_order != 0; }
 
-cudaError_t launch_gemm_tcgen05(const LayerView &L, const void *x, int B, void *out, void *ws, cudaStream_t st)
+cudaError_t launch_gemm_tcgen05(const LayerView *Ls, int n, const void *x, int B, void *const *outs, void *ws, cudaStream_t st)
 {
-    const GemmPlan pl = plan_gemm(L, B);
-    uint8_t *w8 = reinterpret_cast<uint8_t *>(ws);
-
-    // FP32 output with 16-byte aligned rows: the epilogue goes through shared memory and TMA
-    CUtensorMap tmap_out;
-    memset(&tmap_out, 0, sizeof(tmap_out));      // not read by the kernel when tma_out == 0
-    if (pl.tma_out) {
-        EncodeTiledFn encode = get_encode_fn();
-        if (encode == nullptr) return cudaErrorNotSupported;
-        const cuuint64_t odim[2] = {(cuuint64_t)L.M, (cuuint64_t)B};
-        const cuuint64_t ostride[1] = {(cuuint64_t)L.M * 4};
-        const cuuint32_t obox[2] = {32, PIECE_TOKENS};
-        const cuuint32_t estr[2] = {1, 1};
-        const CUresult r = encode(&tmap_out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, out, odim, ostride, obox, estr,
-                                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-        if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
-    }
-
-    PrepassParams Q;
-    memset(&Q, 0, sizeof(Q));
-    Q.L = L; Q.x = x; Q.B = B; Q.tile_n = pl.tile_n;
-    Q.img_main = pl.kb_main * (pl.ks / IMG_COLS); Q.img_total = pl.kb_total * (pl.ks / IMG_COLS);
-    Q.xs = w8 + pl.off_xs;
-    Q.bpart = reinterpret_cast<float *>(w8 + pl.off_bpart);
-    Q.status = reinterpret_cast<int *>(w8);
-    Q.tile_flags = reinterpret_cast<int *>(w8 + pl.off_flags); Q.n_flags = pl.tiles_m * pl.tiles_t * EPI_WARPS;
-    if (pl.scratch) { Q.zero = reinterpret_cast<float *>(w8 + pl.off_scratch); Q.n_zero = pl.n_scratch; }
-    else if (pl.any_split && !pl.flag_order) { Q.zero = reinterpret_cast<float *>(out); Q.n_zero = (long long)B * L.M; }
-    if (pl.pad_bytes && pl.t1 == TABLE_GLOBAL) Q.pad1 = w8 + pl.off_pad1;
-    if (pl.pad_bytes && pl.t2 == TABLE_GLOBAL) Q.pad2 = w8 + pl.off_pad2;
-    Q.pad_bytes = pl.pad_bytes;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(pl.pre_x, pl.pre_y, 1);
-    cfg.blockDim = dim3(PRE_THREADS, 1, 1);
-    cfg.stream = st;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_prepass_kernel, Q);
-    if (e != cudaSuccess) return e;
-
-    GemmParams P;
-    memset(&P, 0, sizeof(P));
-    P.L = L; P.out = out; P.B = B;
-    P.tiles_m = pl.tiles_m; P.tiles_t = pl.tiles_t; P.tile_n = pl.tile_n; P.n0 = pl.n0;
-    P.kb_main = pl.kb_main; P.kb_total = pl.kb_total; P.shares = pl.shares;
-    P.b_stages = pl.b_stages; P.cb1_shift = pl.cb1_shift; P.cb2_shift = pl.cb2_shift;
-    P.cb1_bytes = pl.cb1_bytes; P.cb2_bytes = pl.cb2_bytes;
-    P.flag_order = pl.flag_order; P.tma_out = pl.tma_out;
-    P.status = Q.status; P.bpart = Q.bpart; P.bias_parts = pl.pre_y; P.tile_flags = Q.tile_flags;
-    P.scratch = pl.scratch ? reinterpret_cast<float *>(w8 + pl.off_scratch) : nullptr;
-    P.xs = Q.xs;
-    P.tab1 = Q.pad1 ? Q.pad1 : reinterpret_cast<const uint8_t *>(L.c1);
-    P.tab2 = Q.pad2 ? Q.pad2 : reinterpret_cast<const uint8_t *>(L.c2);
-    if (L.v == 8) return launch_gemm_v<8>(pl, tmap_out, P, st);
-    if (L.v == 6) return launch_gemm_v<6>(pl, tmap_out, P, st);
-    return pl.t2 == TABLE_NONE ? launch_gemm<12, TABLE_GLOBAL, TABLE_NONE>(pl, tmap_out, P, st)
-                               : launch_gemm<12, TABLE_GLOBAL, TABLE_GLOBAL>(pl, tmap_out, P, st);
+    if (n < 1 || n > MAX_FUSED) return cudaErrorInvalidValue;
+    return n == 1 ? launch_layers<1>(Ls, n, x, B, outs, ws, st) : launch_layers<MAX_FUSED>(Ls, n, x, B, outs, ws, st);
 }
 
 }  // namespace vptq

@@ -105,6 +105,7 @@ LayerView make_view(const vptq_layer_desc *d, const vptq_layer_ptrs *p)
         L.prepared = (d->flags & VPTQ_FLAG_PREPARED) ? p->prepared : nullptr;
     }
     L.prep_parts = (d->flags & VPTQ_FLAG_PREPARED) ? d->prepared_parts : 0;
+    L.permuted = (d->flags & VPTQ_FLAG_COL_PERM) ? 1 : 0;
     L.concurrent = (d->flags & VPTQ_FLAG_CONCURRENT) ? 1 : 0;
     L.deterministic = (d->flags & VPTQ_FLAG_DETERMINISTIC) ? 1 : 0;
     return L;

@@ -59,3 +59,41 @@ def test_batched_kernel_repeats_bit_for_bit_when_asked():
     ys = [det.linear(x).clone() for _ in range(3)]
     assert all(np.array_equal(y.cpu().numpy().view(np.uint16), ys[0].cpu().numpy().view(np.uint16)) for y in ys)
     assert rel_err(ys[0].float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
+
+
+@pytest.mark.parametrize("Ms,N,B,kw,outs", [
+    ((130, 2100, 721), 1003, 65, dict(V6), ("fp16", "fp32", "bf16")),             # the fewest tokens that share a launch
+    ((1024, 8), 2056, 513, dict(v=8, k1=65536, permuted=True), ("fp16", "fp32")),  # two token tiles; a layer of one tile
+    ((600, 1800, 600, 600), 1034, 130, dict(V12, permuted=True), ("fp32",) * 4),
+    ((2048, 2048), 1000, 300, dict(v=8, k1=65536, k2=256), ("fp32", "fp32")),
+    ((520, 130), 1003, 17, dict(V6), ("fp16", "fp32")),                           # small layers at few tokens
+    ((520, 130), 1003, 5, dict(V6), ("fp16", "bf16")),
+    ((1024, 264), 1411, 9, dict(v=8, k1=65536), ("fp16", "fp16")),
+    ((600, 1300), 1034, 3, dict(V12), ("fp32", "bf16")),
+])
+def test_layers_that_share_a_batched_launch(Ms, N, B, kw, outs):
+    import torch
+    from paper_2409_17066_b200 import binding as b
+    ds = [synth.make_layer(synth.LayerSpec("bl%d" % i, M, N, out_dtype=o, **kw), 91 + i, 0, B) for i, (M, o) in enumerate(zip(Ms, outs))]
+    dls = [b.DeviceLayer(d) for d in ds]
+    fused = b.FusedLayers(dls)
+    assert fused.path(B) == "fused_gemm_tcgen05"
+    assert b.vptq_linear_fused_launches([dl.desc for dl in dls], B) == 2
+    types = dict(fp16=torch.float16, fp32=torch.float32, bf16=torch.bfloat16)
+    ys = [torch.empty(B, M, dtype=types[o], device="cuda") for M, o in zip(Ms, outs)]
+    for _ in range(2):
+        fused.linear(dls[0].upload_x(ds[0]["x"]), ys)
+    for d, y, o in zip(ds, ys, outs):
+        y_ref = oracle.Layer.from_synth(d).linear(ds[0]["x"])
+        assert rel_err(y.float().cpu().numpy(), y_ref) <= (TOL if o != "bf16" else 2.0 ** -8)
+
+
+@pytest.mark.parametrize("N,B", [(512, 64), (1003, 257), (12800, 100), (12808, 70), (51201, 66)])
+def test_column_orders_gathered_from_staged_rows(N, B):
+    """4 rows of 12800 columns are the most that fit twice, 2 rows of 51200 the most that fit at all."""
+    from paper_2409_17066_b200 import binding as b
+    spec = synth.LayerSpec("cr", 24, N, v=8, k1=4096, n_out=5, v0=4, k0=64, permuted=True)
+    d = synth.make_layer(spec, 97, 0, B)
+    dl = b.DeviceLayer(d)
+    y = dl.linear(dl.upload_x(d["x"]))
+    assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
