@@ -1,4 +1,4 @@
-// Decode path for codebooks that fit shared memory (k1*16 B <= 128 KB, v <= 8), batch 1..8 per
+// Decode path for codebooks that fit shared memory (k1*16 B <= 128 KB, v <= 8), batch 1..4 per
 // launch, FP32 FMAs.
 //
 // y[t][m] = sum_n x[t][n] * W_hat[m][n]   (App. D.2: lookup fused with the product; the FP16
@@ -17,10 +17,16 @@
 // staged per CTA as FP16, main columns and outlier columns apart.  Outlier columns (a5, Sec.
 // 3.2.3) are a small pass of their own (centroids from global memory through L1).  Warp partial
 // sums meet in shared memory; the epilogue adds the bias term and converts (a7).  No scratch.
+//
+// A task costs about 126 cycles of the SM's shared-memory pipe (10.5 for 32 random main centroids, 4 for
+// 32 residual ones, eight times), which is 38 us for gate+up and down of a 7B layer with v = 6 at one
+// token; with the tables' loads, the staging and two launches it takes 61 us (83 us while the outlier
+// pass waited for memory one row at a time and the activations came in as single columns).
 #include "common.cuh"
 #include "decode.cuh"
 #include "index_words.cuh"
 #include "fused_split.cuh"
+#include "outlier_pass.cuh"
 
 namespace vptq {
 
@@ -29,6 +35,8 @@ namespace {
 constexpr int XS_BUDGET = 96 * 1024;        // bytes of staged main-column activations per CTA
 constexpr int PART_BUDGET = 16 * 1024;      // bytes of per-row partial sums per CTA
 constexpr int SMEM_FMA_MAX_B = 4;
+// 16 warps keep the shared-memory pipe as busy as 32, with twice the registers: one token, v = 6, 11008 x 4096 23.4 -> 20.8 us
+constexpr int WARPS = 16;
 
 struct SmemFmaParams {
     LayerView L[MAX_FUSED];        // a fused launch: layer l is the work of CTAs [cta_begin[l], cta_begin[l + 1])
@@ -49,7 +57,7 @@ __device__ __forceinline__ float2 h2f(uint32_t w)
     return __half22float2(*reinterpret_cast<__half2 *>(&w));
 }
 
-template <int TB, int VV, bool RES, int WARPS, bool FUSED>
+template <int TB, int VV, bool RES, bool FUSED>
 __global__ void __launch_bounds__(WARPS * 32, 1)
 decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 {
@@ -80,6 +88,11 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
     const int m_lo = r0 * L.v;
     const int m_hi = min(L.M, r1 * L.v);
 
+    // first reads of the outlier columns, beside the tables'
+    OutlierPieces outl(L, L.n_out > 0 ? m_lo / L.v0 : 0, L.n_out > 0 ? (m_hi + L.v0 - 1) / L.v0 : 0, warp, WARPS, lane);
+    int outl_id[OutlierPieces::PRE];
+    if (L.n_out > 0) outl.fetch_indices(L, outl.first, lane, outl_id);
+
     // ---- a2: codebooks -> shared memory as 16-byte rows; clear the partial sums -------------------
     // (loads of 4 entries are issued before the first store: one L2 round trip per 4 entries, not per entry)
     for (int e0 = threadIdx.x; e0 < L.k1; e0 += 4 * THREADS) {
@@ -106,6 +119,8 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
     for (int i = threadIdx.x; i < P.part_floats; i += THREADS) part[i] = 0.f;
     if (threadIdx.x < 8) bterm[threadIdx.x] = 0.f;
 
+    if (L.n_out > 0) outl.fetch_rows(L, outl_id);
+
     const int rep = P.cb2_replicated ? (lane & 7) : 0;
     const int rshift = P.cb2_replicated ? 3 : 0;
 
@@ -126,32 +141,87 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
             if (RES) raw2 = load_raw8(L.s2.ptr + (long long)r * L.s2.stride, L.s2.stride, grp, c_end, L.s2.bits);
         }
 
-        // ---- stage x*s (FP16): outlier columns once, the slab's main columns; bias term in slab 0 -----
+        // ---- stage x*s (FP16): outlier columns once, the slab's main columns; bias term in slab 0.  Where rows are 16-byte
+        // aligned a thread takes 8 columns at a time, one wide load per array, and has its first scales and biases before
+        // the wait: 11008 columns 11,000 -> 4,300 cycles -----
+        // columns to visit: all of them in slab 0 (bias term, outlier columns), else the slab's own
+        const int n_first = slab == 0 ? 0 : L.n_out + c_begin;
+        const int n_last = slab == 0 ? L.N : L.n_out + c_end;
+        const bool wide = (L.N & 7) == 0 && L.perm == nullptr;
+        auto stage = [&](int t, int n, __half y) {
+            const int c = n - L.n_out;
+            if (c < 0) xs_out[t * P.n_out_pad + n] = y;
+            else if (c >= c_begin && c < c_end) xs[t * P.slab_cols + (c - c_begin)] = y;
+        };
+        uint4 sc8 = make_uint4(0x3C003C00u, 0x3C003C00u, 0x3C003C00u, 0x3C003C00u), bi8 = make_uint4(0, 0, 0, 0);
+        int n = (n_first & ~7) + 8 * threadIdx.x;
+        if (wide && L.has_scale && n < n_last) {
+            sc8 = __ldg(reinterpret_cast<const uint4 *>(L.scale + n));
+            bi8 = __ldg(reinterpret_cast<const uint4 *>(L.bias + n));
+        }
+        // else every THREADS-th column, KC of them at a time
+        constexpr int KC = TB == 1 ? 8 : 4;
+        int col[KC];
+        __half2 scb[KC];                 // scale, bias
+        auto load_columns = [&](int n0) {
+#pragma unroll
+            for (int k = 0; k < KC; k++) {
+                const int nk = n0 + k * THREADS;
+                scb[k] = __floats2half2_rn(1.f, 0.f);
+                if (nk < n_last) {
+                    col[k] = in_col(L, nk);
+                    if (L.has_scale) scb[k] = __halves2half2(__ldg(L.scale + nk), __ldg(L.bias + nk));
+                }
+            }
+        };
+        if (!wide) load_columns(n_first + threadIdx.x);
         // (the activations may be the previous kernel's output: everything above read weights only)
         pdl_wait();
         {
             float bacc[TB];
 #pragma unroll
             for (int t = 0; t < TB; t++) bacc[t] = 0.f;
-            // columns to visit: all of them in slab 0 (bias term, outlier columns), else the slab's own
-            const int n_first = slab == 0 ? 0 : L.n_out + c_begin;
-            const int n_last = slab == 0 ? L.N : L.n_out + c_end;
-#pragma unroll 4
-            for (int n = n_first + threadIdx.x; n < n_last; n += THREADS) {
-                float sc = 1.f, bi = 0.f;
-                if (L.has_scale) {
-                    sc = __half2float(__ldg(L.scale + n));
-                    bi = __half2float(__ldg(L.bias + n));
-                }
-                const int c = n - L.n_out;
-                const bool mine = c >= c_begin && c < c_end;
+            if (wide) {
+                for (; n < n_last; n += 8 * THREADS) {
+                    uint4 x8[TB];
 #pragma unroll
-                for (int t = 0; t < TB; t++) {
-                    const float xv = t < P.B ? load_act(P.x, (long long)t * L.N + in_col(L, n), L.x_bf16) : 0.f;
-                    const __half hv = __float2half_rn(xv * sc);
-                    if (c < 0) xs_out[t * P.n_out_pad + n] = hv;
-                    else if (mine) xs[t * P.slab_cols + (c - c_begin)] = hv;
-                    if (slab == 0) bacc[t] += xv * bi;
+                    for (int t = 0; t < TB; t++)
+                        x8[t] = t < P.B ? __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(P.x) + (long long)t * L.N + n)) : make_uint4(0, 0, 0, 0);
+                    const uint32_t sw[4] = {sc8.x, sc8.y, sc8.z, sc8.w}, bw[4] = {bi8.x, bi8.y, bi8.z, bi8.w};
+                    if (L.has_scale && n + 8 * THREADS < n_last) {
+                        sc8 = __ldg(reinterpret_cast<const uint4 *>(L.scale + n + 8 * THREADS));
+                        bi8 = __ldg(reinterpret_cast<const uint4 *>(L.bias + n + 8 * THREADS));
+                    }
+#pragma unroll
+                    for (int t = 0; t < TB; t++) {
+                        const uint32_t xw[4] = {x8[t].x, x8[t].y, x8[t].z, x8[t].w};
+#pragma unroll
+                        for (int i = 0; i < 4; i++) {
+                            const float2 a = L.x_bf16 ? __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&xw[i])) : h2f(xw[i]);
+                            const float2 f = h2f(sw[i]), h = h2f(bw[i]);
+                            const __half2 y = __floats2half2_rn(a.x * f.x, a.y * f.y);
+                            stage(t, n + 2 * i, y.x);
+                            stage(t, n + 2 * i + 1, y.y);
+                            if (slab == 0) bacc[t] += a.x * h.x + a.y * h.y;
+                        }
+                    }
+                }
+            } else {
+                for (n = n_first + threadIdx.x; n < n_last; n += KC * THREADS) {
+                    if (n != n_first + (int)threadIdx.x) load_columns(n);
+                    float xv[TB][KC];
+#pragma unroll
+                    for (int t = 0; t < TB; t++)
+#pragma unroll
+                        for (int k = 0; k < KC; k++)
+                            xv[t][k] = t < P.B && n + k * THREADS < n_last ? load_act(P.x, (long long)t * L.N + col[k], L.x_bf16) : 0.f;
+#pragma unroll
+                    for (int k = 0; k < KC; k++)
+#pragma unroll
+                        for (int t = 0; t < TB; t++) {
+                            if (n + k * THREADS < n_last) stage(t, n + k * THREADS, __float2half_rn(xv[t][k] * __low2float(scb[k])));
+                            if (slab == 0) bacc[t] += xv[t][k] * __high2float(scb[k]);
+                        }
                 }
             }
             // zero the ragged end of the slab (columns >= Nc inside the last chunk)
@@ -175,47 +245,8 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
             bterm[threadIdx.x] = a;
         }
 
-        // ---- a5: outlier columns (slab 0 only): FP32, centroids gathered from global memory ------------
-        if (slab == 0 && L.n_out > 0) {
-            const int q_lo = m_lo / L.v0, q_hi = (m_hi + L.v0 - 1) / L.v0;
-            for (int qq = q_lo + warp; qq < q_hi; qq += WARPS) {
-                const uint8_t *row0 = L.s0.ptr + (long long)qq * L.s0.stride;
-#pragma unroll 1
-                for (int t0 = 0; t0 < P.B; t0 += 4) {
-                    float oacc[8][4];
-#pragma unroll
-                    for (int j = 0; j < 8; j++)
-#pragma unroll
-                        for (int t = 0; t < 4; t++) oacc[j][t] = 0.f;
-                    for (int n = lane; n < L.n_out; n += 32) {
-                        const int i0 = clamp_index(load_index(row0, n, L.s0.bits), L.k0);
-                        const uint4 cw = load_centroid_row(L.c0, i0, L.v0);
-                        const float2 c01 = h2f(cw.x), c23 = h2f(cw.y), c45 = h2f(cw.z), c67 = h2f(cw.w);
-                        const float cj[8] = {c01.x, c01.y, c23.x, c23.y, c45.x, c45.y, c67.x, c67.y};
-#pragma unroll
-                        for (int t = 0; t < 4; t++) {
-                            const float xv = (t0 + t < TB) ? __half2float(xs_out[min(t0 + t, TB - 1) * P.n_out_pad + n]) : 0.f;
-#pragma unroll
-                            for (int j = 0; j < 8; j++) oacc[j][t] += xv * cj[j];
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; j++) {
-#pragma unroll
-                        for (int t = 0; t < 4; t++) {
-                            float a = oacc[j][t];
-#pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-                            const int m = qq * L.v0 + j;
-                            if (lane == 0 && j < L.v0 && m >= m_lo && m < m_hi && t0 + t < P.B) {
-                                const int rr = m / L.v, jj = m - rr * L.v;
-                                atomicAdd(part + ((rr - r0) * TB + t0 + t) * 8 + jj, a);
-                            }
-                        }
-                    }
-                }
-            }
-        }
+        // ---- a5: outlier columns (slab 0 only) ------------
+        if (slab == 0 && L.n_out > 0) outl.add<TB, 8>(L, xs_out, P.n_out_pad, part, r0, m_lo, m_hi, lane);
 
         // ---- main tasks -----------------------------------------------------------------------------
         float acc[TB][VV];
@@ -316,18 +347,17 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 }
 
 struct SmemFmaPlan {
-    int slab_cols, n_slabs, cb2_rep, grid, part_floats, n_out_pad, warps;
+    int slab_cols, n_slabs, cb2_rep, grid, part_floats, n_out_pad;
     size_t smem;
     bool ok;
     int cta_begin[MAX_FUSED + 1];   // fused launches only
 };
 
-int fma_token_group(int B) { return B >= 8 ? 8 : (B >= 4 ? 4 : (B >= 2 ? 2 : 1)); }
+int fma_token_group(int B) { return B >= 4 ? 4 : (B >= 2 ? 2 : 1); }
 
 SmemFmaPlan plan_smem_fma(const LayerView &L, int TB)
 {
     SmemFmaPlan p;
-    p.warps = TB >= 4 ? 16 : 32;
     const int G = device_sm_count();
     p.grid = L.R < G ? L.R : G;
     const int rows_cta = ceil_div(L.R, p.grid);
@@ -340,25 +370,25 @@ SmemFmaPlan plan_smem_fma(const LayerView &L, int TB)
     p.n_slabs = slab > 0 ? (nc_pad + slab - 1) / slab : 0;
     p.cb2_rep = (L.k2 > 0 && L.k2 <= 256) ? 1 : 0;
     p.smem = (size_t)L.k1 * 16 + (size_t)L.k2 * 16 * (p.cb2_rep ? 8 : 1) + (size_t)TB * p.n_out_pad * 2 +
-             (size_t)TB * slab * 2 + (size_t)p.part_floats * 4 + 8 * 4 + (size_t)p.warps * 8 * 4;
+             (size_t)TB * slab * 2 + (size_t)p.part_floats * 4 + 8 * 4 + (size_t)WARPS * 8 * 4;
     p.ok = (long long)p.part_floats * 4 <= PART_BUDGET && p.smem <= 224 * 1024 && p.n_slabs > 0;
     return p;
 }
 
-template <int TB, int VV, bool RES, int WARPS, bool FUSED>
+template <int TB, int VV, bool RES, bool FUSED>
 cudaError_t launch_kernel(const SmemFmaParams &P, const SmemFmaPlan &pl, cudaStream_t st)
 {
-    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_fma_kernel<TB, VV, RES, WARPS, FUSED>), pl.smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_fma_kernel<TB, VV, RES, FUSED>), pl.smem);
     if (e != cudaSuccess) return e;
-    return launch_dependent("smem_fma", decode_smem_fma_kernel<TB, VV, RES, WARPS, FUSED>, pl.grid, WARPS * 32, pl.smem, st, P);
+    return launch_dependent("smem_fma", decode_smem_fma_kernel<TB, VV, RES, FUSED>, pl.grid, WARPS * 32, pl.smem, st, P);
 }
 
-template <int TB, int VV, int WARPS>
+template <int TB, int VV>
 cudaError_t launch_one(const SmemFmaParams &P, const SmemFmaPlan &pl, bool res, cudaStream_t st)
 {
     const bool fused = P.n_layers > 1;
-    if (res) return fused ? launch_kernel<TB, VV, true, WARPS, true>(P, pl, st) : launch_kernel<TB, VV, true, WARPS, false>(P, pl, st);
-    return fused ? launch_kernel<TB, VV, false, WARPS, true>(P, pl, st) : launch_kernel<TB, VV, false, WARPS, false>(P, pl, st);
+    if (res) return fused ? launch_kernel<TB, VV, true, true>(P, pl, st) : launch_kernel<TB, VV, true, false>(P, pl, st);
+    return fused ? launch_kernel<TB, VV, false, true>(P, pl, st) : launch_kernel<TB, VV, false, false>(P, pl, st);
 }
 
 // several layers of the same format (apart from M) in one grid
@@ -381,12 +411,12 @@ bool plan_smem_fma_fused(const LayerView *Ls, int n, int TB, SmemFmaPlan *out)
     return true;
 }
 
-template <int TB, int WARPS>
+template <int TB>
 cudaError_t launch_vv(const SmemFmaParams &P, const SmemFmaPlan &pl, int v, bool res, cudaStream_t st)
 {
-    if (v <= 4) return launch_one<TB, 4, WARPS>(P, pl, res, st);
-    if (v <= 6) return launch_one<TB, 6, WARPS>(P, pl, res, st);
-    return launch_one<TB, 8, WARPS>(P, pl, res, st);
+    if (v <= 4) return launch_one<TB, 4>(P, pl, res, st);
+    if (v <= 6) return launch_one<TB, 6>(P, pl, res, st);
+    return launch_one<TB, 8>(P, pl, res, st);
 }
 
 }  // namespace
@@ -426,10 +456,9 @@ cudaError_t launch_decode_smem_fma(const LayerView &L, const void *x, int B, voi
         P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.cb2_replicated = pl.cb2_rep;
         P.n_out_pad = pl.n_out_pad; P.part_floats = pl.part_floats;
         cudaError_t e;
-        if (TB == 8) e = launch_vv<8, 16>(P, pl, L.v, res, st);
-        else if (TB == 4) e = launch_vv<4, 16>(P, pl, L.v, res, st);
-        else if (TB == 2) e = launch_vv<2, 32>(P, pl, L.v, res, st);
-        else e = launch_vv<1, 32>(P, pl, L.v, res, st);
+        if (TB == 4) e = launch_vv<4>(P, pl, L.v, res, st);
+        else if (TB == 2) e = launch_vv<2>(P, pl, L.v, res, st);
+        else e = launch_vv<1>(P, pl, L.v, res, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -463,10 +492,9 @@ cudaError_t launch_decode_smem_fma_fused(const LayerView *Ls, int n, const void 
         P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.cb2_replicated = pl.cb2_rep;
         P.n_out_pad = pl.n_out_pad; P.part_floats = pl.part_floats;
         cudaError_t e;
-        if (TB == 8) e = launch_vv<8, 16>(P, pl, Ls[0].v, res, st);
-        else if (TB == 4) e = launch_vv<4, 16>(P, pl, Ls[0].v, res, st);
-        else if (TB == 2) e = launch_vv<2, 32>(P, pl, Ls[0].v, res, st);
-        else e = launch_vv<1, 32>(P, pl, Ls[0].v, res, st);
+        if (TB == 4) e = launch_vv<4>(P, pl, Ls[0].v, res, st);
+        else if (TB == 2) e = launch_vv<2>(P, pl, Ls[0].v, res, st);
+        else e = launch_vv<1>(P, pl, Ls[0].v, res, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

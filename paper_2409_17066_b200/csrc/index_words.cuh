@@ -88,13 +88,13 @@ __device__ __forceinline__ uint4 load_centroid_row(const __half *__restrict__ ta
 // the call quantity q's total over the 32 lanes sits in v[k] of the lanes with first = the returned index,
 // q = first + k, k < max(1, NV / 32): with NV >= 32 every lane holds NV / 32 distinct totals, with NV < 32 only
 // the lanes whose low log2(32 / NV) bits are clear matter (the others hold copies).  31 shuffles' worth of
-// additions spread over the lanes instead of 5 * NV.
-template <int NV>
+// additions spread over the lanes instead of 5 * NV.  With LANES = 16 the same within each half of the warp.
+template <int NV, int LANES = 32>
 __device__ __forceinline__ int halving_butterfly(float (&v)[NV], int lane)
 {
-    int first = 0, n = NV, o = 16;
+    int first = 0, n = NV, o = LANES / 2;
 #pragma unroll
-    for (int step = 0; step < 5; step++) {
+    for (int step = 0; step < (LANES == 32 ? 5 : 4); step++) {
         if (n > 1) {
             const bool up = (lane & o) != 0;
             const int h = n / 2;

@@ -1,0 +1,32 @@
+"""Decode over tables in shared memory where its staging and its outlier pass have edges: more pieces of outlier rows than a
+warp asks for in advance, rows that are not 16-byte aligned, a stored column order, more columns than one pass of the CTA
+stages, more than one slab."""
+import pytest
+
+from oracle import oracle
+from paper_2409_17066_b200 import synth
+
+from helpers import TOL, rel_err
+
+pytestmark = pytest.mark.gpu
+
+V6 = dict(v=6, k1=4096, k2=256, v0=1, k0=300)
+
+
+@pytest.mark.parametrize("M,N,B,kw", [
+    (7110, 72, 1, dict(V6, n_out=33)),                      # 3 pieces of up to 16 columns in each of 49 outlier rows per CTA
+    (7110, 73, 3, dict(V6, n_out=17, permuted=True)),
+    (1776, 4100, 1, dict(V6, n_out=16, v0=4)),              # staged 8 columns at a time ...
+    (60, 4101, 1, dict(V6, n_out=5, v0=4)),                 # ... and one by one, in more than one round
+    (60, 2056, 2, dict(V6, n_out=1, permuted=True)),
+    (64, 12808, 4, dict(v=8, k1=256)),                      # two slabs
+    (64, 12809, 4, dict(v=8, k1=256, x_dtype="bf16")),
+    (40, 264, 2, dict(v=4, k1=512, k2=17, has_scale=False)),
+])
+def test_smem_decode_edges(M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    d = synth.make_layer(synth.LayerSpec("se", M, N, **kw), 98, B, B)
+    dl = b.DeviceLayer(d)
+    assert b.vptq_linear_path(dl.desc, B) == "decode_smem_fma"
+    y = dl.linear(dl.upload_x(d["x"]))
+    assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
