@@ -16,11 +16,13 @@
 //     the bias becomes one scalar per token.
 // A warp accumulates in registers while its tasks stay in one vector row and reduces the 8*B
 // partial sums with a halving butterfly at a row change.  Two ways to combine the warps (a7):
-//   OWNER    a CTA owns whole vector rows: partial sums meet in shared memory, no scratch;
-//            used when the rows divide well over the SMs;
+//   OWNER    a CTA owns whole vector rows: partial sums meet in shared memory;
 //   balanced tasks are dealt out regardless of rows: partial sums meet in an FP32 scratch array
 //            through atomic adds, and a task counter per block of 16 vector rows tells which warp
-//            completed the block and so converts and stores it.
+//            completed the block and so converts and stores it.  Only for so many rows that their
+//            sums do not fit shared memory: clearing the scratch, the global atomics and the counters
+//            cost more than SMs that get a row less.  One token, 16 warps, as a dependent launch:
+//            1024 x 4096 12.3 -> 4.8 us, 3000 x 4096 18.4 -> 8.9, 5000 x 4096 21.1 -> 12.7.
 // Fused launch (FUSED): up to MAX_FUSED layers that read the same activations (q/k/v, gate/up) in one
 // OWNER-mode grid; the CTAs are dealt out to the layers in proportion to their vector rows and each
 // CTA works on one layer exactly as in a launch of its own.  Small layers no longer pay a launch,
@@ -37,7 +39,7 @@ namespace {
 constexpr int RB_ROWS = 16;                 // vector rows per completion counter (balanced mode)
 constexpr int XS_BUDGET = 64 * 1024;        // bytes of staged activations per CTA
 constexpr int PART_BUDGET = 32 * 1024;      // bytes of per-row partial sums per CTA (OWNER mode)
-constexpr int WARPS_TB4 = 16;               // 4 tokens per launch need 128 registers per thread
+constexpr int WARPS = 16;                   // 4 tokens need 128 registers a thread; for fewer, 4096 x 4096 11.2 -> 10.7 us against 32
 
 struct L2FmaParams {
     LayerView L[MAX_FUSED];
@@ -85,7 +87,7 @@ __device__ __forceinline__ void act8_to_float(uint4 q, int is_bf16, float (&f)[8
     }
 }
 
-template <int TB, bool RES, bool OWNER, int WARPS, bool FUSED>
+template <int TB, bool RES, bool OWNER, bool FUSED>
 __global__ void __launch_bounds__(WARPS * 32, 1)
 decode_l2_fma_kernel(const __grid_constant__ L2FmaParams P)
 {
@@ -381,7 +383,7 @@ decode_l2_fma_kernel(const __grid_constant__ L2FmaParams P)
 }
 
 struct L2Plan {
-    int slab_cols, n_slabs, chunks_total, cb2_rep, grid, owner, part_floats, warps, det, rows_cta;
+    int slab_cols, n_slabs, chunks_total, cb2_rep, grid, owner, part_floats, det, rows_cta;
     size_t smem;
     long long ws_bytes, off_counters;
     int cta_begin[MAX_FUSED + 1];   // fused launches only
@@ -390,7 +392,6 @@ struct L2Plan {
 L2Plan plan_l2(const LayerView &L, int TB)
 {
     L2Plan p;
-    p.warps = TB == 4 ? WARPS_TB4 : 32;     // 64 registers per thread suffice up to 2 tokens
     const int n_pad = (L.N + 255) / 256 * 256;
     int slab = XS_BUDGET / (2 * TB) / 256 * 256;
     if (slab > n_pad) slab = n_pad;
@@ -399,23 +400,22 @@ L2Plan plan_l2(const LayerView &L, int TB)
     p.chunks_total = n_pad / 256;
     const int G = device_sm_count();
     p.cb2_rep = (L.k2 > 0 && L.k2 <= 256) ? 1 : 0;
-    // OWNER mode when whole rows divide well over the SMs (and over the warps of a CTA)
     const int rows_cta = ceil_div(L.R, G);
-    const double eff_cta = (double)L.R / ((double)(L.R < G ? L.R : G) * rows_cta) * (L.R < G ? (double)L.R / G : 1.0);
-    const long long t_cta = (long long)rows_cta * (slab / 256);
-    const double eff_warp = (double)t_cta / ((double)p.warps * (double)((t_cta + p.warps - 1) / p.warps));
     p.part_floats = rows_cta * TB * 8;
     p.rows_cta = rows_cta;
     p.det = L.deterministic ? 1 : 0;
-    // a deterministic call takes row-owner mode whatever the balance (the other mode adds by global atomics)
-    p.owner = ((eff_cta * eff_warp >= 0.80 || p.det) && (long long)p.part_floats * 4 <= PART_BUDGET) ? 1 : 0;
+    p.owner = (long long)p.part_floats * 4 <= PART_BUDGET ? 1 : 0;
     if (!p.owner) p.part_floats = 0;
     p.grid = p.owner ? (L.R < G ? L.R : G) : (G < p.n_slabs ? p.n_slabs : G);
-    p.smem = (size_t)TB * slab * 2 + 4 * 4 + (size_t)p.warps * 4 * 4 + (size_t)L.k2 * 16 * (p.cb2_rep ? 8 : 1) +
-             (size_t)p.part_floats * 4 + (p.det && p.owner ? (size_t)(rows_cta + p.warps) * TB * 8 * 4 : 0);
+    p.smem = (size_t)TB * slab * 2 + 4 * 4 + (size_t)WARPS * 4 * 4 + (size_t)L.k2 * 16 * (p.cb2_rep ? 8 : 1) +
+             (size_t)p.part_floats * 4 + (p.det && p.owner ? (size_t)(rows_cta + WARPS) * TB * 8 * 4 : 0);
     p.ws_bytes = 0;
     p.off_counters = 0;
-    if (!p.owner) {
+    // (callers have sized their scratch by this number; row-owner mode leaves it alone)
+    const double eff_cta = (double)L.R / ((double)(L.R < G ? L.R : G) * rows_cta) * (L.R < G ? (double)L.R / G : 1.0);
+    const long long t_cta = (long long)rows_cta * (slab / 256);
+    const double eff_warp = (double)t_cta / ((double)WARPS * (double)((t_cta + WARPS - 1) / WARPS));
+    if (!p.owner || (eff_cta * eff_warp < 0.80 && !p.det)) {
         p.off_counters = ((long long)TB * L.M * 4 + 255) / 256 * 256;
         p.ws_bytes = p.off_counters + ((long long)ceil_div(L.R, RB_ROWS) * 4 + 255) / 256 * 256;
     }
@@ -426,7 +426,7 @@ int token_group(int B) { return B >= 4 ? 4 : (B >= 2 ? 2 : 1); }
 
 // A fused launch: the SMs are dealt out to the layers in proportion to their vector rows (every layer at
 // least one; leftover SMs go where the most rows per CTA remain).  False when the layers cannot share a
-// launch or whole rows would leave the SMs unevenly loaded.
+// launch.
 bool plan_l2_fused(const LayerView *Ls, int n, int TB, L2Plan *out)
 {
     if (n < 2 || n > MAX_FUSED) return false;
@@ -435,17 +435,13 @@ bool plan_l2_fused(const LayerView *Ls, int n, int TB, L2Plan *out)
     L2Plan p = plan_l2(Ls[0], TB);          // slab geometry, warps, residual table: functions of N, k2, TB
     const int G = device_sm_count();
     int R[MAX_FUSED], rows_cta = 0;
-    long long rows = 0;
-    for (int l = 0; l < n; l++) { R[l] = Ls[l].R; rows += Ls[l].R; }
+    for (int l = 0; l < n; l++) R[l] = Ls[l].R;
     if (!split_ctas(R, n, G, p.cta_begin, &rows_cta)) return false;
-    const double eff_cta = (double)rows / ((double)G * rows_cta);
-    const long long t_cta = (long long)rows_cta * (p.slab_cols / 256);
-    const double eff_warp = (double)t_cta / ((double)p.warps * (double)((t_cta + p.warps - 1) / p.warps));
     p.part_floats = rows_cta * TB * 8;
-    if (eff_cta * eff_warp < 0.80 || (long long)p.part_floats * 4 > PART_BUDGET) return false;
+    if ((long long)p.part_floats * 4 > PART_BUDGET) return false;
     p.owner = 1;
     p.grid = G;
-    p.smem = (size_t)TB * p.slab_cols * 2 + 4 * 4 + (size_t)p.warps * 4 * 4 +
+    p.smem = (size_t)TB * p.slab_cols * 2 + 4 * 4 + (size_t)WARPS * 4 * 4 +
              (size_t)Ls[0].k2 * 16 * (p.cb2_rep ? 8 : 1) + (size_t)p.part_floats * 4;
     p.ws_bytes = 0;
     p.off_counters = 0;
@@ -453,19 +449,15 @@ bool plan_l2_fused(const LayerView *Ls, int n, int TB, L2Plan *out)
     return true;
 }
 
-template <int TB, bool RES, bool OWNER, int WARPS, bool FUSED>
+template <int TB, bool RES, bool OWNER, bool FUSED>
 cudaError_t launch_one(const L2FmaParams &P, const L2Plan &pl, cudaStream_t st)
 {
-    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_l2_fma_kernel<TB, RES, OWNER, WARPS, FUSED>), pl.smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_l2_fma_kernel<TB, RES, OWNER, FUSED>), pl.smem);
     if (e != cudaSuccess) return e;
-    // Launched the ordinary way: as a programmatic dependent this kernel measured slower back to back (the
-    // 70B-shaped layer 377 us per pass instead of 295 us), although its prologue is short.  It still lets the
-    // kernel after it start early (pdl_launch_dependents above), which is where the gain is.
-    decode_l2_fma_kernel<TB, RES, OWNER, WARPS, FUSED><<<pl.grid, WARPS * 32, pl.smem, st>>>(P);
-    return cudaGetLastError();
+    return launch_dependent("l2_fma", decode_l2_fma_kernel<TB, RES, OWNER, FUSED>, pl.grid, WARPS * 32, pl.smem, st, P);
 }
 
-template <int TB, int WARPS>
+template <int TB>
 cudaError_t launch_group(const LayerView &L, const L2Plan &pl, const void *x, int Bg, void *out,
                          void *ws, cudaStream_t st)
 {
@@ -484,11 +476,11 @@ cudaError_t launch_group(const LayerView &L, const L2Plan &pl, const void *x, in
         if (e != cudaSuccess) return e;
     }
     const bool res = L.k2 > 0;
-    if (pl.owner) return res ? launch_one<TB, true, true, WARPS, false>(P, pl, st) : launch_one<TB, false, true, WARPS, false>(P, pl, st);
-    return res ? launch_one<TB, true, false, WARPS, false>(P, pl, st) : launch_one<TB, false, false, WARPS, false>(P, pl, st);
+    if (pl.owner) return res ? launch_one<TB, true, true, false>(P, pl, st) : launch_one<TB, false, true, false>(P, pl, st);
+    return res ? launch_one<TB, true, false, false>(P, pl, st) : launch_one<TB, false, false, false>(P, pl, st);
 }
 
-template <int TB, int WARPS>
+template <int TB>
 cudaError_t launch_group_fused(const LayerView *Ls, int n, const L2Plan &pl, const void *x, int Bg, void *const *outs,
                                cudaStream_t st)
 {
@@ -501,7 +493,7 @@ cudaError_t launch_group_fused(const LayerView *Ls, int n, const L2Plan &pl, con
     P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.chunks_total = pl.chunks_total;
     P.cb2_replicated = pl.cb2_rep; P.part_floats = pl.part_floats;
     P.yacc = nullptr; P.counters = nullptr;
-    return Ls[0].k2 > 0 ? launch_one<TB, true, true, WARPS, true>(P, pl, st) : launch_one<TB, false, true, WARPS, true>(P, pl, st);
+    return Ls[0].k2 > 0 ? launch_one<TB, true, true, true>(P, pl, st) : launch_one<TB, false, true, true>(P, pl, st);
 }
 
 }  // namespace
@@ -545,9 +537,9 @@ cudaError_t launch_decode_l2_fma(const LayerView &L, const void *x, int B, void 
         const void *xg = reinterpret_cast<const uint8_t *>(x) + (size_t)t0 * L.N * xe;
         void *og = reinterpret_cast<uint8_t *>(out) + (size_t)t0 * L.M * oe;
         cudaError_t e;
-        if (TB == 4) e = launch_group<4, WARPS_TB4>(L, pl, xg, Bg, og, ws, st);
-        else if (TB == 2) e = launch_group<2, 32>(L, pl, xg, Bg, og, ws, st);
-        else e = launch_group<1, 32>(L, pl, xg, Bg, og, ws, st);
+        if (TB == 4) e = launch_group<4>(L, pl, xg, Bg, og, ws, st);
+        else if (TB == 2) e = launch_group<2>(L, pl, xg, Bg, og, ws, st);
+        else e = launch_group<1>(L, pl, xg, Bg, og, ws, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -580,9 +572,9 @@ cudaError_t launch_decode_l2_fma_fused(const LayerView *Ls, int n, const void *x
         for (int l = 0; l < n; l++)
             og[l] = reinterpret_cast<uint8_t *>(outs[l]) + (size_t)t0 * Ls[l].M * (Ls[l].out_dtype == VPTQ_DTYPE_FP32 ? 4 : 2);
         cudaError_t e;
-        if (TB == 4) e = launch_group_fused<4, WARPS_TB4>(Ls, n, pl, xg, Bg, og, st);
-        else if (TB == 2) e = launch_group_fused<2, 32>(Ls, n, pl, xg, Bg, og, st);
-        else e = launch_group_fused<1, 32>(Ls, n, pl, xg, Bg, og, st);
+        if (TB == 4) e = launch_group_fused<4>(Ls, n, pl, xg, Bg, og, st);
+        else if (TB == 2) e = launch_group_fused<2>(Ls, n, pl, xg, Bg, og, st);
+        else e = launch_group_fused<1>(Ls, n, pl, xg, Bg, og, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
