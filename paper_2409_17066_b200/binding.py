@@ -244,10 +244,7 @@ def prepared_shares(vector_rows, n_sm: int, n_buckets: int = 16):
 
 
 def vptq_dequant(desc: LayerDesc, ptrs: LayerPtrs, W_out: torch.Tensor) -> torch.Tensor:
-    assert W_out.is_cuda and W_out.dtype == torch.float16 and W_out.is_contiguous()
-    assert tuple(W_out.shape) == (desc.M, desc.N)
-    _check(lib.vptq_dequant(C.byref(desc), C.byref(ptrs), _ptr(W_out), _stream()))
-    return W_out
+    return _native.dequant(desc, ptrs, W_out)
 
 
 def vptq_assign_path(M: int, N: int, v: int, k: int, flags: int = 0) -> str:

@@ -354,14 +354,15 @@ decode_l2_fma_kernel(const __grid_constant__ L2FmaParams P)
         if (OWNER) __syncthreads();      // the slab's xs is dead; part[] complete after the last slab
         if (OWNER && P.det) {
             // one thread per sum adds the slab's warp partial sums in warp order: the warps whose task range
-            // [n_tasks*w/WARPS, n_tasks*(w+1)/WARPS) meets the row's tasks [rho*chunks, (rho+1)*chunks)
+            // [n_tasks*w/WARPS, n_tasks*(w+1)/WARPS) meets the row's tasks [rho*chunks, (rho+1)*chunks); a warp
+            // without tasks has written no slot
             for (int i = threadIdx.x; i < (r1 - r0) * TB * 8; i += THREADS) {
                 const int rho = i / (TB * 8), e = i % (TB * 8);
                 const long long lo = (long long)rho * chunks, hi = lo + chunks;
                 float a = part[i];
                 for (int w = 0; w < WARPS; w++) {
                     const long long qa = n_tasks * w / WARPS, qb = n_tasks * (w + 1) / WARPS;
-                    if (qa < hi && qb > lo) a += slots[(rho + w) * (TB * 8) + e];
+                    if (qa < qb && qa < hi && qb > lo) a += slots[(rho + w) * (TB * 8) + e];
                 }
                 part[i] = a;
             }
