@@ -24,7 +24,7 @@ __host__ __device__ inline long long row_bytes(int cols, int k)
     return (bytes + 15) / 16 * 16;
 }
 
-inline int ceil_div(int a, int b) { return (a + b - 1) / b; }
+inline int ceil_div(int a, int b) { return a / b + (a % b > 0); }      // (no sum that could pass INT_MAX)
 
 // One packed index stream as the kernels see it.
 struct Stream {

@@ -72,7 +72,7 @@ long long linear_workspace_bytes(const LayerView &L, int B, int flags)
 
 int linear_launches(const LayerView &L, int B, int flags)
 {
-    const int groups = (B + DECODE_MAX_B - 1) / DECODE_MAX_B;
+    const int groups = ceil_div(B, DECODE_MAX_B);
     const int last = B - (groups - 1) * DECODE_MAX_B;
     const LinearPath path = choose_path(L, B, flags);
     if (batched_decode(path, L, B)) return gemm_tcgen05_launches(L, B);

@@ -1137,8 +1137,9 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
     sh.kb = p.kb_total; sh.whole_tiles = L.deterministic ? 1 : 0;
     sh.len = p.kb_total + DRAIN_COLS * p.tile_n / MAX_TILE_N / p.ks;
     // (a share of a few k blocks is not worth a CTA of its own: it costs a piece of the output and its meeting)
-    const unsigned most = L.deterministic ? tiles : (tiles * sh.kb * p.ks + 127) / 128;
-    if (most < (unsigned)workers) workers = (int)most;
+    const long long columns = (long long)tiles * sh.kb * p.ks;            // (of all tiles: past 32 bits for large calls)
+    const long long most = L.deterministic ? tiles : (columns + 127) / 128;
+    if (most < workers) workers = (int)most;
     sh.workers = p.grid = workers;
     const unsigned line = sh.whole_tiles ? tiles : tiles * sh.len;
     sh.each = line / workers; sh.rest = line % workers;
@@ -1147,7 +1148,7 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
     p.tma_out = (L.out_dtype == VPTQ_DTYPE_FP32 && (L.M & 3) == 0) ? 1 : 0;
     p.scratch = p.any_split && !p.tma_out;
     // flag order makes CTAs wait for one another: only for a call that has the GPU to itself
-    p.flag_order = (p.any_split && p.tma_out && tiles * sh.kb / workers * p.ks >= FLAG_ORDER_MIN_COLS && !L.concurrent) ? 1 : 0;
+    p.flag_order = (p.any_split && p.tma_out && columns / workers >= FLAG_ORDER_MIN_COLS && !L.concurrent) ? 1 : 0;
     // Shared memory: tables, A ring, then a B ring of up to 96 KB.  Three stages of it come before
     // copies of the residual table (eight copies are free of bank conflicts).  A table in L2
     // needs the L1 that is left, whose lines hold the reads in flight: past 196 KB a CTA (with the 1 KB the system keeps)
@@ -1169,10 +1170,11 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
     }
     // pre-pass: enough blocks to fill the GPU (each of them is one part of eight tokens' bias terms)
     const int images = p.kb_total * (p.ks / IMG_COLS);
-    const int row_bytes = (L.N + 7) / 8 * 16;
+    const long long row_bytes = (L.N + 7LL) / 8 * 16;
     p.pre_rows = !L.permuted || (long long)B * L.N * n_layers < PRE_ROWS_MIN ? 0 : 4 * row_bytes <= 100 * 1024 ? 4 : 2 * row_bytes <= 200 * 1024 ? 2 : 0;
     p.pre_x = p.tiles_t * p.tile_n / (p.pre_rows ? p.pre_rows : 8);
-    p.pre_y = p.pre_rows ? 2 * device_sm_count() / (p.pre_x * n_layers) : ceil_div(4 * device_sm_count(), p.pre_x * n_layers);
+    const long long sms = device_sm_count(), blocks = (long long)p.pre_x * n_layers;
+    p.pre_y = (int)(p.pre_rows ? 2 * sms / blocks : (4 * sms + blocks - 1) / blocks);
     if (p.pre_y < 1) p.pre_y = 1;
     if (p.pre_y > ceil_div(images, 8)) p.pre_y = ceil_div(images, 8);
     p.pad_bytes = (V != 8 && (p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL)) ? (V <= 8 ? 16 : 32) : 0;
@@ -1335,9 +1337,10 @@ cudaError_t launch_layers(const LayerView *Ls, int n, const void *x, int B, void
 
 bool gemm_tcgen05_supported(const LayerView &L, int B)
 {
-    if (B < 1 || L.scale_rows || L.Nc <= 0) return false;
-    // (unit numbers are 32-bit: more than any batch that fits the device's memory needs)
-    return (L.v == 6 || L.v == 8 || L.v == 12) && ((long long)L.M / 96 + 1) * (B / 256 + 1) * (L.N / 16 + 16) < 0x7fffffffLL;
+    if (B < 1 || B > (1 << 30) || L.scale_rows || L.Nc <= 0) return false;       // (token numbers, padded to whole tiles, are 32-bit)
+    // (so are unit numbers: more than any batch that fits the device's memory needs)
+    const long long tiles = (L.M / 96 + 1LL) * (B / 256 + 1), blocks = L.N / 16 + 16;
+    return (L.v == 6 || L.v == 8 || L.v == 12) && tiles <= 0x7fffffffLL / blocks;
 }
 
 long long gemm_tcgen05_workspace_bytes(const LayerView *Ls, int n, int B)

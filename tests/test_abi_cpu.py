@@ -3,6 +3,8 @@ its host-only format arithmetic agrees with the oracle's and with the paper's fo
 import ctypes as C
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -191,3 +193,31 @@ def test_calls_that_share_the_gpu_never_wait_between_ctas(binding):
     half = b.make_desc(4096, 14336, 8, 65536, 256, x_dtype="bf16", out_dtype="fp16")
     assert b.lib.vptq_linear_waits_between_ctas(C.byref(half), 512) == 0
     assert b.lib.vptq_linear_waits_between_ctas(C.byref(down), 0) == b.E_SHAPE
+
+
+@pytest.mark.parametrize("M,N,B,kw", [
+    (524288, 8192, 65536, dict(v=8, k1=65536, k2=256, out_dtype="fp32")),        # tiles x k blocks x 32 columns = 2^32
+    (4194304, 1024, 65536, dict(v=8, k1=65536, k2=256, out_dtype="fp32", flags=33)),
+    (2 ** 30, 2 ** 28, 2 ** 28, dict(v=6, k1=5000, k2=5000)),                    # ... and some that pass 64 bits
+    (2 ** 30, 2 ** 30, 2 ** 28, dict(v=6, k1=5000, k2=5000)),
+    (32, 64, 2 ** 30, dict(v=8, k1=4096, flags=9)),                              # a column order: 2^29 blocks of the pre-pass, times four layers
+    (32, 64, 2 ** 31 - 1, dict(v=12, k1=4096, k2=4096)),
+    (64, 2 ** 31 - 1, 20, dict(v=8, k1=65536, flags=9)),
+    (2 ** 31 - 1, 64, 1, dict(v=8, k1=65536, k2=256)),
+])
+def test_size_queries_of_very_large_calls_answer(M, N, B, kw):
+    # sizes whose products pass 32 bits.  In a process of its own: an arithmetic fault ends it
+    code = f"""
+import ctypes as C
+from paper_2409_17066_b200 import binding as b
+d = b.make_desc({M}, {N}, **{kw!r})
+four = (b.LayerDesc * 4)(d, d, d, d)
+print(b.lib.vptq_linear_workspace_bytes(C.byref(d), {B}), b.lib.vptq_linear_fused_workspace_bytes(four, 4, {B}),
+      b.lib.vptq_linear_waits_between_ctas(C.byref(d), {B}), b.vptq_linear_path(d, {B}))
+"""
+    r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    one, fused, waits, path = r.stdout.split()
+    assert 0 <= int(one) <= int(fused) and int(waits) >= 0
+    if path == "gemm_tcgen05":
+        assert int(one) >= 2 * B * N                        # the activations' images are part of it
