@@ -181,14 +181,17 @@ int64_t vptq_linear_workspace_bytes(const vptq_layer_desc *desc, int32_t B);
  * FP16 rounding of W_hat; FP32 accumulation; the result differs from the FP64 product
  * over the FP16-rounded weights by at most ~1e-3 of max|out|).
  *   x    [B][N] row-major, desc->x_dtype;  out [B][M] row-major, desc->out_dtype.
- * B <= 16 runs the split-K decode kernels; larger B runs the tensor-core path
+ * B <= 16 runs the decode kernels; larger B runs the tensor-core path
  * (tcgen05) when the layer qualifies (v = 6, 8 or 12, any codebook sizes, groups and outlier columns, scale and
- * bias per input column), otherwise the decode kernels over groups of 16 tokens.  From 5 tokens on the paths
- * "decode_l2_fma" and "decode_gl_fma" run the tensor-core kernel as well.  Calls on one stream are ordered; calls
- * on different streams must not share a workspace.
- * The tensor-core path splits the input dimension of some output tiles over CTAs.  With long shares the CTA
+ * bias per input column), otherwise the decode kernels over groups of 16 tokens.  The tensor-core kernel also takes
+ * such layers on the path "decode_l2_fma" from 5 tokens on and on the path "decode_gl_fma" from 3 tokens on (not
+ * with VPTQ_FLAG_DETERMINISTIC): vptq_linear_path() goes on naming the family, and what is said of the tensor-core
+ * kernel here holds for these calls too.  Calls on one stream are ordered; calls on different streams must not share
+ * a workspace.
+ * The tensor-core kernel splits the input dimension of some output tiles over CTAs.  With long shares the CTA
  * that holds a tile's last piece stores it and raises a flag, and the CTAs that hold the other pieces wait for
- * that flag (bounded: about two seconds, then VPTQ_E_TIMEOUT in the status word) before they add theirs.  That
+ * that flag (bounded: about two seconds, then VPTQ_E_TIMEOUT in the status word) before they add theirs
+ * (vptq_linear_waits_between_ctas() tells which calls do).  That
  * is only live while every CTA of the grid (one per SM of the current device) is resident at once, i.e. while
  * the call has the GPU to itself.  A call that may overlap other GPU work — another stream, another process, an
  * SM limit — must set VPTQ_FLAG_CONCURRENT: the output is then cleared first and every piece is added, and no
@@ -211,17 +214,19 @@ int vptq_linear(const vptq_layer_desc *desc, const void *x, int32_t B,
  *   outs         host array of n_layers DEVICE pointers, outs[l] = [B][M_l] row-major
  * When every layer takes the same one of the decode paths "decode_l2_fma" (B <= 8), "decode_smem_fma"
  * or "decode_gl_fma" (B <= 4; for these two the layers must also share their format apart from M: v,
- * codebook sizes, outlier columns, groups, scale flag) and whole vector rows of the layers spread evenly
- * over the SMs, one kernel per token group serves all layers (no launch, prologue and ragged tail per
+ * codebook sizes, outlier columns, groups, scale flag) and have together at least as many vector rows as
+ * there are SMs, one kernel per token group serves all layers (no launch, prologue and ragged tail per
  * layer; no scratch).  Layers of one format apart from M that the batched tensor-core kernel takes share
  * one launch of it and of its pre-pass from 65 tokens on, and from 3 tokens on where that is faster than
- * their own launches; its scratch starts with a status word like that of "gemm_tcgen05".  Otherwise the
+ * their own launches; as in vptq_linear it may let CTAs wait for one another (unless one of the layers carries
+ * VPTQ_FLAG_CONCURRENT: a launch shares the GPU or does not), and its scratch starts with a status word:
+ * vptq_linear_fused_waits_between_ctas() and vptq_linear_fused_has_status() answer for a call.  Otherwise the
  * layers run one after the other on `stream`, sharing the workspace.
  * vptq_linear_fused_path() names which: "fused_decode_l2_fma", "fused_decode_smem_fma",
- * "fused_decode_gl_fma", "fused_gemm_tcgen05" (up to 8 tokens over a table in L2 still
- * "fused_decode_l2_fma") or "one_by_one" ("invalid" for arguments the call would reject).  Each layer's
- * result is the one vptq_linear gives for it (same arithmetic, same summation order within a vector
- * row).  Errors as for vptq_linear; nothing is launched when an argument is rejected. */
+ * "fused_decode_gl_fma", "fused_decode_bucket_fma" (prepared images), "fused_gemm_tcgen05" (its launch of up to
+ * 8 tokens over a table in L2 goes by the family's name, "fused_decode_l2_fma") or "one_by_one" ("invalid" for
+ * arguments the call would reject).  Each layer's result agrees with the one vptq_linear gives for it to FP32
+ * summation order.  Errors as for vptq_linear; nothing is launched when an argument is rejected. */
 #define VPTQ_MAX_FUSED_LAYERS 4
 int64_t vptq_linear_fused_workspace_bytes(const vptq_layer_desc *descs, int32_t n_layers, int32_t B);
 int vptq_linear_fused(const vptq_layer_desc *descs, const vptq_layer_ptrs *ptrs, int32_t n_layers,
@@ -427,26 +432,34 @@ int vptq_kmeans_update(const void *W, int32_t M, int32_t N, int32_t v, const int
 
 const char *vptq_status_string(int code);
 const char *vptq_last_cuda_error(void);
-/* Three paths — vptq_linear on "gemm_tcgen05" and on "decode_bucket_fma" (prepared images), and vptq_assign on
- * "assign_tcgen05" — keep an int32 status word at byte 0 of their workspace; after any other call the workspace holds no status and
- * this call has no meaning.  It synchronises `stream`, reads the word and returns VPTQ_E_TIMEOUT if a
+/* Three kernels — the batched tensor-core kernel and the one over prepared images, behind vptq_linear and
+ * vptq_linear_fused, and "assign_tcgen05" behind vptq_assign — keep an int32 status word at byte 0 of their workspace;
+ * vptq_linear_has_status() and vptq_linear_fused_has_status() tell for which calls.  After any other call the workspace holds
+ * no status and this call has no meaning.  It synchronises `stream`, reads the word and returns VPTQ_E_TIMEOUT if a
  * bounded device-side wait gave up during the call (the output is then invalid; the context stays
  * usable), VPTQ_E_UNSUPPORTED if the prepared-image kernel refused its image, else VPTQ_OK.  A null
  * workspace returns VPTQ_OK. */
 int vptq_workspace_status(const void *workspace, void *stream);
+/* 1 when the workspace of vptq_linear / vptq_linear_fused for these arguments starts with a status word (see
+ * vptq_workspace_status), 0 when not, negative VPTQ_E_* on bad arguments.  Not always apparent from the path's name: the
+ * tensor-core kernel also takes calls of "decode_l2_fma" and "decode_gl_fma" (see vptq_linear).  Where a fused call runs its
+ * layers one by one, the answer and the word are the last layer's. */
+int vptq_linear_has_status(const vptq_layer_desc *desc, int32_t B);
+int vptq_linear_fused_has_status(const vptq_layer_desc *descs, int32_t n_layers, int32_t B);
 /* For tests of the error path: the kernels' device-side waits (on mbarriers and flags) give up after about
  * two seconds; this sets the limit, in SM clock cycles, for the kernels launched afterwards by any thread
  * (0 restores the default).  With a limit of a few cycles a healthy kernel abandons its first wait that is
  * not already satisfied, reports VPTQ_E_TIMEOUT in its status word, leaves no copy in flight and returns;
  * the context stays usable.  Honoured by the path "decode_bucket_fma".  Process-wide; not for production. */
 void vptq_debug_set_wait_limit(uint64_t cycles);
-/* 1 when the kernels of vptq_linear for (desc, B) let one CTA wait for a flag that another CTA of the same grid
- * raises, 0 when no CTA waits for another, negative VPTQ_E_* on bad arguments.  Only the batched path does this
- * (see vptq_linear), and VPTQ_FLAG_CONCURRENT switches it off. */
+/* 1 when the kernels of vptq_linear / vptq_linear_fused for these arguments let one CTA wait for a flag that another CTA of
+ * the same grid raises, 0 when no CTA waits for another, negative VPTQ_E_* on bad arguments.  Only the tensor-core kernel
+ * does this, under whatever path's name it runs (see vptq_linear), and VPTQ_FLAG_CONCURRENT switches it off. */
 int vptq_linear_waits_between_ctas(const vptq_layer_desc *desc, int32_t B);
+int vptq_linear_fused_waits_between_ctas(const vptq_layer_desc *descs, int32_t n_layers, int32_t B);
 /* Name of the kernel family vptq_linear picks for (desc, B): "generic", "decode_smem_fma",
  * "decode_smem_mma", "decode_l2_fma", "decode_gl_fma", "gemm_tcgen05", "decode_bucket_fma".  For tests and
- * benchmark logs. */
+ * benchmark logs (a family, not a kernel: see vptq_linear). */
 const char *vptq_linear_path(const vptq_layer_desc *desc, int32_t B);
 /* Number of kernels one vptq_linear call launches (scratch memsets are not counted). */
 int vptq_linear_launches(const vptq_layer_desc *desc, int32_t B);

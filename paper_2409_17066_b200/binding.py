@@ -100,6 +100,9 @@ EXPORTS = {
     "vptq_workspace_status": (C.c_int, [C.c_void_p, C.c_void_p]),
     "vptq_debug_set_wait_limit": (None, [C.c_uint64]),
     "vptq_linear_waits_between_ctas": (C.c_int, [C.POINTER(LayerDesc), C.c_int32]),
+    "vptq_linear_fused_waits_between_ctas": (C.c_int, [C.POINTER(LayerDesc), C.c_int32, C.c_int32]),
+    "vptq_linear_has_status": (C.c_int, [C.POINTER(LayerDesc), C.c_int32]),
+    "vptq_linear_fused_has_status": (C.c_int, [C.POINTER(LayerDesc), C.c_int32, C.c_int32]),
     "vptq_linear_path": (C.c_char_p, [C.POINTER(LayerDesc), C.c_int32]),
     "vptq_linear_launches": (C.c_int, [C.POINTER(LayerDesc), C.c_int32]),
 }

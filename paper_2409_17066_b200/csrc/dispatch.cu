@@ -34,12 +34,25 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
     return PATH_GENERIC;
 }
 
-// The families whose main tables are in L2 or group-wise take at most four or two tokens per launch and gather every centroid
+// Whether a call of this family runs in the batched kernel.  The families whose main tables are in L2 or group-wise take at most four or two tokens per launch and gather every centroid
 // again for the next ones; the batched kernel gathers it once whatever the batch.  4096 x 4096 over the 1 MiB table: 25 us
 // at any batch up to 64, against 14-17 us per four tokens; 11008 x 4096, v = 12 in four groups: 52 us against 31 us per two.
-static bool batched_decode(LinearPath path, const LayerView &L, int B)
+static bool takes_batched(LinearPath path, const LayerView &L, int B)
 {
+    if (path == PATH_GEMM_TCGEN05) return true;
     return ((path == PATH_DECODE_L2_FMA && B >= 5) || (path == PATH_DECODE_GL_FMA && B >= 3)) && !L.deterministic && gemm_tcgen05_supported(L, B);
+}
+
+// (answers for the kernel that runs, whatever the family is called)
+bool linear_waits_between_ctas(const LayerView &L, int B, int flags)
+{
+    return takes_batched(choose_path(L, B, flags), L, B) && gemm_tcgen05_waits_between_ctas(&L, 1, B);
+}
+
+bool linear_has_status(const LayerView &L, int B, int flags)
+{
+    const LinearPath path = choose_path(L, B, flags);
+    return path == PATH_DECODE_BUCKET_FMA || takes_batched(path, L, B);
 }
 
 const char *linear_path_name(const LayerView &L, int B, int flags)
@@ -58,13 +71,12 @@ const char *linear_path_name(const LayerView &L, int B, int flags)
 long long linear_workspace_bytes(const LayerView &L, int B, int flags)
 {
     const LinearPath path = choose_path(L, B, flags);
-    if (batched_decode(path, L, B)) return gemm_tcgen05_workspace_bytes(&L, 1, B);
+    if (takes_batched(path, L, B)) return gemm_tcgen05_workspace_bytes(&L, 1, B);
     switch (path) {
     case PATH_DECODE_SMEM_FMA: return 0;
     case PATH_DECODE_SMEM_MMA: return smem_mma_workspace_bytes(L, decode_group(B));
     case PATH_DECODE_L2_FMA: return l2_fma_workspace_bytes(L, decode_group(B));
     case PATH_DECODE_GL_FMA: return 0;
-    case PATH_GEMM_TCGEN05: return gemm_tcgen05_workspace_bytes(&L, 1, B);
     case PATH_DECODE_BUCKET_FMA: return (long long)bucket_fma_workspace_bytes(&L, &L.prep_parts, 1);
     default: return generic_workspace_bytes(L, B);
     }
@@ -75,12 +87,11 @@ int linear_launches(const LayerView &L, int B, int flags)
     const int groups = ceil_div(B, DECODE_MAX_B);
     const int last = B - (groups - 1) * DECODE_MAX_B;
     const LinearPath path = choose_path(L, B, flags);
-    if (batched_decode(path, L, B)) return gemm_tcgen05_launches(L, B);
+    if (takes_batched(path, L, B)) return gemm_tcgen05_launches(L, B);
     switch (path) {
     case PATH_DECODE_SMEM_FMA:
         return (groups - 1) * smem_fma_launches(L, DECODE_MAX_B) + smem_fma_launches(L, last);
     case PATH_DECODE_SMEM_MMA: return groups * (smem_tc_supported(L, decode_group(B)) ? 2 : 1);      // pre-pass + main kernel
-    case PATH_GEMM_TCGEN05: return gemm_tcgen05_launches(L, B);
     case PATH_DECODE_BUCKET_FMA: return 1;
     case PATH_DECODE_L2_FMA:
         return (groups - 1) * l2_fma_launches(L, DECODE_MAX_B) + l2_fma_launches(L, last);
@@ -97,7 +108,7 @@ int linear_dispatch(const LayerView &L, int flags, const void *x, int B, void *o
     const LinearPath path = choose_path(L, B, flags);
     if (path == PATH_GENERIC) {
         e = launch_linear_generic(L, x, B, out, ws, st);
-    } else if (path == PATH_GEMM_TCGEN05 || batched_decode(path, L, B)) {
+    } else if (takes_batched(path, L, B)) {
         e = launch_gemm_tcgen05(&L, 1, x, B, &out, ws, st);
     } else if (path == PATH_DECODE_BUCKET_FMA) {
         const void *img = L.prepared;
@@ -145,7 +156,7 @@ LinearPath fused_path(const LayerView *Ls, const int *flags, int n, int B)
     const LinearPath path = choose_path(Ls[0], B, flags[0]);
     for (int l = 1; l < n; l++)
         if (choose_path(Ls[l], B, flags[l]) != path) return PATH_GENERIC;
-    if (path == PATH_GEMM_TCGEN05 || batched_decode(path, Ls[0], B) || path == PATH_DECODE_SMEM_MMA) {
+    if (takes_batched(path, Ls[0], B) || path == PATH_DECODE_SMEM_MMA) {
         if (fused_batched(path, Ls, n, B) && gemm_tcgen05_fused_supported(Ls, n, B)) return PATH_GEMM_TCGEN05;
         if (path != PATH_DECODE_L2_FMA || B > 8) return PATH_GENERIC;
     }
@@ -168,7 +179,8 @@ LinearPath fused_path(const LayerView *Ls, const int *flags, int n, int B)
 const char *linear_fused_path_name(const LayerView *Ls, const int *flags, int n, int B)
 {
     const LinearPath path = fused_path(Ls, flags, n, B);
-    // (up to 8 tokens callers know these layers by the decode family's name, whichever kernel takes them)
+    // (a family's name, as in linear_path_name: up to 8 tokens over a table in L2 the decode family's, whichever kernel takes them;
+    // linear_fused_has_status and linear_fused_waits_between_ctas answer for the kernel)
     if (path == PATH_GEMM_TCGEN05 && B <= 8 && choose_path(Ls[0], B, flags[0]) == PATH_DECODE_L2_FMA) return "fused_decode_l2_fma";
     switch (path) {
     case PATH_DECODE_L2_FMA: return "fused_decode_l2_fma";
@@ -178,6 +190,24 @@ const char *linear_fused_path_name(const LayerView *Ls, const int *flags, int n,
     case PATH_GEMM_TCGEN05: return "fused_gemm_tcgen05";
     default: return "one_by_one";
     }
+}
+
+bool linear_fused_waits_between_ctas(const LayerView *Ls, const int *flags, int n, int B)
+{
+    const LinearPath path = fused_path(Ls, flags, n, B);
+    if (path == PATH_GEMM_TCGEN05) return gemm_tcgen05_waits_between_ctas(Ls, n, B);
+    if (path != PATH_GENERIC) return false;
+    for (int l = 0; l < n; l++)
+        if (linear_waits_between_ctas(Ls[l], B, flags[l])) return true;
+    return false;
+}
+
+// (one layer after the other: the word, if any, is the last layer's)
+bool linear_fused_has_status(const LayerView *Ls, const int *flags, int n, int B)
+{
+    const LinearPath path = fused_path(Ls, flags, n, B);
+    if (path == PATH_GENERIC) return linear_has_status(Ls[n - 1], B, flags[n - 1]);
+    return path == PATH_GEMM_TCGEN05 || path == PATH_DECODE_BUCKET_FMA;
 }
 
 long long linear_fused_workspace_bytes(const LayerView *Ls, const int *flags, int n, int B)

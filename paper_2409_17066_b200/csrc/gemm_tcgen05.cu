@@ -1112,7 +1112,7 @@ struct GemmPlan {
 
 // `workers` CTAs at most, in a launch of n_layers layers
 template <int V>
-GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
+GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool concurrent)
 {
     GemmPlan p;
     memset(&p, 0, sizeof(p));
@@ -1148,7 +1148,7 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
     p.tma_out = (L.out_dtype == VPTQ_DTYPE_FP32 && (L.M & 3) == 0) ? 1 : 0;
     p.scratch = p.any_split && !p.tma_out;
     // flag order makes CTAs wait for one another: only for a call that has the GPU to itself
-    p.flag_order = (p.any_split && p.tma_out && columns / workers >= FLAG_ORDER_MIN_COLS && !L.concurrent) ? 1 : 0;
+    p.flag_order = (p.any_split && p.tma_out && columns / workers >= FLAG_ORDER_MIN_COLS && !concurrent) ? 1 : 0;
     // Shared memory: tables, A ring, then a B ring of up to 96 KB.  Three stages of it come before
     // copies of the residual table (eight copies are free of bank conflicts).  A table in L2
     // needs the L1 that is left, whose lines hold the reads in flight: past 196 KB a CTA (with the 1 KB the system keeps)
@@ -1190,10 +1190,11 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers)
     return p;
 }
 
-GemmPlan plan_gemm(const LayerView &L, int B, int workers, int n_layers)
+GemmPlan plan_gemm(const LayerView &L, int B, int workers, int n_layers, bool concurrent)
 {
-    return L.v == 8 ? plan_gemm_v<8>(L, B, workers, n_layers) : L.v == 6 ? plan_gemm_v<6>(L, B, workers, n_layers)
-                                                                         : plan_gemm_v<12>(L, B, workers, n_layers);
+    return L.v == 8   ? plan_gemm_v<8>(L, B, workers, n_layers, concurrent)
+           : L.v == 6 ? plan_gemm_v<6>(L, B, workers, n_layers, concurrent)
+                      : plan_gemm_v<12>(L, B, workers, n_layers, concurrent);
 }
 
 // The plans of the layers of one launch (n = 1: a launch of its own): the SMs are dealt out to the layers in proportion to
@@ -1203,7 +1204,11 @@ long long plan_launch(const LayerView *Ls, int n, int B, GemmPlan *pl)
     const int G = device_sm_count();
     int ctas[MAX_FUSED], used = 0;
     long long total = 0, ws = 0;
-    for (int l = 0; l < n; l++) total += Ls[l].R;
+    bool concurrent = false;                         // one layer's flag speaks for the launch
+    for (int l = 0; l < n; l++) {
+        total += Ls[l].R;
+        concurrent = concurrent || Ls[l].concurrent;
+    }
     for (int l = 0; l < n; l++) {
         ctas[l] = (int)(G * (long long)Ls[l].R / total);
         if (ctas[l] < 1) ctas[l] = 1;
@@ -1216,7 +1221,7 @@ long long plan_launch(const LayerView *Ls, int n, int B, GemmPlan *pl)
         ctas[most]++;
     }
     for (int l = 0; l < n; l++) {
-        pl[l] = plan_gemm(Ls[l], B, ctas[l], n);
+        pl[l] = plan_gemm(Ls[l], B, ctas[l], n, concurrent);
         ws += pl[l].ws_bytes;
     }
     return ws;
@@ -1361,7 +1366,14 @@ bool gemm_tcgen05_fused_supported(const LayerView *Ls, int n, int B)
 
 int gemm_tcgen05_launches(const LayerView &, int) { return 2; }   // pre-pass + GEMM
 
-bool gemm_tcgen05_waits_between_ctas(const LayerView &L, int B) { return plan_gemm(L, B, device_sm_count(), 1).flag_order != 0; }
+bool gemm_tcgen05_waits_between_ctas(const LayerView *Ls, int n, int B)
+{
+    GemmPlan pl[MAX_FUSED];
+    plan_launch(Ls, n, B, pl);
+    for (int l = 0; l < n; l++)
+        if (pl[l].flag_order) return true;
+    return false;
+}
 
 cudaError_t launch_gemm_tcgen05(const LayerView *Ls, int n, const void *x, int B, void *const *outs, void *ws, cudaStream_t st)
 {

@@ -9,7 +9,6 @@
 #include "paths.cuh"
 #include "assign.cuh"
 #include "prepared.cuh"
-#include "gemm.cuh"
 
 #include <vector>
 
@@ -586,7 +585,34 @@ int vptq_linear_waits_between_ctas(const vptq_layer_desc *desc, int32_t B)
     if (rc != VPTQ_OK) return rc;
     if (B <= 0) return VPTQ_E_SHAPE;
     LayerView L = make_view(desc, nullptr);
-    return choose_path(L, B, desc->flags) == PATH_GEMM_TCGEN05 && gemm_tcgen05_waits_between_ctas(L, B) ? 1 : 0;
+    return linear_waits_between_ctas(L, B, desc->flags) ? 1 : 0;
+}
+
+int vptq_linear_has_status(const vptq_layer_desc *desc, int32_t B)
+{
+    const int rc = check_desc(desc);
+    if (rc != VPTQ_OK) return rc;
+    if (B <= 0) return VPTQ_E_SHAPE;
+    LayerView L = make_view(desc, nullptr);
+    return linear_has_status(L, B, desc->flags) ? 1 : 0;
+}
+
+int vptq_linear_fused_waits_between_ctas(const vptq_layer_desc *descs, int32_t n_layers, int32_t B)
+{
+    LayerView Ls[VPTQ_MAX_FUSED_LAYERS];
+    int flags[VPTQ_MAX_FUSED_LAYERS];
+    const int rc = fused_views(descs, nullptr, n_layers, B, Ls, flags);
+    if (rc != VPTQ_OK) return rc;
+    return linear_fused_waits_between_ctas(Ls, flags, n_layers, B) ? 1 : 0;
+}
+
+int vptq_linear_fused_has_status(const vptq_layer_desc *descs, int32_t n_layers, int32_t B)
+{
+    LayerView Ls[VPTQ_MAX_FUSED_LAYERS];
+    int flags[VPTQ_MAX_FUSED_LAYERS];
+    const int rc = fused_views(descs, nullptr, n_layers, B, Ls, flags);
+    if (rc != VPTQ_OK) return rc;
+    return linear_fused_has_status(Ls, flags, n_layers, B) ? 1 : 0;
 }
 
 int vptq_linear_launches(const vptq_layer_desc *desc, int32_t B)

@@ -221,3 +221,39 @@ print(b.lib.vptq_linear_workspace_bytes(C.byref(d), {B}), b.lib.vptq_linear_fuse
     assert 0 <= int(one) <= int(fused) and int(waits) >= 0
     if path == "gemm_tcgen05":
         assert int(one) >= 2 * B * N                        # the activations' images are part of it
+
+
+@pytest.mark.parametrize("fmt,name,first", [
+    (dict(v=8, k1=65536, k2=256), "decode_l2_fma", 5),
+    (dict(v=12, k1=4096, k2=4096, n_outlier=82, v0=4, k0=8192, n_groups=4), "decode_gl_fma", 3),
+])
+def test_queries_answer_for_the_kernel_that_runs_whatever_the_path_is_called(binding, fmt, name, first):
+    # the tensor-core kernel takes these families' calls from `first` tokens on, with waits between CTAs and a status word
+    b = binding
+
+    def q(B, **kw):
+        d = b.make_desc(28672, 8192, **dict(dict(fmt, out_dtype="fp32"), **kw))
+        return b.vptq_linear_path(d, B), b.lib.vptq_linear_waits_between_ctas(C.byref(d), B), b.lib.vptq_linear_has_status(C.byref(d), B)
+    for B in (1, first - 1, first, 8, 16, 17):
+        batched = int(B >= first)
+        assert q(B) == ("gemm_tcgen05" if B > 16 else name, batched, batched)
+        assert q(B, flags=b.FLAG_SCALE_BIAS | b.FLAG_CONCURRENT)[1:] == (0, batched)
+    assert q(8, flags=b.FLAG_SCALE_BIAS | b.FLAG_DETERMINISTIC)[1:] == (0, 0)
+    assert q(16, out_dtype="fp16")[1:] == (0, 1)              # pieces meet in the scratch: nobody waits
+
+    def fused(B, flags=b.FLAG_SCALE_BIAS):
+        two = [b.make_desc(8184, 8192, **dict(fmt, out_dtype="fp32", flags=f)) for f in (b.FLAG_SCALE_BIAS, flags)]
+        arr = (b.LayerDesc * 2)(*two)
+        return (b.vptq_linear_fused_path(two, B) == "one_by_one", b.lib.vptq_linear_fused_waits_between_ctas(arr, 2, B),
+                b.lib.vptq_linear_fused_has_status(arr, 2, B))
+    for B in (1, first - 1, first, 8, 9, 16, 17, 300):
+        batched = int(B >= first)
+        one_by_one = fused(B)[0]
+        assert fused(B)[1:] == (batched, batched)
+        # the flag of one layer speaks for the launch it is part of
+        assert fused(B, b.FLAG_SCALE_BIAS | b.FLAG_CONCURRENT)[1:] == (int(batched and one_by_one), batched)
+    assert fused(17)[0] and not fused(300)[0]
+    assert b.lib.vptq_linear_fused_waits_between_ctas(None, 2, 8) == b.E_NULL
+    assert b.lib.vptq_linear_fused_has_status((b.LayerDesc * 1)(b.make_desc(64, 64, 8, 256)), 1, 0) == b.E_SHAPE
+    small = b.make_desc(11008, 4096, 6, 4096, 256)
+    assert [b.lib.vptq_linear_has_status(C.byref(small), B) for B in (1, 16, 17)] == [0, 0, 1]

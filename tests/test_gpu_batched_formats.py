@@ -97,3 +97,27 @@ def test_column_orders_gathered_from_staged_rows(N, B):
     dl = b.DeviceLayer(d)
     y = dl.linear(dl.upload_x(d["x"]))
     assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
+
+
+@pytest.mark.parametrize("Ms,B,kw", [((1000,), 5, dict(v=8, k1=65536)), ((1000,), 16, dict(v=8, k1=65536, out_dtype="fp32")), ((600,), 3, V12),
+                                     ((1024, 264), 6, dict(v=8, k1=65536)), ((600, 1300), 3, V12)])
+def test_calls_that_keep_a_status_word_set_it(Ms, B, kw):
+    """What vptq_linear_has_status promises: the word an earlier error left behind is gone after a healthy call."""
+    import torch
+    from paper_2409_17066_b200 import binding as b
+    ds = [synth.make_layer(synth.LayerSpec("st%d" % i, M, 1100, **kw), 98 + i, 0, B) for i, M in enumerate(Ms)]
+    dls = [b.DeviceLayer(d) for d in ds]
+    call = dls[0] if len(Ms) == 1 else b.FusedLayers(dls)
+    if len(Ms) == 1:
+        assert b.lib.vptq_linear_has_status(C.byref(call.desc), B) == 1
+    else:
+        assert b.lib.vptq_linear_fused_has_status(call.descs, call.n, B) == 1
+    ws = call.workspace(B)
+    ws.view(torch.int32)[0] = b.E_TIMEOUT
+    assert b.vptq_workspace_status(ws) == b.E_TIMEOUT
+    x = dls[0].upload_x(ds[0]["x"])
+    outs = [torch.empty(B, M, dtype=b._TORCH_DT[dl.desc.out_dtype], device="cuda") for M, dl in zip(Ms, dls)]
+    call.linear(x, outs[0] if len(Ms) == 1 else outs)
+    assert call.workspace(B) is ws and b.vptq_workspace_status(ws) == b.OK
+    for d, y in zip(ds, outs):
+        assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(ds[0]["x"])) <= TOL
