@@ -37,7 +37,8 @@
 //     (a bounded wait that is normally over before it starts) and reduce-add;
 //   - FP32 output, short shares or a call that shares the GPU: in the output, cleared by the pre-pass, every piece adds;
 //   - any other output: in an FP32 scratch tile cleared by the pre-pass; every piece adds and counts itself in, and
-//     whichever warp finds its part complete converts and stores it (nobody waits).  Whole tiles per CTA, the form before,
+//     whichever warp finds its part complete converts and stores it (nobody waits).  Only split tiles have one, at most one
+//     per cut between two shares, so the scratch does not grow with the call.  Whole tiles per CTA, the form before,
 //     left 84 of 148 SMs idle on an 8192 x 8192 layer at 333 tokens and 140 on a 1024 x 8192 one.
 //
 // Every mbarrier wait is bounded: after about two seconds a waiter records VPTQ_E_TIMEOUT in
@@ -137,7 +138,8 @@ struct GemmParams {
     int bias_parts;
     int *tile_flags;     // [tiles][EPI_WARPS]: flag order: [tile][0] counts the epilogue warps that have stored the last
                          // piece; scratch: arrivals per epilogue warp
-    float *scratch;      // [tiles][4][scratch_rows(tile_n)][32] FP32 sums of split tiles, or null
+    float *scratch;      // [slots][4][scratch_rows(tile_n)][32] FP32 sums of split tiles, or null
+    int slot_per_tile;   // a split tile's slot: 1 = its number, 0 = the worker that holds its first unit
     const uint8_t *xs;   // activation images, [tiles_t][kb_total * KS / 32][tile_n * 64 bytes]
     const uint8_t *tab1, *tab2;     // tables read from global memory: rows of 16 (v <= 8) or 32 bytes
 };
@@ -933,11 +935,13 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             const bool to_scratch = split && P.scratch != nullptr;
             const bool add = P.flag_order ? kb1 != P.kb_total : split;
             const bool announce = P.flag_order && kb0 != 0 && kb1 == P.kb_total;
-            int pieces = 0;                                  // shares that hold some of the tile (worked out while the MMAs run)
+            int pieces = 0, slot = tile;                     // shares that hold some of the tile (worked out while the MMAs run)
             if (to_scratch) {
                 const unsigned first_u = (unsigned)tile * P.kb_total, end_u = first_u + P.kb_total;
-                unsigned at = 0;
-                for (unsigned w = P.shares.worker_of(first_u); at < end_u; w++) {
+                unsigned at = 0, w = P.shares.worker_of(first_u);
+                // (that worker's share ends inside this tile, so no other split tile begins in it, and it is not the last one)
+                if (!P.slot_per_tile) slot = (int)w;
+                for (; at < end_u; w++) {
                     const unsigned next = P.shares.begin(w + 1);
                     pieces += next > at;                                     // (an empty share holds nothing)
                     at = next;
@@ -956,7 +960,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             // rows of this quarter that belong to the tile: a 120-row tile leaves 8 lanes of the last quarter unused, and a
             // 32-row box of the output must not touch the next tile's rows, so that quarter stores element by element
             const bool box = P.tma_out && 32 * q + 32 <= TILE_M;
-            float *sc = to_scratch ? P.scratch + ((long long)tile * 4 + q) * scratch_rows(P.tile_n) * 32 : nullptr;
+            float *sc = to_scratch ? P.scratch + ((long long)slot * 4 + q) * scratch_rows(P.tile_n) * 32 : nullptr;
             for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += 2 * EPI_TOKENS) {
                 uint32_t r[EPI_TOKENS];
                 tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c1, r);
@@ -1100,7 +1104,7 @@ EncodeTiledFn get_encode_fn()
 struct GemmPlan {
     int t1, t2;                      // TableSource of the main and the residual table
     Shares shares;
-    int tiles_m, tiles_t, tile_n, n0, ks, kb_main, kb_total, grid, any_split, flag_order, tma_out, scratch;
+    int tiles_m, tiles_t, tile_n, n0, ks, kb_main, kb_total, grid, any_split, flag_order, tma_out, scratch, slot_per_tile;
     int b_stages, cb1_shift, cb2_shift, cb1_bytes, cb2_bytes;
     int pre_x, pre_y;                // pre-pass grid; pre_y = parts of a bias term
     int pre_rows;                    // tokens per block of the pre-pass that keeps rows in shared memory, 0 = the other one
@@ -1184,7 +1188,10 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     p.off_bpart = take((long long)p.pre_y * p.tiles_t * p.tile_n * 4);
     p.off_pad1 = take(p.pad_bytes && p.t1 == TABLE_GLOBAL ? (long long)L.G * L.k1 * p.pad_bytes : 0);
     p.off_pad2 = take(p.pad_bytes && p.t2 == TABLE_GLOBAL ? (long long)L.G * L.k2 * p.pad_bytes : 0);
-    p.n_scratch = p.scratch ? (long long)tiles * 4 * scratch_rows(p.tile_n) * 32 : 0;
+    // (a slot per tile of a large call would be its whole output in FP32, cleared at every call: 28672 x 8192 at 8192 tokens
+    // 1074 MB of workspace instead of 177)
+    p.slot_per_tile = (long long)tiles < workers;
+    p.n_scratch = p.scratch ? (p.slot_per_tile ? (long long)tiles : workers - 1) * 4 * scratch_rows(p.tile_n) * 32 : 0;
     p.off_scratch = take(p.n_scratch * 4);
     p.off_xs = take((long long)p.tiles_t * images * b_bytes);
     return p;
@@ -1310,6 +1317,7 @@ cudaError_t launch_layers(const LayerView *Ls, int n, const void *x, int B, void
         P.flag_order = pl.flag_order; P.tma_out = pl.tma_out;
         P.status = status; P.bpart = q.bpart; P.bias_parts = pl.pre_y; P.tile_flags = q.tile_flags;
         P.scratch = pl.scratch ? reinterpret_cast<float *>(w8 + pl.off_scratch) : nullptr;
+        P.slot_per_tile = pl.slot_per_tile;
         P.xs = q.xs;
         P.tab1 = q.pad1 ? q.pad1 : reinterpret_cast<const uint8_t *>(L.c1);
         P.tab2 = q.pad2 ? q.pad2 : reinterpret_cast<const uint8_t *>(L.c2);

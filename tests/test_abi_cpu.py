@@ -223,6 +223,28 @@ print(b.lib.vptq_linear_workspace_bytes(C.byref(d), {B}), b.lib.vptq_linear_fuse
         assert int(one) >= 2 * B * N                        # the activations' images are part of it
 
 
+@pytest.mark.parametrize("M,N,B,out", [
+    (28672, 8192, 8192, "fp16"), (28672, 8192, 512, "bf16"), (28674, 8192, 1025, "fp32"), (8192, 8192, 333, "fp16"),
+    (2176, 4096, 61681 * 512, "fp16"),               # tiles x columns = 2^32 + 4096: not 32 CTAs
+])
+def test_batched_scratch_holds_split_tiles_only(binding, M, N, B, out):
+    # FP32 sums of tiles cut between CTAs: a tile per cut at most, whatever the size of the output
+    b = binding
+    whole = b.vptq_linear_workspace_bytes(b.make_desc(M, N, 8, 65536, 256, out_dtype=out, flags=b.FLAG_SCALE_BIAS | b.FLAG_DETERMINISTIC), B)
+    split = b.vptq_linear_workspace_bytes(b.make_desc(M, N, 8, 65536, 256, out_dtype=out), B)
+    token_tiles = -(-B // 512)
+    tokens = -(-B // token_tiles)
+    tile_bytes = 128 * (-(-tokens // 32) * 32) * 4
+    tiles = -(-M // 128) * token_tiles
+    n_sm = 148
+    try:
+        import torch
+        n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    except Exception:
+        pass
+    assert split - whole == min(tiles, n_sm - 1) * tile_bytes
+
+
 @pytest.mark.parametrize("fmt,name,first", [
     (dict(v=8, k1=65536, k2=256), "decode_l2_fma", 5),
     (dict(v=12, k1=4096, k2=4096, n_outlier=82, v0=4, k0=8192, n_groups=4), "decode_gl_fma", 3),

@@ -49,6 +49,25 @@ def test_batched_kernel_formats_and_edges(M, N, B, kw):
     assert rel_err(shared.linear(x).float().cpu().numpy(), y_ref) <= tol
 
 
+@pytest.mark.parametrize("M,N,B,kw", [
+    (18816, 520, 40, dict(v=8, k1=65536)),                                        # on 148 SMs: a tile less than SMs, a slot per tile
+    (18944, 520, 40, dict(v=8, k1=65536, out_dtype="bf16")),                      # as many tiles as SMs, a slot per cut
+    (19065, 520, 33, dict(v=8, k1=65536, out_dtype="fp32")),                      # one more; rows of 4 bytes' alignment
+    (9600, 300, 600, dict(v=8, k1=65536, k2=256)),                                # two token tiles
+    (25000, 130, 520, dict(v=6, k1=256)),                                         # tiles of few k blocks: some whole, some cut
+    (600, 9000, 24, dict(v=12, k1=512)),                                          # few tiles, many pieces each
+])
+def test_split_tiles_have_scratch_of_their_own(M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    d = synth.make_layer(synth.LayerSpec("sl", M, N, **kw), 96, 0, B)
+    dl = b.DeviceLayer(d)
+    y_ref = oracle.Layer.from_synth(d).linear(d["x"])
+    x = dl.upload_x(d["x"])
+    tol = TOL if kw.get("out_dtype") != "bf16" else 2.0 ** -8
+    for _ in range(2):                                  # the second call finds the first one's sums and counts
+        assert rel_err(dl.linear(x).float().cpu().numpy(), y_ref) <= tol
+
+
 def test_batched_kernel_repeats_bit_for_bit_when_asked():
     from paper_2409_17066_b200 import binding as b
     spec = synth.LayerSpec("bd", 1210, 2100, **V6)
