@@ -368,11 +368,13 @@ int vptq_prepare(const vptq_layer_desc *desc, const vptq_layer_ptrs *p, int32_t 
  * no allocating library routine.
  *
  * Limits and errors: layers of another geometry return VPTQ_E_UNSUPPORTED.  The kernel
- * needs scratch only when the layer's vector rows do not divide well over the SMs (it then
- * deals the work out regardless of rows and adds partial sums up in scratch): 4 * g * M bytes, g the
- * tokens per launch (4 for B >= 4, 2 for B = 2 or 3, else 1), plus a few KB of counters.  A layer whose need exceeds the array returns
- * VPTQ_E_SCRATCH_LIMIT (M up to about 65000 fits at any B); nothing is launched in either
- * case.  vptq_linear_workspace_bytes() tells the need of a given layer and B.
+ * needs scratch only when the layer has more than 1024 / g vector rows per SM, g the tokens per
+ * launch (4 for B >= 4, 2 for B = 2 or 3, else 1): it then deals the work out regardless of rows and
+ * adds partial sums up in scratch, 4 * g * M bytes plus a few KB of counters.  A layer whose need
+ * exceeds the array returns VPTQ_E_SCRATCH_LIMIT; nothing is launched in either case.  On 148 SMs no
+ * layer of up to 303104 output rows needs scratch at any B, and none that needs it fits the array: it
+ * is used on a partition of a GPU with fewer than 32 SMs.  For B <= 4 vptq_linear_workspace_bytes()
+ * tells the need (larger batches of vptq_linear go to another kernel).
  *
  * Set-up: the first call on each device looks up the array's device address (with that
  * device current) and remembers it; make that first call outside any stream capture.

@@ -20,7 +20,7 @@
 //   balanced tasks are dealt out regardless of rows: partial sums meet in an FP32 scratch array
 //            through atomic adds, and a task counter per block of 16 vector rows tells which warp
 //            completed the block and so converts and stores it.  Only for so many rows that their
-//            sums do not fit shared memory: clearing the scratch, the global atomics and the counters
+//            sums do not fit shared memory (past 1024 / tokens rows a CTA): clearing the scratch, the global atomics and the counters
 //            cost more than SMs that get a row less.  One token, 16 warps, as a dependent launch:
 //            1024 x 4096 12.3 -> 4.8 us, 3000 x 4096 18.4 -> 8.9, 5000 x 4096 21.1 -> 12.7.
 // Fused launch (FUSED): up to MAX_FUSED layers that read the same activations (q/k/v, gate/up) in one
@@ -412,11 +412,7 @@ L2Plan plan_l2(const LayerView &L, int TB)
              (size_t)p.part_floats * 4 + (p.det && p.owner ? (size_t)(rows_cta + WARPS) * TB * 8 * 4 : 0);
     p.ws_bytes = 0;
     p.off_counters = 0;
-    // (callers have sized their scratch by this number; row-owner mode leaves it alone)
-    const double eff_cta = (double)L.R / ((double)(L.R < G ? L.R : G) * rows_cta) * (L.R < G ? (double)L.R / G : 1.0);
-    const long long t_cta = (long long)rows_cta * (slab / 256);
-    const double eff_warp = (double)t_cta / ((double)WARPS * (double)((t_cta + WARPS - 1) / WARPS));
-    if (!p.owner || (eff_cta * eff_warp < 0.80 && !p.det)) {
+    if (!p.owner) {
         p.off_counters = ((long long)TB * L.M * 4 + 255) / 256 * 256;
         p.ws_bytes = p.off_counters + ((long long)ceil_div(L.R, RB_ROWS) * 4 + 255) / 256 * 256;
     }

@@ -1189,7 +1189,7 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     p.off_pad1 = take(p.pad_bytes && p.t1 == TABLE_GLOBAL ? (long long)L.G * L.k1 * p.pad_bytes : 0);
     p.off_pad2 = take(p.pad_bytes && p.t2 == TABLE_GLOBAL ? (long long)L.G * L.k2 * p.pad_bytes : 0);
     // (a slot per tile of a large call would be its whole output in FP32, cleared at every call: 28672 x 8192 at 8192 tokens
-    // 1074 MB of workspace instead of 177)
+    // 1074 MB of workspace instead of 173)
     p.slot_per_tile = (long long)tiles < workers;
     p.n_scratch = p.scratch ? (p.slot_per_tile ? (long long)tiles : workers - 1) * 4 * scratch_rows(p.tile_n) * 32 : 0;
     p.off_scratch = take(p.n_scratch * 4);

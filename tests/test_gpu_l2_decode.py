@@ -1,5 +1,7 @@
 """Decode over a table in L2 at row counts that do not divide over the SMs: fewer rows than SMs, one row more, a ragged last row,
 less than a chunk of columns, two slabs, layers of uneven rows that share a launch, calls back to back without a pause."""
+import ctypes as C
+
 import pytest
 import torch
 
@@ -44,3 +46,40 @@ def test_uneven_rows_share_a_launch(Ms, B):
     fused.linear(dls[0].upload_x(ds[0]["x"]), ys)
     for d, y in zip(ds, ys):
         assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(ds[0]["x"])) <= TOL
+
+
+@pytest.mark.parametrize("M,N,B,k2,out,perm", [
+    (303109, 8200, 4, 256, "fp16", False),              # 37889 rows: the sums of one CTA no longer fit; two slabs; a short last row
+    (303112, 72, 4, 0, "fp32", True),
+    (606300, 40, 3, 0, "bf16", False),                  # two launches over one scratch, a token short
+    (1212500, 300, 1, 200, "fp32", False),
+])
+def test_more_rows_than_their_sums_fit_shared_memory(M, N, B, k2, out, perm):
+    """Tasks dealt out regardless of rows, partial sums in the workspace, against the plain kernel."""
+    from paper_2409_17066_b200 import binding as b
+    g = torch.Generator(device="cuda").manual_seed(M)
+
+    def stream(rows, k):                                # any bytes are indices (clamped where k is no power of two); N % 8 == 0
+        return torch.randint(0, 256, (rows, b.vptq_packed_row_bytes(N, k)), generator=g, dtype=torch.uint8, device="cuda")
+
+    def normal(sd, *shape):
+        return (torch.randn(shape, generator=g, device="cuda") * sd).half()
+    R = -(-M // 8)
+    parts = [stream(R, 65536), normal(0.02, 65536, 8), stream(R, k2) if k2 else None, normal(0.005, k2, 8) if k2 else None, None, None,
+             normal(0.2, N) + 1, normal(0.01, N), torch.randperm(N, generator=g, device="cuda").int() if perm else None]
+    ptrs = b.LayerPtrs(*[None if t is None else t.data_ptr() for t in parts])
+    flags = b.FLAG_SCALE_BIAS | (b.FLAG_COL_PERM if perm else 0)
+    desc = b.make_desc(M, N, 8, 65536, k2, out_dtype=out, flags=flags)
+    plain = b.make_desc(M, N, 8, 65536, k2, out_dtype="fp32", flags=flags | b.FLAG_FORCE_GENERIC)
+    assert b.vptq_linear_path(desc, B) == "decode_l2_fma"
+    ws = torch.full((b.vptq_linear_workspace_bytes(desc, B),), 0x7F, dtype=torch.uint8, device="cuda")
+    assert ws.numel() >= 4 * (4 if B == 4 else 2 if B > 1 else 1) * M
+    ws_plain = torch.empty(b.vptq_linear_workspace_bytes(plain, B), dtype=torch.uint8, device="cuda")
+    for _ in range(2):                                  # the second call finds the first one's sums and counts
+        x = normal(1, B, N)
+        y = torch.full((B, M), float("nan"), dtype=b._TORCH_DT[desc.out_dtype], device="cuda")
+        want = torch.empty((B, M), dtype=torch.float32, device="cuda")
+        b.vptq_linear(desc, x, ptrs, y, ws)
+        b.vptq_linear(plain, x, ptrs, want, ws_plain)
+        err = (y.float() - want).abs().max() / want.abs().max()
+        assert float(err) <= (TOL if out != "bf16" else 2.0 ** -8)
