@@ -83,3 +83,21 @@ def test_more_rows_than_their_sums_fit_shared_memory(M, N, B, k2, out, perm):
         b.vptq_linear(plain, x, ptrs, want, ws_plain)
         err = (y.float() - want).abs().max() / want.abs().max()
         assert float(err) <= (TOL if out != "bf16" else 2.0 ** -8)
+
+
+def test_deterministic_sums_take_nothing_from_the_previous_kernel():
+    """Nine tasks for sixteen warps: the slots of warps without tasks hold what the previous kernel left in shared memory, here
+    the residual table of a layer that leaves large values at that place on every SM."""
+    from paper_2409_17066_b200 import binding as b
+    fill = synth.make_layer(synth.LayerSpec("fill", 8 * 148, 16384, v=8, k1=65536, k2=256), 100, 0, 1)
+    fill["c2"][:] = 60000.0                             # as FP32 pairs: 1.1e36
+    spec = synth.LayerSpec("det", 1030, 2100, v=8, k1=65536, k2=256)
+    d = synth.make_layer(spec, 101, 0, 1)
+    filler, dl = b.DeviceLayer(fill), b.DeviceLayer(d)
+    det = dl.with_flags(dl.desc.flags | b.FLAG_DETERMINISTIC)
+    x, xf = dl.upload_x(d["x"]), filler.upload_x(fill["x"])
+    y_ref = oracle.Layer.from_synth(d).linear(d["x"])
+    for _ in range(3):
+        filler.linear(xf)
+        torch.cuda.synchronize()
+        assert rel_err(det.linear(x).float().cpu().numpy(), y_ref) <= TOL
