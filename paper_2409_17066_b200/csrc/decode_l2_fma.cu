@@ -39,7 +39,6 @@ namespace {
 constexpr int RB_ROWS = 16;                 // vector rows per completion counter (balanced mode)
 constexpr int XS_BUDGET = 64 * 1024;        // bytes of staged activations per CTA
 constexpr int PART_BUDGET = 32 * 1024;      // bytes of per-row partial sums per CTA (OWNER mode)
-constexpr int WARPS = 16;                   // 4 tokens need 128 registers a thread; for fewer, 4096 x 4096 11.2 -> 10.7 us against 32
 
 struct L2FmaParams {
     LayerView L[MAX_FUSED];
@@ -87,7 +86,7 @@ __device__ __forceinline__ void act8_to_float(uint4 q, int is_bf16, float (&f)[8
     }
 }
 
-template <int TB, bool RES, bool OWNER, bool FUSED>
+template <int TB, bool RES, bool OWNER, bool FUSED, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32, 1)
 decode_l2_fma_kernel(const __grid_constant__ L2FmaParams P)
 {
@@ -384,11 +383,18 @@ decode_l2_fma_kernel(const __grid_constant__ L2FmaParams P)
 }
 
 struct L2Plan {
-    int slab_cols, n_slabs, chunks_total, cb2_rep, grid, owner, part_floats, det, rows_cta;
+    int slab_cols, n_slabs, chunks_total, cb2_rep, grid, owner, part_floats, det, rows_cta, warps;
     size_t smem;
     long long ws_bytes, off_counters;
     int cta_begin[MAX_FUSED + 1];   // fused launches only
 };
+
+// Warps of a CTA.  16 take the fewer tasks of a small layer in fewer, longer ranges (64 tasks, 4096 x 4096, one token: 11.7 us
+// against 12.2 with 32); the residual sum makes a task's chain long enough that many tasks want 32 to cover it: from 128 on
+// (2368 x 16384 22.9 -> 21.8 us, 28672 x 8192 111.8 -> 106.8, gate+up of that size in one launch and down 345 -> 318; 96 to 112
+// tasks between 0.96 and 1.06 times the time).  Without a residual the two differ by 2 % either way, and more tokens
+// need the registers.
+int pick_warps(int TB, bool res, int rows_cta, int chunks) { return TB == 1 && res && (long long)rows_cta * chunks >= 128 ? 32 : 16; }
 
 L2Plan plan_l2(const LayerView &L, int TB)
 {
@@ -408,8 +414,9 @@ L2Plan plan_l2(const LayerView &L, int TB)
     p.owner = (long long)p.part_floats * 4 <= PART_BUDGET ? 1 : 0;
     if (!p.owner) p.part_floats = 0;
     p.grid = p.owner ? (L.R < G ? L.R : G) : (G < p.n_slabs ? p.n_slabs : G);
-    p.smem = (size_t)TB * slab * 2 + 4 * 4 + (size_t)WARPS * 4 * 4 + (size_t)L.k2 * 16 * (p.cb2_rep ? 8 : 1) +
-             (size_t)p.part_floats * 4 + (p.det && p.owner ? (size_t)(rows_cta + WARPS) * TB * 8 * 4 : 0);
+    p.warps = pick_warps(TB, L.k2 > 0, rows_cta, p.chunks_total);
+    p.smem = (size_t)TB * slab * 2 + 4 * 4 + (size_t)p.warps * 4 * 4 + (size_t)L.k2 * 16 * (p.cb2_rep ? 8 : 1) +
+             (size_t)p.part_floats * 4 + (p.det && p.owner ? (size_t)(rows_cta + p.warps) * TB * 8 * 4 : 0);
     p.ws_bytes = 0;
     p.off_counters = 0;
     if (!p.owner) {
@@ -438,7 +445,8 @@ bool plan_l2_fused(const LayerView *Ls, int n, int TB, L2Plan *out)
     if ((long long)p.part_floats * 4 > PART_BUDGET) return false;
     p.owner = 1;
     p.grid = G;
-    p.smem = (size_t)TB * p.slab_cols * 2 + 4 * 4 + (size_t)WARPS * 4 * 4 +
+    p.warps = pick_warps(TB, Ls[0].k2 > 0, rows_cta, p.chunks_total);
+    p.smem = (size_t)TB * p.slab_cols * 2 + 4 * 4 + (size_t)p.warps * 4 * 4 +
              (size_t)Ls[0].k2 * 16 * (p.cb2_rep ? 8 : 1) + (size_t)p.part_floats * 4;
     p.ws_bytes = 0;
     p.off_counters = 0;
@@ -446,12 +454,20 @@ bool plan_l2_fused(const LayerView *Ls, int n, int TB, L2Plan *out)
     return true;
 }
 
+template <int TB, bool RES, bool OWNER, bool FUSED, int WARPS>
+cudaError_t launch_warps(const L2FmaParams &P, const L2Plan &pl, cudaStream_t st)
+{
+    auto kern = decode_l2_fma_kernel<TB, RES, OWNER, FUSED, WARPS>;
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), pl.smem);
+    if (e != cudaSuccess) return e;
+    return launch_dependent("l2_fma", kern, pl.grid, WARPS * 32, pl.smem, st, P);
+}
+
 template <int TB, bool RES, bool OWNER, bool FUSED>
 cudaError_t launch_one(const L2FmaParams &P, const L2Plan &pl, cudaStream_t st)
 {
-    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_l2_fma_kernel<TB, RES, OWNER, FUSED>), pl.smem);
-    if (e != cudaSuccess) return e;
-    return launch_dependent("l2_fma", decode_l2_fma_kernel<TB, RES, OWNER, FUSED>, pl.grid, WARPS * 32, pl.smem, st, P);
+    if (TB == 1 && RES && pl.warps == 32) return launch_warps<TB, RES, OWNER, FUSED, TB == 1 && RES ? 32 : 16>(P, pl, st);
+    return launch_warps<TB, RES, OWNER, FUSED, 16>(P, pl, st);
 }
 
 template <int TB>

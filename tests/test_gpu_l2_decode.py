@@ -21,6 +21,10 @@ pytestmark = pytest.mark.gpu
     (2400, 16640, 2, dict(k2=256, out_dtype="fp32")),
     (1000, 8200, 4, dict(out_dtype="bf16")),
     (1300, 1000, 3, dict(k2=200, has_scale=False)),
+    (8, 32512, 1, dict(k2=256)),                        # 127 chunks of one row: 16 warps
+    (8, 32513, 1, dict(k2=256)),                        # 128: 32 warps
+    (2361, 16380, 1, dict(k2=200, x_dtype="bf16", out_dtype="fp32")),
+    (1192, 36000, 1, dict(k2=256, permuted=True)),      # 32 warps, two slabs
 ])
 def test_rows_that_do_not_divide(M, N, B, kw):
     from paper_2409_17066_b200 import binding as b
@@ -83,6 +87,23 @@ def test_more_rows_than_their_sums_fit_shared_memory(M, N, B, k2, out, perm):
         b.vptq_linear(plain, x, ptrs, want, ws_plain)
         err = (y.float() - want).abs().max() / want.abs().max()
         assert float(err) <= (TOL if out != "bf16" else 2.0 ** -8)
+
+
+def test_many_tasks_a_cta_in_shared_and_deterministic_launches():
+    from paper_2409_17066_b200 import binding as b
+    ds = [synth.make_layer(synth.LayerSpec("m%d" % i, M, 16384, v=8, k1=65536, k2=256), 102 + i, 0, 1) for i, M in enumerate((1200, 1181))]
+    dls = [b.DeviceLayer(d) for d in ds]
+    x = dls[0].upload_x(ds[0]["x"])
+    fused = b.FusedLayers(dls)
+    assert fused.path(1) == "fused_decode_l2_fma"
+    ys = [torch.empty(1, d["spec"].M, dtype=torch.float16, device="cuda") for d in ds]
+    fused.linear(x, ys)
+    for d, dl, y in zip(ds, dls, ys):
+        y_ref = oracle.Layer.from_synth(d).linear(ds[0]["x"])
+        assert rel_err(y.float().cpu().numpy(), y_ref) <= TOL
+        det = dl.with_flags(dl.desc.flags | b.FLAG_DETERMINISTIC)
+        zs = [det.linear(x).clone() for _ in range(3)]
+        assert all(torch.equal(z, zs[0]) for z in zs) and rel_err(zs[0].float().cpu().numpy(), y_ref) <= TOL
 
 
 def test_deterministic_sums_take_nothing_from_the_previous_kernel():
