@@ -911,6 +911,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
         const int q = warp & 3;                                  // TMEM lane quarter this warp may read
         const int padded_b = P.tiles_t * P.tile_n;
         int seg_no = 0, bias_tile = -1;
+        unsigned piece = 0;                                      // staged pieces so far, over all segments: the buffers alternate
         grid_dependency_wait();                                  // bias terms, flags and cleared sums come from the pre-pass
         FOR_EACH_SEGMENT {
             const int mt = tile % P.tiles_m, tt = tile / P.tiles_m;
@@ -959,7 +960,8 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             const int m0 = mt * TILE_M + 32 * q;
             // rows of this quarter that belong to the tile: a 120-row tile leaves 8 lanes of the last quarter unused, and a
             // 32-row box of the output must not touch the next tile's rows, so that quarter stores element by element
-            const bool box = P.tma_out && 32 * q + 32 <= TILE_M;
+            // (a quarter past the last row stages nothing: a piece without a copy would break the count of copies in flight)
+            const bool box = P.tma_out && 32 * q + 32 <= TILE_M && m0 < L.M;
             float *sc = to_scratch ? P.scratch + ((long long)slot * 4 + q) * scratch_rows(P.tile_n) * 32 : nullptr;
             for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += 2 * EPI_TOKENS) {
                 uint32_t r[EPI_TOKENS];
@@ -980,12 +982,12 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                     // lane hands it to the copy engine (store or reduce-add); two staging buffers per warp, so the copy of
                     // one piece overlaps the next.  The buffer written two pieces ago must have been read by its copy.
 #pragma unroll
-                    for (int p = 0; p < EPI_TOKENS / PIECE_TOKENS; p++) {
+                    for (int p = 0; p < EPI_TOKENS / PIECE_TOKENS; p++, piece++) {
                         const int c2 = c1 + p * PIECE_TOKENS;
                         if (c2 >= t_cnt) break;
                         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
                         __syncwarp();
-                        const uint32_t buf = ebuf + (uint32_t)(p & 1) * EPI_BUF_BYTES;
+                        const uint32_t buf = ebuf + (piece & 1u) * EPI_BUF_BYTES;
 #pragma unroll
                         for (int j = 0; j < PIECE_TOKENS; j++)
                             asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + j * 128u + lane * 4u), "r"(r[p * PIECE_TOKENS + j]) : "memory");
@@ -993,7 +995,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                         __syncwarp();
                         if (lane == 0) {
                             if (to_scratch) bulk_add(sc + c2 * 32, buf);
-                            else if (m0 < L.M) tma_store_2d(&tmap_out, buf, m0, t0 + c2, add);
+                            else tma_store_2d(&tmap_out, buf, m0, t0 + c2, add);
                         }
                     }
                 } else if (m_ok) {

@@ -56,6 +56,8 @@ def test_batched_kernel_formats_and_edges(M, N, B, kw):
     (9600, 300, 600, dict(v=8, k1=65536, k2=256)),                                # two token tiles
     (25000, 130, 520, dict(v=6, k1=256)),                                         # tiles of few k blocks: some whole, some cut
     (600, 9000, 24, dict(v=12, k1=512)),                                          # few tiles, many pieces each
+    (40000, 72, 16, dict(v=8, k1=65536, out_dtype="fp32")),                       # segment after segment of one staged piece
+    (40032, 40, 33, dict(v=8, k1=65536, out_dtype="fp32")),                       # ... of three; a quarter without rows at the end
 ])
 def test_split_tiles_have_scratch_of_their_own(M, N, B, kw):
     from paper_2409_17066_b200 import binding as b
