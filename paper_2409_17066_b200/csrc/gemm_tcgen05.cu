@@ -18,8 +18,8 @@
 // (small ones as several skewed copies); larger or group-wise ones are read out of L2, rows of 12 and 24 bytes from a copy
 // with rows padded to 16 and 32 bytes that the pre-pass writes (one load instruction and one 32-byte sector per row).
 //
-// Warp roles: warp 0 bulk loads of B; warp 1 TMEM allocation + MMA issue (one thread); warps 4-19 the dequant producers in
-// GROUPS groups, a k block each in turn (the next visit's packed indices in flight); warps 20-27 the epilogue
+// Warp roles: warp 0 bulk loads of B; warp 1 TMEM allocation + MMA issue (an elected lane); 10 (v = 8) or 12 producer warps in
+// GROUPS groups, a k block each in turn (the next visit's packed indices in flight); 8 warps the epilogue
 // (tcgen05.ld -> + bias term -> output), two per TMEM lane quarter.
 // What bounds the k loop is the SM's shared-memory/L1 data pipe (128 bytes per clock), which everything passes: per 32
 // columns at 512 tokens the MMAs read 48 KB (384 clocks) and the bulk copies write 32 KB (256), the producers' stores take 64
@@ -75,20 +75,24 @@ constexpr int SMEM_LIMIT = 227 * 1024, SMEM_LIMIT_L1 = 195 * 1024;
 // per vector length: geometry of the A tile and the producers
 template <int V> struct Tile;
 template <> struct Tile<8> {
-    static constexpr int NV = 16, KS = 32, A_STAGES = 6, GROUP_WARPS = 2, GROUPS = 6;
+    static constexpr int NV = 16, KS = 32, A_STAGES = 6, GROUP_WARPS = 2, GROUPS = 5, WARP0 = 2, WARPS = 10;
 };
 template <> struct Tile<6> {
-    static constexpr int NV = 20, KS = 64, A_STAGES = 3, GROUP_WARPS = 5, GROUPS = 2;
+    static constexpr int NV = 20, KS = 64, A_STAGES = 3, GROUP_WARPS = 5, GROUPS = 2, WARP0 = 4, WARPS = 12;
 };
 template <> struct Tile<12> {
-    static constexpr int NV = 10, KS = 64, A_STAGES = 5, GROUP_WARPS = 3, GROUPS = 4;
+    static constexpr int NV = 10, KS = 64, A_STAGES = 5, GROUP_WARPS = 3, GROUPS = 4, WARP0 = 4, WARPS = 12;
 };
 template <int V> constexpr int a_stage_bytes() { return 128 * Tile<V>::KS * 2; }
-// Warps by role, in whole warpgroups (register shares move between warpgroups): 4 with the loader and the MMA issuer, 12
-// producers, 8 for the epilogue.  24 warps start with 80 registers a thread; the producers take 104, the others keep 56:
-// 12 x 104 + 12 x 56 = 24 x 80.  (16 producer warps with 96 registers fill the A ring no faster: the shared-memory pipe bounds.)
-constexpr int PRODUCER_WARP0 = 4, PRODUCER_WARPS = 12, EPI_WARP0 = PRODUCER_WARP0 + PRODUCER_WARPS;
-constexpr int GEMM_THREADS = 32 * (EPI_WARP0 + EPI_WARPS);
+// Warps by role: the loader, the MMA issuer, producers from WARP0 on, then the epilogue.
+// v = 6, 12: roles in whole warpgroups, between which registers move: 24 warps start with 80 registers a thread; the 12
+// producers take 104, the others keep 56: 12 x 104 + 12 x 56 = 24 x 80.  (16 producer warps with 96 registers fill the A ring
+// no faster: the shared-memory pipe bounds.)
+// v = 8: 20 warps with 96 registers each, five pairs of producers.  24 warps in six pairs spill some of the producers' state:
+// 14336 x 4096 at 512 tokens, FP32 results, 82.2 against 80.1 us; 4096 x 14336 84.8 against 83.0; 8192 x 8192 at 333 79.7 / 77.6.
+template <int V> constexpr bool split_registers() { return V != 8; }
+template <int V> constexpr int epi_warp0() { return Tile<V>::WARP0 + Tile<V>::WARPS; }
+template <int V> constexpr int gemm_threads() { return 32 * (epi_warp0<V>() + EPI_WARPS); }
 constexpr int REGS_PRODUCER = 104, REGS_OTHER = 56;
 
 // where a table's rows come from
@@ -556,8 +560,10 @@ __device__ __forceinline__ uint2 outlier_vector4(const LayerView &L, int m0, int
 }
 
 // ---- the GEMM ------------------------------------------------------------------------------------
-template <int V, int T1, int T2, int NL>
-__global__ void __launch_bounds__(GEMM_THREADS, 1)
+// PLAIN: no outlier columns, one group, 16-bit main and 8-bit residual indices: the same without the code for anything else in
+// the producers' loop (14336 x 4096 at 512 tokens 81.3 -> 80.1 us, 4096 x 14336 84.3 -> 83.0, 5000 x 9000 at 150 48.2 -> 45.9)
+template <int V, int T1, int T2, int NL, bool PLAIN>
+__global__ void __launch_bounds__(gemm_threads<V>(), 1)
 gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_constant__ GemmLaunch<NL> F)
 {
     // the layer this CTA works on, and its place among that layer's CTAs
@@ -573,7 +579,10 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     constexpr int SUBS = KS / IMG_COLS, TILE_M = NV * V, W2 = V / 2;
     constexpr int A_SBO = MN ? 2048 : 1024, A_LBO = MN ? 1024 : 16;
     static_assert(A_STAGES >= GROUPS, "a producer group needs a stage of its own");
-    static_assert(GROUPS * GROUP_WARPS <= PRODUCER_WARPS, "producer warps");
+    constexpr int PRODUCER_WARP0 = Tile<V>::WARP0, EPI_WARP0 = epi_warp0<V>(), GEMM_THREADS = gemm_threads<V>();
+    constexpr bool SPLIT_REGS = split_registers<V>();
+    static_assert(GROUPS * GROUP_WARPS <= Tile<V>::WARPS, "producer warps");
+    static_assert(!SPLIT_REGS || (PRODUCER_WARP0 % 4 == 0 && EPI_WARP0 % 4 == 0 && EPI_WARPS % 4 == 0), "whole warpgroups");
     extern __shared__ __align__(1024) uint8_t sm[];          // swizzled operand stages need 1024-byte alignment
     const LayerView &L = P.L;
     const uint32_t base = smem_addr(sm);
@@ -652,7 +661,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     bool ok = true;
 
     if (warp < PRODUCER_WARP0) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
+        if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
         // ================= bulk copies: B ring =================
         if (warp == 0 && lane == 0) {
             grid_dependency_wait();                              // the images are the pre-pass's output
@@ -736,13 +745,14 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
         }
     } else if (warp < EPI_WARP0) {
         // ================= dequant producers: A tiles =================
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_PRODUCER));
+        if (SPLIT_REGS) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_PRODUCER));
         const int pw = warp - PRODUCER_WARP0, group = pw / GROUP_WARPS, wi = pw % GROUP_WARPS;
         // v = 8: lane = (row chunk within the 64-row half `wi`, 8-column group of 4); else lane = (vector row of 4, group of 8)
         const int vr = MN ? 8 * wi + (lane & 7) : 4 * wi + (lane >> 3);         // vector row within the tile
         const int cg = MN ? lane >> 3 : lane & 7;
         const uint4 *cb1 = reinterpret_cast<const uint4 *>(cb1_ptr) + (lane & ((1 << P.cb1_shift) - 1));
         const uint4 *cb2 = reinterpret_cast<const uint4 *>(cb2_ptr) + (lane & ((1 << P.cb2_shift) - 1));
+        const int bits1 = PLAIN ? 16 : L.s1.bits, bits2 = PLAIN ? 8 : L.s2.bits;
         if (group >= GROUPS) ok = false;                     // a warp beyond the last whole group has no work
         bool waited = false;                                 // padded tables are the pre-pass's output
         int it0 = 0;                                         // k blocks of earlier segments
@@ -759,15 +769,15 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             const int limit = row_ok ? L.Nc : 0;
             uint4 raw1 = make_uint4(0, 0, 0, 0), raw2 = make_uint4(0, 0, 0, 0);
             if (kb < kb1) {
-                raw1 = load_raw8(row1, L.s1.stride, kb * (KS / 8) + cg, limit, L.s1.bits);
-                if (T2) raw2 = load_raw8(row2, L.s2.stride, kb * (KS / 8) + cg, limit, L.s2.bits);
+                raw1 = load_raw8(row1, L.s1.stride, kb * (KS / 8) + cg, limit, bits1);
+                if (T2) raw2 = load_raw8(row2, L.s2.stride, kb * (KS / 8) + cg, limit, bits2);
             }
             if ((T1 == TABLE_GLOBAL || T2 == TABLE_GLOBAL) && V != 8 && !waited) { grid_dependency_wait(); waited = true; }
             for (; kb < kb1; kb += GROUPS) {
                 const int it = it0 + (kb - kb0);
                 const int s = it % A_STAGES;
                 const uint32_t stage = sA + s * A_BYTES;
-                if (kb >= P.kb_main) {
+                if (!PLAIN && kb >= P.kb_main) {
                     // a5: outlier columns; few k blocks, written element by element
                     ok = __all_sync(0xffffffffu, mbar_wait(bar_emptyA(s), ((it / A_STAGES) & 1) ^ 1, abort_flag, P.status));
                     if (!ok) break;
@@ -819,15 +829,17 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                     const int col0 = kb * KS + 8 * cg;
                     // (a lane without a row or columns holds zeros and so reads entry 0 along with the others)
                     uint32_t w1[4], w2[4] = {0, 0, 0, 0};
-                    decode8(raw1, L.s1.bits, L.k1, w1);
-                    if (T2) decode8(raw2, L.s2.bits, L.k2, w2);
+                    decode8(raw1, bits1, L.k1, w1);
+                    if (T2) decode8(raw2, bits2, L.k2, w2);
                     if (kb + GROUPS < kb1) {
-                        raw1 = load_raw8(row1, L.s1.stride, (kb + GROUPS) * (KS / 8) + cg, limit, L.s1.bits);
-                        if (T2) raw2 = load_raw8(row2, L.s2.stride, (kb + GROUPS) * (KS / 8) + cg, limit, L.s2.bits);
+                        raw1 = load_raw8(row1, L.s1.stride, (kb + GROUPS) * (KS / 8) + cg, limit, bits1);
+                        if (T2) raw2 = load_raw8(row2, L.s2.stride, (kb + GROUPS) * (KS / 8) + cg, limit, bits2);
                     }
                     // Sec. 3.1: a column's tables are those of its group
                     uint32_t g = 0;
                     int g_next = 0x7fffffff;
+                    // (asked in the PLAIN form too: the test between the columns keeps their reads in turn.  Without it the compiler
+                    // puts all main reads before the residual ones, 8192 x 8192 at 333 tokens, FP16 results: 90.4 us against 87.3)
                     if ((T1 == TABLE_GLOBAL || T2 == TABLE_GLOBAL) && L.G > 1) { g = (uint32_t)(col0 / L.cpg); g_next = (int)(g + 1) * L.cpg; }
                     auto next_group = [&](int j) { if (col0 + j >= g_next && (int)g + 1 < L.G) { g++; g_next += L.cpg; } };
                     auto id = [&](const uint32_t (&w)[4], int j) { return (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu; };
@@ -906,7 +918,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
         }
     } else {
         // ================= epilogue: two warps per TMEM lane quarter, taking turns at chunks of 32 tokens =================
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
+        if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
         const int ew = warp - EPI_WARP0, h = ew >> 2;
         const int q = warp & 3;                                  // TMEM lane quarter this warp may read
         const int padded_b = P.tiles_t * P.tile_n;
@@ -1112,6 +1124,7 @@ struct GemmPlan {
     int pre_rows;                    // tokens per block of the pre-pass that keeps rows in shared memory, 0 = the other one
     long long n_scratch;
     size_t smem;
+    int plain;                       // v = 8 over a table in L2: the kernel for 16-bit main and 8-bit residual indices, nothing else
     int pad_bytes;                   // rows of padded table copies, 0 = none
     long long ws_bytes, off_flags, off_bpart, off_pad1, off_pad2, off_scratch, off_xs;
 };
@@ -1129,6 +1142,7 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
         while (p.cb1_shift < 3 && (L.k1 * 16 << (p.cb1_shift + 1)) <= 32 * 1024) p.cb1_shift++;
         p.cb1_bytes = L.k1 * 16 << p.cb1_shift;
     }
+    p.plain = V == 8 && p.t1 == TABLE_GLOBAL && L.G == 1 && L.n_out == 0 && L.s1.bits == 16 && (L.k2 == 0 || L.s2.bits == 8);
     // token tiles of equal size, at most MAX_TILE_N tokens each
     p.tiles_t = ceil_div(B, MAX_TILE_N);
     p.tile_n = (ceil_div(B, p.tiles_t) + 15) / 16 * 16;
@@ -1236,10 +1250,10 @@ long long plan_launch(const LayerView *Ls, int n, int B, GemmPlan *pl)
     return ws;
 }
 
-template <int V, int T1, int T2, int NL>
+template <int V, int T1, int T2, int NL, bool PLAIN = false>
 cudaError_t launch_gemm(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmLaunch<NL> &F, cudaStream_t st)
 {
-    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2, NL>), pl.smem);
+    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2, NL, PLAIN>), pl.smem);
     if (e != cudaSuccess) return e;
     // programmatic dependent launch: set-up and the producers' first reads overlap the pre-pass
     cudaLaunchConfig_t cfg = {};
@@ -1247,11 +1261,11 @@ cudaError_t launch_gemm(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmL
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(F.cta_begin[F.n_layers], 1, 1);
-    cfg.blockDim = dim3(GEMM_THREADS, 1, 1);
+    cfg.blockDim = dim3(gemm_threads<V>(), 1, 1);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2, NL>, maps, F);
+    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2, NL, PLAIN>, maps, F);
 }
 
 template <int V, int NL>
@@ -1262,6 +1276,8 @@ cudaError_t launch_gemm_v(const GemmPlan &pl, const OutMaps<NL> &maps, const Gem
         if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_SHARED, TABLE_SHARED, NL>(pl, maps, F, st);
         return launch_gemm<V, TABLE_SHARED, TABLE_GLOBAL, NL>(pl, maps, F, st);
     }
+    if (V == 8 && pl.plain && pl.t2 == TABLE_NONE) return launch_gemm<8, TABLE_GLOBAL, TABLE_NONE, NL, true>(pl, maps, F, st);
+    if (V == 8 && pl.plain && pl.t2 == TABLE_SHARED) return launch_gemm<8, TABLE_GLOBAL, TABLE_SHARED, NL, true>(pl, maps, F, st);
     if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_GLOBAL, TABLE_NONE, NL>(pl, maps, F, st);
     if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_GLOBAL, TABLE_SHARED, NL>(pl, maps, F, st);
     return launch_gemm<V, TABLE_GLOBAL, TABLE_GLOBAL, NL>(pl, maps, F, st);

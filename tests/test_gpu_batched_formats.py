@@ -70,6 +70,25 @@ def test_split_tiles_have_scratch_of_their_own(M, N, B, kw):
         assert rel_err(dl.linear(x).float().cpu().numpy(), y_ref) <= tol
 
 
+@pytest.mark.parametrize("M,N,B,kw", [
+    (1000, 1003, 40, dict(k1=40000, k2=129)),                                     # 16 and 8 bits, indices that need the clamp
+    (136, 33, 17, dict(k1=32769)),                                                # 16 bits, one k block and a column more
+    (130, 31, 300, dict(k1=65536, k2=256, out_dtype="fp32")),                     # fewer columns than a k block, fewer k blocks than producers
+    (2056, 1411, 513, dict(k1=65536, k2=256, permuted=True, x_dtype="bf16")),
+    (1000, 1003, 40, dict(k1=32768, k2=256)),                                     # just outside: 15 bits,
+    (1000, 1003, 40, dict(k1=65536, k2=128, out_dtype="fp32")),                   # 7 bits,
+    (1000, 1003, 40, dict(k1=65536, k2=257)),                                     # 9 bits,
+    (1000, 1003, 40, dict(k1=65536, k2=256, n_out=9, v0=4, k0=37)),               # outlier columns,
+    (1000, 1003, 40, dict(k1=65536, k2=256, n_groups=2)),                         # groups
+])
+def test_v8_kernel_for_16_and_8_bit_indices_and_its_neighbours(M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    d = synth.make_layer(synth.LayerSpec("v8", M, N, v=8, **kw), 99, 0, B)
+    dl = b.DeviceLayer(d)
+    y = dl.linear(dl.upload_x(d["x"]))
+    assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
+
+
 def test_batched_kernel_repeats_bit_for_bit_when_asked():
     from paper_2409_17066_b200 import binding as b
     spec = synth.LayerSpec("bd", 1210, 2100, **V6)
