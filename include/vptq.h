@@ -402,9 +402,9 @@ int vptq_linear_noalloc(const vptq_layer_desc *desc, const void *x, int32_t B,
  * wins (all NaN: index 0); components beyond row M-1 (short last vector row) are left out.
  * Two kernels give these same indices: "assign_fp32" evaluates the definition for every pair;
  * "assign_tcgen05" (v <= 14, v divides M, k >= 1024, at least 4096 vectors) computes
- * ||c||^2 - 2 x.c on the tensor cores only to find, per vector, the group of 32 centroids that holds
- * the minimum, evaluates that group by the definition, and hands every vector whose candidate group is
- * not clearly the only one (within a bound on the tensor core's rounding) to the first kernel.
+ * ||x||^2 + ||c||^2 - 2 x.c on the tensor cores only to find, per vector, the groups of 32 centroids whose
+ * minimum may be the smallest (within a bound on the rounding), and evaluates these groups by the definition;
+ * a vector with more of them than its list holds, or out of the FP16 range, is scanned in full by a second kernel.
  * vptq_assign_path() names the kernel; VPTQ_FLAG_FORCE_GENERIC in `flags` selects "assign_fp32".
  * The tensor-core kernel needs a workspace of vptq_assign_workspace_bytes() bytes (256-byte aligned;
  * its first int32 is a status word read by vptq_workspace_status()); the other needs none.

@@ -27,7 +27,7 @@
 // branch.  The next step's A tiles are written before a step's scan.
 // What bounds it: the round trip of a TMEM buffer.  The accumulators of 256 vectors x 256 centroids fill TMEM, and from the
 // release of a buffer to the signal of its next MMA pass about 500 clocks, whatever the MMA's size (the handshake alone, with
-// nothing read or reduced, takes 640 clocks per 256 centroids; with both it is 830, where the ALU pipe needs about 400, the
+// nothing read or reduced, takes 640 clocks per 256 centroids; with both it is 760, where the ALU pipe needs about 400, the
 // TMEM reads and the MMAs 256 each).  Buffers of 64 columns were slower (an MMA of 64 takes 48 clocks, one of 128 takes 64).
 // 4096 x 4096, v = 8, 65536 centroids: 6.1 ms; with FP32 accumulators, two-input minima and a full scan of the 0.7 % of vectors
 // with a second candidate group 13.7 ms.

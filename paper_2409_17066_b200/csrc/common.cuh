@@ -175,7 +175,7 @@ void unpack_host(const uint8_t *packed, int rows, int cols, int k, int32_t *idx)
 cudaError_t launch_dequant(const LayerView &L, __half *W, cudaStream_t st);
 // assignment step of the quantizer (Eq. 2): idx [ceil(M/v)][N]
 bool assign_supported(int v, int k);
-// (weighted) k-means centroid update (Sec. 3.2.1); workspace = 2*k*v floats
+// (weighted) k-means centroid update (Sec. 3.2.1); workspace = FP32 sums of components (padded rows) and of weights
 long long kmeans_update_workspace_bytes(int v, int k);
 cudaError_t launch_kmeans_update(const __half *W, int M, int N, int v, const int *idx, const float *h, int k,
                                  __half *C, void *ws, cudaStream_t st);

@@ -402,7 +402,7 @@ cudaError_t launch_decode_smem_tc(const LayerView &L, const void *x, int B, void
     P.image = reinterpret_cast<uint8_t *>(ws);
     const bool res = L.k2 > 0;
     P.pre_grid = pl.pre_grid;
-    // (a dependent launch, and no memset in front of it: 1024 x 1024, v = 6, 5 tokens 14.3 -> 10.9 us, 4096 x 4096 22.5 -> 20.4)
+    // (a dependent launch, and no memset in front of it: 4096 x 4096, v = 6, 5 tokens 23.1 -> 21.4 us, 11008 x 4096, 16 tokens 47.5 -> 44.9)
     cudaError_t e = launch_dependent("smem_tc", NT == 2 ? smem_tc_prepass_kernel<2> : smem_tc_prepass_kernel<1>, pl.pre_grid, PRE_THREADS, 0, st, P);
     if (e != cudaSuccess) return e;
     if (NT == 2) {

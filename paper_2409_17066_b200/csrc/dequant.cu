@@ -12,7 +12,7 @@
 // skewed copies (conflict free).  The three roundings (add, multiply, add) are those of the definition: the residual is
 // added by a mixed-precision fma with factor one (f16 x 1 is exact), scale and bias are applied one
 // after the other (packed f32x2 multiply and add were contracted to one rounding by the assembler, so they are not used).
-// What bounds it: with the 1 MiB table the shared-memory/L1 data pipe (73 % busy: a random 16-byte read out of L2 is
+// What bounds it: with the 1 MiB table the shared-memory/L1 data pipe (72 % busy: a random 16-byte read out of L2 is
 // a wavefront of its own there, 29.4 M of them for 8192 x 28672, and the stores pass through it too), else the writes.
 // Measured against one thread per column with 2-byte centroid loads: 8192 x 28672 over the 1 MiB table 684.6 -> 182.8 us,
 // 8192 x 8192 over a 256-entry table 147.5 -> 30.8 us (4.6 TB/s), 11008 x 4096 with v = 6 / v = 12 and outlier columns

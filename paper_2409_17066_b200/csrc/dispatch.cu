@@ -34,8 +34,9 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
     return PATH_GENERIC;
 }
 
-// Whether a call of this family runs in the batched kernel.  The families whose main tables are in L2 or group-wise take at most four or two tokens per launch and gather every centroid
-// again for the next ones; the batched kernel gathers it once whatever the batch.  4096 x 4096 over the 1 MiB table: 25 us
+// Whether a call of this family runs in the batched kernel.  The families whose main tables are in L2 or group-wise take at
+// most four or two tokens per launch and gather every centroid again for the next ones; the batched kernel gathers it once
+// whatever the batch.  4096 x 4096 over the 1 MiB table: 25 us
 // at any batch up to 64, against 14-17 us per four tokens; 11008 x 4096, v = 12 in four groups: 52 us against 31 us per two.
 static bool takes_batched(LinearPath path, const LayerView &L, int B)
 {
