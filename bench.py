@@ -48,17 +48,17 @@ def read_peaks():
 # An entry is removed (-> null in the output) when its kernel changes after the capture.
 NCU_DRAM_BYTES_PER_ALGORITHMIC_BYTE = {
     # kernel: (ratio, source file of the kernel, first 12 hex digits of its SHA-1 when the capture was taken)
-    # profiles/decode_l2_fma_kernel_config3_gate_up_fused_B1.md: (178.38 + 3.18) MB DRAM / 178.33 MB algorithmic
-    "decode_l2_fma_kernel": (1.018, "decode_l2_fma.cu", "15af2fb60845"),
+    # profiles/decode_l2_fma_kernel_config3_gate_up_fused_B1.md: (178.41 + 3.89) MB DRAM / 178.33 MB algorithmic
+    "decode_l2_fma_kernel": (1.022, "decode_l2_fma.cu", "95179ce9e05e"),
     # profiles/decode_smem_fma_kernel_config2_gate_proj_B1.md: 19.00 MB / 18.92 MB
-    "decode_smem_fma_kernel": (1.004, "decode_smem_fma.cu", "160ad3290bed"),
-    # profiles/decode_smem_tc_kernel_config2_gate_proj_B8.md: 21.46 MB / 19.0 MB (the 0.5 MB fragment image and the
+    "decode_smem_fma_kernel": (1.004, "decode_smem_fma.cu", "6b2df8aed37f"),
+    # profiles/decode_smem_tc_kernel_config2_gate_proj_B8.md: 21.47 MB / 19.0 MB (the 0.5 MB fragment image and the
     # pre-pass's traffic included)
-    "decode_smem_tc_kernel": (1.13, "decode_smem_tc.cu", "ccf102769587"),
-    # profiles/decode_bucket_fma_kernel_config3_gate_up_fused_B1.md: (291.95 + 3.35) MB DRAM / 178.33 MB canonical
+    "decode_smem_tc_kernel": (1.13, "decode_smem_tc.cu", "0d06328cffc6"),
+    # profiles/decode_bucket_fma_kernel_config3_gate_up_fused_B1.md: (291.97 + 3.96) MB DRAM / 178.33 MB canonical
     # compressed bytes: the kernel reads the prepared image (4 bytes per slot, 21 % padding at N = 8192; the
     # N = 28672 image of down_proj is 1.47 x its canonical bytes, so this overstates that launch by a tenth)
-    "decode_bucket_fma_kernel": (1.656, "decode_bucket_fma.cu", "5da8f01fa7c4"),
+    "decode_bucket_fma_kernel": (1.659, "decode_bucket_fma.cu", "154b5b0e81ce"),
 }
 
 ROOFLINE_KERNEL = {"decode_l2_fma": "decode_l2_fma_kernel", "decode_smem_fma": "decode_smem_fma_kernel", "decode_gl_fma": "decode_gl_fma_kernel", "decode_smem_mma": "decode_smem_tc_kernel",
