@@ -86,14 +86,15 @@ template <> struct Tile<12> {
 template <int V> constexpr int a_stage_bytes() { return 128 * Tile<V>::KS * 2; }
 // Warps by role: the loader, the MMA issuer, producers from WARP0 on, then the epilogue.
 // v = 6, 12: roles in whole warpgroups, between which registers move: 24 warps start with 80 registers a thread; the 12
-// producers take 104, the others keep 56: 12 x 104 + 12 x 56 = 24 x 80.  (16 producer warps with 96 registers fill the A ring
-// no faster: the shared-memory pipe bounds.)
+// producers take 104, the epilogue keeps 64, loader and issuer 40: 12 x 104 + 8 x 64 + 4 x 40 = 24 x 80.  With 56 for the last two the
+// epilogue spills its place in the scratch: FP16 results, v = 6, 4096 x 4096 at 512 tokens 60.5 against 59.4 us, 8192 x 8192 at 24 60.8 / 59.5.
+// (16 producer warps with 96 registers fill the A ring no faster: the shared-memory pipe bounds.)
 // v = 8: 20 warps with 96 registers each, five pairs of producers.  24 warps in six pairs spill some of the producers' state:
 // 14336 x 4096 at 512 tokens, FP32 results, 82.2 against 80.1 us; 4096 x 14336 84.8 against 83.0; 8192 x 8192 at 333 79.7 / 77.6.
 template <int V> constexpr bool split_registers() { return V != 8; }
 template <int V> constexpr int epi_warp0() { return Tile<V>::WARP0 + Tile<V>::WARPS; }
 template <int V> constexpr int gemm_threads() { return 32 * (epi_warp0<V>() + EPI_WARPS); }
-constexpr int REGS_PRODUCER = 104, REGS_OTHER = 56;
+constexpr int REGS_PRODUCER = 104, REGS_EPILOGUE = 64, REGS_ISSUE = 40;
 
 // where a table's rows come from
 enum TableSource { TABLE_NONE = 0, TABLE_SHARED = 1, TABLE_GLOBAL = 2 };
@@ -582,6 +583,8 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     constexpr int PRODUCER_WARP0 = Tile<V>::WARP0, EPI_WARP0 = epi_warp0<V>(), GEMM_THREADS = gemm_threads<V>();
     constexpr bool SPLIT_REGS = split_registers<V>();
     static_assert(GROUPS * GROUP_WARPS <= Tile<V>::WARPS, "producer warps");
+    static_assert(PRODUCER_WARP0 * REGS_ISSUE + Tile<V>::WARPS * REGS_PRODUCER + EPI_WARPS * REGS_EPILOGUE <= 65536 / GEMM_THREADS / 8 * 8 * (GEMM_THREADS / 32) || !SPLIT_REGS,
+                  "a split takes no more than the launch has");
     static_assert(!SPLIT_REGS || (PRODUCER_WARP0 % 4 == 0 && EPI_WARP0 % 4 == 0 && EPI_WARPS % 4 == 0), "whole warpgroups");
     extern __shared__ __align__(1024) uint8_t sm[];          // swizzled operand stages need 1024-byte alignment
     const LayerView &L = P.L;
@@ -661,7 +664,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     bool ok = true;
 
     if (warp < PRODUCER_WARP0) {
-        if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
+        if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_ISSUE));
         // ================= bulk copies: B ring =================
         if (warp == 0 && lane == 0) {
             grid_dependency_wait();                              // the images are the pre-pass's output
@@ -918,7 +921,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
         }
     } else {
         // ================= epilogue: two warps per TMEM lane quarter, taking turns at chunks of 32 tokens =================
-        if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_OTHER));
+        if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_EPILOGUE));
         const int ew = warp - EPI_WARP0, h = ew >> 2;
         const int q = warp & 3;                                  // TMEM lane quarter this warp may read
         const int padded_b = P.tiles_t * P.tile_n;
