@@ -20,7 +20,9 @@
 //
 // Warp roles: warp 0 bulk loads of B; warp 1 TMEM allocation + MMA issue (an elected lane); 10 (v = 8) or 12 producer warps in
 // GROUPS groups, a k block each in turn (the next visit's packed indices in flight); 8 warps the epilogue
-// (tcgen05.ld -> + bias term -> output), two per TMEM lane quarter.
+// (tcgen05.ld -> + bias term -> output), two per TMEM lane quarter.  A form for few tokens has more producers (see Tile).
+// Up to 256 tokens TMEM holds two sets of accumulators, so the next piece's MMAs do not wait for the epilogue
+// (8192 x 8192, v = 6, 16 tokens 54.5 -> 53.1 us).
 // What bounds the k loop is the SM's shared-memory/L1 data pipe (128 bytes per clock), which everything passes: per 32
 // columns at 512 tokens the MMAs read 48 KB (384 clocks) and the bulk copies write 32 KB (256), the producers' stores take 64
 // and 512 gathers out of L2 a wavefront each (512) plus the residual reads: about 1280 of the 1070-1330 clocks measured
@@ -29,7 +31,8 @@
 // shared memory were slower (117 us against 88 us on 14336 x 4096 at 512 tokens).
 //
 // Persistent grid, one CTA per SM.  The work is the list of (tile, k block) units, tile = (token tile, row tile); every
-// CTA takes an equal, contiguous share of the units, whatever tile they fall in (a deterministic call: whole tiles).
+// CTA takes an equal, contiguous share of the units, whatever tile they fall in (a deterministic call: whole tiles; a call of
+// few tiles: every tile cut among CTAs of its own).
 // The pieces of a split tile meet
 //   - FP32 output with 16-byte rows, long shares (FLAG_ORDER_MIN_COLS columns): in the output, without a zero-fill: the
 //     piece that holds the tile's last k blocks is the first thing its CTA works on, so it finishes early; it stores and
@@ -61,28 +64,46 @@ using namespace tc;
 constexpr int MAX_TILE_N = 512;                          // tokens of a tile: all TMEM columns
 constexpr int IMG_COLS = 32;                             // columns of a B ring element
 constexpr int MAX_B_STAGES = 8;
-constexpr int EPI_WARPS = 8;
+constexpr int MAX_EPI_WARPS = 8;
 constexpr int EPI_TOKENS = 32;                            // tokens an epilogue warp reads out of TMEM at a time
 constexpr int PIECE_TOKENS = 16;                          // ... and hands to the copy engine at a time
 constexpr int EPI_BUF_BYTES = PIECE_TOKENS * 32 * 4;      // one staged piece of the output: 16 tokens x 32 rows, FP32
-constexpr int EPI_STAGE_BYTES = EPI_WARPS * 2 * EPI_BUF_BYTES;   // two buffers per epilogue warp: 32 KB
 constexpr int B_SBO = 512;    // bytes between consecutive 8-token groups of a B element (8 x 64 B)
 constexpr int WS_STATUS_BYTES = 256;
 constexpr int DRAIN_COLS = 160;                          // columns of a k loop that take as long as draining 512 tokens of a tile
+// ... and the columns that a piece which meets others in a scratch tile takes besides (bulk add, its completion, the count).  4096 x 11008, 16
+// tokens: v = 8 without 39.7 us, with 128 38.8, 224 39.2; v = 6 41.7, 40.7, 40.1; v = 12 52.1, 50.4, 50.1.
+constexpr int MEET_COLS_8 = 128, MEET_COLS = 224;
+// Columns by which the longest share may grow for the sake of whole CTAs per tile: scratch tiles (plus an eighth of the tokens),
+// FP32 sums.  1024 x 2048 (v = 6, 16 tokens, 16-bit results; 64 columns longer) 25.4 -> 13.0 us, 4096 x 4096 with v = 12 at 512
+// tokens (105 longer) 60.4 -> 55.2; v = 8: 4096 x 4096 (138 longer) 21.4 / 21.6 at 16 tokens, 50.3 / 47.4 at 512, 8192 x 8192 (554 longer)
+// 52.3 / 57.6.  FP32 sums: 1024 x 8192, v = 12, 512 tokens (70 longer) 61.7 -> 45.9, 200 tokens x 1024 x 2048 (64 longer) 18.8 / 19.6.
+constexpr int LONGER_COLS = 128, LONGER_COLS_SUM = 96;
 constexpr int FLAG_ORDER_MIN_COLS = 768;                 // columns of a share from which split tiles meet by flag order
 constexpr int SMEM_LIMIT = 227 * 1024, SMEM_LIMIT_L1 = 195 * 1024;
 
 // per vector length: geometry of the A tile and the producers
-template <int V> struct Tile;
-template <> struct Tile<8> {
-    static constexpr int NV = 16, KS = 32, A_STAGES = 6, GROUP_WARPS = 2, GROUPS = 5, WARP0 = 2, WARPS = 10;
+template <int V, bool FEW = false> struct Tile;
+template <> struct Tile<8, false> {
+    static constexpr int NV = 16, KS = 32, A_STAGES = 6, GROUP_WARPS = 2, GROUPS = 5, WARP0 = 2, WARPS = 10, EPI = 8;
 };
-template <> struct Tile<6> {
-    static constexpr int NV = 20, KS = 64, A_STAGES = 3, GROUP_WARPS = 5, GROUPS = 2, WARP0 = 4, WARPS = 12;
+template <> struct Tile<8, true> {
+    static constexpr int NV = 16, KS = 32, A_STAGES = 8, GROUP_WARPS = 2, GROUPS = 7, WARP0 = 2, WARPS = 14, EPI = 4;
 };
-template <> struct Tile<12> {
-    static constexpr int NV = 10, KS = 64, A_STAGES = 5, GROUP_WARPS = 3, GROUPS = 4, WARP0 = 4, WARPS = 12;
+template <> struct Tile<6, false> {
+    static constexpr int NV = 20, KS = 64, A_STAGES = 3, GROUP_WARPS = 5, GROUPS = 2, WARP0 = 4, WARPS = 12, EPI = 8;
 };
+template <> struct Tile<6, true> {
+    static constexpr int NV = 20, KS = 64, A_STAGES = 5, GROUP_WARPS = 5, GROUPS = 4, WARP0 = 4, WARPS = 20, EPI = 4;
+};
+template <> struct Tile<12, false> {
+    static constexpr int NV = 10, KS = 64, A_STAGES = 5, GROUP_WARPS = 3, GROUPS = 4, WARP0 = 4, WARPS = 12, EPI = 8;
+};
+// The form for FEW tokens (up to few_tokens() of a tile): the MMAs and the epilogue need little, and the producers are bound by the
+// latency of their table reads, so there are more of them: v = 6: four groups (20 warps) in place of two, five stages of A; v = 8: seven pairs,
+// eight stages; four epilogue warps.  v = 6, gate+up of 2 x 11008 x 4096 at 16 tokens 83 -> 73 us; v = 8, 1 MiB table, 8192 x 8192 at 16 48.4 -> 46.8,
+// at 64 52.8 / 52.6, 4096 x 4096 at 64 22.9 / 24.0 (an epilogue of four warps).  v = 12 reads two 32-byte rows a pair out of L2, whose rate bounds it.
+template <int V> constexpr int few_tokens() { return V == 8 ? 32 : V == 6 ? 64 : 0; }
 template <int V> constexpr int a_stage_bytes() { return 128 * Tile<V>::KS * 2; }
 // Warps by role: the loader, the MMA issuer, producers from WARP0 on, then the epilogue.
 // v = 6, 12: roles in whole warpgroups, between which registers move: 24 warps start with 80 registers a thread; the 12
@@ -91,10 +112,12 @@ template <int V> constexpr int a_stage_bytes() { return 128 * Tile<V>::KS * 2; }
 // (16 producer warps with 96 registers fill the A ring no faster: the shared-memory pipe bounds.)
 // v = 8: 20 warps with 96 registers each, five pairs of producers.  24 warps in six pairs spill some of the producers' state:
 // 14336 x 4096 at 512 tokens, FP32 results, 82.2 against 80.1 us; 4096 x 14336 84.8 against 83.0; 8192 x 8192 at 333 79.7 / 77.6.
+// v = 6, few tokens: 28 warps start with 72 registers: 20 x 80 + 4 x 64 + 4 x 40 = 28 x 72.
 template <int V> constexpr bool split_registers() { return V != 8; }
-template <int V> constexpr int epi_warp0() { return Tile<V>::WARP0 + Tile<V>::WARPS; }
-template <int V> constexpr int gemm_threads() { return 32 * (epi_warp0<V>() + EPI_WARPS); }
-constexpr int REGS_PRODUCER = 104, REGS_EPILOGUE = 64, REGS_ISSUE = 40;
+template <int V, bool FEW> constexpr int epi_warp0() { return Tile<V, FEW>::WARP0 + Tile<V, FEW>::WARPS; }
+template <int V, bool FEW> constexpr int gemm_threads() { return 32 * (epi_warp0<V, FEW>() + Tile<V, FEW>::EPI); }
+template <bool FEW> constexpr int regs_producer() { return FEW ? 80 : 104; }
+constexpr int REGS_EPILOGUE = 64, REGS_ISSUE = 40;
 
 // where a table's rows come from
 enum TableSource { TABLE_NONE = 0, TABLE_SHARED = 1, TABLE_GLOBAL = 2 };
@@ -108,9 +131,14 @@ __host__ __device__ __forceinline__ int scratch_rows(int tile_n) { return (tile_
 // us.  whole_tiles: cuts only between tiles.
 struct Shares {
     unsigned kb, len, workers, whole_tiles;      // k blocks of a tile; its length on the line, kb + drain
-    unsigned each, rest;                         // line (or tiles) per worker, and how many workers get one more
+    unsigned per_tile;                           // not 0: that many workers for each tile, none works on two
+    unsigned each, rest;                         // line (or tiles, or k blocks of a tile) per worker, and how many workers get one more
     __host__ __device__ unsigned begin(unsigned w) const        // first unit of worker w (w = workers: the end)
     {
+        if (per_tile) {
+            const unsigned tile = w / per_tile, part = w - tile * per_tile;
+            return tile * kb + part * each + (part < rest ? part : rest);
+        }
         const unsigned at = w * each + (w < rest ? w : rest);
         if (whole_tiles) return at * kb;
         const unsigned tile = at / len, off = at - tile * len;
@@ -119,7 +147,7 @@ struct Shares {
     __host__ __device__ unsigned worker_of(unsigned u) const    // the worker whose share holds unit u
     {
         const unsigned tile = u / kb, at = whole_tiles ? tile : tile * len + (u - tile * kb);
-        unsigned w = at / (each + 1);
+        unsigned w = per_tile ? tile * per_tile + (u - tile * kb) / (each + 1) : at / (each + 1);
         while (w + 1 < workers && begin(w + 1) <= u) w++;
         return w;
     }
@@ -141,7 +169,7 @@ struct GemmParams {
     int *status;         // workspace status word
     const float *bpart;  // [bias_parts][tiles_t * tile_n]: partial sums of x*b
     int bias_parts;
-    int *tile_flags;     // [tiles][EPI_WARPS]: flag order: [tile][0] counts the epilogue warps that have stored the last
+    int *tile_flags;     // [tiles][MAX_EPI_WARPS]: flag order: [tile][0] counts the epilogue warps that have stored the last
                          // piece; scratch: arrivals per epilogue warp
     float *scratch;      // [slots][4][scratch_rows(tile_n)][32] FP32 sums of split tiles, or null
     int slot_per_tile;   // a split tile's slot: 1 = its number, 0 = the worker that holds its first unit
@@ -555,16 +583,31 @@ __device__ __forceinline__ uint32_t outlier_bits(const LayerView &L, int m, int 
 // four output rows m0 .. m0+3 (m0 a multiple of 4) of column n as two words, for v0 = 4
 __device__ __forceinline__ uint2 outlier_vector4(const LayerView &L, int m0, int n)
 {
-    if (m0 >= L.M || n >= L.n_out) return make_uint2(0u, 0u);
-    const int i = clamp_index(load_index(L.s0.ptr + (long long)(m0 >> 2) * L.s0.stride, n, L.s0.bits), L.k0);
-    return __ldg(reinterpret_cast<const uint2 *>(L.c0) + i);
+    // (a place outside reads the first one's entry and drops it: no branch, so that a caller's reads are in flight together)
+    const bool in = m0 < L.M && n < L.n_out;
+    const int i = clamp_index(load_index(L.s0.ptr + (long long)(in ? m0 >> 2 : 0) * L.s0.stride, in ? n : 0, L.s0.bits), L.k0);
+    const uint2 c = __ldg(reinterpret_cast<const uint2 *>(L.c0) + i);
+    return make_uint2(in ? c.x : 0u, in ? c.y : 0u);
+}
+// ... of columns 8g .. 8g + 7: the eight indices, then the eight centroids in flight at once (column by column, behind branches, a k block
+// of them held the whole ring up: v = 6, gate+up and down of a 7B MLP at 16 tokens 116.5 -> 109.0 us)
+__device__ __forceinline__ void outlier_vectors4(const LayerView &L, int m0, int g, uint2 (&a)[8])
+{
+    const int cols = m0 < L.M ? L.n_out : 0;
+    uint32_t w[4];
+    decode8(load_raw8(L.s0.ptr + (long long)(m0 < L.M ? m0 >> 2 : 0) * L.s0.stride, L.s0.stride, g, cols, L.s0.bits), L.s0.bits, L.k0, w);
+#pragma unroll
+    for (int j = 0; j < 8; j++) a[j] = __ldg(reinterpret_cast<const uint2 *>(L.c0) + ((w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu));
+#pragma unroll
+    for (int j = 0; j < 8; j++)
+        if (8 * g + j >= cols) a[j] = make_uint2(0u, 0u);
 }
 
 // ---- the GEMM ------------------------------------------------------------------------------------
 // PLAIN: no outlier columns, one group, 16-bit main and 8-bit residual indices: the same without the code for anything else in
 // the producers' loop (14336 x 4096 at 512 tokens 81.3 -> 80.1 us, 4096 x 14336 84.3 -> 83.0, 5000 x 9000 at 150 48.2 -> 45.9)
-template <int V, int T1, int T2, int NL, bool PLAIN>
-__global__ void __launch_bounds__(gemm_threads<V>(), 1)
+template <int V, int T1, int T2, int NL, bool PLAIN, bool FEW>
+__global__ void __launch_bounds__(gemm_threads<V, FEW>(), 1)
 gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_constant__ GemmLaunch<NL> F)
 {
     // the layer this CTA works on, and its place among that layer's CTAs
@@ -575,15 +618,16 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     const CUtensorMap &tmap_out = maps.layer[NL > 1 ? li : 0];
     const unsigned worker = blockIdx.x - (NL > 1 ? F.cta_begin[li] : 0);
     constexpr bool MN = V == 8;                              // A layout
-    constexpr int KS = Tile<V>::KS, NV = Tile<V>::NV, A_STAGES = Tile<V>::A_STAGES, A_BYTES = a_stage_bytes<V>();
-    constexpr int GROUPS = Tile<V>::GROUPS, GROUP_WARPS = Tile<V>::GROUP_WARPS;
+    using T = Tile<V, FEW>;
+    constexpr int KS = T::KS, NV = T::NV, A_STAGES = T::A_STAGES, A_BYTES = a_stage_bytes<V>();
+    constexpr int GROUPS = T::GROUPS, GROUP_WARPS = T::GROUP_WARPS, EPI_WARPS = T::EPI;
     constexpr int SUBS = KS / IMG_COLS, TILE_M = NV * V, W2 = V / 2;
     constexpr int A_SBO = MN ? 2048 : 1024, A_LBO = MN ? 1024 : 16;
     static_assert(A_STAGES >= GROUPS, "a producer group needs a stage of its own");
-    constexpr int PRODUCER_WARP0 = Tile<V>::WARP0, EPI_WARP0 = epi_warp0<V>(), GEMM_THREADS = gemm_threads<V>();
+    constexpr int PRODUCER_WARP0 = T::WARP0, EPI_WARP0 = epi_warp0<V, FEW>(), GEMM_THREADS = gemm_threads<V, FEW>(), REGS_PRODUCER = regs_producer<FEW>();
     constexpr bool SPLIT_REGS = split_registers<V>();
-    static_assert(GROUPS * GROUP_WARPS <= Tile<V>::WARPS, "producer warps");
-    static_assert(PRODUCER_WARP0 * REGS_ISSUE + Tile<V>::WARPS * REGS_PRODUCER + EPI_WARPS * REGS_EPILOGUE <= 65536 / GEMM_THREADS / 8 * 8 * (GEMM_THREADS / 32) || !SPLIT_REGS,
+    static_assert(GROUPS * GROUP_WARPS <= T::WARPS, "producer warps");
+    static_assert(PRODUCER_WARP0 * REGS_ISSUE + T::WARPS * REGS_PRODUCER + EPI_WARPS * REGS_EPILOGUE <= 65536 / GEMM_THREADS / 8 * 8 * (GEMM_THREADS / 32) || !SPLIT_REGS,
                   "a split takes no more than the launch has");
     static_assert(!SPLIT_REGS || (PRODUCER_WARP0 % 4 == 0 && EPI_WARP0 % 4 == 0 && EPI_WARPS % 4 == 0), "whole warpgroups");
     extern __shared__ __align__(1024) uint8_t sm[];          // swizzled operand stages need 1024-byte alignment
@@ -600,7 +644,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     uint8_t *cb1_ptr = sm + A_STAGES * A_BYTES + b_stages * b_bytes;
     uint8_t *cb2_ptr = cb1_ptr + P.cb1_bytes;
     const uint32_t sEpi = smem_addr(cb2_ptr + P.cb2_bytes);     // EPI_WARPS x 2 x 2 KB output staging
-    float *bias = reinterpret_cast<float *>(cb2_ptr + P.cb2_bytes + EPI_STAGE_BYTES);       // [tile_n] bias terms of the token tile
+    float *bias = reinterpret_cast<float *>(cb2_ptr + P.cb2_bytes + EPI_WARPS * 2 * EPI_BUF_BYTES);       // [tile_n] bias terms of the token tile
     uint64_t *bars = reinterpret_cast<uint64_t *>(bias + MAX_TILE_N);   // fullA[] emptyA[] fullB[] emptyB[] accum_full accum_empty
     const uint32_t bar0 = smem_addr(bars);
     auto bar_fullA = [&](int s) { return bar0 + 8u * s; };
@@ -608,9 +652,13 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     auto bar_fullB = [&](int s) { return bar0 + 8u * (2 * A_STAGES + s); };
     auto bar_emptyB = [&](int s) { return bar0 + 8u * (2 * A_STAGES + MAX_B_STAGES + s); };
     constexpr int N_RING_BARS = 2 * A_STAGES + 2 * MAX_B_STAGES;
-    const uint32_t bar_accum_full = bar0 + 8u * N_RING_BARS;
-    const uint32_t bar_accum_empty = bar0 + 8u * (N_RING_BARS + 1);
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + N_RING_BARS + 2);
+    // accumulators: two sets of them, which the segments take in turn, where they fit TMEM
+    const int two = P.tile_n <= MAX_TILE_N / 2;
+    auto acc_set = [&](int seg) { return seg & two; };
+    auto acc_parity = [&](int seg) { return (uint32_t)(seg >> two) & 1u; };
+    auto bar_accum_full = [&](int set) { return bar0 + 8u * (N_RING_BARS + set); };
+    auto bar_accum_empty = [&](int set) { return bar0 + 8u * (N_RING_BARS + 2 + set); };
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + N_RING_BARS + 4);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -623,8 +671,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             mbar_init(bar_fullB(s), 1);       // the expect_tx arrival
             mbar_init(bar_emptyB(s), 1);      // tcgen05.commit
         }
-        mbar_init(bar_accum_full, 1);
-        mbar_init(bar_accum_empty, EPI_WARPS);
+        for (int i = 0; i < 2; i++) { mbar_init(bar_accum_full(i), 1); mbar_init(bar_accum_empty(i), EPI_WARPS); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -700,14 +747,15 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             const int n1 = P.tile_n - P.n0;
             const uint32_t id0 = instr_desc(MN, P.n0), id1 = instr_desc(MN, n1);
             const uint32_t bh = (uint32_t)((P.n0 * 64) >> 4);        // second MMA's token rows
-            const uint32_t tmem0 = __shfl_sync(0xffffffffu, tmem_base, 0), tmem1 = tmem0 + (uint32_t)P.n0;
+            const uint32_t tmem_all = __shfl_sync(0xffffffffu, tmem_base, 0);
             int sa = 0, sb = 0;                                      // ring positions and their phase parities
             uint32_t pa = 0, pb = 0, gave_up = 0;
             int seg_no = 0;
             FOR_EACH_SEGMENT {
-                // the accumulators must have been drained by the epilogues of the previous segment
-                mbar_wait_uniform(bar_accum_empty, (seg_no & 1) ^ 1, gave_up);
+                // the accumulators must have been drained by the epilogues of the segment that had them before
+                mbar_wait_uniform(bar_accum_empty(acc_set(seg_no)), acc_parity(seg_no) ^ 1u, gave_up);
                 tc_fence_after();
+                const uint32_t tmem0 = tmem_all + (uint32_t)(acc_set(seg_no) * (MAX_TILE_N / 2)), tmem1 = tmem0 + (uint32_t)P.n0;
                 uint32_t acc = 0;
                 for (int kb = kb0; kb < kb1; kb++) {
                     mbar_wait_uniform(bar_fullA(sa), pa, gave_up);
@@ -740,7 +788,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                     if (lane == 0) { grid_dependency_wait(); atomicExch(P.status, VPTQ_E_TIMEOUT); }
                     ok = false;
                 } else if (elect_one()) {
-                    umma_commit(bar_accum_full);                     // accumulators complete
+                    umma_commit(bar_accum_full(acc_set(seg_no)));                     // accumulators complete
                 }
                 __syncwarp();
                 seg_no++;
@@ -805,8 +853,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                         for (int i = wi * 32 + lane; i < (TILE_M / 4) * 8; i += GROUP_WARPS * 32) {
                             const int q = i & 7, m = (i >> 3) * 4;
                             uint2 a[8];
-#pragma unroll
-                            for (int j = 0; j < 8; j++) a[j] = outlier_vector4(L, m_tile + m, n0c + q * 8 + j);
+                            outlier_vectors4(L, m_tile + m, (n0c >> 3) + q, a);
 #pragma unroll
                             for (int r = 0; r < 4; r++) {
                                 uint32_t w[4];
@@ -847,7 +894,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                     auto next_group = [&](int j) { if (col0 + j >= g_next && (int)g + 1 < L.G) { g++; g_next += L.cpg; } };
                     auto id = [&](const uint32_t (&w)[4], int j) { return (w[j >> 1] >> (16 * (j & 1))) & 0xFFFFu; };
                     uint32_t cw[8][W2];
-                    if (V <= 8) {
+                    if (V <= 8 && !(FEW && V == 6)) {
                         // a3: main centroids, a4: residual centroids; all reads in flight before the wait (they do not touch the stage)
                         uint32_t rv[8][W2];
 #pragma unroll
@@ -868,7 +915,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                                 for (int i = 0; i < W2; i++) cw[j][i] = hadd2_bits(cw[j][i], rv[j][i]);
                         }
                     } else {
-                        // two 32-byte rows per column: four columns in flight at a time
+                        // v = 12: two 32-byte rows per column; few tokens: more warps with fewer registers.  Four columns in flight at a time
 #pragma unroll
                         for (int j0 = 0; j0 < 8; j0 += 4) {
                             uint32_t rv[4][W2];
@@ -876,8 +923,10 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                             for (int u = 0; u < 4; u++) {
                                 const int j = j0 + u;
                                 next_group(j);
-                                row_global<V>(P.tab1, g * (uint32_t)L.k1 + id(w1, j), cw[j]);
-                                if (T2) row_global<V>(P.tab2, g * (uint32_t)L.k2 + id(w2, j), rv[u]);
+                                if (T1 == TABLE_SHARED) row_shared<V>(cb1, id(w1, j) << P.cb1_shift, cw[j]);
+                                else row_global<V>(P.tab1, g * (uint32_t)L.k1 + id(w1, j), cw[j]);
+                                if (T2 == TABLE_SHARED) row_shared<V>(cb2, id(w2, j) << P.cb2_shift, rv[u]);
+                                else if (T2 == TABLE_GLOBAL) row_global<V>(P.tab2, g * (uint32_t)L.k2 + id(w2, j), rv[u]);
                             }
                             if (T2) {
 #pragma unroll
@@ -963,11 +1012,11 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                     at = next;
                 }
             }
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_accum_full, seg_no & 1, abort_flag, P.status));
+            ok = __all_sync(0xffffffffu, mbar_wait(bar_accum_full(acc_set(seg_no)), acc_parity(seg_no), abort_flag, P.status));
             if (!ok) break;
             tc_fence_after();
             if (add && P.flag_order) {
-                ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(P.tile_flags + tile * EPI_WARPS, EPI_WARPS, abort_flag, P.status));
+                ok = __all_sync(0xffffffffu, lane != 0 || flag_wait(P.tile_flags + tile * MAX_EPI_WARPS, EPI_WARPS, abort_flag, P.status));
                 if (!ok) break;
                 asm volatile("fence.proxy.async;" ::: "memory");     // the reduce-adds below go through the async proxy
             }
@@ -978,9 +1027,9 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             // (a quarter past the last row stages nothing: a piece without a copy would break the count of copies in flight)
             const bool box = P.tma_out && 32 * q + 32 <= TILE_M && m0 < L.M;
             float *sc = to_scratch ? P.scratch + ((long long)slot * 4 + q) * scratch_rows(P.tile_n) * 32 : nullptr;
-            for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += 2 * EPI_TOKENS) {
+            for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += EPI_WARPS / 4 * EPI_TOKENS) {
                 uint32_t r[EPI_TOKENS];
-                tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)c1, r);
+                tmem_ld32(tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(acc_set(seg_no) * (MAX_TILE_N / 2) + c1), r);
                 if (kb0 == 0) {
                     const float4 *b4 = reinterpret_cast<const float4 *>(bias + c1);
 #pragma unroll
@@ -1029,7 +1078,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_accum_empty);
+            if (lane == 0) mbar_arrive(bar_accum_empty(acc_set(seg_no)));
             if (announce) {
                 // this warp's part of the tile is in memory before the flag counts it
                 if (lane == 0 && P.tma_out) {
@@ -1038,7 +1087,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                 }
                 __threadfence();
                 __syncwarp();
-                if (lane == 0) atomicAdd(P.tile_flags + tile * EPI_WARPS, 1);
+                if (lane == 0) atomicAdd(P.tile_flags + tile * MAX_EPI_WARPS, 1);
             }
             if (to_scratch) {
                 // count this warp's part in; the CTA that finds all pieces counted converts and stores the part
@@ -1047,14 +1096,14 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                     asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
                     asm volatile("fence.proxy.async;" ::: "memory");
                     __threadfence();
-                    before = atomicAdd(P.tile_flags + tile * EPI_WARPS + ew, 1);
+                    before = atomicAdd(P.tile_flags + tile * MAX_EPI_WARPS + ew, 1);
                     __threadfence();
                 }
                 before = __shfl_sync(0xffffffffu, before, 0);
                 if (before == pieces - 1) {
                     const int rq = 4 * (lane & 7), mq = m0 + rq;              // this lane's four rows
                     const bool rows4 = 32 * q + rq + 4 <= TILE_M && mq + 4 <= L.M && (L.M & 3) == 0;
-                    for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += 2 * EPI_TOKENS)
+                    for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += EPI_WARPS / 4 * EPI_TOKENS)
 #pragma unroll
                     for (int c2 = c1; c2 < c1 + EPI_TOKENS; c2 += 16) {
                         float4 v[4];
@@ -1127,6 +1176,7 @@ struct GemmPlan {
     int pre_rows;                    // tokens per block of the pre-pass that keeps rows in shared memory, 0 = the other one
     long long n_scratch;
     size_t smem;
+    int few;                         // the kernel for few tokens
     int plain;                       // v = 8 over a table in L2: the kernel for 16-bit main and 8-bit residual indices, nothing else
     int pad_bytes;                   // rows of padded table copies, 0 = none
     long long ws_bytes, off_flags, off_bpart, off_pad1, off_pad2, off_scratch, off_xs;
@@ -1158,20 +1208,33 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     Shares &sh = p.shares;
     const unsigned tiles = (unsigned)p.tiles_m * p.tiles_t;
     sh.kb = p.kb_total; sh.whole_tiles = L.deterministic ? 1 : 0;
-    sh.len = p.kb_total + DRAIN_COLS * p.tile_n / MAX_TILE_N / p.ks;
+    p.tma_out = (L.out_dtype == VPTQ_DTYPE_FP32 && (L.M & 3) == 0) ? 1 : 0;
     // (a share of a few k blocks is not worth a CTA of its own: it costs a piece of the output and its meeting)
     const long long columns = (long long)tiles * sh.kb * p.ks;            // (of all tiles: past 32 bits for large calls)
     const long long most = L.deterministic ? tiles : (columns + 127) / 128;
     if (most < workers) workers = (int)most;
+    // flag order makes CTAs wait for one another: only for a call that has the GPU to itself
+    const bool in_order = p.tma_out && columns / workers >= FLAG_ORDER_MIN_COLS && !concurrent;
+    const int drain_cols = DRAIN_COLS * p.tile_n / MAX_TILE_N + (p.tma_out ? 0 : V == 8 ? MEET_COLS_8 : MEET_COLS);
+    sh.len = p.kb_total + drain_cols / p.ks;
+    // With fewer tiles than CTAs every tile can have as many CTAs to itself (per_tile): no CTA then drains two pieces and
+    // meets others twice.  Worth it while the longest share grows by less than that costs (see LONGER_COLS); under flag order
+    // a second piece costs next to nothing (4096 x 4096 over the 1 MiB table, 512 tokens, FP32: 40.0 us, 41.4 per tile).
+    if (!sh.whole_tiles && !in_order && tiles < (unsigned)workers) {
+        const unsigned per_tile = workers / tiles;
+        const long long longer = (long long)((sh.kb + per_tile - 1) / per_tile) * p.ks - columns / workers;
+        if (longer <= (p.tma_out ? LONGER_COLS_SUM : LONGER_COLS + p.tile_n / 8)) {
+            sh.per_tile = per_tile;
+            workers = (int)(tiles * per_tile);
+        }
+    }
     sh.workers = p.grid = workers;
-    const unsigned line = sh.whole_tiles ? tiles : tiles * sh.len;
-    sh.each = line / workers; sh.rest = line % workers;
+    const unsigned line = sh.per_tile ? sh.kb : sh.whole_tiles ? tiles : tiles * sh.len, parts = sh.per_tile ? sh.per_tile : workers;
+    sh.each = line / parts; sh.rest = line % parts;
     for (int c = 1; c < workers; c++)
         if (sh.begin(c) % p.kb_total != 0) p.any_split = 1;
-    p.tma_out = (L.out_dtype == VPTQ_DTYPE_FP32 && (L.M & 3) == 0) ? 1 : 0;
     p.scratch = p.any_split && !p.tma_out;
-    // flag order makes CTAs wait for one another: only for a call that has the GPU to itself
-    p.flag_order = (p.any_split && p.tma_out && columns / workers >= FLAG_ORDER_MIN_COLS && !concurrent) ? 1 : 0;
+    p.flag_order = p.any_split && in_order ? 1 : 0;
     // Shared memory: tables, A ring, then a B ring of up to 96 KB.  Three stages of it come before
     // copies of the residual table (eight copies are free of bank conflicts).  A table in L2
     // needs the L1 that is left, whose lines hold the reads in flight: past 196 KB a CTA (with the 1 KB the system keeps)
@@ -1179,11 +1242,14 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     const int b_bytes = p.tile_n * 64;
     const int limit = p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL ? SMEM_LIMIT_L1 : SMEM_LIMIT;
     const bool copies = p.t2 == TABLE_SHARED && L.k2 <= 256;
+    p.few = p.tile_n <= few_tokens<V>() && !(V == 6 && p.t1 == TABLE_GLOBAL);
+    constexpr bool HAS_FEW = V != 12;
+    const int a_stages = p.few ? Tile<V, HAS_FEW>::A_STAGES : Tile<V>::A_STAGES, epi = p.few ? Tile<V, HAS_FEW>::EPI : Tile<V>::EPI;
     p.cb2_shift = copies ? 3 : 0;
     while (true) {
         p.cb2_bytes = p.t2 == TABLE_SHARED ? L.k2 * 16 << p.cb2_shift : 0;
-        const int fixed = Tile<V>::A_STAGES * a_stage_bytes<V>() + p.cb1_bytes + p.cb2_bytes + EPI_STAGE_BYTES +
-                          MAX_TILE_N * 4 + 8 * (2 * Tile<V>::A_STAGES + 2 * MAX_B_STAGES + 2) + 16;
+        const int fixed = a_stages * a_stage_bytes<V>() + p.cb1_bytes + p.cb2_bytes + epi * 2 * EPI_BUF_BYTES +
+                          MAX_TILE_N * 4 + 8 * (2 * a_stages + 2 * MAX_B_STAGES + 4) + 16;
         int room = limit - fixed;
         if (room > 96 * 1024) room = 96 * 1024;
         p.b_stages = room / b_bytes < MAX_B_STAGES ? room / b_bytes : MAX_B_STAGES;
@@ -1203,7 +1269,7 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     p.pad_bytes = (V != 8 && (p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL)) ? (V <= 8 ? 16 : 32) : 0;
     auto take = [&](long long bytes) { const long long at = p.ws_bytes; p.ws_bytes += (bytes + 255) / 256 * 256; return at; };
     take(WS_STATUS_BYTES);
-    p.off_flags = take((long long)tiles * EPI_WARPS * 4);
+    p.off_flags = take((long long)tiles * MAX_EPI_WARPS * 4);
     p.off_bpart = take((long long)p.pre_y * p.tiles_t * p.tile_n * 4);
     p.off_pad1 = take(p.pad_bytes && p.t1 == TABLE_GLOBAL ? (long long)L.G * L.k1 * p.pad_bytes : 0);
     p.off_pad2 = take(p.pad_bytes && p.t2 == TABLE_GLOBAL ? (long long)L.G * L.k2 * p.pad_bytes : 0);
@@ -1253,10 +1319,10 @@ long long plan_launch(const LayerView *Ls, int n, int B, GemmPlan *pl)
     return ws;
 }
 
-template <int V, int T1, int T2, int NL, bool PLAIN = false>
+template <int V, int T1, int T2, int NL, bool PLAIN, bool FEW>
 cudaError_t launch_gemm(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmLaunch<NL> &F, cudaStream_t st)
 {
-    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2, NL, PLAIN>), pl.smem);
+    const cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(gemm_tcgen05_kernel<V, T1, T2, NL, PLAIN, FEW>), pl.smem);
     if (e != cudaSuccess) return e;
     // programmatic dependent launch: set-up and the producers' first reads overlap the pre-pass
     cudaLaunchConfig_t cfg = {};
@@ -1264,26 +1330,27 @@ cudaError_t launch_gemm(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmL
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(F.cta_begin[F.n_layers], 1, 1);
-    cfg.blockDim = dim3(gemm_threads<V>(), 1, 1);
+    cfg.blockDim = dim3(gemm_threads<V, FEW>(), 1, 1);
     cfg.dynamicSmemBytes = pl.smem;
     cfg.stream = st;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2, NL, PLAIN>, maps, F);
+    return cudaLaunchKernelEx(&cfg, gemm_tcgen05_kernel<V, T1, T2, NL, PLAIN, FEW>, maps, F);
 }
 
-template <int V, int NL>
+template <int V, int NL, bool FEW>
 cudaError_t launch_gemm_v(const GemmPlan &pl, const OutMaps<NL> &maps, const GemmLaunch<NL> &F, cudaStream_t st)
 {
     if (pl.t1 == TABLE_SHARED) {
-        if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_SHARED, TABLE_NONE, NL>(pl, maps, F, st);
-        if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_SHARED, TABLE_SHARED, NL>(pl, maps, F, st);
-        return launch_gemm<V, TABLE_SHARED, TABLE_GLOBAL, NL>(pl, maps, F, st);
+        if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_SHARED, TABLE_NONE, NL, false, FEW>(pl, maps, F, st);
+        if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_SHARED, TABLE_SHARED, NL, false, FEW>(pl, maps, F, st);
+        return launch_gemm<V, TABLE_SHARED, TABLE_GLOBAL, NL, false, FEW>(pl, maps, F, st);
     }
-    if (V == 8 && pl.plain && pl.t2 == TABLE_NONE) return launch_gemm<8, TABLE_GLOBAL, TABLE_NONE, NL, true>(pl, maps, F, st);
-    if (V == 8 && pl.plain && pl.t2 == TABLE_SHARED) return launch_gemm<8, TABLE_GLOBAL, TABLE_SHARED, NL, true>(pl, maps, F, st);
-    if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_GLOBAL, TABLE_NONE, NL>(pl, maps, F, st);
-    if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_GLOBAL, TABLE_SHARED, NL>(pl, maps, F, st);
-    return launch_gemm<V, TABLE_GLOBAL, TABLE_GLOBAL, NL>(pl, maps, F, st);
+    constexpr bool G = FEW && V == 8;               // (v = 6 over a table in L2 has the one kernel)
+    if (V == 8 && pl.plain && pl.t2 == TABLE_NONE) return launch_gemm<8, TABLE_GLOBAL, TABLE_NONE, NL, true, G>(pl, maps, F, st);
+    if (V == 8 && pl.plain && pl.t2 == TABLE_SHARED) return launch_gemm<8, TABLE_GLOBAL, TABLE_SHARED, NL, true, G>(pl, maps, F, st);
+    if (pl.t2 == TABLE_NONE) return launch_gemm<V, TABLE_GLOBAL, TABLE_NONE, NL, false, G>(pl, maps, F, st);
+    if (pl.t2 == TABLE_SHARED) return launch_gemm<V, TABLE_GLOBAL, TABLE_SHARED, NL, false, G>(pl, maps, F, st);
+    return launch_gemm<V, TABLE_GLOBAL, TABLE_GLOBAL, NL, false, G>(pl, maps, F, st);
 }
 
 template <int NL>
@@ -1322,7 +1389,7 @@ cudaError_t launch_layers(const LayerView *Ls, int n, const void *x, int B, void
         q.xs = w8 + pl.off_xs;
         q.bpart = reinterpret_cast<float *>(w8 + pl.off_bpart);
         q.status = status;
-        q.tile_flags = reinterpret_cast<int *>(w8 + pl.off_flags); q.n_flags = pl.tiles_m * pl.tiles_t * EPI_WARPS;
+        q.tile_flags = reinterpret_cast<int *>(w8 + pl.off_flags); q.n_flags = pl.tiles_m * pl.tiles_t * MAX_EPI_WARPS;
         if (pl.scratch) { q.zero = reinterpret_cast<float *>(w8 + pl.off_scratch); q.n_zero = pl.n_scratch; }
         else if (pl.any_split && !pl.flag_order) { q.zero = reinterpret_cast<float *>(outs[l]); q.n_zero = (long long)B * L.M; }
         if (pl.pad_bytes && pl.t1 == TABLE_GLOBAL) q.pad1 = w8 + pl.off_pad1;
@@ -1361,10 +1428,10 @@ cudaError_t launch_layers(const LayerView *Ls, int n, const void *x, int B, void
     cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(pre), cfg.dynamicSmemBytes);
     if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, pre, Q);
     if (e != cudaSuccess) return e;
-    if (Ls[0].v == 8) return launch_gemm_v<8, NL>(pl, maps, F, st);
-    if (Ls[0].v == 6) return launch_gemm_v<6, NL>(pl, maps, F, st);
-    return pl.t2 == TABLE_NONE ? launch_gemm<12, TABLE_GLOBAL, TABLE_NONE, NL>(pl, maps, F, st)
-                               : launch_gemm<12, TABLE_GLOBAL, TABLE_GLOBAL, NL>(pl, maps, F, st);
+    if (Ls[0].v == 8) return pl.few ? launch_gemm_v<8, NL, true>(pl, maps, F, st) : launch_gemm_v<8, NL, false>(pl, maps, F, st);
+    if (Ls[0].v == 6) return pl.few ? launch_gemm_v<6, NL, true>(pl, maps, F, st) : launch_gemm_v<6, NL, false>(pl, maps, F, st);
+    return pl.t2 == TABLE_NONE ? launch_gemm<12, TABLE_GLOBAL, TABLE_NONE, NL, false, false>(pl, maps, F, st)
+                               : launch_gemm<12, TABLE_GLOBAL, TABLE_GLOBAL, NL, false, false>(pl, maps, F, st);
 }
 
 }  // namespace
