@@ -384,6 +384,8 @@ bool smem_tc_supported(const LayerView &L, int B)
     return plan_smem_tc(L, B <= 8 ? 1 : 2).ok;
 }
 
+int smem_tc_slabs(const LayerView &L, int B) { return plan_smem_tc(L, B <= 8 ? 1 : 2).n_slabs; }
+
 long long smem_tc_workspace_bytes(const LayerView &L, int B)
 {
     return plan_smem_tc(L, B <= 8 ? 1 : 2).ws_bytes;

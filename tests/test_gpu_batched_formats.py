@@ -71,6 +71,30 @@ def test_split_tiles_have_scratch_of_their_own(M, N, B, kw):
 
 
 @pytest.mark.parametrize("M,N,B,kw", [
+    (1000, 1100, 32, dict(v=8, k1=65536, k2=256)),                                # the last tokens of the form for few tokens,
+    (1000, 1100, 33, dict(v=8, k1=65536, k2=256)),                                # the first of the other one
+    (726, 1100, 64, V6), (726, 1100, 65, V6),
+    (724, 1100, 17, dict(V6, out_dtype="fp32")),                                  # pieces that add up in the output
+    (1450, 2100, 256, V6), (1450, 2100, 257, V6),                                 # two sets of accumulators, one
+    (9600, 200, 20, dict(v=6, k1=512)),                                           # one k block more than CTAs per tile; short segments in turn
+    (600, 70, 20, V12),                                                           # fewer k blocks than CTAs per tile
+    (2048, 2048, 64, dict(v=8, k1=256, n_out=40, v0=4, k0=300)),                  # outlier columns past a k block of 32
+    (700, 9000, 9, dict(V6, n_out=65, k0=5000)),                                  # 13-bit outlier indices, a k block and a column of them;
+    (700, 9000, 8, dict(V6, n_out=8, k0=200)),                                    # ... 8 bits, in a call of the decode family's name
+    (300, 9000, 16, dict(v=8, k1=512, out_dtype="bf16")),
+])
+def test_few_tokens_and_cuts_within_tiles(M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    d = synth.make_layer(synth.LayerSpec("ft", M, N, **kw), 101, 0, B)
+    dl = b.DeviceLayer(d)
+    x, y_ref = dl.upload_x(d["x"]), oracle.Layer.from_synth(d).linear(d["x"])
+    for _ in range(2):
+        y = dl.linear(x)
+        assert b.lib.vptq_linear_has_status(C.byref(dl.desc), B) == 1 and b.vptq_workspace_status(dl.workspace(B)) == b.OK
+        assert rel_err(y.float().cpu().numpy(), y_ref) <= (TOL if kw.get("out_dtype") != "bf16" else 2.0 ** -8)
+
+
+@pytest.mark.parametrize("M,N,B,kw", [
     (1000, 1003, 40, dict(k1=40000, k2=129)),                                     # 16 and 8 bits, indices that need the clamp
     (136, 33, 17, dict(k1=32769)),                                                # 16 bits, one k block and a column more
     (130, 31, 300, dict(k1=65536, k2=256, out_dtype="fp32")),                     # fewer columns than a k block, fewer k blocks than producers
