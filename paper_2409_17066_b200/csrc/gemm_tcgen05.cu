@@ -182,7 +182,7 @@ struct GemmParams {
 // their address is taken, and with them in one struct 17 tokens x 8192 columns took 26.5 us instead of 24.)
 template <int NL>
 struct OutMaps {
-    CUtensorMap layer[NL];
+    CUtensorMap layer[NL], tail[NL];         // boxes of 32 rows; of the rows of a tile's last quarter, where it has fewer
 };
 template <int NL>
 struct GemmLaunch {
@@ -615,7 +615,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     if (NL > 1)
         while (li + 1 < F.n_layers && (int)blockIdx.x >= F.cta_begin[li + 1]) li++;
     const GemmParams P = F.layer[NL > 1 ? li : 0];           // (a copy: through a reference gate+up of 11008 x 4096 at 300 tokens took 7 us more)
-    const CUtensorMap &tmap_out = maps.layer[NL > 1 ? li : 0];
+    const CUtensorMap &tmap_out = maps.layer[NL > 1 ? li : 0], &tmap_tail = maps.tail[NL > 1 ? li : 0];
     const unsigned worker = blockIdx.x - (NL > 1 ? F.cta_begin[li] : 0);
     constexpr bool MN = V == 8;                              // A layout
     using T = Tile<V, FEW>;
@@ -1022,10 +1022,12 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             }
             const uint32_t ebuf = sEpi + (uint32_t)(ew * 2 * EPI_BUF_BYTES);
             const int m0 = mt * TILE_M + 32 * q;
-            // rows of this quarter that belong to the tile: a 120-row tile leaves 8 lanes of the last quarter unused, and a
-            // 32-row box of the output must not touch the next tile's rows, so that quarter stores element by element
+            // A 120-row tile leaves 8 lanes of the last quarter unused, and a box of the output must not touch the next tile's rows:
+            // that quarter has a map with boxes of 24 rows.  (Stored and added element by element, it held the others up:
+            // 4096 x 4096 at 512 tokens, FP32 results, v = 6 61.8 us instead of 47.4, v = 12 59.1 instead of 48.0.)
             // (a quarter past the last row stages nothing: a piece without a copy would break the count of copies in flight)
-            const bool box = P.tma_out && 32 * q + 32 <= TILE_M && m0 < L.M;
+            const bool box = P.tma_out && m0 < L.M;
+            const bool tail = TILE_M < 128 && q == 3;
             float *sc = to_scratch ? P.scratch + ((long long)slot * 4 + q) * scratch_rows(P.tile_n) * 32 : nullptr;
             for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += EPI_WARPS / 4 * EPI_TOKENS) {
                 uint32_t r[EPI_TOKENS];
@@ -1054,12 +1056,13 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                         const uint32_t buf = ebuf + (piece & 1u) * EPI_BUF_BYTES;
 #pragma unroll
                         for (int j = 0; j < PIECE_TOKENS; j++)
-                            asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + j * 128u + lane * 4u), "r"(r[p * PIECE_TOKENS + j]) : "memory");
+                            if (!(tail && box) || lane < TILE_M - 96)
+                                asm volatile("st.shared.b32 [%0], %1;" ::"r"(buf + j * (tail && box ? (TILE_M - 96) * 4u : 128u) + lane * 4u), "r"(r[p * PIECE_TOKENS + j]) : "memory");
                         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                         __syncwarp();
                         if (lane == 0) {
                             if (to_scratch) bulk_add(sc + c2 * 32, buf);
-                            else tma_store_2d(&tmap_out, buf, m0, t0 + c2, add);
+                            else tma_store_2d(tail ? &tmap_tail : &tmap_out, buf, m0, t0 + c2, add);
                         }
                     }
                 } else if (m_ok) {
@@ -1101,16 +1104,19 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                 }
                 before = __shfl_sync(0xffffffffu, before, 0);
                 if (before == pieces - 1) {
+                    // eight 512-byte reads of a warp in flight: with four, 4096 x 4096 (v = 8) at 512 tokens 47.4 us instead of 45.8; the form
+                    // of 72 registers keeps four (14336 x 4096 at 16 tokens 49.2 / 50.3)
+                    constexpr int LOADS = SPLIT_REGS && FEW ? 4 : 8;
                     const int rq = 4 * (lane & 7), mq = m0 + rq;              // this lane's four rows
                     const bool rows4 = 32 * q + rq + 4 <= TILE_M && mq + 4 <= L.M && (L.M & 3) == 0;
                     for (int c1 = EPI_TOKENS * h; c1 < t_cnt; c1 += EPI_WARPS / 4 * EPI_TOKENS)
 #pragma unroll
-                    for (int c2 = c1; c2 < c1 + EPI_TOKENS; c2 += 16) {
-                        float4 v[4];
+                    for (int c2 = c1; c2 < c1 + EPI_TOKENS; c2 += 4 * LOADS) {
+                        float4 v[LOADS];
 #pragma unroll
-                        for (int i = 0; i < 4; i++) v[i] = __ldcg(reinterpret_cast<const float4 *>(sc + (c2 + 4 * i + (lane >> 3)) * 32 + rq));
+                        for (int i = 0; i < LOADS; i++) v[i] = __ldcg(reinterpret_cast<const float4 *>(sc + (c2 + 4 * i + (lane >> 3)) * 32 + rq));
 #pragma unroll
-                        for (int i = 0; i < 4; i++) {
+                        for (int i = 0; i < LOADS; i++) {
                             const int t = c2 + 4 * i + (lane >> 3);
                             if (t >= t_cnt) continue;
                             const long long o = (long long)(t0 + t) * L.M + mq;
@@ -1376,12 +1382,15 @@ cudaError_t launch_layers(const LayerView *Ls, int n, const void *x, int B, void
             if (encode == nullptr) return cudaErrorNotSupported;
             const cuuint64_t odim[2] = {(cuuint64_t)L.M, (cuuint64_t)B};
             const cuuint64_t ostride[1] = {(cuuint64_t)L.M * 4};
-            const cuuint32_t obox[2] = {32, PIECE_TOKENS};
-            const cuuint32_t estr[2] = {1, 1};
-            const CUresult r = encode(&maps.layer[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, outs[l], odim, ostride, obox, estr,
-                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+            const cuuint32_t tail_rows = (L.v == 8 ? Tile<8>::NV * 8 : L.v == 6 ? Tile<6>::NV * 6 : Tile<12>::NV * 12) - 96u;
+            for (int k = 0; k < (tail_rows < 32 ? 2 : 1); k++) {
+                const cuuint32_t obox[2] = {k ? tail_rows : 32u, PIECE_TOKENS};
+                const cuuint32_t estr[2] = {1, 1};
+                const CUresult r = encode(k ? &maps.tail[l] : &maps.layer[l], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, outs[l], odim, ostride, obox, estr,
+                                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                          CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                if (r != CUDA_SUCCESS) return cudaErrorInvalidValue;
+            }
         }
         PrepassParams &q = Q.layer[l];
         q.L = L; q.x = x; q.B = B; q.tile_n = pl.tile_n;
