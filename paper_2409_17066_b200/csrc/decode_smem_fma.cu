@@ -18,7 +18,7 @@
 // 3.2.3) are a small pass of their own (centroids from global memory through L1).  Warp partial
 // sums meet in shared memory; the epilogue adds the bias term and converts (a7).  No scratch.
 //
-// A task costs about 126 cycles of the SM's shared-memory pipe (10.5 for 32 random main centroids, 4 for
+// A task costs about 126 cycles of the SM's shared-memory pipe (10.5 for 32 random main centroids, 4 out of a small table in eight copies, 4 for
 // 32 residual ones, eight times), which is 38 us for gate+up and down of a 7B layer with v = 6 at one
 // token; with the tables' loads, the staging and two launches it takes 61 us (83 us while the outlier
 // pass waited for memory one row at a time and the activations came in as single columns).
@@ -47,6 +47,7 @@ struct SmemFmaParams {
     int B;                 // tokens in this launch (<= TB)
     int slab_cols;         // main columns per slab (multiple of 256)
     int n_slabs;
+    int cb1_shift;         // log2 of the copies of the main table: [k1][copies][16 B]
     int cb2_replicated;    // 1: [k2][8 replicas][16 B], 0: [k2][16 B]
     int n_out_pad;         // outlier columns rounded up to 8
     int part_floats;
@@ -74,8 +75,8 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
     const int gdim = FUSED ? P.cta_begin[li + 1] - P.cta_begin[li] : (int)gridDim.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    uint4 *cb1 = reinterpret_cast<uint4 *>(smem);                                            // [k1]
-    uint4 *cb2 = cb1 + L.k1;                                                                 // [k2][rep]
+    uint4 *cb1 = reinterpret_cast<uint4 *>(smem);                                            // [k1][copies]
+    uint4 *cb2 = cb1 + (L.k1 << P.cb1_shift);                                                                 // [k2][rep]
     __half *xs_out = reinterpret_cast<__half *>(cb2 + (RES ? (size_t)L.k2 * (P.cb2_replicated ? 8 : 1) : 0));   // [TB][n_out_pad]
     __half *xs = xs_out + (size_t)TB * P.n_out_pad;                                          // [TB][slab_cols]
     float *part = reinterpret_cast<float *>(xs + (size_t)TB * P.slab_cols);                  // [rows][TB][8]
@@ -95,14 +96,15 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 
     // ---- a2: codebooks -> shared memory as 16-byte rows; clear the partial sums -------------------
     // (loads of 4 entries are issued before the first store: one L2 round trip per 4 entries, not per entry)
-    for (int e0 = threadIdx.x; e0 < L.k1; e0 += 4 * THREADS) {
+    const int sh1 = P.cb1_shift, n1 = L.k1 << sh1;
+    for (int e0 = threadIdx.x; e0 < n1; e0 += 4 * THREADS) {
         uint4 row[4];
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (e0 + u * THREADS < L.k1) row[u] = load_centroid_row(L.c1, e0 + u * THREADS, L.v);
+            if (e0 + u * THREADS < n1) row[u] = load_centroid_row(L.c1, (e0 + u * THREADS) >> sh1, L.v);
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (e0 + u * THREADS < L.k1) cb1[e0 + u * THREADS] = row[u];
+            if (e0 + u * THREADS < n1) cb1[e0 + u * THREADS] = row[u];
     }
     if (RES) {
         const int n2 = P.cb2_replicated ? L.k2 * 8 : L.k2, sh = P.cb2_replicated ? 3 : 0;
@@ -121,6 +123,7 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 
     if (L.n_out > 0) outl.fetch_rows(L, outl_id);
 
+    const uint4 *cb1_lane = cb1 + (lane & ((1 << sh1) - 1));
     const int rep = P.cb2_replicated ? (lane & 7) : 0;
     const int rshift = P.cb2_replicated ? 3 : 0;
 
@@ -273,7 +276,7 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
                 // a3: 8 main centroids
                 uint4 cw[8];
 #pragma unroll
-                for (int s = 0; s < 8; s++) cw[s] = cb1[(w1[s >> 1] >> (16 * (s & 1))) & 0xFFFFu];
+                for (int s = 0; s < 8; s++) cw[s] = cb1_lane[((w1[s >> 1] >> (16 * (s & 1))) & 0xFFFFu) << sh1];
                 // this lane's 8 scaled activations per token
                 uint4 xv4[TB];
 #pragma unroll
@@ -347,13 +350,30 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 }
 
 struct SmemFmaPlan {
-    int slab_cols, n_slabs, cb2_rep, grid, part_floats, n_out_pad;
+    int slab_cols, n_slabs, cb1_shift, cb2_rep, grid, part_floats, n_out_pad;
     size_t smem;
     bool ok;
     int cta_begin[MAX_FUSED + 1];   // fused launches only
 };
 
 int fma_token_group(int B) { return B >= 4 ? 4 : (B >= 2 ? 2 : 1); }
+
+// Copies of a small main table side by side, lane l reading copy l mod copies: of the eight lanes that read 16-byte rows at random in
+// one wavefront those of one copy share 8 / copies of the 8 banks of that width; eight copies are free of conflicts.  256 centroids, v = 8,
+// one token: 11008 x 4096 10.6 -> 7.9 us, 4096 x 4096 6.25 -> 5.34.  As many as fit COPIES_BYTES, where a CTA reads as many rows as
+// it stages at one token, 2 * tokens as many at more (products bound there: 4 tokens, 4096 x 4096 8.51 / 8.42, 2048 x 2048, which reads
+// twice as many, 5.46 / 5.71).  Two copies of 64 KB do not pay: k1 = 4096, 4096 x 4096 7.18 / 7.73, 11008 x 4096 11.70 / 11.93.
+constexpr size_t COPIES_BYTES = 32 * 1024;
+void plan_copies(SmemFmaPlan &p, const LayerView &L, int TB, int rows_cta)
+{
+    const size_t table = (size_t)L.k1 * 16, rest = p.smem - table;
+    const long long reads = (long long)rows_cta * L.Nc / (TB == 1 ? 1 : 2 * TB);
+    p.cb1_shift = 0;
+    while (p.cb1_shift < 3 && table << (p.cb1_shift + 1) <= COPIES_BYTES && rest + (table << (p.cb1_shift + 1)) <= 224 * 1024 &&
+           reads >= (long long)L.k1 << (p.cb1_shift + 1))
+        p.cb1_shift++;
+    p.smem = rest + (table << p.cb1_shift);
+}
 
 SmemFmaPlan plan_smem_fma(const LayerView &L, int TB)
 {
@@ -372,6 +392,7 @@ SmemFmaPlan plan_smem_fma(const LayerView &L, int TB)
     p.smem = (size_t)L.k1 * 16 + (size_t)L.k2 * 16 * (p.cb2_rep ? 8 : 1) + (size_t)TB * p.n_out_pad * 2 +
              (size_t)TB * slab * 2 + (size_t)p.part_floats * 4 + 8 * 4 + (size_t)WARPS * 8 * 4;
     p.ok = (long long)p.part_floats * 4 <= PART_BUDGET && p.smem <= 224 * 1024 && p.n_slabs > 0;
+    plan_copies(p, L, TB, rows_cta);
     return p;
 }
 
@@ -403,10 +424,11 @@ bool plan_smem_fma_fused(const LayerView *Ls, int n, int TB, SmemFmaPlan *out)
     for (int l = 0; l < n; l++) R[l] = Ls[l].R;
     if (!split_ctas(R, n, device_sm_count(), p.cta_begin, &rows_cta)) return false;
     p.grid = device_sm_count();
-    p.smem -= (size_t)p.part_floats * 4;
+    p.smem -= (size_t)p.part_floats * 4 + ((size_t)Ls[0].k1 * 16 << p.cb1_shift) - (size_t)Ls[0].k1 * 16;
     p.part_floats = rows_cta * TB * 8;
     p.smem += (size_t)p.part_floats * 4;
     if ((long long)p.part_floats * 4 > PART_BUDGET || p.smem > 224 * 1024) return false;
+    plan_copies(p, Ls[0], TB, rows_cta);
     *out = p;
     return true;
 }
@@ -453,7 +475,7 @@ cudaError_t launch_decode_smem_fma(const LayerView &L, const void *x, int B, voi
         P.B = (B - t0 < TB) ? (B - t0) : TB;
         P.x = reinterpret_cast<const uint8_t *>(x) + (size_t)t0 * L.N * xe;
         P.out[0] = reinterpret_cast<uint8_t *>(out) + (size_t)t0 * L.M * oe;
-        P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.cb2_replicated = pl.cb2_rep;
+        P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.cb1_shift = pl.cb1_shift; P.cb2_replicated = pl.cb2_rep;
         P.n_out_pad = pl.n_out_pad; P.part_floats = pl.part_floats;
         cudaError_t e;
         if (TB == 4) e = launch_vv<4>(P, pl, L.v, res, st);
@@ -489,7 +511,7 @@ cudaError_t launch_decode_smem_fma_fused(const LayerView *Ls, int n, const void 
         P.n_layers = n;
         P.B = (B - t0 < TB) ? (B - t0) : TB;
         P.x = reinterpret_cast<const uint8_t *>(x) + (size_t)t0 * Ls[0].N * 2;
-        P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.cb2_replicated = pl.cb2_rep;
+        P.slab_cols = pl.slab_cols; P.n_slabs = pl.n_slabs; P.cb1_shift = pl.cb1_shift; P.cb2_replicated = pl.cb2_rep;
         P.n_out_pad = pl.n_out_pad; P.part_floats = pl.part_floats;
         cudaError_t e;
         if (TB == 4) e = launch_vv<4>(P, pl, Ls[0].v, res, st);

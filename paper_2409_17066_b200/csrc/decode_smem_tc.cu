@@ -29,6 +29,9 @@ namespace {
 
 constexpr int TC_WARPS = 32, TC_THREADS = TC_WARPS * 32;
 constexpr int TC_SMEM_BUDGET = 224 * 1024;
+// bytes of copies of a small main table: lane l reads copy l mod copies, so with eight the 8 rows of a matrix come from 8 different 16-byte
+// banks.  256 centroids, v = 8: 11008 x 4096 20.0 -> 16.0 us at 8 tokens, 24.0 -> 20.1 at 16; v = 6 with a residual table 31.0 -> 26.8, 35.8 -> 31.9.
+constexpr int TC_COPIES_BYTES = 32 * 1024;
 
 constexpr int PRE_THREADS = 512;       // pre-pass: 32 columns of 16 tokens
 
@@ -39,6 +42,7 @@ struct SmemTcParams {
     int B;
     int slab_chunks;     // 256-column chunks per slab
     int n_slabs;
+    int cb1_shift;       // log2 of the copies of the main table
     int cb2_replicated;
     int n_out_pad;
     int pre_grid;          // blocks of the pre-pass, each with a part of the bias terms
@@ -120,8 +124,8 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
     constexpr int CHUNK_BYTES = 16 * 32 * FRAG;                    // 8 steps x 2 mma x 32 lanes
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-    uint4 *cb1 = reinterpret_cast<uint4 *>(smem);                                                        // [k1]
-    uint4 *cb2 = cb1 + L.k1;                                                                             // [k2][rep]
+    uint4 *cb1 = reinterpret_cast<uint4 *>(smem);                                                        // [k1][copies]
+    uint4 *cb2 = cb1 + (L.k1 << P.cb1_shift);                                                                             // [k2][rep]
     uint8_t *afrag = reinterpret_cast<uint8_t *>(cb2 + (RES ? (size_t)L.k2 * (P.cb2_replicated ? 8 : 1) : 0));   // [slab_chunks][16][32][FRAG]
     __half *xs_out = reinterpret_cast<__half *>(afrag + (size_t)P.slab_chunks * CHUNK_BYTES);            // [TP][n_out_pad]
     float *part = reinterpret_cast<float *>(xs_out + (size_t)TP * P.n_out_pad);                          // [rows_cta][TP][8]
@@ -132,14 +136,15 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
     const int m_lo = r0 * L.v, m_hi = min(L.M, r1 * L.v);
 
     // ---- a2: codebooks -> shared memory as 16-byte rows (4 entries per thread in flight); clear the sums ----
-    for (int e0 = threadIdx.x; e0 < L.k1; e0 += 4 * TC_THREADS) {
+    const int sh1 = P.cb1_shift, n1 = L.k1 << sh1;
+    for (int e0 = threadIdx.x; e0 < n1; e0 += 4 * TC_THREADS) {
         uint4 row[4];
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (e0 + u * TC_THREADS < L.k1) row[u] = load_centroid_row(L.c1, e0 + u * TC_THREADS, L.v);
+            if (e0 + u * TC_THREADS < n1) row[u] = load_centroid_row(L.c1, (e0 + u * TC_THREADS) >> sh1, L.v);
 #pragma unroll
         for (int u = 0; u < 4; u++)
-            if (e0 + u * TC_THREADS < L.k1) cb1[e0 + u * TC_THREADS] = row[u];
+            if (e0 + u * TC_THREADS < n1) cb1[e0 + u * TC_THREADS] = row[u];
     }
     if (RES) {
         const int n2 = P.cb2_replicated ? L.k2 * 8 : L.k2, sh = P.cb2_replicated ? 3 : 0;
@@ -148,7 +153,7 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
     for (int i = threadIdx.x; i < P.rows_cta * TP * 8; i += TC_THREADS) part[i] = 0.f;
     if (threadIdx.x < TP) tok[threadIdx.x] = 0.f;
 
-    const uint32_t cb1_addr = tc_saddr(cb1);
+    const uint32_t cb1_lane = tc_saddr(cb1) + (uint32_t)(lane & ((1 << sh1) - 1)) * 16u, cb1_shift = 4u + (uint32_t)sh1;
     const uint32_t cb2_lane = tc_saddr(cb2) + (P.cb2_replicated ? (uint32_t)(lane & 7) * 16u : 0u);
     const uint32_t cb2_shift = P.cb2_replicated ? 7u : 4u;       // bytes per residual entry: 128 (8 copies) or 16
     const uint32_t afrag_lane = tc_saddr(afrag) + (uint32_t)lane * FRAG;
@@ -295,7 +300,7 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
                     for (int s = 0; s < 8; s++) {
                         const uint32_t i1 = (w1[s >> 1] >> (16 * (s & 1))) & 0xFFFFu;
                         uint32_t b0, b1, b2, b3;
-                        tc_ldmatrix_x4_trans(cb1_addr + i1 * 16u, b0, b1, b2, b3);
+                        tc_ldmatrix_x4_trans(cb1_lane + (i1 << cb1_shift), b0, b1, b2, b3);
                         if (RES) {
                             const uint32_t i2 = (w2[s >> 1] >> (16 * (s & 1))) & 0xFFFFu;
                             uint32_t q0, q1, q2, q3;
@@ -335,7 +340,7 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
 }
 
 struct SmemTcPlan {
-    int slab_chunks, n_slabs, cb2_rep, n_out_pad, rows_cta, grid, chunks_total;
+    int slab_chunks, n_slabs, cb1_shift, cb2_rep, n_out_pad, rows_cta, grid, chunks_total;
     int pre_grid;
     size_t smem;
     long long ws_bytes;
@@ -351,7 +356,9 @@ SmemTcPlan plan_smem_tc(const LayerView &L, int NT)
     p.rows_cta = ceil_div(L.R, p.grid);
     p.n_out_pad = (L.n_out + 7) / 8 * 8;
     p.cb2_rep = (L.k2 > 0 && L.k2 <= 256) ? 1 : 0;
-    const long long fixed = (long long)L.k1 * 16 + (long long)L.k2 * 16 * (p.cb2_rep ? 8 : 1) + (long long)TP * p.n_out_pad * 2 +
+    p.cb1_shift = 0;
+    while (p.cb1_shift < 3 && (L.k1 * 16 << (p.cb1_shift + 1)) <= TC_COPIES_BYTES) p.cb1_shift++;
+    const long long fixed = ((long long)L.k1 * 16 << p.cb1_shift) + (long long)L.k2 * 16 * (p.cb2_rep ? 8 : 1) + (long long)TP * p.n_out_pad * 2 +
                             (long long)p.rows_cta * TP * 8 * 4 + TP * 4 + 64;
     const int chunk_bytes = 16 * 32 * 8 * NT;
     const int n_chunks = (L.Nc + 255) / 256;
@@ -398,7 +405,7 @@ cudaError_t launch_decode_smem_tc(const LayerView &L, const void *x, int B, void
     SmemTcParams P;
     memset(&P, 0, sizeof(P));
     P.L = L; P.x = x; P.out = out; P.B = B;
-    P.slab_chunks = pl.slab_chunks; P.n_slabs = pl.n_slabs; P.cb2_replicated = pl.cb2_rep;
+    P.slab_chunks = pl.slab_chunks; P.n_slabs = pl.n_slabs; P.cb1_shift = pl.cb1_shift; P.cb2_replicated = pl.cb2_rep;
     P.n_out_pad = pl.n_out_pad; P.rows_cta = pl.rows_cta;
     P.chunks_total = pl.chunks_total;
     P.image = reinterpret_cast<uint8_t *>(ws);

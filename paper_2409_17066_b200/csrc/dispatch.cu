@@ -39,15 +39,17 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
 // whatever the batch.  4096 x 4096 over the 1 MiB table: 25 us
 // at any batch up to 64, against 14-17 us per four tokens; 11008 x 4096, v = 12 in four groups: 52 us against 31 us per two.
 // Tables in shared memory: the decode kernel stages the activations slab by slab, which nothing overlaps, and reads outlier
-// columns one after the other.  Past one slab and 8 tokens the batched kernel is faster for v = 6 (4096 x 4096 with outlier columns at 16
-// tokens 27.6 -> 23.1 us, 11008 x 4096 45.0 -> 41.0, 4096 x 11008 56.6 -> 40.7) and for v = 8 up to 4096 rows (256 centroids, 2048 x 8192
-// 20.0 -> 16.7, 4096 x 11008 30.5 / 29.6; 8192 x 8192 slower), up to 8 tokens only with outlier columns and a residual table (2048 x 8192 27.0 ->
-// 22.7, 4096 x 11008 43.8 -> 40.2; without outliers 36.8 / 38.1); in one slab at 8 tokens 21.3 / 22.7 (4096 x 4096).  It has a quick way for outlier vectors of 4.
+// columns one after the other.  Past one slab and 8 tokens the batched kernel is faster for v = 6 with a residual table (4096 x 4096 with outlier
+// columns at 16 tokens 27.6 -> 23.1 us, 11008 x 4096 45.0 -> 41.0, 4096 x 11008 56.6 -> 40.7) and otherwise up to 2048 rows (v = 8, 256 centroids, 2048 x
+// 8192 18.6 -> 16.5, but 4096 x 11008 26.7 / 29.3), up to 8 tokens only for v = 6 with outlier columns and a residual table (2048 x 8192 27.0 -> 22.7,
+// 4096 x 11008 43.8 -> 40.2; without outliers 36.8 / 38.1); in one slab at 8 tokens 21.3 / 22.7 (4096 x 4096).  It has a quick way for outlier
+// vectors of 4.
 static bool smem_takes_batched(const LayerView &L, int B)
 {
     const int Bg = decode_group(B);
     if (!smem_tc_supported(L, Bg) || (L.n_out > 0 && L.v0 != 4) || smem_tc_slabs(L, Bg) < 2) return false;
-    return Bg > 8 ? L.v < 8 || L.M <= 4096 : L.v < 8 && L.n_out > 0 && L.k2 > 0;
+    const bool gathers = L.v < 8 && L.k2 > 0;
+    return Bg > 8 ? gathers || L.M <= 2048 : gathers && L.n_out > 0;
 }
 
 static bool takes_batched(LinearPath path, const LayerView &L, int B)

@@ -81,7 +81,7 @@ def test_split_tiles_have_scratch_of_their_own(M, N, B, kw):
     (2048, 2048, 64, dict(v=8, k1=256, n_out=40, v0=4, k0=300)),                  # outlier columns past a k block of 32
     (700, 9000, 9, dict(V6, n_out=65, k0=5000)),                                  # 13-bit outlier indices, a k block and a column of them;
     (700, 9000, 8, dict(V6, n_out=8, k0=200)),                                    # ... 8 bits, in a call of the decode family's name
-    (300, 9000, 16, dict(v=8, k1=512, out_dtype="bf16")),
+    (300, 9000, 16, dict(v=8, k1=512, out_dtype="bf16")),                         # a small layer of many slabs
 ])
 def test_few_tokens_and_cuts_within_tiles(M, N, B, kw):
     from paper_2409_17066_b200 import binding as b

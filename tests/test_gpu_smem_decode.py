@@ -30,3 +30,20 @@ def test_smem_decode_edges(M, N, B, kw):
     assert b.vptq_linear_path(dl.desc, B) == "decode_smem_fma"
     y = dl.linear(dl.upload_x(d["x"]))
     assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
+
+
+@pytest.mark.parametrize("k1", [200, 256, 257, 512, 1024, 1025])
+@pytest.mark.parametrize("M,N,B,kw", [
+    (4800, 2300, 1, dict(v=8)),                             # eight copies of a main table of up to 256 rows, four of 512, two of 1024
+    (4001, 2303, 4, dict(v=6, k2=256, n_out=9, v0=4, k0=64)),
+    (900, 700, 2, dict(v=4, out_dtype="fp32")),             # fewer reads, fewer copies
+    (1000, 2300, 8, dict(v=8, k2=100)),                     # the tensor-core kernel
+    (1000, 1003, 13, dict(v=6)),
+])
+def test_small_tables_in_copies(k1, M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    d = synth.make_layer(synth.LayerSpec("sc", M, N, k1=k1, **kw), 102, B, B)
+    dl = b.DeviceLayer(d)
+    assert b.vptq_linear_path(dl.desc, B) == ("decode_smem_fma" if B <= 4 else "decode_smem_mma")
+    y = dl.linear(dl.upload_x(d["x"]))
+    assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
