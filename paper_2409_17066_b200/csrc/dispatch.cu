@@ -40,7 +40,8 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
 // at any batch up to 64, against 14-17 us per four tokens; 11008 x 4096, v = 12 in four groups: 52 us against 31 us per two.
 // Tables in shared memory: the decode kernel stages the activations slab by slab, which nothing overlaps, and reads outlier
 // columns one after the other.  Past one slab and 8 tokens the batched kernel is faster for v = 6 with a residual table (4096 x 4096 with outlier
-// columns at 16 tokens 27.6 -> 23.1 us, 11008 x 4096 45.0 -> 41.0, 4096 x 11008 56.6 -> 40.7) and otherwise up to 2048 rows (v = 8, 256 centroids, 2048 x
+// columns at 16 tokens 27.6 -> 23.1 us, 11008 x 4096 45.0 -> 41.0, 4096 x 11008 56.6 -> 40.7; without them up to twice as many rows as columns: 11008 x 4096
+// 40.4 / 39.2) and otherwise up to 2048 rows (v = 8, 256 centroids, 2048 x
 // 8192 18.6 -> 16.5, but 4096 x 11008 26.7 / 29.3), up to 8 tokens only for v = 6 with outlier columns and a residual table (2048 x 8192 27.0 -> 22.7,
 // 4096 x 11008 43.8 -> 40.2; without outliers 36.8 / 38.1); in one slab at 8 tokens 21.3 / 22.7 (4096 x 4096).  It has a quick way for outlier
 // vectors of 4.
@@ -49,7 +50,16 @@ static bool smem_takes_batched(const LayerView &L, int B)
     const int Bg = decode_group(B);
     if (!smem_tc_supported(L, Bg) || (L.n_out > 0 && L.v0 != 4) || smem_tc_slabs(L, Bg) < 2) return false;
     const bool gathers = L.v < 8 && L.k2 > 0;
-    return Bg > 8 ? gathers || L.M <= 2048 : gathers && L.n_out > 0;
+    return Bg > 8 ? (gathers && (L.n_out > 0 || L.M <= 2 * L.N)) || L.M <= 2048 : gathers && L.n_out > 0;
+}
+
+// The layer as the batched kernel takes it.  Calls of the family of tables in shared memory have never had CTAs that wait for one
+// another, so they may share the GPU without saying so.
+static LayerView batched_view(LinearPath path, const LayerView &L)
+{
+    LayerView v = L;
+    if (path == PATH_DECODE_SMEM_MMA) v.concurrent = true;
+    return v;
 }
 
 static bool takes_batched(LinearPath path, const LayerView &L, int B)
@@ -62,7 +72,9 @@ static bool takes_batched(LinearPath path, const LayerView &L, int B)
 // (answers for the kernel that runs, whatever the family is called)
 bool linear_waits_between_ctas(const LayerView &L, int B, int flags)
 {
-    return takes_batched(choose_path(L, B, flags), L, B) && gemm_tcgen05_waits_between_ctas(&L, 1, B);
+    const LinearPath path = choose_path(L, B, flags);
+    const LayerView view = batched_view(path, L);
+    return takes_batched(path, L, B) && gemm_tcgen05_waits_between_ctas(&view, 1, B);
 }
 
 bool linear_has_status(const LayerView &L, int B, int flags)
@@ -87,7 +99,10 @@ const char *linear_path_name(const LayerView &L, int B, int flags)
 long long linear_workspace_bytes(const LayerView &L, int B, int flags)
 {
     const LinearPath path = choose_path(L, B, flags);
-    if (takes_batched(path, L, B)) return gemm_tcgen05_workspace_bytes(&L, 1, B);
+    if (takes_batched(path, L, B)) {
+        const LayerView view = batched_view(path, L);
+        return gemm_tcgen05_workspace_bytes(&view, 1, B);
+    }
     switch (path) {
     case PATH_DECODE_SMEM_FMA: return 0;
     case PATH_DECODE_SMEM_MMA: return smem_mma_workspace_bytes(L, decode_group(B));
@@ -125,7 +140,8 @@ int linear_dispatch(const LayerView &L, int flags, const void *x, int B, void *o
     if (path == PATH_GENERIC) {
         e = launch_linear_generic(L, x, B, out, ws, st);
     } else if (takes_batched(path, L, B)) {
-        e = launch_gemm_tcgen05(&L, 1, x, B, &out, ws, st);
+        const LayerView view = batched_view(path, L);
+        e = launch_gemm_tcgen05(&view, 1, x, B, &out, ws, st);
     } else if (path == PATH_DECODE_BUCKET_FMA) {
         const void *img = L.prepared;
         void *o = out;

@@ -279,3 +279,11 @@ def test_queries_answer_for_the_kernel_that_runs_whatever_the_path_is_called(bin
     assert b.lib.vptq_linear_fused_has_status((b.LayerDesc * 1)(b.make_desc(64, 64, 8, 256)), 1, 0) == b.E_SHAPE
     small = b.make_desc(11008, 4096, 6, 4096, 256)
     assert [b.lib.vptq_linear_has_status(C.byref(small), B) for B in (1, 16, 17)] == [0, 0, 1]
+
+
+def test_shared_memory_tables_in_the_batched_kernel_have_no_waits_between_ctas(binding):
+    b = binding
+    for B, out in ((9, "fp32"), (16, "fp32"), (16, "fp16"), (8, "fp32")):
+        d = b.make_desc(4096, 11008, 6, 4096, 256, n_outlier=110, v0=4, k0=4096, out_dtype=out)
+        assert b.vptq_linear_path(d, B) == "decode_smem_mma" and b.lib.vptq_linear_has_status(C.byref(d), B) == 1
+        assert b.lib.vptq_linear_waits_between_ctas(C.byref(d), B) == 0
