@@ -29,7 +29,7 @@
 // release of a buffer to the signal of its next MMA pass about 500 clocks, whatever the MMA's size (the handshake alone, with
 // nothing read or reduced, takes 640 clocks per 256 centroids; with both it is 760, where the ALU pipe needs about 400, the
 // TMEM reads and the MMAs 256 each).  Buffers of 64 columns were slower (an MMA of 64 takes 48 clocks, one of 128 takes 64).
-// 4096 x 4096, v = 8, 65536 centroids: 6.1 ms; with FP32 accumulators, two-input minima and a full scan of the 0.7 % of vectors
+// 4096 x 4096, v = 8, 65536 centroids: 5.9 ms; with FP32 accumulators, two-input minima and a full scan of the 0.7 % of vectors
 // with a second candidate group 13.7 ms.
 // Every mbarrier wait is bounded; a wait that gives up sets the status word of the workspace.
 #include "common.cuh"
@@ -54,6 +54,9 @@ constexpr int AHEAD = B_STAGES - 3;             // stages loaded ahead of the on
 constexpr int STEP_VECTORS = 256;             // two A tiles
 constexpr int GROUP = 32;                     // centroids of a candidate group: every other one of 64
 constexpr int LIST_LEN = 24, LIST_STRIDE = 2 * STEP_VECTORS;    // candidates kept per vector and buffer
+constexpr unsigned long long NO_RESULT = 0x7F8000007FFFFFFFull;            // infinite distance, no index
+// centroids from which on a lane evaluates a group by itself (16384: 2.06 -> 1.92 ms; below that the warp does: 8192 1.35 -> 1.23)
+constexpr int WARP_GROUP_MAX_K = 16384;
 constexpr uint32_t NO_THRESHOLD = 0x7C007C00u, GAVE_UP = 0x80008000u;      // infinity; below every value
 constexpr float PAD_NORM = 60000.f;           // norm of the padding rows of the last centroid tile: never the minimum
 constexpr float X_LIMIT = 3.0e4f, C_LIMIT = 1.5e4f;      // scaled ||x||^2 and max ||c||^2 up to which no real distance reaches the padding's
@@ -70,7 +73,7 @@ constexpr int SCAN_SMEM = OFF_BARS + N_BARS * 8 + 16;
 struct ScanParams {
     const __half *W;
     int M, N, v, k;
-    const __half *C;          // [k_tiles * KT][8 or 16]: centroids padded with zeros
+    const __half *C;          // [k_tiles * KT][8 or 16]: centroids padded with zeros, of every 64 the even ones first
     const uint8_t *Bimg;      // [k_tiles][TILE_BYTES]
     const float *cmax;        // max ||c||^2
     int *idx;                 // [n_vectors]
@@ -211,13 +214,14 @@ assign_prepare_kernel(const __half *__restrict__ C, int k, int v, uint8_t *__res
     const uint4 *src = reinterpret_cast<const uint4 *>(row), *rsrc = reinterpret_cast<const uint4 *>(raw);
     *reinterpret_cast<uint4 *>(tile + image_offset(i % KT, 0)) = src[0];
     *reinterpret_cast<uint4 *>(tile + image_offset(i % KT, 1)) = src[1];
-    uint4 *dst = reinterpret_cast<uint4 *>(Cpad + (long long)i * pad);
+    // (a group's 32 centroids, the even or the odd ones of 64, next to each other)
+    uint4 *dst = reinterpret_cast<uint4 *>(Cpad + (long long)((i & ~63) | ((i & 1) << 5) | ((i & 63) >> 1)) * pad);
     dst[0] = rsrc[0];
     if (pad == 16) dst[1] = rsrc[1];
 }
 
 // ---- the scan ---------------------------------------------------------------------------------------------
-template <int VMAX>
+template <int VMAX, bool WARP_GROUP>
 __global__ void __launch_bounds__(SCAN_THREADS, 1)
 assign_scan_kernel(ScanParams P)
 {
@@ -228,7 +232,7 @@ assign_scan_kernel(ScanParams P)
     const uint32_t sA = smem_addr(sm), sB = sA + OFF_B;
     uint2 *lists = reinterpret_cast<uint2 *>(sm + OFF_CAND);               // [LIST_LEN][2 buffers][256] candidates
     int2 *bound = reinterpret_cast<int2 *>(sm + OFF_BOUND);               // [256][2 buffers] threshold, length of the list
-    int2 *result = reinterpret_cast<int2 *>(sm + OFF_BEST);               // [256] distance bits, index
+    unsigned long long *result = reinterpret_cast<unsigned long long *>(sm + OFF_BEST);     // [256] distance bits, index below them
 
     uint32_t *xsave = reinterpret_cast<uint32_t *>(sm + OFF_X);           // [2 steps][256][8] components as they are
 
@@ -331,8 +335,8 @@ assign_scan_kernel(ScanParams P)
         const float scale = exp2f((float)scale_exponent(__ldg(P.cmax)));
         const float cmax = __ldg(P.cmax) * scale * scale;      // in the filter's units
         const float abs_c = P.v <= 13 ? ABS : ABS + ABS_NO_LO;
-        // this lane's column of the candidate lists, and that of the other warp of its vector
-        uint2 *mine = lists + b * (LIST_STRIDE / 2) + a * 128 + row, *others = lists + (b ^ 1) * (LIST_STRIDE / 2) + a * 128 + row;
+        // this lane's column of the candidate lists
+        uint2 *mine = lists + b * (LIST_STRIDE / 2) + a * 128 + row;
         // components of this lane's vector of a step, packed as they are (zeros beyond v and beyond the last vector)
         constexpr int XW = (VMAX + 1) / 2;
         auto load_x = [&](long long step, uint32_t (&xw)[XW]) {
@@ -436,58 +440,78 @@ assign_scan_kernel(ScanParams P)
                 break;
             }
 
-            // ---- the two warps of a vector put their candidates together; each evaluates half of every candidate group ----
+            // ---- the two warps of a vector agree on the threshold; each evaluates the candidates of its own lists ----
             const int slot = a * 128 + row;
             const long long g = step * STEP_VECTORS + slot;
             bound[slot * 2 + b] = make_int2((int)(thr & 0xffff0000u), cnt);
+            if (b == 0) result[slot] = NO_RESULT;
             if (!(ok = meet(0))) break;
-            const int2 other = bound[slot * 2 + (b ^ 1)];
-            const int t = min((int)(thr & 0xffff0000u), other.x);
+            const int t = min((int)(thr & 0xffff0000u), bound[slot * 2 + (b ^ 1)].x);
             // (no candidate below infinity, or a vector or table out of the filter's range: the full scan decides)
             const bool full = t <= 0 || !(xn < X_LIMIT) || !(cmax < C_LIMIT);
             const bool valid = g < P.n_vectors;
-            int best = 0x7fffffff;
-            float best_d = __int_as_float(0x7f800000);
-            if (valid && !full) {
-                float x[VMAX];
-                const uint32_t *xr = xsave + (step_no & 1) * (STEP_VECTORS * 8) + slot * 8;
-#pragma unroll
-                for (int w = 0; w < XW; w++) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(xr + w));
-                    x[2 * w] = f.x; x[2 * w + 1] = f.y;
+            // the groups still below the common threshold, two to an entry, to the front of the lane's list
+            int n = 0;
+            auto put = [&](uint32_t group) { reinterpret_cast<uint32_t *>(mine + (n >> 1) * LIST_STRIDE)[n & 1] = group; n++; };
+            if (valid && !full)
+                for (int i = 0; i < cnt; i++) {
+                    const uint2 e = mine[i * LIST_STRIDE];
+                    if ((int)(e.x << 16) < t) put(e.y);
+                    if ((int)(e.x & 0xffff0000u) < t) put(e.y | 1u);
                 }
-                // this warp's list, then the other's: the entries still below the common threshold, even columns before odd ones
-                const uint32_t t2 = (uint32_t)(t >> 16) * 0x10001u;
-                const int total = cnt + other.y;
-                int i = 0;
-                uint2 e = make_uint2(0u, 0u);
-                bool odd = false;
-                while (true) {
-                    int grp = -1;
-                    if (odd) { grp = (int)e.y | 1; odd = false; }
-                    for (; i < total && grp < 0; i++) {
-                        e = i < cnt ? mine[i * LIST_STRIDE] : others[(i - cnt) * LIST_STRIDE];
-                        if (__vmins2(e.x, t2) == t2) continue;
-                        odd = (int)(e.x & 0xffff0000u) < t;
-                        if ((int)(e.x << 16) < t) grp = (int)e.y;
-                        else { grp = (int)e.y | 1; odd = false; }
+            // The warp's groups are numbered through, whosever they are.  A table of few centroids: the warp takes one after the other, a
+            // lane a centroid, 512 bytes side by side.  Else 32 at a time, a lane a group: with 65536 centroids a vector has so many that the
+            // lanes are busy that way.  (With a lane to a vector a warp took as long as its longest list, and read single centroids.
+            // 4096 x 4096, one iteration, k = 65536, v = 8: 6.21 -> 6.04 ms; k = 4096, v = 8: 1.00 -> 0.89, v = 12: 0.88 -> 0.72; 65536 the first way 6.31, 4096
+            // (v = 8) the second 1.07.)
+            int first = n;                                             // groups of the lanes before this one
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, first, o);
+                if (lane >= o) first += v;
+            }
+            const int total = __shfl_sync(0xffffffffu, first, 31);
+            first -= n;
+            __syncwarp();
+            // (distances are not negative, so their bits are ordered like them; the lowest index wins a tie)
+            auto pack = [](uint32_t d, int c) { return (unsigned long long)d << 32 | (unsigned)c; };
+            unsigned long long best = NO_RESULT;                       // of this lane's vector (WARP_GROUP)
+            for (int i0 = 0; i0 < total; i0 += 32) {
+                // lane i finds the vector and the group of item i0 + i
+                const int i = i0 + lane;
+                int owner = 0;                                         // the last lane whose groups begin at or before i
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const int v = __shfl_sync(0xffffffffu, first, owner + o);
+                    if (v <= i) owner += o;
+                }
+                const int k = i - __shfl_sync(0xffffffffu, first, owner);
+                uint32_t group = 0;
+                if (i < total) group = reinterpret_cast<const uint32_t *>(lists + b * (LIST_STRIDE / 2) + a * 128 + 32 * q + owner + (k >> 1) * LIST_STRIDE)[k & 1];
+                if (!WARP_GROUP) {
+                    if (i >= total) continue;
+                    const int os = a * 128 + 32 * q + owner, c0 = (int)(group >> 1) * 64 + (int)(group & 1u);
+                    float x[VMAX];
+                    const uint32_t *xr = xsave + (step_no & 1) * (STEP_VECTORS * 8) + os * 8;
+#pragma unroll
+                    for (int w = 0; w < XW; w++) {
+                        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(xr + w));
+                        x[2 * w] = f.x; x[2 * w + 1] = f.y;
                     }
-                    if (grp < 0) break;
-                    const int base = (grp >> 1) * 64 + (grp & 1) + b * GROUP;       // 16 of the group's 32 centroids, two apart
+                    unsigned long long least = NO_RESULT;
                     constexpr int AT_ONCE = VMAX > 8 ? 4 : 8;
 #pragma unroll 1
-                    for (int u0 = 0; u0 < GROUP / 2; u0 += AT_ONCE) {
+                    for (int u0 = 0; u0 < GROUP; u0 += AT_ONCE) {
                         uint4 w[AT_ONCE][VMAX > 8 ? 2 : 1];
 #pragma unroll
                         for (int u = 0; u < AT_ONCE; u++) {
-                            const uint4 *cr = reinterpret_cast<const uint4 *>(P.C) + (long long)(base + 2 * (u0 + u)) * (VMAX > 8 ? 2 : 1);
+                            const uint4 *cr = reinterpret_cast<const uint4 *>(P.C) + (long long)(group * GROUP + u0 + u) * (VMAX > 8 ? 2 : 1);
                             w[u][0] = __ldg(cr);
                             if (VMAX > 8) w[u][VMAX > 8 ? 1 : 0] = __ldg(cr + 1);
                         }
 #pragma unroll
                         for (int u = 0; u < AT_ONCE; u++) {
                             const uint32_t *wu = reinterpret_cast<const uint32_t *>(w[u]);
-                            const int ci = base + 2 * (u0 + u);
                             float dd = 0.f;
 #pragma unroll
                             for (int j = 0; j < VMAX; j++) {
@@ -495,19 +519,54 @@ assign_scan_kernel(ScanParams P)
                                 const float tt = __fsub_rn(x[j], (j & 1) ? cv.y : cv.x);
                                 dd = __fmaf_rn(tt, tt, dd);
                             }
-                            if (ci < P.k && (dd < best_d || (dd == best_d && ci < best))) { best_d = dd; best = ci; }
+                            const int ci = c0 + 2 * (u0 + u);
+                            if (ci < P.k) least = min(least, pack(__float_as_uint(dd), ci));
                         }
+                    }
+                    atomicMin(result + os, least);
+                    continue;
+                }
+                const int items = min(32, total - i0);
+                constexpr int AT_ONCE = 4;
+#pragma unroll 1
+                for (int j0 = 0; j0 < items; j0 += AT_ONCE) {
+                    uint4 w[AT_ONCE][VMAX > 8 ? 2 : 1];
+                    uint32_t gj[AT_ONCE];
+#pragma unroll
+                    for (int u = 0; u < AT_ONCE; u++) {
+                        gj[u] = __shfl_sync(0xffffffffu, group, j0 + u);          // (items past the last are group 0, and dropped)
+                        const uint4 *cr = reinterpret_cast<const uint4 *>(P.C) + (long long)(gj[u] * GROUP + lane) * (VMAX > 8 ? 2 : 1);
+                        w[u][0] = __ldg(cr);
+                        if (VMAX > 8) w[u][VMAX > 8 ? 1 : 0] = __ldg(cr + 1);
+                    }
+#pragma unroll
+                    for (int u = 0; u < AT_ONCE; u++) {
+                        const int oj = __shfl_sync(0xffffffffu, owner, j0 + u);
+                        const uint32_t *xr = xsave + (step_no & 1) * (STEP_VECTORS * 8) + (a * 128 + 32 * q + oj) * 8;
+                        const uint32_t *wu = reinterpret_cast<const uint32_t *>(w[u]);
+                        float dd = 0.f;
+#pragma unroll
+                        for (int j = 0; j < XW; j++) {
+                            const float2 xv = __half22float2(*reinterpret_cast<const __half2 *>(xr + j));
+                            const float2 cv = __half22float2(*reinterpret_cast<const __half2 *>(&wu[j]));
+                            const float t0 = __fsub_rn(xv.x, cv.x), t1 = __fsub_rn(xv.y, cv.y);
+                            dd = __fmaf_rn(t0, t0, dd);
+                            if (2 * j + 1 < VMAX) dd = __fmaf_rn(t1, t1, dd);
+                        }
+                        const int c0 = (int)(gj[u] >> 1) * 64 + (int)(gj[u] & 1u);           // the group's centroids are two apart
+                        const uint32_t key = c0 + 2 * lane < P.k ? __float_as_uint(dd) : 0xffffffffu;
+                        const uint32_t least = __reduce_min_sync(0xffffffffu, key);
+                        const int ci = c0 + 2 * (__ffs(__ballot_sync(0xffffffffu, key == least)) - 1);     // the lowest index wins a tie
+                        if (lane == oj && j0 + u < items) best = min(best, pack(least, ci));
                     }
                 }
             }
-            if (b == 1) result[slot] = make_int2(__float_as_int(best_d), best);
+            if (WARP_GROUP) atomicMin(result + slot, best);
             if (!(ok = meet(1))) break;
             if (b == 0 && valid) {
-                const int2 o = result[slot];
-                const float od = __int_as_float(o.x);
-                if (od < best_d || (od == best_d && o.y < best)) best = o.y;
-                if (full || best == 0x7fffffff) P.list[atomicAdd(P.count, 1)] = (int)g;      // the full scan decides
-                else P.idx[g] = best;
+                const int nearest = (int)(unsigned)result[slot];
+                if (full || nearest == 0x7fffffff) P.list[atomicAdd(P.count, 1)] = (int)g;      // the full scan decides
+                else P.idx[g] = nearest;
             }
         }
     }
@@ -585,7 +644,9 @@ cudaError_t launch_assign_tcgen05(const __half *W, int M, int N, int v, const __
     if (e != cudaSuccess) return e;
     const long long n_steps = (n_vectors + STEP_VECTORS - 1) / STEP_VECTORS;
     const int grid = (int)(n_steps < device_sm_count() ? n_steps : device_sm_count());
-    auto kern = v <= 8 ? assign_scan_kernel<8> : assign_scan_kernel<14>;
+    const bool warp_group = k < WARP_GROUP_MAX_K;
+    auto kern = v <= 8 ? (warp_group ? assign_scan_kernel<8, true> : assign_scan_kernel<8, false>)
+                       : (warp_group ? assign_scan_kernel<14, true> : assign_scan_kernel<14, false>);
     e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), SCAN_SMEM);
     if (e != cudaSuccess) return e;
     kern<<<grid, SCAN_THREADS, SCAN_SMEM, st>>>(P);

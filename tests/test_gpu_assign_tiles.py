@@ -29,6 +29,19 @@ def test_assign_tiles(M, N, v, k, sigma):
     assert np.array_equal(b.vptq_assign(torch.from_numpy(W).cuda(), v, torch.from_numpy(Cb).cuda()).cpu().numpy(), oracle.assign(W, v, Cb))
 
 
+@pytest.mark.parametrize("k", [16383, 16384])                 # a warp a group, a lane a group
+@pytest.mark.parametrize("copies,noise", [(1, 0.02), (3, 0.02), (8, 0.0)])
+def test_assign_with_several_candidate_groups_a_vector(k, copies, noise):
+    # centroids that come more than once, far apart in the table, and vectors that are centroids: ties and near ties across groups
+    from paper_2409_17066_b200 import binding as b
+    rng = np.random.default_rng(k + copies)
+    base = rng.normal(0, 1, (k // copies + 1, 8))
+    Cb = np.tile(base, (copies, 1))[rng.permutation((k // copies + 1) * copies)[:k]].astype(np.float16)
+    W = (Cb[rng.integers(0, k, 4100)].astype(np.float64) + noise * rng.normal(0, 1, (4100, 8))).T.astype(np.float16)
+    assert b.vptq_assign_path(8, 4100, 8, k) == "assign_tcgen05"
+    assert np.array_equal(b.vptq_assign(torch.from_numpy(W.copy()).cuda(), 8, torch.from_numpy(Cb).cuda()).cpu().numpy(), oracle.assign(W.copy(), 8, Cb))
+
+
 @pytest.mark.parametrize("spread", [0.0, 1e-3])
 def test_assign_with_more_candidates_than_a_list_holds(spread):
     # all centroids (nearly) equal: every group stays within the filter's error of the best one
