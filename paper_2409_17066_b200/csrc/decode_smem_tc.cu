@@ -112,7 +112,8 @@ smem_tc_prepass_kernel(const __grid_constant__ SmemTcParams P)
 }
 
 // NT = 1: up to 8 tokens (A fragments of 8 bytes per lane), NT = 2: up to 16 tokens (16 bytes per lane)
-template <int NT, bool RES>
+// (COPIES: a kernel of its own, since a variable shift of every index costs the others 1-2 %)
+template <int NT, bool RES, bool COPIES>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
 {
@@ -136,7 +137,7 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
     const int m_lo = r0 * L.v, m_hi = min(L.M, r1 * L.v);
 
     // ---- a2: codebooks -> shared memory as 16-byte rows (4 entries per thread in flight); clear the sums ----
-    const int sh1 = P.cb1_shift, n1 = L.k1 << sh1;
+    const int sh1 = COPIES ? P.cb1_shift : 0, n1 = L.k1 << sh1;
     for (int e0 = threadIdx.x; e0 < n1; e0 += 4 * TC_THREADS) {
         uint4 row[4];
 #pragma unroll
@@ -414,13 +415,11 @@ cudaError_t launch_decode_smem_tc(const LayerView &L, const void *x, int B, void
     // (a dependent launch, and no memset in front of it: 4096 x 4096, v = 6, 5 tokens 23.1 -> 21.4 us, 11008 x 4096, 16 tokens 47.5 -> 44.9)
     cudaError_t e = launch_dependent("smem_tc", NT == 2 ? smem_tc_prepass_kernel<2> : smem_tc_prepass_kernel<1>, pl.pre_grid, PRE_THREADS, 0, st, P);
     if (e != cudaSuccess) return e;
-    if (NT == 2) {
-        auto kern = res ? decode_smem_tc_kernel<2, true> : decode_smem_tc_kernel<2, false>;
-        e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), pl.smem);
-        if (e != cudaSuccess) return e;
-        return launch_dependent("smem_tc", kern, pl.grid, TC_THREADS, pl.smem, st, P);
-    }
-    auto kern = res ? decode_smem_tc_kernel<1, true> : decode_smem_tc_kernel<1, false>;
+    const bool copies = pl.cb1_shift > 0;
+    auto kern = NT == 2 ? (res ? (copies ? decode_smem_tc_kernel<2, true, true> : decode_smem_tc_kernel<2, true, false>)
+                               : (copies ? decode_smem_tc_kernel<2, false, true> : decode_smem_tc_kernel<2, false, false>))
+                        : (res ? (copies ? decode_smem_tc_kernel<1, true, true> : decode_smem_tc_kernel<1, true, false>)
+                               : (copies ? decode_smem_tc_kernel<1, false, true> : decode_smem_tc_kernel<1, false, false>));
     e = allow_dynamic_smem(reinterpret_cast<const void *>(kern), pl.smem);
     if (e != cudaSuccess) return e;
     return launch_dependent("smem_tc", kern, pl.grid, TC_THREADS, pl.smem, st, P);

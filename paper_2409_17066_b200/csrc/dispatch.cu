@@ -42,15 +42,15 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
 // columns one after the other.  Past one slab and 8 tokens the batched kernel is faster for v = 6 with a residual table (4096 x 4096 with outlier
 // columns at 16 tokens 27.6 -> 23.1 us, 11008 x 4096 45.0 -> 41.0, 4096 x 11008 56.6 -> 40.7; without them up to twice as many rows as columns: 11008 x 4096
 // 40.4 / 39.2) and otherwise up to 2048 rows (v = 8, 256 centroids, 2048 x
-// 8192 18.6 -> 16.5, but 4096 x 11008 26.7 / 29.3), up to 8 tokens only for v = 6 with outlier columns and a residual table (2048 x 8192 27.0 -> 22.7,
-// 4096 x 11008 43.8 -> 40.2; without outliers 36.8 / 38.1); in one slab at 8 tokens 21.3 / 22.7 (4096 x 4096).  It has a quick way for outlier
+// 8192 18.6 -> 16.5, but 4096 x 11008 26.7 / 29.3), up to 8 tokens only for v = 6 with outlier columns and a residual table and at most half as many rows as
+// columns (2048 x 8192 27.0 -> 22.7, 4096 x 11008 43.8 -> 40.2; without outliers 36.8 / 38.1, 8192 x 8192 slower); in one slab at 8 tokens 21.3 / 22.7 (4096 x 4096).  It has a quick way for outlier
 // vectors of 4.
 static bool smem_takes_batched(const LayerView &L, int B)
 {
     const int Bg = decode_group(B);
     if (!smem_tc_supported(L, Bg) || (L.n_out > 0 && L.v0 != 4) || smem_tc_slabs(L, Bg) < 2) return false;
     const bool gathers = L.v < 8 && L.k2 > 0;
-    return Bg > 8 ? (gathers && (L.n_out > 0 || L.M <= 2 * L.N)) || L.M <= 2048 : gathers && L.n_out > 0;
+    return Bg > 8 ? (gathers && (L.n_out > 0 || L.M <= 2 * L.N)) || L.M <= 2048 : gathers && L.n_out > 0 && 2 * L.M <= L.N;
 }
 
 // The layer as the batched kernel takes it.  Calls of the family of tables in shared memory have never had CTAs that wait for one
