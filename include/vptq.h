@@ -184,7 +184,8 @@ int64_t vptq_linear_workspace_bytes(const vptq_layer_desc *desc, int32_t B);
  * B <= 16 runs the decode kernels; larger B runs the tensor-core path
  * (tcgen05) when the layer qualifies (v = 6, 8 or 12, any codebook sizes, groups and outlier columns, scale and
  * bias per input column), otherwise the decode kernels over groups of 16 tokens.  The tensor-core kernel also takes
- * such layers on the path "decode_l2_fma" from 5 tokens on and on the path "decode_gl_fma" from 3 tokens on (not
+ * such layers on the path "decode_l2_fma" from 5 tokens on and on the path "decode_gl_fma" from 3 tokens on, and some
+ * of 5 to 16 tokens on the path "decode_smem_mma", these without waits between CTAs (none of them
  * with VPTQ_FLAG_DETERMINISTIC): vptq_linear_path() goes on naming the family, and what is said of the tensor-core
  * kernel here holds for these calls too.  Calls on one stream are ordered; calls on different streams must not share
  * a workspace.
