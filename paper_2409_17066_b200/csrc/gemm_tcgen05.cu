@@ -641,10 +641,13 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
     const int b_bytes = P.tile_n * 64, b_stages = P.b_stages;
     const uint32_t sA = base;
     const uint32_t sB = sA + A_STAGES * A_BYTES;
-    uint8_t *cb1_ptr = sm + A_STAGES * A_BYTES + b_stages * b_bytes;
+    // Output staging, EPI_WARPS x 2 x 2 KB: before the tables, whose sizes are multiples of 16 bytes only, since a tensor copy reads
+    // shared memory from a multiple of 128.
+    const uint32_t sEpi = sB + b_stages * b_bytes;
+    static_assert(A_BYTES % 1024 == 0 && EPI_BUF_BYTES % 128 == 0, "a piece begins on a multiple of 128 bytes (a stage of B is tile_n / 16 KB)");
+    uint8_t *cb1_ptr = sm + A_STAGES * A_BYTES + b_stages * b_bytes + EPI_WARPS * 2 * EPI_BUF_BYTES;
     uint8_t *cb2_ptr = cb1_ptr + P.cb1_bytes;
-    const uint32_t sEpi = smem_addr(cb2_ptr + P.cb2_bytes);     // EPI_WARPS x 2 x 2 KB output staging
-    float *bias = reinterpret_cast<float *>(cb2_ptr + P.cb2_bytes + EPI_WARPS * 2 * EPI_BUF_BYTES);       // [tile_n] bias terms of the token tile
+    float *bias = reinterpret_cast<float *>(cb2_ptr + P.cb2_bytes);       // [tile_n] bias terms of the token tile
     uint64_t *bars = reinterpret_cast<uint64_t *>(bias + MAX_TILE_N);   // fullA[] emptyA[] fullB[] emptyB[] accum_full accum_empty
     const uint32_t bar0 = smem_addr(bars);
     auto bar_fullA = [&](int s) { return bar0 + 8u * s; };

@@ -94,6 +94,33 @@ def test_few_tokens_and_cuts_within_tiles(M, N, B, kw):
         assert rel_err(y.float().cpu().numpy(), y_ref) <= (TOL if kw.get("out_dtype") != "bf16" else 2.0 ** -8)
 
 
+ANY = dict(V6, k1=1100, out_dtype="fp32")
+
+
+@pytest.mark.parametrize("Ms,N,B,kw", [                     # staged tables of sizes that are no multiple of 128 bytes, FP32 results
+    ((720,), 12000, 8, ANY), ((724,), 9000, 16, ANY),                             # calls of the decode family's name
+    ((724,), 1003, 40, dict(ANY, k1=4096, k2=300)), ((720,), 1100, 100, dict(ANY, k1=1001)),
+    ((1000,), 1100, 20, dict(v=8, k1=1100, k2=300, out_dtype="fp32")),
+    ((1000,), 1100, 70, dict(v=8, k1=4095, out_dtype="fp32")), ((264,), 1003, 40, dict(v=8, k1=65536, k2=300, out_dtype="fp32")),
+    ((520, 132), 1003, 17, ANY), ((520, 136), 1003, 70, dict(v=8, k1=1001, k2=75, out_dtype="fp32")),
+])
+def test_fp32_pieces_are_staged_where_the_copy_engine_can_read(Ms, N, B, kw):
+    import torch
+    from paper_2409_17066_b200 import binding as b
+    ds = [synth.make_layer(synth.LayerSpec("al%d" % i, M, N, **kw), 103 + i, 0, B) for i, M in enumerate(Ms)]
+    dls = [b.DeviceLayer(d) for d in ds]
+    x, ys = dls[0].upload_x(ds[0]["x"]), [torch.empty(B, M, dtype=torch.float32, device="cuda") for M in Ms]
+    if len(Ms) == 1:
+        assert b.lib.vptq_linear_has_status(C.byref(dls[0].desc), B) == 1
+        dls[0].linear(x, ys[0])
+    else:
+        fused = b.FusedLayers(dls)
+        assert fused.path(B) == "fused_gemm_tcgen05"
+        fused.linear(x, ys)
+    for d, y in zip(ds, ys):
+        assert rel_err(y.cpu().numpy(), oracle.Layer.from_synth(d).linear(ds[0]["x"])) <= TOL
+
+
 @pytest.mark.parametrize("M,N,B,kw", [
     (1000, 1003, 40, dict(k1=40000, k2=129)),                                     # 16 and 8 bits, indices that need the clamp
     (136, 33, 17, dict(k1=32769)),                                                # 16 bits, one k block and a column more
