@@ -20,6 +20,7 @@ cudaError_t launch_decode_smem_mma(const LayerView &L, const void *x, int B, voi
 // activations staged in shared memory in mma A-fragment order, 32 warps (decode_smem_tc.cu)
 bool smem_tc_supported(const LayerView &L, int B);
 int smem_tc_slabs(const LayerView &L, int B);        // slabs of columns whose activations it stages one after the other
+bool smem_tc_tight(const LayerView &L, int B);       // more than one, or one only without copies of the main table
 long long smem_tc_workspace_bytes(const LayerView &L, int B);
 cudaError_t launch_decode_smem_tc(const LayerView &L, const void *x, int B, void *out, void *ws, cudaStream_t st);
 

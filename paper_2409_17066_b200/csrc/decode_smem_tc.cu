@@ -29,8 +29,13 @@ namespace {
 
 constexpr int TC_WARPS = 32, TC_THREADS = TC_WARPS * 32;
 constexpr int TC_SMEM_BUDGET = 224 * 1024;
-// bytes of copies of a small main table: lane l reads copy l mod copies, so with eight the 8 rows of a matrix come from 8 different 16-byte
-// banks.  256 centroids, v = 8: 11008 x 4096 20.0 -> 16.0 us at 8 tokens, 24.0 -> 20.1 at 16; v = 6 with a residual table 31.0 -> 26.8, 35.8 -> 31.9.
+// Copies of a small main table: lane l reads copy l mod copies, so with eight the 8 rows of a matrix come from 8 different 16-byte
+// banks.  As many as TC_COPIES_BYTES hold, four at least (eight of 256 rows, four of 512; two of 1024 gain nothing and cost up to 0.2 us), where a CTA reads 1.5
+// rows for each that it stages and they cost no slab.  256 centroids, v = 8: 11008 x 4096 20.0 -> 16.0 us at 8 tokens, 24.0 -> 20.1 at 16;
+// v = 6 with a residual table 31.0 -> 26.8, 35.8 -> 31.9; 512, v = 8, 16 tokens: 4096 x 5632 20.3 -> 19.6; but v = 6, 1792 x 768 at 5 tokens 7.51 / 7.67.
+// A slab more takes 1.2-2 us, which eight copies win back from TC_SLAB_READS reads on (v = 8, 16 tokens: 4096 x 6400 20.3 -> 19.4, 4096 x 13000 34.1 -> 30.5, v = 4
+// 2048 x 6600 20.6 -> 19.3, but v = 8 2048 x 6600 16.2 / 16.6, 2048 x 6144 15.4 / 16.2), four do not (512, 4096 x 6400 22.9 / 23.4, 11008 x 6400 39.2 / 40.8).
+constexpr int TC_SLAB_READS = 20000;
 constexpr int TC_COPIES_BYTES = 32 * 1024;
 
 constexpr int PRE_THREADS = 512;       // pre-pass: 32 columns of 16 tokens
@@ -126,7 +131,8 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     uint4 *cb1 = reinterpret_cast<uint4 *>(smem);                                                        // [k1][copies]
-    uint4 *cb2 = cb1 + (L.k1 << P.cb1_shift);                                                                             // [k2][rep]
+    const int sh1 = COPIES ? P.cb1_shift : 0, n1 = L.k1 << sh1;
+    uint4 *cb2 = cb1 + n1;                                                                               // [k2][rep]
     uint8_t *afrag = reinterpret_cast<uint8_t *>(cb2 + (RES ? (size_t)L.k2 * (P.cb2_replicated ? 8 : 1) : 0));   // [slab_chunks][16][32][FRAG]
     __half *xs_out = reinterpret_cast<__half *>(afrag + (size_t)P.slab_chunks * CHUNK_BYTES);            // [TP][n_out_pad]
     float *part = reinterpret_cast<float *>(xs_out + (size_t)TP * P.n_out_pad);                          // [rows_cta][TP][8]
@@ -137,7 +143,6 @@ decode_smem_tc_kernel(const __grid_constant__ SmemTcParams P)
     const int m_lo = r0 * L.v, m_hi = min(L.M, r1 * L.v);
 
     // ---- a2: codebooks -> shared memory as 16-byte rows (4 entries per thread in flight); clear the sums ----
-    const int sh1 = COPIES ? P.cb1_shift : 0, n1 = L.k1 << sh1;
     for (int e0 = threadIdx.x; e0 < n1; e0 += 4 * TC_THREADS) {
         uint4 row[4];
 #pragma unroll
@@ -346,6 +351,7 @@ struct SmemTcPlan {
     size_t smem;
     long long ws_bytes;
     bool ok;
+    bool tight;          // more than one slab, or would be with the copies that TC_COPIES_BYTES hold
 };
 
 SmemTcPlan plan_smem_tc(const LayerView &L, int NT)
@@ -357,19 +363,30 @@ SmemTcPlan plan_smem_tc(const LayerView &L, int NT)
     p.rows_cta = ceil_div(L.R, p.grid);
     p.n_out_pad = (L.n_out + 7) / 8 * 8;
     p.cb2_rep = (L.k2 > 0 && L.k2 <= 256) ? 1 : 0;
-    p.cb1_shift = 0;
-    while (p.cb1_shift < 3 && (L.k1 * 16 << (p.cb1_shift + 1)) <= TC_COPIES_BYTES) p.cb1_shift++;
-    const long long fixed = ((long long)L.k1 * 16 << p.cb1_shift) + (long long)L.k2 * 16 * (p.cb2_rep ? 8 : 1) + (long long)TP * p.n_out_pad * 2 +
-                            (long long)p.rows_cta * TP * 8 * 4 + TP * 4 + 64;
     const int chunk_bytes = 16 * 32 * 8 * NT;
     const int n_chunks = (L.Nc + 255) / 256;
-    long long room = (TC_SMEM_BUDGET - fixed) / chunk_bytes;
-    if (room > n_chunks) room = n_chunks;
-    p.ok = room >= 1;
-    if (!p.ok) room = 1;
-    p.n_slabs = ceil_div(n_chunks, (int)room);
+    auto fixed = [&](int shift) {
+        return ((long long)L.k1 * 16 << shift) + (long long)L.k2 * 16 * (p.cb2_rep ? 8 : 1) + (long long)TP * p.n_out_pad * 2 +
+               (long long)p.rows_cta * TP * 8 * 4 + TP * 4 + 64;
+    };
+    auto slabs = [&](int shift) {                             // 0: the tables leave no room for activations
+        const long long room = (TC_SMEM_BUDGET - fixed(shift)) / chunk_bytes;
+        return room < 1 ? 0 : room >= n_chunks ? 1 : ceil_div(n_chunks, (int)room);
+    };
+    p.n_slabs = slabs(0);
+    p.ok = p.n_slabs > 0;
+    if (!p.ok) p.n_slabs = n_chunks;
+    // see TC_COPIES_BYTES
+    int most = 3;
+    while (most > 0 && (long long)L.k1 * 16 << most > TC_COPIES_BYTES) most--;
+    if (!p.ok || most < 2) most = 0;
+    const long long reads = (long long)p.rows_cta * L.Nc;
+    p.tight = p.n_slabs > 1 || slabs(most) != 1;
+    p.cb1_shift = 0;
+    while (p.cb1_shift < most && slabs(p.cb1_shift + 1) == p.n_slabs && 2 * reads >= 3LL * L.k1 << (p.cb1_shift + 1)) p.cb1_shift++;
+    if (p.cb1_shift < most && most == 3 && reads >= TC_SLAB_READS && slabs(3) == p.n_slabs + 1) { p.cb1_shift = 3; p.n_slabs++; }
     p.slab_chunks = ceil_div(n_chunks, p.n_slabs);            // equal slabs
-    p.smem = (size_t)(fixed + (long long)p.slab_chunks * chunk_bytes);
+    p.smem = (size_t)(fixed(p.cb1_shift) + (long long)p.slab_chunks * chunk_bytes);
     p.chunks_total = n_chunks;
     p.pre_grid = ceil_div(L.n_out + n_chunks * 256, PRE_THREADS / 16);
     if (p.pre_grid > 4 * G) p.pre_grid = 4 * G;
@@ -393,6 +410,8 @@ bool smem_tc_supported(const LayerView &L, int B)
 }
 
 int smem_tc_slabs(const LayerView &L, int B) { return plan_smem_tc(L, B <= 8 ? 1 : 2).n_slabs; }
+
+bool smem_tc_tight(const LayerView &L, int B) { return plan_smem_tc(L, B <= 8 ? 1 : 2).tight; }
 
 long long smem_tc_workspace_bytes(const LayerView &L, int B)
 {

@@ -38,23 +38,30 @@ LinearPath choose_path(const LayerView &L, int B, int flags)
 // most four or two tokens per launch and gather every centroid again for the next ones; the batched kernel gathers it once
 // whatever the batch.  4096 x 4096 over the 1 MiB table: 25 us
 // at any batch up to 64, against 14-17 us per four tokens; 11008 x 4096, v = 12 in four groups: 52 us against 31 us per two.
-// Tables in shared memory: the decode kernel stages the activations slab by slab, which nothing overlaps, and reads outlier
-// columns one after the other.  Past one slab and 8 tokens the batched kernel is faster for v = 6 with a residual table (4096 x 4096 with outlier
-// columns at 16 tokens 27.6 -> 23.1 us, 11008 x 4096 45.0 -> 41.0, 4096 x 11008 56.6 -> 40.7; without them up to twice as many rows as columns: 11008 x 4096
-// 40.4 / 39.2) and otherwise up to 2048 rows (v = 8, 256 centroids, 2048 x
-// 8192 18.6 -> 16.5, but 4096 x 11008 26.7 / 29.3), up to 8 tokens only for v = 6 with outlier columns and a residual table and at most half as many rows as
-// columns (2048 x 8192 27.0 -> 22.7, 4096 x 11008 43.8 -> 40.2; without outliers 36.8 / 38.1, 8192 x 8192 slower); in one slab at 8 tokens 21.3 / 22.7 (4096 x 4096).  It has a quick way for outlier
-// vectors of 4.
+//
+// Of the family of tables in shared memory it takes, with outlier vectors of 4 or none, the calls whose tables, copies of a small
+// main one among them, leave no room for all activations at once (smem_tc_tight), and of these
+//   up to 8 tokens    v < 8 with a residual table and outlier columns and at most half as many rows as columns;
+//   9 to 16 tokens    up to 2048 rows; v < 8 with a residual table: with outlier columns any, without them up to twice as many
+//                     rows as columns where the decode kernel takes more than one slab.
+// The decode kernel stages the activations slab by slab, which nothing overlaps, and reads outlier columns one after the other; the
+// batched one has a set-up to pay and reads a centroid per 128 rows whatever the batch.  Both in us, decode / batched:
+//   v = 6, residual, outliers, 16 tokens   4096 x 4096 27.6 / 23.1, 11008 x 4096 45.0 / 41.0, 4096 x 11008 56.6 / 40.7
+//   ... 8 tokens                           2048 x 8192 27.0 / 22.7, 4096 x 11008 43.8 / 40.2; one slab, 4096 x 4096: 21.3 / 22.7
+//   v = 6, residual, 16 tokens             11008 x 4096 40.4 / 39.2, 12 tokens 2048 x 6144 24.3 / 21.8; one slab, 4096 x 6400 (512 centroids): 34.7 / 35.7
+//   ... 8 tokens                           4096 x 11008 36.8 / 38.1
+//   v = 8, 256 centroids, 16 tokens        2048 x 8192 18.6 / 16.5, 2048 x 6600 16.2 / 15.0, 1024 x 6600 14.5 / 12.2; 4096 x 11008 26.7 / 29.3
 static bool smem_takes_batched(const LayerView &L, int B)
 {
     const int Bg = decode_group(B);
-    if (!smem_tc_supported(L, Bg) || (L.n_out > 0 && L.v0 != 4) || smem_tc_slabs(L, Bg) < 2) return false;
+    if (!smem_tc_supported(L, Bg) || (L.n_out > 0 && L.v0 != 4) || !smem_tc_tight(L, Bg)) return false;
     const bool gathers = L.v < 8 && L.k2 > 0;
-    return Bg > 8 ? (gathers && (L.n_out > 0 || L.M <= 2 * L.N)) || L.M <= 2048 : gathers && L.n_out > 0 && 2 * L.M <= L.N;
+    if (Bg <= 8) return gathers && L.n_out > 0 && 2 * L.M <= L.N;
+    return L.M <= 2048 || (gathers && (L.n_out > 0 || (L.M <= 2 * L.N && smem_tc_slabs(L, Bg) > 1)));
 }
 
-// The layer as the batched kernel takes it.  Calls of the family of tables in shared memory have never had CTAs that wait for one
-// another, so they may share the GPU without saying so.
+// The layer as the batched kernel takes it.  A call of one layer of the family of tables in shared memory has never had CTAs that wait
+// for one another, so it may share the GPU without saying so (launches that several layers share may wait: linear_fused_waits_between_ctas).
 static LayerView batched_view(LinearPath path, const LayerView &L)
 {
     LayerView v = L;

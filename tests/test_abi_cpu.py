@@ -287,3 +287,18 @@ def test_shared_memory_tables_in_the_batched_kernel_have_no_waits_between_ctas(b
         d = b.make_desc(4096, 11008, 6, 4096, 256, n_outlier=110, v0=4, k0=4096, out_dtype=out)
         assert b.vptq_linear_path(d, B) == "decode_smem_mma" and b.lib.vptq_linear_has_status(C.byref(d), B) == 1
         assert b.lib.vptq_linear_waits_between_ctas(C.byref(d), B) == 0
+
+
+@pytest.mark.parametrize("M,N,B,k1,launches,status", [
+    (449920, 512, 16, 256, 2, 0), (497280, 512, 16, 256, 2, 0),       # many rows: without copies of the table there is room for them
+    (520960, 512, 16, 256, 1, 0),                                     # ... and here no longer
+    (4096, 6144, 12, 1024, 2, 0), (2048, 6144, 12, 1024, 2, 0),       # two copies of 1024 rows would cost a slab
+    (4096, 6400, 16, 256, 2, 0), (2048, 6600, 16, 256, 2, 1),         # tight beside eight copies of 256 rows: up to 2048 rows batched
+    (2048, 5632, 16, 256, 2, 0), (2052, 6600, 16, 256, 2, 0),
+])
+def test_copies_of_a_small_table_do_not_move_calls_to_other_kernels(binding, M, N, B, k1, launches, status):
+    b = binding
+    d = b.make_desc(M, N, 8, k1)
+    assert b.vptq_linear_path(d, B) == "decode_smem_mma"
+    assert b.vptq_linear_launches(d, B) == launches            # the pre-pass of decode_smem_tc and of the batched kernel; the older one has none
+    assert b.lib.vptq_linear_has_status(C.byref(d), B) == status

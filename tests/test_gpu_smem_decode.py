@@ -1,6 +1,8 @@
 """Decode over tables in shared memory where its staging and its outlier pass have edges: more pieces of outlier rows than a
 warp asks for in advance, rows that are not 16-byte aligned, a stored column order, more columns than one pass of the CTA
 stages, more than one slab."""
+import ctypes as C
+
 import pytest
 
 from oracle import oracle
@@ -47,3 +49,28 @@ def test_small_tables_in_copies(k1, M, N, B, kw):
     assert b.vptq_linear_path(dl.desc, B) == ("decode_smem_fma" if B <= 4 else "decode_smem_mma")
     y = dl.linear(dl.upload_x(d["x"]))
     assert rel_err(y.float().cpu().numpy(), oracle.Layer.from_synth(d).linear(d["x"])) <= TOL
+
+
+@pytest.mark.parametrize("M,N,B,kw", [                      # on 148 SMs:
+    (2056, 9001, 16, dict(v=8, k1=256)),                    # two slabs, eight copies
+    (4096, 6600, 16, dict(v=8, k1=256, out_dtype="fp32")),  # two slabs, one of them for the sake of eight copies
+    (2056, 6700, 9, dict(v=8, k1=256)),                     # one slab that is nearly full, no copies
+    (4096, 13000, 13, dict(v=8, k1=256, x_dtype="bf16")),   # three slabs
+    (2500, 14300, 16, dict(v=7, k1=300)),                   # three slabs, four copies
+    (2056, 20000, 16, dict(v=8, k1=4096, out_dtype="bf16")),    # five slabs
+    (4600, 9003, 8, dict(v=6, k1=4096, k2=256, n_out=9, v0=4, k0=300)),    # two, outlier columns, up to 8 tokens
+    (4096, 19000, 5, dict(v=8, k1=200, k2=100)),
+    (500, 9000, 16, dict(v=4, k1=256)),
+    (1000, 14001, 8, dict(v=4, k1=1024, k2=256)),
+    (2400, 13000, 12, dict(v=4, k1=4096, k2=256)),          # four slabs
+])
+def test_tensor_core_decode_slab_by_slab(M, N, B, kw):
+    from paper_2409_17066_b200 import binding as b
+    d = synth.make_layer(synth.LayerSpec("sl", M, N, **kw), 104, B, B)
+    dl = b.DeviceLayer(d)
+    assert b.vptq_linear_path(dl.desc, B) == "decode_smem_mma" and b.vptq_linear_launches(dl.desc, B) == 2
+    assert b.lib.vptq_linear_has_status(C.byref(dl.desc), B) == 0           # not the batched kernel
+    y_ref = oracle.Layer.from_synth(d).linear(d["x"])
+    for _ in range(2):
+        y = dl.linear(dl.upload_x(d["x"]))
+        assert rel_err(y.float().cpu().numpy(), y_ref) <= (TOL if kw.get("out_dtype") != "bf16" else 2.0 ** -8)
