@@ -58,7 +58,8 @@ __device__ __forceinline__ float2 h2f(uint32_t w)
     return __half22float2(*reinterpret_cast<__half2 *>(&w));
 }
 
-template <int TB, int VV, bool RES, bool FUSED>
+// (COPIES: a kernel of its own, since a variable shift of every index costs the others up to 3 %)
+template <int TB, int VV, bool RES, bool FUSED, bool COPIES>
 __global__ void __launch_bounds__(WARPS * 32, 1)
 decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 {
@@ -76,7 +77,8 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     uint4 *cb1 = reinterpret_cast<uint4 *>(smem);                                            // [k1][copies]
-    uint4 *cb2 = cb1 + (L.k1 << P.cb1_shift);                                                                 // [k2][rep]
+    const int sh1 = COPIES ? P.cb1_shift : 0, n1 = L.k1 << sh1;
+    uint4 *cb2 = cb1 + n1;                                                                   // [k2][rep]
     __half *xs_out = reinterpret_cast<__half *>(cb2 + (RES ? (size_t)L.k2 * (P.cb2_replicated ? 8 : 1) : 0));   // [TB][n_out_pad]
     __half *xs = xs_out + (size_t)TB * P.n_out_pad;                                          // [TB][slab_cols]
     float *part = reinterpret_cast<float *>(xs + (size_t)TB * P.slab_cols);                  // [rows][TB][8]
@@ -96,7 +98,6 @@ decode_smem_fma_kernel(const __grid_constant__ SmemFmaParams P)
 
     // ---- a2: codebooks -> shared memory as 16-byte rows; clear the partial sums -------------------
     // (loads of 4 entries are issued before the first store: one L2 round trip per 4 entries, not per entry)
-    const int sh1 = P.cb1_shift, n1 = L.k1 << sh1;
     for (int e0 = threadIdx.x; e0 < n1; e0 += 4 * THREADS) {
         uint4 row[4];
 #pragma unroll
@@ -360,18 +361,28 @@ int fma_token_group(int B) { return B >= 4 ? 4 : (B >= 2 ? 2 : 1); }
 
 // Copies of a small main table side by side, lane l reading copy l mod copies: of the eight lanes that read 16-byte rows at random in
 // one wavefront those of one copy share 8 / copies of the 8 banks of that width; eight copies are free of conflicts.  256 centroids, v = 8,
-// one token: 11008 x 4096 10.6 -> 7.9 us, 4096 x 4096 6.25 -> 5.34.  As many as fit COPIES_BYTES, where a CTA reads as many rows as
-// it stages at one token, 2 * tokens as many at more (products bound there: 4 tokens, 4096 x 4096 8.51 / 8.42, 2048 x 2048, which reads
-// twice as many, 5.46 / 5.71).  Two copies of 64 KB do not pay: k1 = 4096, 4096 x 4096 7.18 / 7.73, 11008 x 4096 11.70 / 11.93.
+// one token: 11008 x 4096 10.6 -> 7.9 us.  Eight of 256 rows or four of 512 fit COPIES_BYTES; two of 1024 gain nothing (v = 4,
+// 6661 x 2512 19.4 / 19.6).  Staging them takes 0.1-0.5 us.  A CTA has to read 2 rows for each that it stages at one token, 4 at two and 16 at
+// four, where products bound, half as many again beside a residual table, twice as many of four copies, and half a row where
+// less than half of the SMs stage:
+//   1 token    1408 x 2112, v = 8 4.60 -> 4.44; 827 x 2880, v = 8 3.99 / 4.10; 1664 x 994, v = 6 4.59 / 5.11
+//   2 tokens   1536 x 9600, v = 6 9.74 -> 9.21; 11136 x 545, v = 8 5.57 / 5.65
+//   4 tokens   8987 x 8512, v = 8 24.9 -> 23.9; 2368 x 1964, v = 8 7.01 / 7.37; 448 x 8399, v = 4 16.5 / 16.7
+//   residual   5158 x 7360, v = 6 19.3 -> 17.1; 2624 x 1216, v = 8 4.95 / 5.14 (one token)
+//   512 rows   7424 x 5201, v = 8 18.3 -> 17.7; 5299 x 625, v = 6 8.44 / 8.65 (one token)
+//   54 CTAs    320 x 1536, v = 6 3.04 -> 2.89
 constexpr size_t COPIES_BYTES = 32 * 1024;
 void plan_copies(SmemFmaPlan &p, const LayerView &L, int TB, int rows_cta)
 {
     const size_t table = (size_t)L.k1 * 16, rest = p.smem - table;
-    const long long reads = (long long)rows_cta * L.Nc / (TB == 1 ? 1 : 2 * TB);
-    p.cb1_shift = 0;
-    while (p.cb1_shift < 3 && table << (p.cb1_shift + 1) <= COPIES_BYTES && rest + (table << (p.cb1_shift + 1)) <= 224 * 1024 &&
-           reads >= (long long)L.k1 << (p.cb1_shift + 1))
-        p.cb1_shift++;
+    int shift = 3;
+    while (shift > 0 && (table << shift > COPIES_BYTES || rest + (table << shift) > 224 * 1024)) shift--;
+    long long halves = TB == 1 ? 4 : TB == 2 ? 8 : 32;           // twice the rows to read for each that is staged
+    if (L.k2 > 0) halves += halves / 2;
+    if (shift == 2) halves *= 2;
+    if (2 * p.grid <= device_sm_count()) halves = 1;
+    const long long staged = (table << shift) / 16 > 2048 ? (table << shift) / 16 : 2048;
+    p.cb1_shift = shift >= 2 && 2LL * rows_cta * L.Nc >= staged * halves ? shift : 0;
     p.smem = rest + (table << p.cb1_shift);
 }
 
@@ -396,20 +407,20 @@ SmemFmaPlan plan_smem_fma(const LayerView &L, int TB)
     return p;
 }
 
-template <int TB, int VV, bool RES, bool FUSED>
+template <int TB, int VV, bool RES, bool FUSED, bool COPIES>
 cudaError_t launch_kernel(const SmemFmaParams &P, const SmemFmaPlan &pl, cudaStream_t st)
 {
-    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_fma_kernel<TB, VV, RES, FUSED>), pl.smem);
+    cudaError_t e = allow_dynamic_smem(reinterpret_cast<const void *>(decode_smem_fma_kernel<TB, VV, RES, FUSED, COPIES>), pl.smem);
     if (e != cudaSuccess) return e;
-    return launch_dependent("smem_fma", decode_smem_fma_kernel<TB, VV, RES, FUSED>, pl.grid, WARPS * 32, pl.smem, st, P);
+    return launch_dependent("smem_fma", decode_smem_fma_kernel<TB, VV, RES, FUSED, COPIES>, pl.grid, WARPS * 32, pl.smem, st, P);
 }
 
-template <int TB, int VV>
+template <int TB, int VV, bool COPIES>
 cudaError_t launch_one(const SmemFmaParams &P, const SmemFmaPlan &pl, bool res, cudaStream_t st)
 {
     const bool fused = P.n_layers > 1;
-    if (res) return fused ? launch_kernel<TB, VV, true, true>(P, pl, st) : launch_kernel<TB, VV, true, false>(P, pl, st);
-    return fused ? launch_kernel<TB, VV, false, true>(P, pl, st) : launch_kernel<TB, VV, false, false>(P, pl, st);
+    if (res) return fused ? launch_kernel<TB, VV, true, true, COPIES>(P, pl, st) : launch_kernel<TB, VV, true, false, COPIES>(P, pl, st);
+    return fused ? launch_kernel<TB, VV, false, true, COPIES>(P, pl, st) : launch_kernel<TB, VV, false, false, COPIES>(P, pl, st);
 }
 
 // several layers of the same format (apart from M) in one grid
@@ -433,12 +444,18 @@ bool plan_smem_fma_fused(const LayerView *Ls, int n, int TB, SmemFmaPlan *out)
     return true;
 }
 
+template <int TB, bool COPIES>
+cudaError_t launch_vv(const SmemFmaParams &P, const SmemFmaPlan &pl, int v, bool res, cudaStream_t st)
+{
+    if (v <= 4) return launch_one<TB, 4, COPIES>(P, pl, res, st);
+    if (v <= 6) return launch_one<TB, 6, COPIES>(P, pl, res, st);
+    return launch_one<TB, 8, COPIES>(P, pl, res, st);
+}
+
 template <int TB>
 cudaError_t launch_vv(const SmemFmaParams &P, const SmemFmaPlan &pl, int v, bool res, cudaStream_t st)
 {
-    if (v <= 4) return launch_one<TB, 4>(P, pl, res, st);
-    if (v <= 6) return launch_one<TB, 6>(P, pl, res, st);
-    return launch_one<TB, 8>(P, pl, res, st);
+    return pl.cb1_shift > 0 ? launch_vv<TB, true>(P, pl, v, res, st) : launch_vv<TB, false>(P, pl, v, res, st);
 }
 
 }  // namespace
