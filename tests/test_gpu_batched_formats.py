@@ -9,7 +9,7 @@ import pytest
 from oracle import oracle
 from paper_2409_17066_b200 import synth
 
-from helpers import TOL, rel_err
+from helpers import TOL, batched_segments, rel_err
 
 pytestmark = pytest.mark.gpu
 
@@ -50,8 +50,8 @@ def test_batched_kernel_formats_and_edges(M, N, B, kw):
 
 
 @pytest.mark.parametrize("M,N,B,kw", [
-    (18816, 520, 40, dict(v=8, k1=65536)),                                        # on 148 SMs: a tile less than SMs, a slot per tile
-    (18944, 520, 40, dict(v=8, k1=65536, out_dtype="bf16")),                      # as many tiles as SMs, a slot per cut
+    (18816, 520, 40, dict(v=8, k1=65536)),                                        # on 148 SMs: a tile less than SMs, whole ones, one CTA each
+    (18944, 520, 40, dict(v=8, k1=65536, out_dtype="bf16")),                      # as many tiles as SMs: the same
     (19065, 520, 33, dict(v=8, k1=65536, out_dtype="fp32")),                      # one more; rows of 4 bytes' alignment
     (9600, 300, 600, dict(v=8, k1=65536, k2=256)),                                # two token tiles
     (25000, 130, 520, dict(v=6, k1=256)),                                         # tiles of few k blocks: some whole, some cut
@@ -75,9 +75,11 @@ def test_split_tiles_have_scratch_of_their_own(M, N, B, kw):
     (1000, 1100, 33, dict(v=8, k1=65536, k2=256)),                                # the first of the other one
     (726, 1100, 64, V6), (726, 1100, 65, V6),
     (724, 1100, 17, dict(V6, out_dtype="fp32")),                                  # pieces that add up in the output
-    (1450, 2100, 256, V6), (1450, 2100, 257, V6),                                 # two sets of accumulators, one
-    (9600, 200, 20, dict(v=6, k1=512)),                                           # one k block more than CTAs per tile; short segments in turn
-    (600, 70, 20, V12),                                                           # fewer k blocks than CTAs per tile
+    (1450, 2100, 256, V6), (1450, 2100, 257, V6),                                 # room for two sets of accumulators, for one; a piece a CTA
+    (9600, 200, 20, dict(v=6, k1=512)),                                           # whole tiles, one CTA each
+    (600, 70, 20, V12),                                                           # ... of two k blocks
+    (7200, 2600, 20, dict(v=6, k1=4096, k2=5000)),                                # few tokens, residual table in L2: rows of 12 bytes, padded
+    (1000, 1100, 20, dict(v=8, k1=1024, k2=4096)),                                # ... of 16
     (2048, 2048, 64, dict(v=8, k1=256, n_out=40, v0=4, k0=300)),                  # outlier columns past a k block of 32
     (700, 9000, 9, dict(V6, n_out=65, k0=5000)),                                  # 13-bit outlier indices, a k block and a column of them;
     (700, 9000, 8, dict(V6, n_out=8, k0=200)),                                    # ... 8 bits, in a call of the decode family's name
@@ -92,6 +94,49 @@ def test_few_tokens_and_cuts_within_tiles(M, N, B, kw):
         y = dl.linear(x)
         assert b.lib.vptq_linear_has_status(C.byref(dl.desc), B) == 1 and b.vptq_workspace_status(dl.workspace(B)) == b.OK
         assert rel_err(y.float().cpu().numpy(), y_ref) <= (TOL if kw.get("out_dtype") != "bf16" else 2.0 ** -8)
+
+
+FP32 = dict(out_dtype="fp32")
+
+
+@pytest.mark.parametrize("M,N,B,kw,pieces,in_order", [      # on 148 SMs
+    (71990, 130, 40, dict(v=6, k1=512), 5, False),                                # accumulators in turn, both phases of both sets: v = 6, few tokens
+    (71996, 130, 40, dict(v=6, k1=512, **FP32), 5, True),
+    (71990, 130, 200, dict(v=6, k1=512, out_dtype="bf16"), 5, False),             # ... the other form
+    (71996, 130, 200, dict(v=6, k1=512, **FP32), 5, True),
+    (71990, 130, 200, dict(v=12, k1=512), 5, False),
+    (71996, 130, 200, dict(v=12, k1=512, **FP32), 5, True),
+    (76780, 66, 16, dict(v=8, k1=65536), 5, False),
+    (76780, 66, 100, dict(v=8, k1=65536, **FP32), 5, False),
+    (12797, 1500, 16, dict(v=8, k1=65536), 2, False),                             # fewer tiles than SMs, shares across their boundaries: a CTA ends one cut
+    (12797, 1500, 40, dict(v=8, k1=65536, out_dtype="bf16"), 2, False),           # tile and begins the next, a slot per tile
+    (11990, 1500, 16, V6, 2, False), (11989, 1900, 100, dict(V6, out_dtype="bf16"), 2, False),
+    (9000, 1700, 100, dict(v=12, k1=4096), 2, False),
+    (1300, 13000, 40, dict(v=6, k1=4096, **FP32), 2, True),                       # flag order, tiles of 120 rows: the last one ends in its quarter of 24
+    (1300, 13000, 100, dict(v=6, k1=4096, **FP32), 2, True),
+    (1304, 13000, 40, dict(v=12, k1=4096, **FP32), 2, True),
+    (10550, 878, 256, dict(v=8, k1=4096, k2=256), 1, False),                      # whole tiles, one CTA each
+])
+def test_pieces_that_a_cta_takes_in_turn(M, N, B, kw, pieces, in_order):
+    import torch
+    from paper_2409_17066_b200 import binding as b
+    spec = synth.LayerSpec("pt", M, N, **kw)
+    d = synth.make_layer(spec, 105, 0, B)
+    dl = b.DeviceLayer(d)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    ctas, kb, tile_n, flags = batched_segments(spec, B, n_sm)
+    assert b.lib.vptq_linear_waits_between_ctas(C.byref(dl.desc), B) == int(flags)
+    if n_sm == 148:
+        assert max(map(len, ctas)) == pieces and flags == in_order and (pieces < 5 or tile_n <= 256)
+        assert pieces != 2 or any(len(c) == 2 and c[0][1] > 0 and c[1][2] < kb for c in ctas)
+    y_ref = oracle.Layer.from_synth(d).linear(d["x"])
+    x, tol = dl.upload_x(d["x"]), TOL if kw.get("out_dtype") != "bf16" else 2.0 ** -8
+    for _ in range(2):
+        y = dl.linear(x)
+        assert b.vptq_workspace_status(dl.workspace(B)) == b.OK and rel_err(y.float().cpu().numpy(), y_ref) <= tol
+    shared = dl.with_flags(dl.desc.flags | b.FLAG_CONCURRENT)
+    assert b.lib.vptq_linear_waits_between_ctas(C.byref(shared.desc), B) == 0
+    assert rel_err(shared.linear(x).float().cpu().numpy(), y_ref) <= tol
 
 
 ANY = dict(V6, k1=1100, out_dtype="fp32")
