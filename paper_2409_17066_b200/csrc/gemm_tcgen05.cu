@@ -20,7 +20,8 @@
 //
 // Warp roles: warp 0 bulk loads of B; warp 1 TMEM allocation + MMA issue (an elected lane); 10 (v = 8) or 12 producer warps in
 // GROUPS groups, a k block each in turn (the next visit's packed indices in flight); 8 warps the epilogue
-// (tcgen05.ld -> + bias term -> output), two per TMEM lane quarter.  A form for few tokens has more producers (see Tile).
+// (tcgen05.ld -> + bias term -> output), two per TMEM lane quarter.  A form for few tokens has more producers and one
+// epilogue warp per quarter (see Tile).
 // Up to 256 tokens TMEM holds two sets of accumulators, so the next piece's MMAs do not wait for the epilogue
 // (8192 x 8192, v = 6, 16 tokens 54.5 -> 53.1 us).
 // What bounds the k loop is the SM's shared-memory/L1 data pipe (128 bytes per clock), which everything passes: per 32
@@ -77,8 +78,15 @@ constexpr int MEET_COLS_8 = 128, MEET_COLS = 224;
 // Columns by which the longest share may grow for the sake of whole CTAs per tile: scratch tiles (plus an eighth of the tokens),
 // FP32 sums.  1024 x 2048 (v = 6, 16 tokens, 16-bit results; 64 columns longer) 25.4 -> 13.0 us, 4096 x 4096 with v = 12 at 512
 // tokens (105 longer) 60.4 -> 55.2; v = 8: 4096 x 4096 (138 longer) 21.4 / 21.6 at 16 tokens, 50.3 / 47.4 at 512, 8192 x 8192 (554 longer)
-// 52.3 / 57.6.  FP32 sums: 1024 x 8192, v = 12, 512 tokens (70 longer) 61.7 -> 45.9, 200 tokens x 1024 x 2048 (64 longer) 18.8 / 19.6.
+// 52.3 / 57.6.  Over 208 layers of v = 6, 8 and 12 at 5 to 512 tokens, all result types, the cuts taken are within 2 % of the better ones in 195, 49 of
+// up to 16 tokens among them 45 (worst: v = 12, 3705 x 4728 at 5 tokens, 224 longer, 21.7 / 19.8; v = 6, 6101 x 918 at 64, 160 longer, 22.8 / 18.9).
+// FP32 sums: 1024 x 8192, v = 12, 512 tokens (70 longer) 61.7 -> 45.9, 200 tokens x 1024 x 2048 (64 longer) 18.8 / 19.6.
 constexpr int LONGER_COLS = 128, LONGER_COLS_SUM = 96;
+// ... and where that is one CTA a tile, so that no piece meets another and nothing is cleared: that many and 5/4 of the tokens.  v = 8: 10550 x 878 at 256
+// tokens (394 columns longer) 45.0 -> 25.0 us, 14463 x 397 at 32 (99) 19.7 -> 12.1, 12809 x 969 at 512 (284, v = 6) 56.5 -> 39.4, 13256 x 2119 at 512
+// (638) 55.6 -> 44.9, 15702 x 2408 at 16 (411) 33.3 / 32.7, 15316 x 2793 at 64 (533) 44.3 / 46.4, 15689 x 3469 at 17 (590) 36.7 / 36.5, 13022 x 1073 at
+// 64 (339) 25.8 -> 21.2; FP32 sums: 10224 x 1234 at 64 (574) 18.9 / 22.4.
+constexpr int WHOLE_COLS = 400;
 constexpr int FLAG_ORDER_MIN_COLS = 768;                 // columns of a share from which split tiles meet by flag order
 constexpr int SMEM_LIMIT = 227 * 1024, SMEM_LIMIT_L1 = 195 * 1024;
 
@@ -972,7 +980,7 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
             it0 += kb1 - kb0;
         }
     } else {
-        // ================= epilogue: two warps per TMEM lane quarter, taking turns at chunks of 32 tokens =================
+        // ============ epilogue: two warps per TMEM lane quarter (few tokens: one), taking turns at chunks of 32 tokens ============
         if (SPLIT_REGS) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_EPILOGUE));
         const int ew = warp - EPI_WARP0, h = ew >> 2;
         const int q = warp & 3;                                  // TMEM lane quarter this warp may read
@@ -1071,6 +1079,8 @@ gemm_tcgen05_kernel(const __grid_constant__ OutMaps<NL> maps, const __grid_const
                 } else if (m_ok) {
                     const int nt = min(EPI_TOKENS, t_cnt - c1);                // tokens of this chunk that exist
                     const long long o0 = (long long)(t0 + c1) * L.M + m;
+                    // (`add` does not come here: pieces of a tile meet in the scratch or in boxes.  Without it ptxas does worse by the rest: v = 6, FP32
+                    // results, 3757 + 939 rows x 3757 at 333 tokens 59.6 -> 62.3 us, 1299 + 324 x 1299 at 65 18.9 -> 20.0; with a loop a type 62.9, 20.0.)
                     if (add) {
 #pragma unroll
                         for (int j = 0; j < EPI_TOKENS; j++)
@@ -1232,7 +1242,8 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     if (!sh.whole_tiles && !in_order && tiles < (unsigned)workers) {
         const unsigned per_tile = workers / tiles;
         const long long longer = (long long)((sh.kb + per_tile - 1) / per_tile) * p.ks - columns / workers;
-        if (longer <= (p.tma_out ? LONGER_COLS_SUM : LONGER_COLS + p.tile_n / 8)) {
+        const int limit = per_tile == 1 ? WHOLE_COLS + p.tile_n * 5 / 4 : p.tma_out ? LONGER_COLS_SUM : LONGER_COLS + p.tile_n / 8;
+        if (longer <= limit) {
             sh.per_tile = per_tile;
             workers = (int)(tiles * per_tile);
         }

@@ -302,3 +302,15 @@ def test_copies_of_a_small_table_do_not_move_calls_to_other_kernels(binding, M, 
     assert b.vptq_linear_path(d, B) == "decode_smem_mma"
     assert b.vptq_linear_launches(d, B) == launches            # the pre-pass of decode_smem_tc and of the batched kernel; the older one has none
     assert b.lib.vptq_linear_has_status(C.byref(d), B) == status
+
+
+@pytest.mark.parametrize("M,N,B,v,whole", [
+    (10550, 878, 256, 8, True), (14463, 397, 32, 8, True), (13256, 2119, 512, 8, True),     # a whole tile for each of 83, 113 and 104 CTAs
+    (12797, 1500, 16, 8, False), (14798, 5343, 16, 8, False),                               # too long a share for that
+    (9400, 700, 64, 8, False),                                                              # 74 tiles: two CTAs each
+])
+def test_batched_tiles_are_not_cut_where_a_cta_each_will_do(binding, M, N, B, v, whole):
+    # nothing is cut: no scratch tiles, as with VPTQ_FLAG_DETERMINISTIC
+    b = binding
+    need = [b.vptq_linear_workspace_bytes(b.make_desc(M, N, v, 65536, flags=b.FLAG_SCALE_BIAS | f), B) for f in (0, b.FLAG_DETERMINISTIC)]
+    assert (need[0] == need[1]) == whole
