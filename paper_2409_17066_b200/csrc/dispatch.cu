@@ -174,15 +174,28 @@ int linear_dispatch(const LayerView &L, int flags, const void *x, int B, void *o
 
 // Whether layers whose own calls would take `path` are better off in one launch of the batched kernel, which costs one
 // set-up for all of them: a 7B layer's q+k+v+o (1024 rows of k and v) at 16 tokens takes 50 us instead of 76 over the 1 MiB
-// table, 70 instead of 100 with v = 12 in four groups.  Tables in shared memory have a decode kernel that takes a weight
-// for a little over half of the time, after 9 us (18 us with a residual table and 16 tokens) a layer: q+k+v+o with v = 6
-// 102 -> 65 us at 16 tokens, 82 -> 58 at 8, but gate+up of 11008 x 4096 79 -> 87 us at 8, and with 256 centroids and no
-// residual 42 -> 56.  From 17 to 64 tokens large layers, which fill the SMs on their own, keep sharing one layer's scratch.
+// table, 70 instead of 100 with v = 12 in four groups.  From 17 to 64 tokens large layers, which fill the SMs on their own, keep sharing
+// one layer's scratch.
+// Tables in shared memory have a decode kernel that takes a weight in a little over half of the time (v = 8 over eight copies of a
+// table: in half), after 8 us a layer (13 past 8 tokens, 4 more beside a residual table): shared up to 2^25 weights for each layer but one,
+// twice as many past 8 tokens, twice as many with a residual table, 5/8 of all that for v = 8 with up to 256 centroids.  One by one /
+// shared, us (* what is taken; of 192 calls of 5 to 16 tokens 189 are within 5 % of the better one):
+//                                                     q+k+v, 4096 + 2 x 1024 rows x 4096   2 x 11008 x 4096   2 x 8192 x 3072
+//   v = 6, 4096 + 256 centroids, outliers, 8 tokens   53.7 / 29.2*                         69.0* / 66.4       48.5 / 45.7*
+//   ... 16 tokens                                     52.0 / 29.8*                         81.4 / 66.7*       60.5 / 46.4*
+//   v = 8, 4096 centroids, 8 tokens                   33.0 / 21.6*                         41.5* / 49.5       29.7* / 33.8
+//   ... 16 tokens                                     38.3 / 21.8*                         50.3* / 49.9       37.4 / 34.0*
+//   v = 8, 256 centroids, 8 tokens                    30.1 / 20.5*                         31.6* / 48.3       24.1* / 32.5
+//   ... 16 tokens                                     34.3 / 20.5*                         39.4* / 48.6       30.9* / 32.7
+//   v = 8, 256 + 256 centroids, 8 tokens              35.2 / 22.8*                         43.0* / 52.4       31.2* / 35.3
 static bool fused_batched(LinearPath path, const LayerView *Ls, int n, int B)
 {
     long long weights = 0;
     for (int l = 0; l < n; l++) weights += (long long)Ls[l].M * Ls[l].N;
-    if (path == PATH_DECODE_SMEM_MMA) return weights <= ((n - 1LL) << (25 + (B > 8) + (Ls[0].k2 > 0)));
+    if (path == PATH_DECODE_SMEM_MMA) {
+        const int eighths = Ls[0].v == 8 && Ls[0].k1 <= 256 ? 5 : 8;
+        return 8 * weights <= eighths * ((n - 1LL) << (25 + (B > 8) + (Ls[0].k2 > 0)));
+    }
     return path != PATH_GEMM_TCGEN05 || B > 64 || weights <= ((n - 1LL) << 26);
 }
 

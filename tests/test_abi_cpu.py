@@ -314,3 +314,14 @@ def test_batched_tiles_are_not_cut_where_a_cta_each_will_do(binding, M, N, B, v,
     b = binding
     need = [b.vptq_linear_workspace_bytes(b.make_desc(M, N, v, 65536, flags=b.FLAG_SCALE_BIAS | f), B) for f in (0, b.FLAG_DETERMINISTIC)]
     assert (need[0] == need[1]) == whole
+
+
+@pytest.mark.parametrize("v,k1,k2,B,Ms,N,shared", [
+    (8, 256, 0, 8, (4096, 1024, 1024), 4096, True), (8, 256, 0, 16, (8192, 8192), 3072, False), (8, 256, 256, 8, (8192, 8192), 3072, False),
+    (8, 257, 0, 16, (8192, 8192), 3072, True), (6, 256, 0, 16, (8192, 8192), 3072, True), (8, 256, 256, 16, (8192, 8192), 3072, True),
+    (6, 4096, 256, 8, (8192, 8192), 3072, True), (6, 4096, 256, 8, (11008, 11008), 4096, False), (8, 4096, 0, 8, (8192, 8192), 3072, False),
+])
+def test_layers_over_tables_in_shared_memory_share_a_launch_up_to_a_size(binding, v, k1, k2, B, Ms, N, shared):
+    b = binding
+    path = b.vptq_linear_fused_path([b.make_desc(M, N, v, k1, k2) for M in Ms], B)
+    assert path == ("fused_gemm_tcgen05" if shared else "one_by_one")
