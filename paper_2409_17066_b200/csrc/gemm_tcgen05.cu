@@ -1207,6 +1207,7 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
 {
     GemmPlan p;
     memset(&p, 0, sizeof(p));
+    const int ctas = workers;
     // tables: small ones of a single group in shared memory, with copies where that costs little
     p.t1 = (V <= 8 && L.G == 1 && (long long)L.k1 * 16 <= 64 * 1024) ? TABLE_SHARED : TABLE_GLOBAL;
     p.t2 = L.k2 == 0 ? TABLE_NONE : (V <= 8 && L.G == 1 && L.k2 * 16 <= 16 * 1024) ? TABLE_SHARED : TABLE_GLOBAL;
@@ -1297,7 +1298,9 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     // 1074 MB of workspace instead of 173)
     p.slot_per_tile = (long long)tiles < workers;
     p.n_scratch = p.scratch ? (p.slot_per_tile ? (long long)tiles : workers - 1) * 4 * scratch_rows(p.tile_n) * 32 : 0;
-    p.off_scratch = take(p.n_scratch * 4);
+    // (as much for calls that are not cut: a workspace for a larger batch, whose tiles may be whole, serves a smaller one)
+    const long long slots = L.deterministic || p.tma_out ? 0 : (long long)tiles < ctas ? (long long)tiles : ctas - 1;
+    p.off_scratch = take(slots * 4 * scratch_rows(p.tile_n) * 32 * 4);
     p.off_xs = take((long long)p.tiles_t * images * b_bytes);
     return p;
 }

@@ -304,16 +304,14 @@ def test_copies_of_a_small_table_do_not_move_calls_to_other_kernels(binding, M, 
     assert b.lib.vptq_linear_has_status(C.byref(d), B) == status
 
 
-@pytest.mark.parametrize("M,N,B,v,whole", [
-    (10550, 878, 256, 8, True), (14463, 397, 32, 8, True), (13256, 2119, 512, 8, True),     # a whole tile for each of 83, 113 and 104 CTAs
-    (12797, 1500, 16, 8, False), (14798, 5343, 16, 8, False),                               # too long a share for that
-    (9400, 700, 64, 8, False),                                                              # 74 tiles: two CTAs each
-])
-def test_batched_tiles_are_not_cut_where_a_cta_each_will_do(binding, M, N, B, v, whole):
-    # nothing is cut: no scratch tiles, as with VPTQ_FLAG_DETERMINISTIC
+@pytest.mark.parametrize("M,N,v,k1,k2", [(12797, 1500, 8, 65536, 0), (14798, 2300, 8, 65536, 256), (9400, 700, 6, 4096, 256), (10550, 878, 8, 4096, 256),
+                                         (2048, 6600, 8, 256, 0), (16000, 1700, 12, 4096, 0), (64, 300, 6, 256, 0)])
+def test_a_workspace_for_a_batch_serves_smaller_ones(binding, M, N, v, k1, k2):
+    # also where a larger batch's tiles are whole and a smaller one's cut
     b = binding
-    need = [b.vptq_linear_workspace_bytes(b.make_desc(M, N, v, 65536, flags=b.FLAG_SCALE_BIAS | f), B) for f in (0, b.FLAG_DETERMINISTIC)]
-    assert (need[0] == need[1]) == whole
+    for out in ("fp16", "fp32"):
+        need = [b.vptq_linear_workspace_bytes(b.make_desc(M, N, v, k1, k2, out_dtype=out), B) for B in range(1, 513)]
+        assert need == sorted(need)
 
 
 @pytest.mark.parametrize("v,k1,k2,B,Ms,N,shared", [
