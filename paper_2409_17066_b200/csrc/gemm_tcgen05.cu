@@ -112,6 +112,13 @@ template <> struct Tile<12, false> {
 // eight stages; four epilogue warps.  v = 6, gate+up of 2 x 11008 x 4096 at 16 tokens 83 -> 73 us; v = 8, 1 MiB table, 8192 x 8192 at 16 48.4 -> 46.8,
 // at 64 52.8 / 52.6, 4096 x 4096 at 64 22.9 / 24.0 (an epilogue of four warps).  v = 12 reads two 32-byte rows a pair out of L2, whose rate bounds it.
 template <int V> constexpr int few_tokens() { return V == 8 ? 32 : V == 6 ? 64 : 0; }
+// v = 6: a CTA's share from which on it is the form to take: in shorter ones four epilogue warps hold the tile's end up.  The other form / it:
+// 1521 x 1024 at 48 tokens (128 columns) 12.4 / 15.1 us, 3341 x 1170 at 64 (230) 16.0 / 18.5, 1916 x 5650 at 48 (615) 20.5 / 21.8, 833 x 3843 at
+// 16 (184) 13.5 / 14.6, 4096 x 4096 at 64 (983) 22.3 / 23.5; but 7488 x 2844 at 64 (1198) 28.8 / 27.3, 7232 x 5760 at 64 (2400) 42.4 / 37.8, 3 layers'
+// 4500 rows x 3000 at 12 (809) 25.6 / 24.7, 5824 x 4980 at 12 (1652) 28.6 / 26.9.  Past 32 tokens not over eight copies of a small table, whose
+// reads have less to wait for: 256 centroids, 11008 x 4096 at 64 (2585) 35.9 / 37.9, at 32 34.0 / 33.4.  Indices of other widths than 8, 12 and 16 bits
+// are read one by one, which takes more producers at any share: 512 + 64 centroids, 2 x 3803 x 1664 at 32 tokens 29.0 / 24.2, 640 x 4014 at 21 15.7 / 14.7.
+inline int few_min_cols(int tile_n) { return 18 * tile_n > 768 ? 18 * tile_n : 768; }
 template <int V> constexpr int a_stage_bytes() { return 128 * Tile<V>::KS * 2; }
 // Warps by role: the loader, the MMA issuer, producers from WARP0 on, then the epilogue.
 // v = 6, 12: roles in whole warpgroups, between which registers move: 24 warps start with 80 registers a thread; the 12
@@ -1201,9 +1208,9 @@ struct GemmPlan {
     long long ws_bytes, off_flags, off_bpart, off_pad1, off_pad2, off_scratch, off_xs;
 };
 
-// `workers` CTAs at most, in a launch of n_layers layers
+// `workers` CTAs at most, in a launch of n_layers layers with `rows` vector rows
 template <int V>
-GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool concurrent)
+GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, long long rows, bool concurrent)
 {
     GemmPlan p;
     memset(&p, 0, sizeof(p));
@@ -1263,7 +1270,11 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     const int b_bytes = p.tile_n * 64;
     const int limit = p.t1 == TABLE_GLOBAL || p.t2 == TABLE_GLOBAL ? SMEM_LIMIT_L1 : SMEM_LIMIT;
     const bool copies = p.t2 == TABLE_SHARED && L.k2 <= 256;
-    p.few = p.tile_n <= few_tokens<V>() && !(V == 6 && p.t1 == TABLE_GLOBAL);
+    // (the layers of a launch take the same kernel, so by the share that a CTA has of all of them)
+    const long long share = (rows + Tile<V>::NV - 1) / Tile<V>::NV * p.tiles_t * p.kb_total * p.ks / device_sm_count();
+    auto quick = [](int bits) { return bits == 8 || bits == 12 || bits == 16; };
+    const bool long_enough = share >= few_min_cols(p.tile_n) && (p.tile_n <= 32 || p.cb1_shift < 3);
+    p.few = p.tile_n <= few_tokens<V>() && (V != 6 || (p.t1 == TABLE_SHARED && (long_enough || !quick(L.s1.bits) || (L.k2 > 0 && !quick(L.s2.bits)))));
     constexpr bool HAS_FEW = V != 12;
     const int a_stages = p.few ? Tile<V, HAS_FEW>::A_STAGES : Tile<V>::A_STAGES, epi = p.few ? Tile<V, HAS_FEW>::EPI : Tile<V>::EPI;
     p.cb2_shift = copies ? 3 : 0;
@@ -1305,11 +1316,11 @@ GemmPlan plan_gemm_v(const LayerView &L, int B, int workers, int n_layers, bool 
     return p;
 }
 
-GemmPlan plan_gemm(const LayerView &L, int B, int workers, int n_layers, bool concurrent)
+GemmPlan plan_gemm(const LayerView &L, int B, int workers, int n_layers, long long rows, bool concurrent)
 {
-    return L.v == 8   ? plan_gemm_v<8>(L, B, workers, n_layers, concurrent)
-           : L.v == 6 ? plan_gemm_v<6>(L, B, workers, n_layers, concurrent)
-                      : plan_gemm_v<12>(L, B, workers, n_layers, concurrent);
+    return L.v == 8   ? plan_gemm_v<8>(L, B, workers, n_layers, rows, concurrent)
+           : L.v == 6 ? plan_gemm_v<6>(L, B, workers, n_layers, rows, concurrent)
+                      : plan_gemm_v<12>(L, B, workers, n_layers, rows, concurrent);
 }
 
 // The plans of the layers of one launch (n = 1: a launch of its own): the SMs are dealt out to the layers in proportion to
@@ -1336,7 +1347,7 @@ long long plan_launch(const LayerView *Ls, int n, int B, GemmPlan *pl)
         ctas[most]++;
     }
     for (int l = 0; l < n; l++) {
-        pl[l] = plan_gemm(Ls[l], B, ctas[l], n, concurrent);
+        pl[l] = plan_gemm(Ls[l], B, ctas[l], n, total, concurrent);
         ws += pl[l].ws_bytes;
     }
     return ws;

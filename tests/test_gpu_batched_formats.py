@@ -100,8 +100,8 @@ FP32 = dict(out_dtype="fp32")
 
 
 @pytest.mark.parametrize("M,N,B,kw,pieces,in_order", [      # on 148 SMs
-    (71990, 130, 40, dict(v=6, k1=512), 5, False),                                # accumulators in turn, both phases of both sets: v = 6, few tokens
-    (71996, 130, 40, dict(v=6, k1=512, **FP32), 5, True),
+    (71990, 200, 40, dict(v=6, k1=512), 5, False),                                # accumulators in turn, both phases of both sets: v = 6, few tokens
+    (71996, 200, 40, dict(v=6, k1=512, **FP32), 5, True),
     (71990, 130, 200, dict(v=6, k1=512, out_dtype="bf16"), 5, False),             # ... the other form
     (71996, 130, 200, dict(v=6, k1=512, **FP32), 5, True),
     (71990, 130, 200, dict(v=12, k1=512), 5, False),
